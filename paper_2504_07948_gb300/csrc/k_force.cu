@@ -19,104 +19,212 @@
 // is O(n^2 n_basis + n^3 + N n_basis) per walker, independent of N_atom.
 // Basis derivatives to third order are recomputed per walker rather than
 // stored.  The e-n Jastrow, V_en and V_nn terms are added directly.
+#include <type_traits>
+
 #include "batch.cuh"
+#include "fixed64.cuh"
 #include "qmc_internal.cuh"
 
 namespace qmc {
 
 constexpr int kForceTile = 32;  // basis functions per tile of M and Y
 
-// First derivatives d_q Phi, derivatives of the Laplacian d_q lap Phi and
-// the Hessian applied to a vector, (Hess Phi . g)_q, of one function of a
-// shell at offset x (f0..f3: the radial sums at t = |x|^2).  With
-// Phi = P S, S_k = d_k S = 2 x_k f1, S_kq = 4 x_k x_q f2 + 2 delta_kq f1:
-//   d_q Phi        = P S_q + P_q S,
-//   d_q lap Phi    = P_q lap S + P d_q lap S + 2 sum_k (P_kq S_k + P_k S_kq) + S_q lap P,
-//   (Hess Phi g)_q = P sum_k S_kq g_k + S_q (grad P . g) + P_q (grad S . g) + S (Hess P g)_q,
-// with sum_k S_kq g_k = 4 x_q f2 (x . g) + 2 f1 g_q: the Hessian is never
-// formed, only its product with g (the adjoint needs nothing else).
-template <typename F>
-struct Deriv3 {
-    F d1[3];   // d/dq Phi
-    F hg[3];   // (Hess Phi . g)_q
-    F dl[3];   // d/dq lap Phi
+// Adjoint terms of one shell at one electron.  Let x be the offset from the
+// centre, t = |x|^2, f0..f3 the radial sums and g = grad_i J.  With M, Y the
+// basis-space weights of the shell's functions Phi_m = P_m S, the sums over m
+//   v_q = sum_m M_m (1/2 d_q lap Phi_m + (Hess Phi_m g)_q) + Y_m d_q Phi_m,
+//   w_q = sum_m M_m d_q Phi_m
+// are linear in the polynomials, so they are taken once for the combined
+// polynomial sum_m M_m P_m (value U, gradient G, Hessian H; UY, GY those of
+// sum_m Y_m P_m) instead of once per function.  P_m is homogeneous of degree
+// l, so G.x = l U and H x = (l - 1) G, and
+//   v_q = x_q [U ((10 + 4 l) f2 + 4 t f3 + 4 f2 (x.g)) + 2 f1 (G.g + UY) + f1 tr H]
+//       + g_q [2 f1 U] + G_q [(3 + 2 l) f1 + 2 t f2 + 2 f1 (x.g)] + f0 ((H g)_q + GY_q),
+//   w_q = x_q [2 f1 U] + G_q f0.
+// The coefficients of x_q and g_q are scalars that add over all shells of a
+// centre; only the G, H g terms stay vectors.  (One evaluation per function
+// instead took 135 FP64 instructions per p shell and 300 per d shell, against
+// 28 and 65 here.)
+template <typename T>
+struct RunTerms {
+    T ax = T(0), ag = T(0);                  // coefficients of x_q and g_q in v; ag is also that of x_q in w
+    T v[3] = {T(0), T(0), T(0)}, w[3] = {T(0), T(0), T(0)};
 };
 
-__device__ __forceinline__ int hidx(int a, int b) {
-    // symmetric index into (xx, xy, xz, yy, yz, zz)
-    const int lo = a < b ? a : b, hi = a < b ? b : a;
-    return lo == 0 ? hi : (lo == 1 ? 2 + hi : 5);
-}
-
-template <typename F>
-__device__ __forceinline__ void shell_d3(int l, int pure, const F x[3], const F g[3], int fi, F f0, F f1, F f2,
-                                         F f3, Deriv3<F>& out) {
-    const F t = x[0] * x[0] + x[1] * x[1] + x[2] * x[2];
-    const AngPoly<F> a = angular<F>(l, pure, fi, x[0], x[1], x[2]);
-    const F Pk[3] = {a.Px, a.Py, a.Pz};
-    const F HP[6] = {a.Hxx, a.Hxy, a.Hxz, a.Hyy, a.Hyz, a.Hzz};
-    const F LP = a.Hxx + a.Hyy + a.Hzz;
-    F Sk[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) Sk[k] = F(2) * x[k] * f1;
-    const F LS = F(6) * f1 + F(4) * t * f2;
-    const F Px = Pk[0] * x[0] + Pk[1] * x[1] + Pk[2] * x[2];
-    const F Pg = Pk[0] * g[0] + Pk[1] * g[1] + Pk[2] * g[2];
-    const F xg = x[0] * g[0] + x[1] * g[1] + x[2] * g[2];
-    const F c3 = F(20) * f2 + F(8) * t * f3;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        const F HSk = HP[hidx(0, q)] * Sk[0] + HP[hidx(1, q)] * Sk[1] + HP[hidx(2, q)] * Sk[2];
-        const F Hg = HP[hidx(0, q)] * g[0] + HP[hidx(1, q)] * g[1] + HP[hidx(2, q)] * g[2];
-        out.d1[q] = a.P * Sk[q] + Pk[q] * f0;
-        // sum_k (P_kq S_k + P_k S_kq) = (Hess P S)_q + 4 x_q f2 (grad P . x) + 2 f1 P_q
-        const F acc = HSk + F(4) * x[q] * f2 * Px + F(2) * f1 * Pk[q];
-        out.dl[q] = Pk[q] * LS + a.P * x[q] * c3 + F(2) * acc + Sk[q] * LP;
-        out.hg[q] = a.P * (F(4) * x[q] * f2 * xg + F(2) * f1 * g[q]) + Sk[q] * Pg + Pk[q] * (F(2) * f1 * xg) +
-                    f0 * Hg;
-    }
-}
-
-// Adjoint terms of the functions of one shell at one electron: with M, Y
-// the basis-space weights of the function rows (m = Mrow[fi * ld], y =
-// Yrow[fi * ld]) and gj = grad_i J,
-//   vt[q]     += -m (-1/2 d_q lap Phi - gj . d_q grad Phi) + y d_q Phi,
-//   vt[3 + q] +=  m d_q Phi
-// (derivatives with respect to the electron coordinate; the callers turn
-// them into nuclear ones).  L = 0 or 1 fixes the angular momentum at compile
-// time, so the constant angular factors of s and p shells fold away (on
-// GB300 every FP64 instruction counts); L = -1 takes l, pure, nf at run time.
-template <typename T, int L>
-__device__ __forceinline__ void shell_terms(int l, int pure, int nf, const T x[3], T f0, T f1, T f2, T f3,
-                                            const T gj[3], const T* Mrow, const T* Yrow, int ld, T (&vt)[6]) {
-    auto body = [&](int fi) {
-        Deriv3<T> D;
-        shell_d3<T>(L >= 0 ? L : l, pure, x, gj, fi, f0, f1, f2, f3, D);
-        const T m = Mrow[(size_t)fi * ld], y = Yrow[(size_t)fi * ld];
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            vt[q] += -m * (T(-0.5) * D.dl[q] - D.hg[q]) + y * D.d1[q];
-            vt[3 + q] += m * D.d1[q];
-        }
-    };
-    if constexpr (L >= 0) {
-#pragma unroll
-        for (int fi = 0; fi < (L == 0 ? 1 : 3); ++fi) body(fi);
-    } else {
-        for (int fi = 0; fi < nf; ++fi) body(fi);
-    }
-}
-
 template <typename T>
-__device__ __forceinline__ void shell_terms_any(int l, int pure, int nf, const T x[3], T f0, T f1, T f2, T f3,
-                                                const T gj[3], const T* Mrow, const T* Yrow, int ld, T (&vt)[6]) {
-    if (l == 0)
-        shell_terms<T, 0>(l, pure, nf, x, f0, f1, f2, f3, gj, Mrow, Yrow, ld, vt);
-    else if (l == 1)
-        shell_terms<T, 1>(l, pure, nf, x, f0, f1, f2, f3, gj, Mrow, Yrow, ld, vt);
-    else
-        shell_terms<T, -1>(l, pure, nf, x, f0, f1, f2, f3, gj, Mrow, Yrow, ld, vt);
+__device__ __forceinline__ void shell_terms(int l, int pure, const T x[3], const T g[3], T xg, T t, T f0, T f1, T f2,
+                                            T f3, const T* M, const T* Y, size_t ld, RunTerms<T>& o) {
+    const T f12 = T(2) * f1;
+    if (l == 0) {
+        const T m = M[0];
+        o.ax += m * (f2 * (T(10) + T(4) * xg) + T(4) * t * f3) + f12 * Y[0];
+        o.ag += f12 * m;
+        return;
+    }
+    if (l == 1) {
+        const T m[3] = {M[0], M[ld], M[2 * ld]}, y[3] = {Y[0], Y[ld], Y[2 * ld]};
+        const T U = m[0] * x[0] + m[1] * x[1] + m[2] * x[2];
+        const T q = m[0] * g[0] + m[1] * g[1] + m[2] * g[2] + y[0] * x[0] + y[1] * x[1] + y[2] * x[2];
+        o.ax += U * (f2 * (T(14) + T(4) * xg) + T(4) * t * f3) + f12 * q;
+        o.ag += f12 * U;
+        const T cG = f1 * (T(5) + T(2) * xg) + T(2) * t * f2;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            o.v[c] += m[c] * cG + f0 * y[c];
+            o.w[c] += m[c] * f0;
+        }
+        return;
+    }
+    // d: Hessians (xx, xy, xz, yy, yz, zz) of the combined polynomials
+    const T s3 = T(1.7320508075688772);
+    T H[6], K[6], tr = T(0);
+    if (pure) {
+        const T a2 = M[2 * ld], a4 = s3 * M[4 * ld], b2 = Y[2 * ld], b4 = s3 * Y[4 * ld];
+        H[0] = a4 - a2; H[1] = s3 * M[0]; H[2] = s3 * M[3 * ld]; H[3] = -a2 - a4; H[4] = s3 * M[ld]; H[5] = T(2) * a2;
+        K[0] = b4 - b2; K[1] = s3 * Y[0]; K[2] = s3 * Y[3 * ld]; K[3] = -b2 - b4; K[4] = s3 * Y[ld]; K[5] = T(2) * b2;
+    } else {
+        H[0] = T(2) * M[0]; H[1] = s3 * M[ld]; H[2] = s3 * M[2 * ld];
+        H[3] = T(2) * M[3 * ld]; H[4] = s3 * M[4 * ld]; H[5] = T(2) * M[5 * ld];
+        K[0] = T(2) * Y[0]; K[1] = s3 * Y[ld]; K[2] = s3 * Y[2 * ld];
+        K[3] = T(2) * Y[3 * ld]; K[4] = s3 * Y[4 * ld]; K[5] = T(2) * Y[5 * ld];
+        tr = H[0] + H[3] + H[5];
+    }
+    const T G[3] = {H[0] * x[0] + H[1] * x[1] + H[2] * x[2], H[1] * x[0] + H[3] * x[1] + H[4] * x[2],
+                    H[2] * x[0] + H[4] * x[1] + H[5] * x[2]};
+    const T R[3] = {K[0] * x[0] + K[1] * x[1] + K[2] * x[2], K[1] * x[0] + K[3] * x[1] + K[4] * x[2],
+                    K[2] * x[0] + K[4] * x[1] + K[5] * x[2]};
+    const T Hg[3] = {H[0] * g[0] + H[1] * g[1] + H[2] * g[2], H[1] * g[0] + H[3] * g[1] + H[4] * g[2],
+                     H[2] * g[0] + H[4] * g[1] + H[5] * g[2]};
+    const T U = T(0.5) * (G[0] * x[0] + G[1] * x[1] + G[2] * x[2]);
+    const T UY = T(0.5) * (R[0] * x[0] + R[1] * x[1] + R[2] * x[2]);
+    const T Gg = G[0] * g[0] + G[1] * g[1] + G[2] * g[2];
+    o.ax += U * (f2 * (T(18) + T(4) * xg) + T(4) * t * f3) + f12 * (Gg + UY) + f1 * tr;
+    o.ag += f12 * U;
+    const T cG = f1 * (T(7) + T(2) * xg) + T(2) * t * f2;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        o.v[c] += G[c] * cG + f0 * (Hg[c] + R[c]);
+        o.w[c] += G[c] * f0;
+    }
 }
+
+// Radial sums of one shell for the 32 electrons of a warp, FP64: about a
+// third of the (primitive, electron) pairs are unscreened, so the live pairs
+// of up to kRadialPrims primitives are listed and each exponential is taken
+// once on consecutive lanes, instead of one masked exponential per primitive
+// and warp.  The screening test runs in FP32 (a pair near the threshold is
+// below 1e-26 either way).  Called by whole warps; `on` marks the lanes that
+// hold an electron.  scr: kRadialScratch bytes of the warp's shared memory.
+constexpr int kRadialPrims = 4;
+constexpr int kRadialScratch = kRadialPrims * 32 * (int)(sizeof(double) + sizeof(short));
+__device__ __forceinline__ void warp_radial3(const DevSys& s, int p0, int np, double t, bool on, void* scr, double& f0,
+                                             double& f1, double& f2, double& f3) {
+    double* ev = (double*)scr;
+    short* lst = (short*)(ev + kRadialPrims * 32);
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    const float tf = on ? (float)t : 3.0e38f;
+    f0 = f1 = f2 = f3 = 0.0;
+    for (int q0 = 0; q0 < np; q0 += kRadialPrims) {
+        const int nq = min(kRadialPrims, np - q0);
+        int cnt = 0;
+        unsigned mine = 0;
+        for (int q = 0; q < nq; ++q) {
+            const bool live = on && !(s.alpha_f[p0 + q0 + q] * tf > (float)kScreenExponent);
+            const unsigned m = __ballot_sync(0xffffffffu, live);
+            if (live) {
+                lst[cnt + __popc(m & below)] = (short)(q * 32 + lane);
+                mine |= 1u << q;
+            }
+            cnt += __popc(m);
+        }
+        if (cnt == 0) continue;
+        __syncwarp();
+        for (int k = 0; k < cnt; k += 32) {
+            const int e = k + lane < cnt ? lst[k + lane] : 0;
+            const double te = __shfl_sync(0xffffffffu, t, e & 31);
+            if (k + lane < cnt) {
+                const int p = p0 + q0 + (e >> 5);
+                ev[e] = s.cn[p] * exp(-s.alpha[p] * te);
+            }
+        }
+        __syncwarp();
+        for (int q = 0; q < nq; ++q)
+            if (mine & (1u << q)) {
+                const double a = s.alpha[p0 + q0 + q], e = ev[q * 32 + lane];
+                const double e1 = a * e, e2 = a * e1;
+                f0 += e;
+                f1 -= e1;
+                f2 += e2;
+                f3 -= a * e2;
+            }
+        __syncwarp();
+    }
+}
+
+// Sum over a warp of 8 values per lane by a transposing butterfly: 9 adds
+// per lane instead of 40; v[0] of the lanes with (lane & 3) == 0 becomes the
+// total of value fold8_index(lane).
+__device__ __forceinline__ int fold8_index(int lane) {
+    return ((lane >> 2) & 1) | (((lane >> 3) & 1) << 1) | (((lane >> 4) & 1) << 2);
+}
+template <typename A>
+__device__ __forceinline__ A warp_fold8(const A (&v)[8]) {
+    const int lane = threadIdx.x & 31;
+    A a[4];
+    const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) a[i] = (h4 ? v[i + 4] : v[i]) + __shfl_xor_sync(0xffffffffu, h4 ? v[i] : v[i + 4], 16);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) a[i] = (h3 ? a[i + 2] : a[i]) + __shfl_xor_sync(0xffffffffu, h3 ? a[i] : a[i + 2], 8);
+    A r = (h2 ? a[1] : a[0]) + __shfl_xor_sync(0xffffffffu, h2 ? a[0] : a[1], 4);
+    r += __shfl_xor_sync(0xffffffffu, r, 2);
+    r += __shfl_xor_sync(0xffffffffu, r, 1);
+    return r;
+}
+
+// Terms of the shells [sh0, sh1) of one centre at one electron per lane (the
+// whole warp calls; `on`: the lane holds an electron): derivatives v, w with
+// respect to the electron coordinate (see RunTerms).  M, Y: weights of the
+// functions from shell sh0 on, row stride ld.
+template <typename T>
+__device__ __forceinline__ void run_terms(const DevSys& s, int sh0, int sh1, bool on, const T x[3], const T g[3],
+                                          const T* M, const T* Y, size_t ld, void* scr, T (&v)[8]) {
+    const T t = x[0] * x[0] + x[1] * x[1] + x[2] * x[2];
+    const T xg = x[0] * g[0] + x[1] * g[1] + x[2] * g[2];
+    const int fn0 = s.shell_fn[sh0];
+    RunTerms<T> o;
+    for (int sh = sh0; sh < sh1; ++sh) {
+        const int4 d = s.shell[sh];
+        T f0 = T(0), f1 = T(0), f2 = T(0), f3 = T(0);
+        if constexpr (sizeof(T) == 8) {
+            warp_radial3(s, d.z, d.w, t, on, scr, f0, f1, f2, f3);
+        } else {
+            if (on) radial<T, true>(s.alpha_f, s.cn_f, d.z, d.w, t, f0, f1, f2, f3);
+        }
+        if (f0 == T(0) && f1 == T(0) && f2 == T(0) && f3 == T(0)) continue;   // screened (or no electron)
+        const size_t row = (size_t)(s.shell_fn[sh] - fn0) * ld;
+        shell_terms<T>(d.y & 0xff, d.y >> 8, x, g, xg, t, f0, f1, f2, f3, M + row, Y + row, ld, o);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        v[c] = o.ax * x[c] + o.ag * g[c] + o.v[c];
+        v[3 + c] = o.ag * x[c] + o.w[c];
+    }
+    v[6] = v[7] = T(0);
+}
+
+// Reciprocal of a value known to be finite and at least 1: the FP64 form
+// refines the hardware's 20-bit approximation y by 1/x = y (1 + e + e^2 +
+// ...), e = 1 - x y, to the last bit or two (3 FP64 instructions instead of a
+// division's 7).
+__device__ __forceinline__ double rcp_ge1(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ float rcp_ge1(float x) { return 1.0f / x; }
 
 // Shared-memory head of every force kernel: positions (FP64), the per-atom
 // sums acc[nn][6] (FP64: dT (3), dlnpsi (3)), grad_i J and grad_i ln|psi|
@@ -191,7 +299,7 @@ __device__ __forceinline__ void force_gradients_en(const DevSys& s, const DevWal
         const int k = spin ? i - nu : i;
         const T* Ai = (const T*)wk.Ainv[spin] + ((size_t)w * n + k) * n;
         const T* Gi = (const T*)wk.G[spin] + ((size_t)w * n + k) * 4 * n;
-        T v[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};   // grad ln|D| (3), grad J (3)
+        T v[8] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};   // grad ln|D| (3), grad J (3)
         for (int j = lane; j < n; j += 32) {
             const T a = Ai[j];
             v[0] += Gi[j] * a;
@@ -215,18 +323,16 @@ __device__ __forceinline__ void force_gradients_en(const DevSys& s, const DevWal
             }
             const T r2 = x[0] * x[0] + x[1] * x[1] + x[2] * x[2];
             const T ir = rsqrt_t(r2);
-            const T qd = T(1) / (T(1) + b * r2 * ir);
+            const T qd = rcp_ge1(T(1) + b * r2 * ir);
             const T gr = a * qd * qd * ir;  // u'(r) / r
 #pragma unroll
             for (int c = 0; c < 3; ++c) v[3 + c] += gr * x[c];
         }
 #pragma unroll
-        for (int q = 0; q < 6; ++q) v[q] = warp_sum(v[q]);
-        if (lane == 0)
-            for (int c = 0; c < 3; ++c) {
-                h.gJ[3 * i + c] = v[3 + c];
-                h.gt[3 * i + c] = v[3 + c] + v[c];
-            }
+        for (int c = 0; c < 3; ++c) v[c] += v[3 + c];
+        const T sum = warp_fold8(v);
+        const int q = fold8_index(lane);
+        if ((lane & 3) == 0 && q < 6) (q < 3 ? h.gt + q : h.gJ + (q - 3))[3 * i] = sum;
     }
     __syncthreads();
 
@@ -261,48 +367,168 @@ __device__ __forceinline__ void force_gradients_en(const DevSys& s, const DevWal
                 dJ[q] -= du * x[q] * ir;
             }
         }
-        double v[6];
-        for (int q = 0; q < 3; ++q) {
-            v[q] = warp_sum(double(dT[q]));
-            v[3 + q] = warp_sum(double(dJ[q]));
-        }
-        if (lane == 0)
-            for (int q = 0; q < 3; ++q) {
-                h.acc[6 * a + q] = v[q] + dvnn[3 * a + q];
-                h.acc[6 * a + 3 + q] = v[3 + q];
-            }
+        const double v[8] = {double(dT[0]), double(dT[1]), double(dT[2]), double(dJ[0]),
+                             double(dJ[1]), double(dJ[2]), 0.0, 0.0};
+        const double sum = warp_fold8(v);
+        const int q = fold8_index(lane);
+        if ((lane & 3) == 0 && q < 6) h.acc[6 * a + q] = sum + (q < 3 ? dvnn[3 * a + q] : 0.0);
     }
     __syncthreads();
 }
 
-// The transposed inverse and P^T = (B A^-1)^T of a spin are read n times
-// each by the tile products of force_walker; when both fit beside the tiles
-// (at most 100 KB in all, two CTAs per SM) they are staged in shared memory
-// with row stride n + 1 (conflict-free column walks).
-template <typename T>
-__host__ __device__ inline bool force_stage_fits(int N, int nn, int nmax) {
-    const size_t base = force_head_bytes<T>(N, nn) + sizeof(T) * 2 * (size_t)kForceTile * nmax;
-    const size_t extra = sizeof(T) * 2 * (size_t)nmax * (nmax + 1);
-    return base + extra <= 100 * 1024;
+// Rows of dot products of one warp: out(r, i) = sum_k A_r[k] B_i[k] for nl
+// rows r of the left factor (row stride lda) and all n electrons i (row
+// stride ldb).  Lanes take (group of kForceRows rows, electron) items, so one
+// load of B serves kForceRows rows and the rows of A are (nearly) broadcast.
+constexpr int kForceRows = 4;
+
+// FP64 form: operands as limbs (fixed64.cuh); put receives the sum in units
+// of the two rows' scales.
+template <typename Put>
+__device__ __forceinline__ void warp_rows(int nl, int n, const int2* A, int lda, const int2* B, int ldb, Put put) {
+    const int lane = threadIdx.x & 31, items = (nl + kForceRows - 1) / kForceRows * n;
+    for (int o = lane; o < items; o += 32) {
+        const int g = o / n, i = o - g * n, r0 = g * kForceRows, nr = min(kForceRows, nl - r0);
+        const int2* b = B + (size_t)i * ldb;
+        const int2* a[kForceRows];
+#pragma unroll
+        for (int r = 0; r < kForceRows; ++r) a[r] = A + (size_t)(r0 + min(r, nr - 1)) * lda;
+        FxSum sum[kForceRows];
+        for (int k0 = 0; k0 < n; k0 += kFxBlock) {
+            FxDot d[kForceRows];
+            const int k1 = min(n, k0 + kFxBlock);
+#pragma unroll 2
+            for (int k = k0; k < k1; ++k) {
+                const int2 bv = b[k];
+#pragma unroll
+                for (int r = 0; r < kForceRows; ++r) d[r].add(a[r][k], bv);
+            }
+#pragma unroll
+            for (int r = 0; r < kForceRows; ++r) sum[r].fold(d[r]);
+        }
+#pragma unroll
+        for (int r = 0; r < kForceRows; ++r)
+            if (r < nr) put(r0 + r, i, sum[r].value());
+    }
+}
+template <typename Put>
+__device__ __forceinline__ void warp_rows(int nl, int n, const float* A, int lda, const float* B, int ldb, Put put) {
+    const int lane = threadIdx.x & 31, items = (nl + kForceRows - 1) / kForceRows * n;
+    const bool even = ((n | lda) & 1) == 0 && ((uintptr_t)A & 7) == 0;   // the rows of A can be read in pairs
+    for (int o = lane; o < items; o += 32) {
+        const int g = o / n, i = o - g * n, r0 = g * kForceRows, nr = min(kForceRows, nl - r0);
+        const float* b = B + (size_t)i * ldb;
+        const float* a[kForceRows];
+        float v[kForceRows];
+#pragma unroll
+        for (int r = 0; r < kForceRows; ++r) {
+            a[r] = A + (size_t)(r0 + min(r, nr - 1)) * lda;
+            v[r] = 0.f;
+        }
+        if (even) {
+#pragma unroll 2
+            for (int k = 0; k < n; k += 2) {
+                const float b0 = b[k], b1 = b[k + 1];
+#pragma unroll
+                for (int r = 0; r < kForceRows; ++r) {
+                    const float2 av = *reinterpret_cast<const float2*>(a[r] + k);
+                    v[r] += av.x * b0;
+                    v[r] += av.y * b1;
+                }
+            }
+        } else {
+#pragma unroll 2
+            for (int k = 0; k < n; ++k) {
+                const float bv = b[k];
+#pragma unroll
+                for (int r = 0; r < kForceRows; ++r) v[r] += a[r][k] * bv;
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < kForceRows; ++r)
+            if (r < nr) put(r0 + r, i, v[r]);
+    }
 }
 
-template <typename T>
-__host__ __device__ inline size_t force_smem(int N, int nn, int nmax) {
-    const size_t base = force_head_bytes<T>(N, nn) + sizeof(T) * 2 * (size_t)kForceTile * nmax;
-    return base + (force_stage_fits<T>(N, nn, nmax) ? sizeof(T) * 2 * (size_t)nmax * (nmax + 1) : 0);
+// Limbs of n doubles x by one warp into q (x and q may be the same memory:
+// each lane rewrites what it read); returns the row's scale.
+__device__ __forceinline__ double warp_limbs(const double* x, int2* q, int n) {
+    const int lane = threadIdx.x & 31;
+    int e = 0;
+    for (int k = lane; k < n; k += 32) e = max(e, fx_expo(x[k]));
+    e = warp_max_u(e);
+    for (int k = lane; k < n; k += 32) q[k] = fx_limbs(x[k], e);
+    return fx_scale(e);
 }
 
-// Per-electron accumulators of the space-warp form (kE): 3N doubles placed
-// after the force kernel's own shared memory.
-template <typename T>
-__host__ __device__ inline size_t force_smem_e(int N, int nn, int nmax, bool kE) {
-    const size_t b = (force_smem<T>(N, nn, nmax) + 15) & ~(size_t)15;
-    return kE ? b + sizeof(double) * 3 * (size_t)N : force_smem<T>(N, nn, nmax);
+// Groups of kForceRows rows that a warp of force_walker forms together: as
+// many (at most 3, and within the warp's scratch) as fill its lanes best.
+__host__ __device__ inline int force_row_groups(int n) {
+    int best = 1;
+    for (int g = 2; g <= 3; ++g) {
+        if (g * kForceRows * n * 8 > 2560) break;
+        const int used = n * g, lanes = (used + 31) / 32, ub = n * best, lb = (ub + 31) / 32;
+        if (used * lb > ub * lanes) best = g;
+    }
+    return best;
 }
+
+// Shared memory of force_walker.  The transposed inverse and P^T =
+// (B A^-1)^T of a spin are read once per basis function by the products
+// M = C A^-T and Y = M P, so they are staged with an odd row stride ld: as
+// limbs with their row scales in the FP64 form, as floats in the mixed form;
+// a determinant too large for that (stg false) reads A^-T and keeps B and
+// P^T in global memory.  M and Y are formed for F basis functions at a time:
+// all of them where the budget allows (2 CTAs per SM in FP64, 3 mixed), so
+// that the contraction keeps a warp per centre busy.
+// Bound by FP64 issue (FP64 form) and by instruction issue (mixed).  6-water
+// cluster, 2048 walkers: 8.10 -> 3.38 ms FP64 and 0.81 -> 0.45 ms mixed
+// against one derivative evaluation per basis function, FP64 products and a
+// masked exponential per primitive.
+template <typename T>
+struct ForceShape {
+    bool stg;
+    int ld, F, scr;                                      // scr: bytes of scratch per warp
+    size_t AT, PT, sA, scratch, M, Y, gE, total;         // byte offsets
+    __host__ __device__ ForceShape(int N, int nn, int nmax, int nb, bool kE) {
+        const size_t head = (force_head_bytes<T>(N, nn) + 15) & ~(size_t)15;
+        const size_t e_bytes = kE ? sizeof(double) * 3 * (size_t)N : 0;
+        ld = nmax | 1;
+        scr = 0;
+        if (sizeof(T) == 8) {
+            scr = 3 * kForceRows * nmax * 8;
+            if (scr > 2560) scr = 2560 > kForceRows * nmax * 8 ? 2560 : kForceRows * nmax * 8;
+            if (scr < kRadialScratch) scr = kRadialScratch;
+            scr = (scr + 15) & ~15;
+        }
+        const size_t mat = (sizeof(T) * (size_t)nmax * ld + 15) & ~(size_t)15;
+        const size_t row = 2 * sizeof(T) * (size_t)nmax;
+        // the tile also holds B (with its row scales) while P^T is formed
+        int fmin = kForceTile > (ld + 2) / 2 ? kForceTile : (ld + 2) / 2;
+        const size_t fixed = head + 2 * mat + 2 * sizeof(T) * (size_t)nmax + 16 + 8 * (size_t)scr + e_bytes;
+        stg = fixed + row * fmin <= 200 * 1024;
+        if (!stg) fmin = kForceTile;
+        AT = head;
+        PT = AT + (stg ? mat : 0);
+        sA = PT + (stg ? mat : 0);
+        scratch = (sA + (stg ? 2 * sizeof(T) * (size_t)nmax : 0) + 15) & ~(size_t)15;
+        M = scratch + 8 * (size_t)scr;
+        const size_t budget = (sizeof(T) == 8 ? 112 : 74) * 1024;
+        F = fmin;
+        if (stg && budget > M + e_bytes + row * fmin) {
+            const size_t fit = (budget - M - e_bytes) / row;
+            F = fit < (size_t)nb ? (int)fit : nb;
+            if (F < fmin) F = fmin;
+        }
+        Y = M + sizeof(T) * (size_t)F * nmax;
+        gE = (Y + sizeof(T) * (size_t)F * nmax + 15) & ~(size_t)15;
+        total = gE + e_bytes;
+    }
+};
 
 // Adjoint ionic derivatives of walker w (body of k_force).  sm: the
-// dynamic shared memory of launch_force (force_smem_e).  kE: also the
-// determinant part of dE_L/dr_i (the same basis-space terms, every basis
+// dynamic shared memory of launch_force (ForceShape), 256 threads.  kE: also
+// the determinant part of dE_L/dr_i (the same basis-space terms, every basis
 // function moving with the electron, d/dr_i = -d/dR) into gEdet [W][N][3]
 // and grad_i ln|psi| into gtot [W][N][3], for the space warp.
 template <typename T, bool kE = false>
@@ -311,117 +537,176 @@ __device__ __forceinline__ void force_walker(const DevSys& s, const DevWalkers& 
                                              double* gEdet = nullptr, double* gtot = nullptr) {
     const int N = s.N, nu = s.n_up, nn = s.n_nuc;
     const int nmax = nu > s.n_dn ? nu : s.n_dn;
+    constexpr bool kFx = sizeof(T) == 8;
+    using Q = std::conditional_t<kFx, int2, float>;   // staged operands
+    const ForceShape<T> fs(N, nn, nmax, s.n_basis, kE);
+    unsigned char* smb = (unsigned char*)sm;
     const ForceHead<T> h(sm, N, nn);
     double* acc = h.acc;
-    T* Mt = h.end(N);                  // [kForceTile][nmax]
-    T* Yt = Mt + kForceTile * nmax;
+    Q* sAT = (Q*)(smb + fs.AT);
+    Q* sPT = (Q*)(smb + fs.PT);
+    T* sA = (T*)(smb + fs.sA);         // row scales of A^-T and P^T (FP64 form)
+    T* sP = sA + nmax;
+    T* Mt = (T*)(smb + fs.M);          // [F][nmax]
+    T* Yt = (T*)(smb + fs.Y);
+    Q* sB = (Q*)Mt;                    // B while P^T is formed, [n][ld]
+    T* sBs = (T*)(sB + (size_t)nmax * fs.ld);
     T* B = (T*)(Bscr + (size_t)w * nmax * nmax);
     T* PTg = (T*)(Pscr + (size_t)w * nmax * nmax);
-    const bool stg = force_stage_fits<T>(N, nn, nmax);
-    T* sAT = Yt + kForceTile * nmax;
-    T* sPT = sAT + nmax * (nmax + 1);
-    double* gEs = (double*)((unsigned char*)sm + ((force_smem<T>(N, nn, nmax) + 15) & ~(size_t)15));
+    double* gEs = (double*)(smb + fs.gE);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    Q* scr = (Q*)(smb + fs.scratch + (size_t)wid * fs.scr);
 
     force_load_positions(h, wk.R + (size_t)w * 3 * N, N);
     if constexpr (kE)
         for (int q = threadIdx.x; q < 3 * N; q += blockDim.x) gEs[q] = 0.0;
     __syncthreads();
     force_gradients_en<T>(s, wk, w, dvnn, h);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
 
     for (int spin = 0; spin < 2; ++spin) {
         const int n = spin ? s.n_dn : nu;
         if (n == 0) continue;
-        const int i0 = spin ? nu : 0;
+        const int i0 = spin ? nu : 0, ld = fs.ld;
         const T* ATg = (const T*)wk.Ainv[spin] + (size_t)w * n * n;
         const T* Gs = (const T*)wk.G[spin] + (size_t)w * 4 * n * n;
+        const T* nlB = wk.nlB[spin] ? (const T*)wk.nlB[spin] + (size_t)w * n * n : nullptr;
         const T* C = sys_C<T>(s, spin);
-        const int ld = stg ? n + 1 : n;   // row stride of AT and PT as read below
-        const T* AT = stg ? sAT : ATg;
-        T* PT = stg ? sPT : PTg;
-        if (stg)
-            for (int q2 = threadIdx.x; q2 < n * n; q2 += blockDim.x) sAT[(q2 / n) * ld + q2 % n] = ATg[q2];
-        // B_pq = -1/2 lap phi_q(r_p) - grad_p J . grad phi_q(r_p)
-        for (int q2 = threadIdx.x; q2 < n * n; q2 += blockDim.x) {
-            const int pp = q2 / n, qq = q2 - pp * n;
+        // B_pq = -1/2 lap phi_q(r_p) - grad_p J . grad phi_q(r_p), plus the
+        // non-local pseudopotential's rows (E_L gains tr(B_NL A^-1), so the
+        // same -tr(X dA) pull-back covers them)
+        auto b_of = [&](int pp, int qq) {
             const T* Gp = Gs + (size_t)pp * 4 * n;
             const T* gj = h.gJ + 3 * (i0 + pp);
-            B[q2] = T(-0.5) * Gp[3 * n + qq] - gj[0] * Gp[qq] - gj[1] * Gp[n + qq] - gj[2] * Gp[2 * n + qq];
-            // non-local pseudopotential rows: E_L gains tr(B_NL A^-1), so the
-            // same -tr(X dA) pull-back covers them
-            if (wk.nlB[spin]) B[q2] += ((const T*)wk.nlB[spin])[(size_t)w * n * n + q2];
+            T b = T(-0.5) * Gp[3 * n + qq] - gj[0] * Gp[qq] - gj[1] * Gp[n + qq] - gj[2] * Gp[2 * n + qq];
+            if (nlB) b += nlB[(size_t)pp * n + qq];
+            return b;
+        };
+        if (fs.stg) {
+            for (int r = wid; r < n; r += nw) {
+                T* at = (T*)(sAT + (size_t)r * ld);
+                T* bt = (T*)(sB + (size_t)r * ld);
+                for (int q = lane; q < n; q += 32) {
+                    at[q] = ATg[(size_t)r * n + q];
+                    bt[q] = b_of(r, q);
+                }
+                if constexpr (kFx) {
+                    const double a = warp_limbs(at, (int2*)at, n), b = warp_limbs(bt, (int2*)bt, n);
+                    if (lane == 0) {
+                        sA[r] = a;
+                        sBs[r] = b;
+                    }
+                }
+            }
+            __syncthreads();
+            // PT[i][p] = (B A^-1)_{p i} = sum_q AT[i][q] B_pq
+            const int rows = kForceRows * force_row_groups(n);
+            for (int r0 = wid * rows; r0 < n; r0 += nw * rows) {
+                const int nl = min(rows, n - r0);
+                T* pt = (T*)(sPT + (size_t)r0 * ld);
+                warp_rows(nl, n, sAT + (size_t)r0 * ld, ld, sB, ld, [&](int r, int p, T v) {
+                    if constexpr (kFx) v = v * sA[r0 + r] * sBs[p];
+                    pt[r * ld + p] = v;
+                });
+                if constexpr (kFx) {
+                    __syncwarp();
+                    for (int r = 0; r < nl; ++r) {
+                        const double a = warp_limbs(pt + r * ld, (int2*)(pt + r * ld), n);
+                        if (lane == 0) sP[r0 + r] = a;
+                    }
+                }
+            }
+        } else {
+            for (int q2 = threadIdx.x; q2 < n * n; q2 += blockDim.x) B[q2] = b_of(q2 / n, q2 % n);
+            __syncthreads();
+            for (int q2 = threadIdx.x; q2 < n * n; q2 += blockDim.x) {
+                const int i = q2 / n, pp = q2 - i * n;
+                T v = T(0);
+                for (int q = 0; q < n; ++q) v += B[(size_t)pp * n + q] * ATg[(size_t)i * n + q];
+                PTg[q2] = v;
+            }
         }
         __syncthreads();
-        // PT[i][p] = (B A^-1)_{p i} = sum_q B_pq AT[i][q].  With AT staged,
-        // lanes take consecutive i (row p of B is one broadcast address per
-        // step, the AT rows sit at stride n + 1); otherwise consecutive p (the
-        // global AT row is the broadcast one)
-        for (int q2 = threadIdx.x; q2 < n * n; q2 += blockDim.x) {
-            const int r = q2 / n, c = q2 - r * n;
-            const int i = stg ? c : r, pp = stg ? r : c;
-            const T* ATi = AT + (size_t)i * ld;
-            const T* Bp = B + (size_t)pp * n;
-            T v = T(0);
-            for (int q = 0; q < n; ++q) v += Bp[q] * ATi[q];
-            PT[i * ld + pp] = v;
-        }
-        __syncthreads();
-        int sh0 = 0;
+        int sh0 = 0, run0 = 0;
         while (sh0 < s.n_shell) {
             const int fl0 = s.shell_fn[sh0];
             int sh1 = sh0 + 1;
-            while (sh1 < s.n_shell && s.shell_fn[sh1 + 1] - fl0 <= kForceTile) ++sh1;
+            while (sh1 < s.n_shell && s.shell_fn[sh1 + 1] - fl0 <= fs.F) ++sh1;
             const int nfl = s.shell_fn[sh1] - fl0;
-            // M[l][i] = sum_j C[l][j] AT[i][j]
-            for (int q2 = threadIdx.x; q2 < nfl * n; q2 += blockDim.x) {
-                const int l = q2 / n, i = q2 - l * n;
-                const T* Cl = C + (size_t)(fl0 + l) * n;
-                const T* ATi = AT + (size_t)i * ld;
-                T v = T(0);
-                for (int j = 0; j < n; ++j) v += Cl[j] * ATi[j];
-                Mt[l * nmax + i] = v;
+            // M[l][i] = sum_j C[l][j] AT[i][j],  Y[l][i] = sum_p M[l][p] PT[i][p]
+            if (fs.stg) {
+                const int rows = kForceRows * force_row_groups(n);
+                for (int r0 = wid * rows; r0 < nfl; r0 += nw * rows) {
+                    const int nl = min(rows, nfl - r0), l0 = fl0 + r0;
+                    T* m = Mt + (size_t)r0 * nmax;
+                    T* y = Yt + (size_t)r0 * nmax;
+                    if constexpr (kFx) {
+                        const double* sC = s.Cq_s[spin] + l0;
+                        warp_rows(nl, n, s.Cq[spin] + (size_t)l0 * n, n, sAT, ld,
+                                  [&](int r, int i, double v) { m[r * nmax + i] = v * sC[r] * sA[i]; });
+                        __syncwarp();
+                        double sM[3 * kForceRows];
+#pragma unroll
+                        for (int r = 0; r < 3 * kForceRows; ++r)
+                            sM[r] = r < nl ? warp_limbs(m + r * nmax, scr + r * n, n) : 0.0;
+                        __syncwarp();
+                        warp_rows(nl, n, scr, n, sPT, ld, [&](int r, int i, double v) {
+                            double a = 0.0;
+#pragma unroll
+                            for (int q = 0; q < 3 * kForceRows; ++q) a = q == r ? sM[q] : a;
+                            y[r * nmax + i] = v * a * sP[i];
+                        });
+                        __syncwarp();
+                    } else {
+                        warp_rows(nl, n, C + (size_t)l0 * n, n, sAT, ld,
+                                  [&](int r, int i, float v) { m[r * nmax + i] = v; });
+                        __syncwarp();
+                        warp_rows(nl, n, m, nmax, sPT, ld, [&](int r, int i, float v) { y[r * nmax + i] = v; });
+                    }
+                }
+            } else {
+                for (int q2 = threadIdx.x; q2 < nfl * n; q2 += blockDim.x) {
+                    const int l = q2 / n, i = q2 - l * n;
+                    T v = T(0);
+                    for (int j = 0; j < n; ++j) v += C[(size_t)(fl0 + l) * n + j] * ATg[(size_t)i * n + j];
+                    Mt[l * nmax + i] = v;
+                }
+                __syncthreads();
+                for (int q2 = threadIdx.x; q2 < nfl * n; q2 += blockDim.x) {
+                    const int l = q2 / n, i = q2 - l * n;
+                    T v = T(0);
+                    for (int p = 0; p < n; ++p) v += Mt[l * nmax + p] * PTg[(size_t)i * n + p];
+                    Yt[l * nmax + i] = v;
+                }
             }
             __syncthreads();
-            // Y[l][i] = sum_p M[l][p] PT[i][p]
-            for (int q2 = threadIdx.x; q2 < nfl * n; q2 += blockDim.x) {
-                const int l = q2 / n, i = q2 - l * n;
-                const T* Ml = Mt + l * nmax;
-                const T* Pi = PT + (size_t)i * ld;
-                T v = T(0);
-                for (int p = 0; p < n; ++p) v += Ml[p] * Pi[p];
-                Yt[l * nmax + i] = v;
-            }
-            __syncthreads();
-            // warp per shell, lanes over electrons of this spin
-            for (int sh = sh0 + wid; sh < sh1; sh += nw) {
-                const int4 d = s.shell[sh];
-                const int l = d.y & 0xff, pure = d.y >> 8;
-                const int nf = shell_nfn(l, pure);
-                const int lb = s.shell_fn[sh] - fl0;
-                T v[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-                for (int i = lane; i < n; i += 32) {
-                    const T x[3] = {off_en(h, s, i0 + i, d.x, 0), off_en(h, s, i0 + i, d.x, 1),
-                                    off_en(h, s, i0 + i, d.x, 2)};
-                    T f0, f1, f2, f3;
-                    radial<T, true>(sys_alpha<T>(s), sys_cn<T>(s), d.z, d.w, x[0] * x[0] + x[1] * x[1] + x[2] * x[2],
-                                    f0, f1, f2, f3);
-                    if (f0 == T(0) && f1 == T(0) && f2 == T(0) && f3 == T(0)) continue;  // screened
+            // warp per run of shells on one centre (the part of it in this
+            // tile), lanes over the electrons of this spin
+            while (s.run_sh[run0 + 1] <= sh0) ++run0;
+            for (int run = run0 + wid; run < s.n_run && s.run_sh[run] < sh1; run += nw) {
+                const int a0 = max(sh0, s.run_sh[run]), a1 = min(sh1, s.run_sh[run + 1]);
+                const int ctr = s.shell[a0].x, lb = s.shell_fn[a0] - fl0;
+                T v[8] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
+                for (int c0 = 0; c0 < n; c0 += 32) {
+                    const bool on = c0 + lane < n;
+                    const int i = on ? c0 + lane : n - 1;
+                    const T x[3] = {off_en(h, s, i0 + i, ctr, 0), off_en(h, s, i0 + i, ctr, 1),
+                                    off_en(h, s, i0 + i, ctr, 2)};
                     const T gj[3] = {h.gJ[3 * (i0 + i)], h.gJ[3 * (i0 + i) + 1], h.gJ[3 * (i0 + i) + 2]};
-                    // the basis function moves with its nucleus, d/dR = -d/dr:
-                    // dT = sum M (wL dlap + w.dgrad) - Y dPhi with each d -> -d/dr
-                    T vt[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-                    shell_terms_any<T>(l, pure, nf, x, f0, f1, f2, f3, gj, Mt + lb * nmax + i, Yt + lb * nmax + i,
-                                       nmax, vt);
+                    T vt[8];
+                    run_terms<T>(s, a0, a1, on, x, gj, Mt + (size_t)lb * nmax + i, Yt + (size_t)lb * nmax + i, nmax, scr,
+                                 vt);
+                    if (!on) continue;
 #pragma unroll
                     for (int q = 0; q < 6; ++q) v[q] += vt[q];
                     if constexpr (kE)
 #pragma unroll
                         for (int q = 0; q < 3; ++q) atomicAdd(&gEs[3 * (i0 + i) + q], -double(vt[q]));
                 }
-                // one shell's sum over this spin's electrons; shells add in FP64
-                for (int q = 0; q < 6; ++q) v[q] = warp_sum(v[q]);
-                if (lane == 0)
-                    for (int q = 0; q < 6; ++q) atomicAdd(&acc[6 * d.x + q], q < 3 ? double(v[q]) : -double(v[q]));
+                // the basis functions move with their nucleus, d/dR = -d/dr:
+                // dT = sum M (wL dlap + w.dgrad) - Y dPhi with each d -> -d/dr
+                const T sum = warp_fold8(v);
+                const int q = fold8_index(lane);
+                if ((lane & 3) == 0 && q < 6) atomicAdd(&acc[6 * ctr + q], q < 3 ? double(sum) : -double(sum));
             }
             __syncthreads();
             sh0 = sh1;
@@ -507,7 +792,9 @@ __global__ void __launch_bounds__(256) k_force_contract(DevSys s, DevWalkers wk,
     const int N = s.N, nu = s.n_up, nn = s.n_nuc, nb = s.n_basis;
     const ForceHead<T> h(sm, N, nn);
     double* acc = h.acc;
-    double* gEs = (double*)((unsigned char*)sm + ((force_head_bytes<T>(N, nn) + 15) & ~(size_t)15));
+    unsigned char* scr = (unsigned char*)sm + ((force_head_bytes<T>(N, nn) + 15) & ~(size_t)15);
+    double* gEs = (double*)(scr + (sizeof(T) == 8 ? 8 * kRadialScratch : 0));
+    scr += (threadIdx.x >> 5) * kRadialScratch;   // the warp's radial scratch (FP64 form)
     force_load_positions(h, wk.R + (size_t)w * 3 * N, N);
     if constexpr (kE)
         for (int q = threadIdx.x; q < 3 * N; q += blockDim.x) gEs[q] = 0.0;
@@ -521,43 +808,31 @@ __global__ void __launch_bounds__(256) k_force_contract(DevSys s, DevWalkers wk,
         const int i0 = spin ? nu : 0;
         const T* M = Mw + ((size_t)(spin * W + wl)) * nb * n;
         const T* Y = Yw + ((size_t)(spin * W + wl)) * nb * n;
-        // warp per run of shells on one centre, lanes over electrons: the
-        // electron-centre offset is formed once per run, term sums in T, one
-        // FP64 atomic per run and component
+        // warp per run of shells on one centre, lanes over electrons: term
+        // sums in T, one FP64 atomic per run and component
         for (int run = wid; run < s.n_run; run += nw) {
             const int sh0 = s.run_sh[run], sh1 = s.run_sh[run + 1];
             const int ctr = s.shell[sh0].x;
-            T v[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-            for (int i = lane; i < n; i += 32) {
+            const size_t fl = (size_t)s.shell_fn[sh0] * n;
+            T v[8] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
+            for (int c0 = 0; c0 < n; c0 += 32) {
+                const bool on = c0 + lane < n;
+                const int i = on ? c0 + lane : n - 1;
                 const T x[3] = {off_en(h, s, i0 + i, ctr, 0), off_en(h, s, i0 + i, ctr, 1),
                                 off_en(h, s, i0 + i, ctr, 2)};
-                const T t = x[0] * x[0] + x[1] * x[1] + x[2] * x[2];
                 const T gj[3] = {h.gJ[3 * (i0 + i)], h.gJ[3 * (i0 + i) + 1], h.gJ[3 * (i0 + i) + 2]};
-                T ve[3] = {T(0), T(0), T(0)};
-                for (int sh = sh0; sh < sh1; ++sh) {
-                    const int4 d = s.shell[sh];
-                    const int l = d.y & 0xff, pure = d.y >> 8;
-                    const int nf = shell_nfn(l, pure);
-                    const int fl = s.shell_fn[sh];
-                    T f0, f1, f2, f3;
-                    radial<T, true>(sys_alpha<T>(s), sys_cn<T>(s), d.z, d.w, t, f0, f1, f2, f3);
-                    if (f0 == T(0) && f1 == T(0) && f2 == T(0) && f3 == T(0)) continue;  // screened
-                    T vt[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-                    shell_terms_any<T>(l, pure, nf, x, f0, f1, f2, f3, gj, M + (size_t)fl * n + i,
-                                       Y + (size_t)fl * n + i, n, vt);
+                T vt[8];
+                run_terms<T>(s, sh0, sh1, on, x, gj, M + fl + i, Y + fl + i, n, scr, vt);
+                if (!on) continue;
 #pragma unroll
-                    for (int q = 0; q < 6; ++q) v[q] += vt[q];
-                    if constexpr (kE)
-#pragma unroll
-                        for (int q = 0; q < 3; ++q) ve[q] += vt[q];
-                }
+                for (int q = 0; q < 6; ++q) v[q] += vt[q];
                 if constexpr (kE)
 #pragma unroll
-                    for (int q = 0; q < 3; ++q) atomicAdd(&gEs[3 * (i0 + i) + q], -double(ve[q]));
+                    for (int q = 0; q < 3; ++q) atomicAdd(&gEs[3 * (i0 + i) + q], -double(vt[q]));
             }
-            for (int q = 0; q < 6; ++q) v[q] = warp_sum(v[q]);
-            if (lane == 0)
-                for (int q = 0; q < 6; ++q) atomicAdd(&acc[6 * ctr + q], q < 3 ? double(v[q]) : -double(v[q]));
+            const T sum = warp_fold8(v);
+            const int q = fold8_index(lane);
+            if ((lane & 3) == 0 && q < 6) atomicAdd(&acc[6 * ctr + q], q < 3 ? double(sum) : -double(sum));
         }
     }
     __syncthreads();
@@ -594,6 +869,12 @@ cudaError_t launch_force_prep(const DevSys& s, const DevWalkers& wk, int w0, int
     return cudaGetLastError();
 }
 
+template <typename T>
+static size_t contract_smem(int N, int nn, bool kE) {
+    return ((force_head_bytes<T>(N, nn) + 15) & ~(size_t)15) + (sizeof(T) == 8 ? 8 * kRadialScratch : 0) +
+           (kE ? sizeof(double) * 3 * (size_t)N : 0);
+}
+
 // gEdet (may be null): determinant part of dE_L/dr_i [W][N][3] (walker
 // index w0 + local) of the space-warp form.
 template <typename T>
@@ -602,7 +883,7 @@ cudaError_t launch_force_contract(const DevSys& s, const DevWalkers& wk, int w0,
                                   cudaStream_t st) {
     if (W == 0) return cudaSuccess;
     if (gEdet) {
-        const size_t smem = ((force_head_bytes<T>(s.N, s.n_nuc) + 15) & ~(size_t)15) + sizeof(double) * 3 * (size_t)s.N;
+        const size_t smem = contract_smem<T>(s.N, s.n_nuc, true);
         if (smem > 48 * 1024) {
             cudaError_t e = cudaFuncSetAttribute(k_force_contract<T, true>,
                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -612,7 +893,7 @@ cudaError_t launch_force_contract(const DevSys& s, const DevWalkers& wk, int w0,
                                                          dlog, gEdet);
         return cudaGetLastError();
     }
-    const size_t smem = force_head_bytes<T>(s.N, s.n_nuc);
+    const size_t smem = contract_smem<T>(s.N, s.n_nuc, false);
     if (smem > 48 * 1024) {
         cudaError_t e =
             cudaFuncSetAttribute(k_force_contract<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -642,13 +923,13 @@ cudaError_t launch_force(const DevSys& s, const DevWalkers& wk, int W, const dou
     if (W == 0) return cudaSuccess;
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
     if (gEdet) {
-        const size_t smem = force_smem_e<T>(s.N, s.n_nuc, nmax, true);
+        const size_t smem = ForceShape<T>(s.N, s.n_nuc, nmax, s.n_basis, true).total;
         cudaError_t e = cudaFuncSetAttribute(k_force<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         k_force<T, true><<<W, 256, smem, st>>>(s, wk, W, dvnn, Bscr, Pscr, dEL, dlog, gEdet, gtot);
         return cudaGetLastError();
     }
-    const size_t smem = force_smem<T>(s.N, s.n_nuc, nmax);
+    const size_t smem = ForceShape<T>(s.N, s.n_nuc, nmax, s.n_basis, false).total;
     cudaError_t e = cudaFuncSetAttribute(k_force<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     k_force<T, false><<<W, 256, smem, st>>>(s, wk, W, dvnn, Bscr, Pscr, dEL, dlog, nullptr, nullptr);
@@ -856,8 +1137,8 @@ __global__ void __launch_bounds__(256, 2) k_force_batch(const BatchSys* __restri
 
 size_t force_batch_smem_bytes(const DevSys& s, int elem, int space_warp) {
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
-    return elem == 4 ? force_smem_e<float>(s.N, s.n_nuc, nmax, space_warp != 0)
-                     : force_smem_e<double>(s.N, s.n_nuc, nmax, space_warp != 0);
+    return elem == 4 ? ForceShape<float>(s.N, s.n_nuc, nmax, s.n_basis, space_warp != 0).total
+                     : ForceShape<double>(s.N, s.n_nuc, nmax, s.n_basis, space_warp != 0).total;
 }
 
 // Batched space warp: persistent CTAs over the walkers of every system; the

@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "batch.cuh"
+#include "fixed64.cuh"
 #include "qmc.h"
 #include "qmc_internal.cuh"
 #include "sweep_tiled.cuh"
@@ -544,6 +545,19 @@ struct qmc_ctx {
                 for (int j = 0; j < n; ++j) Cs[(size_t)l * n + j] = C[(size_t)occ[j] * n_basis + l];
             s.C[spin] = upload(sys_allocs, Cs);
             s.C_f[spin] = upload(sys_allocs, std::vector<float>(Cs.begin(), Cs.end()));
+            {
+                const size_t n = occ.size();
+                std::vector<int2> q(Cs.size());
+                std::vector<double> sc(n_basis);
+                for (int l = 0; l < n_basis; ++l) {
+                    int e = 0;
+                    for (size_t j = 0; j < n; ++j) e = std::max(e, fx_expo(Cs[l * n + j]));
+                    for (size_t j = 0; j < n; ++j) q[l * n + j] = fx_limbs(Cs[l * n + j], e);
+                    sc[l] = fx_scale(e);
+                }
+                s.Cq[spin] = upload(sys_allocs, q);
+                s.Cq_s[spin] = upload(sys_allocs, sc);
+            }
         }
         if (have_msd) build_multidet(s);
         ds = s;

@@ -47,6 +47,8 @@ struct DevSys {
     const float* cn_f;
     const double* C[2];   // [n_basis][n_s] occupied orbital coefficients per spin
     const float* C_f[2];
+    const int2* Cq[2];     // C as fixed-point limbs per row (fixed64.cuh) and the rows' scales [n_basis]
+    const double* Cq_s[2];
     // Multi-determinant expansion (table method); msd == 0: one determinant.
     // Spin strings are stored relative to the reference determinant: e
     // holes (positions 0..n_s-1 in the reference orbital list, ascending)
