@@ -1,0 +1,243 @@
+// FP64 basis and orbital contraction of one electron position by one CTA
+// (Eq. 2), built around the FP64 pipe: on GB300 an FP64 instruction of a warp
+// takes 16 SM cycles however few lanes are active, so every FP64 step runs on
+// a list that fills its warps and the contraction runs in fixed point
+// (fixed64.cuh).
+//
+//   1. offsets and r^2 from every nucleus (a thread per nucleus);
+//   2. the unscreened primitives and shells are listed (FP32 test; a pair at
+//      the threshold is below 1e-26 either way);
+//   3. one exponential per listed primitive;
+//   4. radial sums per listed shell, whose functions are listed by angular
+//      momentum so that a warp holds functions of one kind;
+//   5. value, gradient and Laplacian of the listed functions, split into
+//      limbs with one scale per component;
+//   6. phi[c][j] = sum_r C[row_r][j] bas[c][r], three 32-bit multiply-adds per
+//      term, slices of the rows on neighbouring lanes.
+// Bound by instruction issue (30 %, with the barriers between the steps) and
+// by the FP64 pipe (50 % at 30 orbitals).  Rebuild of the 32-water cluster, 256
+// walkers: 51 -> 17 ms against a masked basis and FP64 chains; 6-water cluster, 512 walkers: 1.64 -> 0.86 ms.
+// The lists are filled in any order: every sum over them is exact integer
+// arithmetic, so the result does not depend on it.
+#pragma once
+
+#include "fixed64.cuh"
+#include "qmc_internal.cuh"
+
+namespace qmc {
+
+struct Basis64Layout {
+    size_t nuc, ev, fs, bas, plist, slist, flist, rows, cnt, total;
+    int ldb;
+    __host__ __device__ Basis64Layout(int n_nuc, int n_prim, int n_shell, int n_basis) {
+        ldb = (n_basis + 1) & ~1;
+        size_t o = 0;
+        nuc = o;
+        o += sizeof(double) * 4 * (size_t)n_nuc;
+        ev = o;
+        o += sizeof(double) * (size_t)n_prim;
+        fs = o;
+        o += sizeof(double) * 3 * (size_t)n_shell;
+        bas = o;
+        o += sizeof(double) * 5 * (size_t)ldb;
+        plist = o;
+        o += sizeof(int) * (size_t)n_prim;
+        slist = o;
+        o += sizeof(int) * (size_t)n_shell;
+        flist = o;
+        o += sizeof(int) * (size_t)n_basis;
+        rows = o;
+        o += sizeof(int) * (size_t)n_basis;
+        cnt = o;
+        o += sizeof(int) * 16;
+        total = (o + 15) & ~(size_t)15;
+    }
+};
+
+// Largest layout used: 227 KB less the static shared memory of the batched
+// kernels.
+constexpr size_t kBasis64Max = 224 * 1024;
+
+// Steps 1 to 5 at position (r0, r1, r2).  Leaves the limbs in bas [5][ldb]
+// (int2), the functions' indices in rows and returns their number; the
+// components' scales are fx_scale(cnt[8 + c]).  All threads call; ends
+// synchronised.  nuc: the nuclear offsets (x, y, z, r^2) stay valid after it.
+__device__ __forceinline__ int basis64(const DevSys& s, const Basis64Layout& L, unsigned char* sm, double r0, double r1,
+                                       double r2) {
+    double4* nuc = (double4*)(sm + L.nuc);
+    double* ev = (double*)(sm + L.ev);
+    double* fs = (double*)(sm + L.fs);
+    double* bas = (double*)(sm + L.bas);
+    int* plist = (int*)(sm + L.plist);
+    int* slist = (int*)(sm + L.slist);
+    int* flist = (int*)(sm + L.flist);   // functions by kind: s from 0, p from n_fn_s, d from n_fn_s + n_fn_p
+    int* rows = (int*)(sm + L.rows);
+    int* cnt = (int*)(sm + L.cnt);       // [0] primitives, [1] shells, [2..4] functions by kind, [8..12] exponents
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, ldb = L.ldb;
+    const unsigned below = (1u << lane) - 1u;
+    if (tid < 16) cnt[tid] = 0;
+    for (int a = tid; a < s.n_nuc; a += nt) {
+        const double x = r0 - s.Rn[3 * a], y = r1 - s.Rn[3 * a + 1], z = r2 - s.Rn[3 * a + 2];
+        nuc[a] = make_double4(x, y, z, x * x + y * y + z * z);
+    }
+    __syncthreads();
+    const float cut = (float)kScreenExponent;
+    for (int p0 = tid - lane; p0 < s.n_prim; p0 += nt) {
+        const int p = p0 + lane;
+        const bool live = p < s.n_prim && !(s.alpha_f[p] * (float)nuc[s.prim_ctr[p]].w > cut);
+        const unsigned m = __ballot_sync(0xffffffffu, live);
+        int base = 0;
+        if (lane == 0 && m) base = atomicAdd(&cnt[0], __popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (live) plist[base + __popc(m & below)] = p;
+    }
+    for (int q0 = tid - lane; q0 < s.n_shell; q0 += nt) {
+        const int sh = q0 + lane;
+        const bool live = sh < s.n_shell && !(s.shell_amin_f[sh] * (float)nuc[s.shell[sh].x].w > cut);
+        const unsigned m = __ballot_sync(0xffffffffu, live);
+        int base = 0;
+        if (lane == 0 && m) base = atomicAdd(&cnt[1], __popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (live) slist[base + __popc(m & below)] = sh;
+    }
+    __syncthreads();
+    for (int k = tid; k < cnt[0]; k += nt) {
+        const int p = plist[k];
+        ev[p] = s.cn[p] * exp(-s.alpha[p] * nuc[s.prim_ctr[p]].w);
+    }
+    __syncthreads();
+    for (int k = tid; k < cnt[1]; k += nt) {
+        const int sh = slist[k];
+        const int4 d = s.shell[sh];
+        const double t = nuc[d.x].w;
+        const float tf = (float)t;
+        double f0 = 0.0, f1 = 0.0, f2 = 0.0;
+        for (int p = d.z; p < d.z + d.w; ++p) {
+            if (s.alpha_f[p] * tf > cut) continue;
+            const double a = s.alpha[p], e = ev[p], e1 = a * e;
+            f0 += e;
+            f1 -= e1;
+            f2 += a * e1;
+        }
+        // f0, 2 f1 and the radial part of the Laplacian with its 2 grad P . grad S
+        // term folded in (grad P . x = l P): lap = P (6 f1 + 4 t f2 + 4 l f1) + f0 lap P
+        const int l = d.y & 0xff, nf = shell_nfn(l, d.y >> 8);
+        fs[3 * sh] = f0;
+        fs[3 * sh + 1] = 2.0 * f1;
+        fs[3 * sh + 2] = (double)(6 + 4 * l) * f1 + 4.0 * t * f2;
+        const int o = atomicAdd(&cnt[2 + l], nf) + (l > 0 ? s.n_fn_s : 0) + (l > 1 ? s.n_fn_p : 0);
+        for (int f = 0; f < nf; ++f) flist[o + f] = sh * 8 + f;
+    }
+    __syncthreads();
+    // functions of one kind per warp: the kinds' segments padded to 32
+    const int ns = cnt[2], np = cnt[3], nd = cnt[4];
+    const int e0 = (ns + 31) & ~31, e1 = e0 + ((np + 31) & ~31), e2 = e1 + nd;
+    int mx[5] = {0, 0, 0, 0, 0};
+    for (int o = tid; o < e2; o += nt) {
+        const int kind = o < e0 ? 0 : o < e1 ? 1 : 2;
+        const int q = o - (kind == 0 ? 0 : kind == 1 ? e0 : e1);
+        if (q >= (kind == 0 ? ns : kind == 1 ? np : nd)) continue;
+        const int ent = flist[q + (kind == 0 ? 0 : kind == 1 ? s.n_fn_s : s.n_fn_s + s.n_fn_p)];
+        const int sh = ent >> 3, f = ent & 7;
+        const int4 d = s.shell[sh];
+        const double4 x = nuc[d.x];
+        const double f0 = fs[3 * sh], g1 = fs[3 * sh + 1], gl = fs[3 * sh + 2];
+        double v[5];
+        if (kind == 0) {
+            v[0] = f0;
+            v[1] = x.x * g1;
+            v[2] = x.y * g1;
+            v[3] = x.z * g1;
+            v[4] = gl;
+        } else if (kind == 1) {
+            const double P = f == 0 ? x.x : f == 1 ? x.y : x.z, Pg = P * g1;
+            v[0] = P * f0;
+            v[1] = x.x * Pg;
+            v[2] = x.y * Pg;
+            v[3] = x.z * Pg;
+            if (f == 0) v[1] += f0;
+            if (f == 1) v[2] += f0;
+            if (f == 2) v[3] += f0;
+            v[4] = P * gl;
+        } else {
+            const AngPoly<double> a = angular<double>(2, d.y >> 8, f, x.x, x.y, x.z);
+            const double Pg = a.P * g1;
+            v[0] = a.P * f0;
+            v[1] = x.x * Pg + a.Px * f0;
+            v[2] = x.y * Pg + a.Py * f0;
+            v[3] = x.z * Pg + a.Pz * f0;
+            v[4] = a.P * gl;
+            if ((d.y >> 8) == 0) v[4] += (a.Hxx + a.Hyy + a.Hzz) * f0;   // pure d functions are harmonic
+        }
+        const int r = q + (kind == 0 ? 0 : kind == 1 ? ns : ns + np);
+        rows[r] = s.shell_fn[sh] + f;
+#pragma unroll
+        for (int c = 0; c < 5; ++c) {
+            bas[c * ldb + r] = v[c];
+            mx[c] = max(mx[c], fx_expo(v[c]));
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+        const int m = warp_max_u(mx[c]);
+        if (lane == 0 && m) atomicMax(&cnt[8 + c], m);
+    }
+    __syncthreads();
+    const int nrow = ns + np + nd;
+    int em[5];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) em[c] = cnt[8 + c];
+    for (int o = tid; o < 5 * nrow; o += nt) {
+        const int c = o / nrow, q = c * ldb + o - c * nrow;
+        const int e = c == 0 ? em[0] : c == 1 ? em[1] : c == 2 ? em[2] : c == 3 ? em[3] : em[4];
+        ((int2*)bas)[q] = fx_limbs(bas[q], e);
+    }
+    __syncthreads();
+    return nrow;
+}
+
+// Step 6: put(c, j, phi_cj) for c < 5 and every orbital j < n of a
+// coefficient block given as limbs Ck [n_basis][n] with the orbitals' scales
+// sC [n].  S lanes share an orbital, each taking every S-th row: as many as
+// keep n S within the CTA.
+template <typename Put>
+__device__ __forceinline__ void contract64(const Basis64Layout& L, const unsigned char* sm, int nrow,
+                                           const int2* __restrict__ Ck, const double* __restrict__ sC, int n, Put put) {
+    const int2* bas = (const int2*)(sm + L.bas);
+    const int* rows = (const int*)(sm + L.rows);
+    const int* cnt = (const int*)(sm + L.cnt);
+    const int ldb = L.ldb;
+    int lg = 4;
+    while (lg > 0 && (n << lg) > (int)blockDim.x) --lg;
+    const int S = 1 << lg, items = (n << lg);
+    for (int o0 = threadIdx.x & ~31; o0 < items; o0 += blockDim.x) {   // whole warps
+        const int o = o0 + (threadIdx.x & 31), sl = o & (S - 1);
+        const int j = min(o >> lg, n - 1);
+        FxSum sum[5];
+        for (int r0 = sl; r0 < nrow; r0 += kFxBlock * S) {
+            FxDot d[5];
+            const int r1 = min(nrow, r0 + kFxBlock * S);
+#pragma unroll 4
+            for (int r = r0; r < r1; r += S) {
+                const int2 cv = Ck[(size_t)rows[r] * n + j];
+#pragma unroll
+                for (int c = 0; c < 5; ++c) d[c].add(cv, bas[c * ldb + r]);
+            }
+#pragma unroll
+            for (int c = 0; c < 5; ++c) sum[c].fold(d[c]);
+        }
+        for (int k = 1; k < S; k <<= 1)
+#pragma unroll
+            for (int c = 0; c < 5; ++c) {
+                sum[c].hi += __shfl_xor_sync(0xffffffffu, sum[c].hi, k);
+                sum[c].lo += __shfl_xor_sync(0xffffffffu, sum[c].lo, k);
+            }
+        if (o >= items) continue;
+        const double sj = sC[j];
+#pragma unroll
+        for (int c = 0; c < 5; ++c)
+            if ((c & (S - 1)) == sl) put(c, j, sum[c].value() * sj * fx_scale(cnt[8 + c]));   // every lane shares the outputs
+    }
+}
+
+}  // namespace qmc

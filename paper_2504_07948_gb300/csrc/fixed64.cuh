@@ -81,8 +81,9 @@ struct FxSum {
         d.mid = 0;
     }
     __device__ __forceinline__ double value() const {
-        const long long h = hi + (lo >> 32);
-        return (double)h * 4294967296.0 + (double)(lo & 0xffffffffLL);
+        const long long h = hi + (lo >> 32), l = lo & 0xffffffffLL;
+        if (h == (long long)(int)h) return (double)(long long)(((unsigned long long)h << 32) | (unsigned long long)l);
+        return (double)h * 4294967296.0 + (double)l;
     }
 };
 

@@ -3,88 +3,85 @@
 // the Slater matrices, and the local energy.  These kernels serve the
 // parity entry point and the periodic FP64 recompute of the incremental
 // inverse.
+#include "basis64.cuh"
 #include "batch.cuh"
 #include "qmc_internal.cuh"
 
 namespace qmc {
 
-// One CTA per (walker, electron).  Basis value/gradient/Laplacian of every
-// shell at r_i in FP64 (one thread per shell, the "multi-center" flattening
-// of {centres x electrons} onto the grid), then the LCAO contraction
-// phi_j = sum_l C_l^j Phi_l (Eq. 2) for the occupied orbitals of the
-// electron's spin.  A goes to FP64 scratch, the gradient/Laplacian rows to
-// the walker cache in the storage type T.
-// Orbitals of electron i of walker w (body of k_orbitals_all).  sh_bas:
-// 5 n_basis doubles of shared memory.  live (optional, n_shell bytes of
-// shared memory): shells whose values and derivatives are all exactly zero
-// (screened) are left out of the occupied-orbital contraction; the terms
-// that remain are added in the same order, so the result is unchanged.
+// Orbitals of electron i of walker w without lists or limbs (see
+// orbitals_item), for a basis whose lists exceed shared
+// memory (about 2500 functions): 5 n_basis doubles of it.
 template <typename T>
-__device__ __forceinline__ void orbitals_item(const DevSys& s, const DevWalkers& wk, int w, int i, double* sh_bas,
-                                              unsigned char* live = nullptr) {
+__device__ __noinline__ void orbitals_item_plain(const DevSys& s, const DevWalkers& wk, int w, int i, double* bas) {
     const int nb = s.n_basis;
-    double r[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) r[c] = wk.R[((size_t)w * s.N + i) * 3 + c];
-    for (int sh = threadIdx.x; sh < s.n_shell; sh += blockDim.x) shell_vgl<double>(s, sh, r, sh_bas, nb);
+    const double* r = wk.R + ((size_t)w * s.N + i) * 3;
+    for (int sh = threadIdx.x; sh < s.n_shell; sh += blockDim.x) shell_vgl<double>(s, sh, r, bas, nb);
     __syncthreads();
-    if (live) {
-        for (int sh = threadIdx.x; sh < s.n_shell; sh += blockDim.x) {
-            const int f0 = s.shell_fn[sh], f1 = s.shell_fn[sh + 1];
-            bool nz = false;
-            for (int c = 0; c < 5 && !nz; ++c)
-                for (int f = f0; f < f1 && !nz; ++f) nz = sh_bas[c * nb + f] != 0.0;
-            live[sh] = nz ? 1 : 0;
+    const int spin = i < s.n_up ? 0 : 1, n = spin ? s.n_dn : s.n_up, k = spin ? i - s.n_up : i;
+    for (int vir = 0; vir < (s.msd ? 2 : 1); ++vir) {
+        const int nj = vir ? s.n_vir[spin] : n;
+        const double* C = vir ? s.Cv[spin] : s.C[spin];
+        T* G = (T*)(vir ? wk.Gv[spin] : wk.G[spin]) + ((size_t)w * n + k) * 4 * nj;
+        for (int o = threadIdx.x; o < 5 * nj; o += blockDim.x) {
+            const int c = o / nj, j = o - c * nj;
+            double acc = 0.0;
+            for (int l = 0; l < nb; ++l) acc += C[(size_t)l * nj + j] * bas[c * nb + l];
+            if (c)
+                G[(c - 1) * nj + j] = (T)acc;
+            else if (vir)
+                ((T*)wk.Av[spin])[((size_t)w * n + k) * nj + j] = (T)acc;
+            else
+                wk.Ascr[spin][((size_t)w * n + k) * n + j] = acc;
         }
-        __syncthreads();
     }
+}
+
+// Orbitals of electron i of walker w by one CTA (body of k_orbitals_all):
+// the live basis functions at r_i in FP64 and the LCAO contraction phi_j =
+// sum_l C_l^j Phi_l (Eq. 2) in fixed point (basis64.cuh) for the occupied
+// orbitals of the electron's spin.  A goes to FP64 scratch, the gradient and
+// Laplacian rows to the walker cache in the storage type T.  sm:
+// orbitals_smem_bytes of shared memory.
+template <typename T>
+__device__ __forceinline__ void orbitals_item(const DevSys& s, const DevWalkers& wk, int w, int i, unsigned char* sm) {
+    const Basis64Layout L(s.n_nuc, s.n_prim, s.n_shell, s.n_basis);
+    if (L.total > kBasis64Max) {
+        orbitals_item_plain<T>(s, wk, w, i, (double*)sm);
+        return;
+    }
+    const double* r = wk.R + ((size_t)w * s.N + i) * 3;
+    const int nrow = basis64(s, L, sm, r[0], r[1], r[2]);
     const int spin = i < s.n_up ? 0 : 1;
     const int n = spin ? s.n_dn : s.n_up;
     const int k = spin ? i - s.n_up : i;
-    const double* C = s.C[spin];
     T* G = (T*)wk.G[spin] + ((size_t)w * n + k) * 4 * n;
     double* A = wk.Ascr[spin] + ((size_t)w * n + k) * n;
-    for (int o = threadIdx.x; o < 5 * n; o += blockDim.x) {
-        const int c = o / n, j = o - c * n;
-        const double* b = sh_bas + c * nb;
-        double acc = 0.0;
-        if (live) {
-            for (int sh = 0; sh < s.n_shell; ++sh) {
-                if (!live[sh]) continue;
-                for (int l = s.shell_fn[sh]; l < s.shell_fn[sh + 1]; ++l) acc += C[(size_t)l * n + j] * b[l];
-            }
-        } else {
-            for (int l = 0; l < nb; ++l) acc += C[(size_t)l * n + j] * b[l];
-        }
+    contract64(L, sm, nrow, s.Ck[spin], s.Ck_s[spin], n, [&](int c, int j, double v) {
         if (c == 0)
-            A[j] = acc;
+            A[j] = v;
         else
-            G[(c - 1) * n + j] = (T)acc;
-    }
-    if (s.msd) {  // active virtual orbitals of a determinant expansion
+            G[(c - 1) * n + j] = (T)v;
+    });
+    if (s.msd && s.n_vir[spin] > 0) {  // active virtual orbitals of a determinant expansion
         const int nv = s.n_vir[spin];
-        const double* Cv = s.Cv[spin];
         T* Av = (T*)wk.Av[spin] + ((size_t)w * n + k) * nv;
         T* Gv = (T*)wk.Gv[spin] + ((size_t)w * n + k) * 4 * nv;
-        for (int o = threadIdx.x; o < 5 * nv; o += blockDim.x) {
-            const int c = o / nv, p = o - c * nv;
-            const double* b = sh_bas + c * nb;
-            double acc = 0.0;
-            for (int l = 0; l < nb; ++l) acc += Cv[(size_t)l * nv + p] * b[l];
+        contract64(L, sm, nrow, s.Cvk[spin], s.Cvk_s[spin], nv, [&](int c, int j, double v) {
             if (c == 0)
-                Av[p] = (T)acc;
+                Av[j] = (T)v;
             else
-                Gv[(c - 1) * nv + p] = (T)acc;
-        }
+                Gv[(c - 1) * nv + j] = (T)v;
+        });
     }
 }
 
 template <typename T>
 __global__ void k_orbitals_all(DevSys s, DevWalkers wk, int W, const int* only) {
-    extern __shared__ double sh_bas[];  // [5][n_basis], then one live flag per shell
+    extern __shared__ double sh_bas[];
     const int w = blockIdx.x, i = blockIdx.y;
     if (w >= W || (only && !only[w])) return;
-    orbitals_item<T>(s, wk, w, i, sh_bas, reinterpret_cast<unsigned char*>(sh_bas + 5 * s.n_basis));
+    orbitals_item<T>(s, wk, w, i, (unsigned char*)sh_bas);
 }
 
 // In-place Gauss-Jordan inversion with partial (row) pivoting, FP64, one
@@ -573,11 +570,17 @@ __global__ void k_weighted_sum(const double* x, const double* g, int W, int K, d
     if (threadIdx.x == 0) out[k] = (accumulate ? out[k] : 0.0) + v[0];
 }
 
+size_t orbitals_smem_bytes(const DevSys& s) {
+    const size_t b = Basis64Layout(s.n_nuc, s.n_prim, s.n_shell, s.n_basis).total;
+    return b <= kBasis64Max ? b : sizeof(double) * 5 * (size_t)s.n_basis;
+}
+
 template <typename T>
 cudaError_t launch_orbitals_all(const DevSys& s, const DevWalkers& wk, int W, cudaStream_t st, const int* only) {
     if (W == 0 || s.N == 0) return cudaSuccess;
-    const size_t smem = sizeof(double) * 5 * s.n_basis + (size_t)s.n_shell;
-    const int nt = s.n_up > 32 ? 256 : 128;
+    const size_t smem = orbitals_smem_bytes(s);
+    const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
+    const int nt = nmax > 128 ? (nmax > 256 ? 256 : (nmax + 31) & ~31) : 128;   // a thread per orbital
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_orbitals_all<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem);
@@ -636,7 +639,7 @@ __global__ void k_orbitals_batch(const BatchSys* __restrict__ sys, BatchPlan* pl
         batch_load(&bs, sys + q);
         __syncthreads();
         const int N = bs.s.N;
-        orbitals_item<T>(bs.s, bs.wk[parity], s_idx / N, s_idx % N, sh_bas);
+        orbitals_item<T>(bs.s, bs.wk[parity], s_idx / N, s_idx % N, (unsigned char*)sh_bas);
         __syncthreads();
     }
 }

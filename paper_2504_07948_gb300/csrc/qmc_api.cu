@@ -535,6 +535,16 @@ struct qmc_ctx {
             s.shell_amin = upload(sys_allocs, am);
             s.shell_amin_f = upload(sys_allocs, amf);
         }
+        {
+            std::vector<int> pc(alpha.size());
+            s.n_fn_s = s.n_fn_p = 0;
+            for (int q = 0; q < s.n_shell; ++q) {
+                for (int p = sh[q].z; p < sh[q].z + sh[q].w; ++p) pc[p] = sh[q].x;
+                if (sh_l[q] == 0) s.n_fn_s += 1;
+                if (sh_l[q] == 1) s.n_fn_p += 3;
+            }
+            s.prim_ctr = upload(sys_allocs, pc);
+        }
         s.alpha_f = upload(sys_allocs, std::vector<float>(alpha.begin(), alpha.end()));
         s.cn_f = upload(sys_allocs, std::vector<float>(cn.begin(), cn.end()));
         for (int spin = 0; spin < 2; ++spin) {
@@ -558,6 +568,7 @@ struct qmc_ctx {
                 s.Cq[spin] = upload(sys_allocs, q);
                 s.Cq_s[spin] = upload(sys_allocs, sc);
             }
+            upload_columns(Cs, n_basis, n, &s.Ck[spin], &s.Ck_s[spin]);
         }
         if (have_msd) build_multidet(s);
         ds = s;
@@ -570,6 +581,21 @@ struct qmc_ctx {
         for (int b = 0; b < 64 * msd_words; ++b)
             if ((w[b / 64] >> (b % 64)) & 1ULL) o.push_back(b);
         return o;
+    }
+
+    // Fixed-point limbs (fixed64.cuh) of a coefficient block C [rows][n], one
+    // scale per column, to the device.
+    void upload_columns(const std::vector<double>& Cm, int rows, int n, const int2** limbs, const double** scales) {
+        std::vector<int2> q(Cm.size());
+        std::vector<double> sc(n);
+        for (int j = 0; j < n; ++j) {
+            int e = 0;
+            for (int l = 0; l < rows; ++l) e = std::max(e, fx_expo(Cm[(size_t)l * n + j]));
+            for (int l = 0; l < rows; ++l) q[(size_t)l * n + j] = fx_limbs(Cm[(size_t)l * n + j], e);
+            sc[j] = fx_scale(e);
+        }
+        *limbs = upload(sys_allocs, q);
+        *scales = upload(sys_allocs, sc);
     }
 
     // Unique spin strings of the expansion relative to the reference:
@@ -680,6 +706,7 @@ struct qmc_ctx {
                 for (size_t q = 0; q < vir.size(); ++q) Cv[l * vir.size() + q] = C[(size_t)vir[q] * n_basis + l];
             s.Cv[spin] = upload(sys_allocs, Cv);
             s.Cv_f[spin] = upload(sys_allocs, std::vector<float>(Cv.begin(), Cv.end()));
+            upload_columns(Cv, n_basis, (int)vir.size(), &s.Cvk[spin], &s.Cvk_s[spin]);
         }
         for (int spin = 0; spin < 2; ++spin) {
             const int ns = s.n_str[spin];
@@ -2404,7 +2431,7 @@ struct qmc_batch {
         for (int q = 0; q < n; ++q) {
             const DevSys& s = sys[q]->ds;
             const int nmax = std::max(s.n_up, s.n_dn);
-            orb = std::max(orb, sizeof(double) * 5 * (size_t)s.n_basis);
+            orb = std::max(orb, orbitals_smem_bytes(s));
             inv = std::max(inv, sizeof(double) * ((size_t)nmax * nmax + nmax + 1));
             el = std::max(el, (sizeof(double) + sizeof(float)) * 3 * (size_t)s.N);
             fo = std::max(fo, force_batch_smem_bytes(s, elem(), warp[q]));

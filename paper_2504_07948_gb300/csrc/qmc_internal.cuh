@@ -49,6 +49,10 @@ struct DevSys {
     const float* C_f[2];
     const int2* Cq[2];     // C as fixed-point limbs per row (fixed64.cuh) and the rows' scales [n_basis]
     const double* Cq_s[2];
+    const int2* Ck[2];     // C as limbs per column, [n_basis][n_s], and the columns' scales [n_s]
+    const double* Ck_s[2];
+    const int* prim_ctr;   // [n_prim] nucleus of each primitive
+    int n_fn_s, n_fn_p;    // basis functions of s and of p shells
     // Multi-determinant expansion (table method); msd == 0: one determinant.
     // Spin strings are stored relative to the reference determinant: e
     // holes (positions 0..n_s-1 in the reference orbital list, ascending)
@@ -59,6 +63,8 @@ struct DevSys {
     int n_vir[2];             // active virtual orbitals per spin
     const double* Cv[2];      // [n_basis][n_vir] virtual orbital coefficients
     const float* Cv_f[2];
+    const int2* Cvk[2];       // Cv as limbs per column and the columns' scales [n_vir]
+    const double* Cvk_s[2];
     int n_str[2];             // unique strings per spin (string 0 = reference)
     const int4* str[2];       // x = e | (phase < 0) << 8, y = holes, z = particles (4 x 8 bit)
     const int* csr_off[2];    // [n_str + 1]: the determinants that contain each string
@@ -1269,6 +1275,7 @@ struct SweepParams {
     int g_smem;      // keep the gradient/Laplacian cache in shared memory
 };
 
+size_t orbitals_smem_bytes(const DevSys& s);
 template <typename T>
 cudaError_t launch_orbitals_all(const DevSys& s, const DevWalkers& wk, int W, cudaStream_t st,
                                 const int* only = nullptr);
