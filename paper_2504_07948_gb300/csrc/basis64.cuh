@@ -19,6 +19,13 @@
 // walkers: 51 -> 17 ms against a masked basis and FP64 chains; 6-water cluster, 512 walkers: 1.64 -> 0.86 ms.
 // The lists are filled in any order: every sum over them is exact integer
 // arithmetic, so the result does not depend on it.
+//
+// Accuracy: the contraction's error is about sqrt(rows) 2^-60 of the largest
+// basis value times the orbital's largest coefficient.  Where no orbital of
+// the block reaches 2^-4 of that (occupied orbitals without weight on the
+// functions that are large at this point), orbitals64 takes the orbitals
+// again in FP64, so that the row of orbital values keeps the accuracy of an
+// FP64 sum relative to its largest entry.
 #pragma once
 
 #include "fixed64.cuh"
@@ -49,7 +56,7 @@ struct Basis64Layout {
         rows = o;
         o += sizeof(int) * (size_t)n_basis;
         cnt = o;
-        o += sizeof(int) * 16;
+        o += sizeof(int) * 32;
         total = (o + 15) & ~(size_t)15;
     }
 };
@@ -72,10 +79,11 @@ __device__ __forceinline__ int basis64(const DevSys& s, const Basis64Layout& L, 
     int* slist = (int*)(sm + L.slist);
     int* flist = (int*)(sm + L.flist);   // functions by kind: s from 0, p from n_fn_s, d from n_fn_s + n_fn_p
     int* rows = (int*)(sm + L.rows);
-    int* cnt = (int*)(sm + L.cnt);       // [0] primitives, [1] shells, [2..4] functions by kind, [8..12] exponents
+    int* cnt = (int*)(sm + L.cnt);       // [0] primitives, [1] shells, [2..4] functions by kind, [8..12] exponents,
+                                         // [16..20], [24..28] exponents of the sums (orbitals64)
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, ldb = L.ldb;
     const unsigned below = (1u << lane) - 1u;
-    if (tid < 16) cnt[tid] = 0;
+    for (int q = tid; q < 32; q += nt) cnt[q] = 0;
     for (int a = tid; a < s.n_nuc; a += nt) {
         const double x = r0 - s.Rn[3 * a], y = r1 - s.Rn[3 * a + 1], z = r2 - s.Rn[3 * a + 2];
         nuc[a] = make_double4(x, y, z, x * x + y * y + z * z);
@@ -199,10 +207,12 @@ __device__ __forceinline__ int basis64(const DevSys& s, const Basis64Layout& L, 
 // Step 6: put(c, j, phi_cj) for c < 5 and every orbital j < n of a
 // coefficient block given as limbs Ck [n_basis][n] with the orbitals' scales
 // sC [n].  S lanes share an orbital, each taking every S-th row: as many as
-// keep n S within the CTA.
+// keep n S within the CTA.  big: five counters (zero before the call) that
+// receive the largest exponent of the integer sums per component.
 template <typename Put>
 __device__ __forceinline__ void contract64(const Basis64Layout& L, const unsigned char* sm, int nrow,
-                                           const int2* __restrict__ Ck, const double* __restrict__ sC, int n, Put put) {
+                                           const int2* __restrict__ Ck, const double* __restrict__ sC, int n, int* big,
+                                           Put put) {
     const int2* bas = (const int2*)(sm + L.bas);
     const int* rows = (const int*)(sm + L.rows);
     const int* cnt = (const int*)(sm + L.cnt);
@@ -210,6 +220,7 @@ __device__ __forceinline__ void contract64(const Basis64Layout& L, const unsigne
     int lg = 4;
     while (lg > 0 && (n << lg) > (int)blockDim.x) --lg;
     const int S = 1 << lg, items = (n << lg);
+    int mx[5] = {0, 0, 0, 0, 0};
     for (int o0 = threadIdx.x & ~31; o0 < items; o0 += blockDim.x) {   // whole warps
         const int o = o0 + (threadIdx.x & 31), sl = o & (S - 1);
         const int j = min(o >> lg, n - 1);
@@ -231,12 +242,69 @@ __device__ __forceinline__ void contract64(const Basis64Layout& L, const unsigne
             for (int c = 0; c < 5; ++c) {
                 sum[c].hi += __shfl_xor_sync(0xffffffffu, sum[c].hi, k);
                 sum[c].lo += __shfl_xor_sync(0xffffffffu, sum[c].lo, k);
+                sum[c].rem += __shfl_xor_sync(0xffffffffu, sum[c].rem, k);
             }
         if (o >= items) continue;
         const double sj = sC[j];
 #pragma unroll
         for (int c = 0; c < 5; ++c)
-            if ((c & (S - 1)) == sl) put(c, j, sum[c].value() * sj * fx_scale(cnt[8 + c]));   // every lane shares the outputs
+            if ((c & (S - 1)) == sl) {   // every lane takes its share of the outputs
+                const double v = sum[c].value();
+                mx[c] = max(mx[c], fx_expo(v));
+                put(c, j, v * sj * fx_scale(cnt[8 + c]));
+            }
+    }
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+        const int m = warp_max_u(mx[c]);
+        if ((threadIdx.x & 31) == 0 && m) atomicMax(&big[c], m);
+    }
+}
+
+// The same orbitals from every basis function in FP64 (bas: 5 n_basis doubles
+// of shared memory).  Starts and ends synchronised.
+template <typename Put>
+__device__ __noinline__ void orbitals_plain(const DevSys& s, const double r[3], const double* __restrict__ C, int n,
+                                            double* bas, Put put) {
+    const int nb = s.n_basis;
+    __syncthreads();
+    for (int sh = threadIdx.x; sh < s.n_shell; sh += blockDim.x) shell_vgl<double>(s, sh, r, bas, nb);
+    __syncthreads();
+    for (int o = threadIdx.x; o < 5 * n; o += blockDim.x) {
+        const int c = o / n, j = o - c * n;
+        double acc = 0.0;
+        for (int l = 0; l < nb; ++l) acc += C[(size_t)l * n + j] * bas[c * nb + l];
+        put(c, j, acc);
+    }
+    __syncthreads();
+}
+
+// Basis and orbitals at (r0, r1, r2) of one or two (C2, n2 > 0) coefficient
+// blocks, all threads; ends synchronised.  The first block's nuclear offsets
+// stay in nuc (basis64).
+template <typename Put, typename Put2>
+__device__ __forceinline__ void orbitals64(const DevSys& s, const Basis64Layout& L, unsigned char* sm, double r0,
+                                           double r1, double r2, const int2* Ck, const double* sC, const double* C,
+                                           int n, Put put, const int2* Ck2, const double* sC2, const double* C2, int n2,
+                                           Put2 put2) {
+    int* cnt = (int*)(sm + L.cnt);
+    const int nrow = basis64(s, L, sm, r0, r1, r2);
+    contract64(L, sm, nrow, Ck, sC, n, cnt + 16, put);
+    if (n2 > 0) contract64(L, sm, nrow, Ck2, sC2, n2, cnt + 24, put2);
+    __syncthreads();
+    // integer sums of the largest possible product: 2^56 (biased 1079)
+    bool low = false, low2 = false;
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+        const int e = cnt[8 + c];
+        if (e == 0 || e == 2047) continue;   // an all-zero component, or not finite
+        low |= cnt[16 + c] < 1079 - 4;
+        low2 |= cnt[24 + c] < 1079 - 4;
+    }
+    if (low || (low2 && n2 > 0)) {
+        const double r[3] = {r0, r1, r2};
+        orbitals_plain(s, r, C, n, (double*)(sm + L.bas), put);
+        if (n2 > 0) orbitals_plain(s, r, C2, n2, (double*)(sm + L.bas), put2);
     }
 }
 

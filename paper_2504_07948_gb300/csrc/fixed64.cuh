@@ -66,22 +66,23 @@ struct FxDot {
         mid += (long long)a.x * b.y;
         mid += (long long)a.y * b.x;
     }
-    // the block's sum in units of 2^58, below 2^62 in magnitude
-    __device__ __forceinline__ long long block() const { return hh + ((mid + (1LL << (kFxLimb - 1))) >> kFxLimb); }
 };
 
-// Sum of blocks: 32-bit split, so that any number of them adds exactly.
+// Sum of blocks, exact (the order of the terms does not matter): units of
+// 2^58 split in 32-bit halves, and the part below.
 struct FxSum {
-    long long hi = 0, lo = 0;
+    long long hi = 0, lo = 0, rem = 0;
     __device__ __forceinline__ void fold(FxDot& d) {
-        const long long v = d.block();
+        const long long v = d.hh + (d.mid >> kFxLimb);   // below 2^62 in magnitude
         hi += v >> 32;
         lo += v & 0xffffffffLL;
+        rem += d.mid & ((1LL << kFxLimb) - 1);
         d.hh = 0;
         d.mid = 0;
     }
     __device__ __forceinline__ double value() const {
-        const long long h = hi + (lo >> 32), l = lo & 0xffffffffLL;
+        const long long t = lo + ((rem + (1LL << (kFxLimb - 1))) >> kFxLimb);
+        const long long h = hi + (t >> 32), l = t & 0xffffffffLL;
         if (h == (long long)(int)h) return (double)(long long)(((unsigned long long)h << 32) | (unsigned long long)l);
         return (double)h * 4294967296.0 + (double)l;
     }

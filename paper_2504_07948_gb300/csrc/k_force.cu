@@ -214,18 +214,6 @@ __device__ __forceinline__ void run_terms(const DevSys& s, int sh0, int sh1, boo
     v[6] = v[7] = T(0);
 }
 
-// Reciprocal of a value known to be finite and at least 1: the FP64 form
-// refines the hardware's 20-bit approximation y by 1/x = y (1 + e + e^2 +
-// ...), e = 1 - x y, to the last bit or two (3 FP64 instructions instead of a
-// division's 7).
-__device__ __forceinline__ double rcp_ge1(double x) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
-__device__ __forceinline__ float rcp_ge1(float x) { return 1.0f / x; }
-
 // Shared-memory head of every force kernel: positions (FP64), the per-atom
 // sums acc[nn][6] (FP64: dT (3), dlnpsi (3)), grad_i J and grad_i ln|psi|
 // in the form's type T, and the positions split as hi + lo floats, from
@@ -461,6 +449,12 @@ __device__ __forceinline__ double warp_limbs(const double* x, int2* q, int n) {
     return fx_scale(e);
 }
 
+// Reciprocal of a scale (a power of two from fx_scale; NaN and 0 to NaN).
+__device__ __forceinline__ double fx_inverse(double scale) {
+    const int e = fx_expo(scale);
+    return e == 0 || e == 2047 ? fx_double(0x7ff8000000000000LL) : fx_double((long long)(2046 - e) << 52);
+}
+
 // Groups of kForceRows rows that a warp of force_walker forms together: as
 // many (at most 3, and within the warp's scratch) as fill its lanes best.
 __host__ __device__ inline int force_row_groups(int n) {
@@ -586,8 +580,13 @@ __device__ __forceinline__ void force_walker(const DevSys& s, const DevWalkers& 
                 T* at = (T*)(sAT + (size_t)r * ld);
                 T* bt = (T*)(sB + (size_t)r * ld);
                 for (int q = lane; q < n; q += 32) {
-                    at[q] = ATg[(size_t)r * n + q];
-                    bt[q] = b_of(r, q);
+                    T a = ATg[(size_t)r * n + q], b = b_of(r, q);
+                    if constexpr (kFx) {   // orbital q in units of its largest coefficient
+                        a *= s.Ck_s[spin][q];
+                        b *= fx_inverse(s.Ck_s[spin][q]);
+                    }
+                    at[q] = a;
+                    bt[q] = b;
                 }
                 if constexpr (kFx) {
                     const double a = warp_limbs(at, (int2*)at, n), b = warp_limbs(bt, (int2*)bt, n);
@@ -603,8 +602,11 @@ __device__ __forceinline__ void force_walker(const DevSys& s, const DevWalkers& 
             for (int r0 = wid * rows; r0 < n; r0 += nw * rows) {
                 const int nl = min(rows, n - r0);
                 T* pt = (T*)(sPT + (size_t)r0 * ld);
+                // (FP64 form: column p in units of electron p's row of A^-T, as
+                // the limbs of M take it below, so that an electron far out, whose
+                // row of A^-T is large, leaves the others their bits)
                 warp_rows(nl, n, sAT + (size_t)r0 * ld, ld, sB, ld, [&](int r, int p, T v) {
-                    if constexpr (kFx) v = v * sA[r0 + r] * sBs[p];
+                    if constexpr (kFx) v = v * sA[r0 + r] * sBs[p] * sA[p];
                     pt[r * ld + p] = v;
                 });
                 if constexpr (kFx) {
@@ -642,12 +644,14 @@ __device__ __forceinline__ void force_walker(const DevSys& s, const DevWalkers& 
                     if constexpr (kFx) {
                         const double* sC = s.Cq_s[spin] + l0;
                         warp_rows(nl, n, s.Cq[spin] + (size_t)l0 * n, n, sAT, ld,
-                                  [&](int r, int i, double v) { m[r * nmax + i] = v * sC[r] * sA[i]; });
+                                  [&](int r, int i, double v) { m[r * nmax + i] = v * sC[r]; });
                         __syncwarp();
                         double sM[3 * kForceRows];
 #pragma unroll
                         for (int r = 0; r < 3 * kForceRows; ++r)
                             sM[r] = r < nl ? warp_limbs(m + r * nmax, scr + r * n, n) : 0.0;
+                        for (int r = 0; r < nl; ++r)
+                            for (int i = lane; i < n; i += 32) m[r * nmax + i] *= sA[i];
                         __syncwarp();
                         warp_rows(nl, n, scr, n, sPT, ld, [&](int r, int i, double v) {
                             double a = 0.0;

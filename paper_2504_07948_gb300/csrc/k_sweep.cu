@@ -12,7 +12,7 @@
 // form, in float in the mixed form) and, when accepted, applies
 //   A^-1 <- A^-1 - (A^-1 e_e)(phi'^T A^-1 - e_e^T) / rho
 // row by row (one warp per row of the transposed inverse).
-#include "sweep_sm.cuh"
+#include "sweep64.cuh"
 
 namespace qmc {
 
@@ -29,6 +29,25 @@ __global__ void __launch_bounds__(kNt, sizeof(T) == 4 ? (kNt == 128 ? 7 : 3) : (
     sweep_walker<T, (kNt > 128), kJ3>(s, wk, w, p, smem);   // 128 threads: n <= 64 only
 }
 
+// The FP64 form (sweep64.cuh); k_sweep<double> is left for bases whose lists
+// exceed shared memory.
+template <int kNt, bool kJ3>
+__global__ void __launch_bounds__(kNt, kNt == 128 ? 5 : 2) k_sweep64(DevSys s, DevWalkers wk, int W, SweepParams p) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    if ((int)blockIdx.x >= W) return;
+    sweep_walker64<kJ3>(s, wk, blockIdx.x, p, smem);
+}
+
+template <int kNt>
+static cudaError_t launch_sweep64(const DevSys& s, const DevWalkers& wk, int W, const SweepParams& p, size_t smem,
+                                  cudaStream_t st) {
+    const auto f = s.n3 > 0 ? k_sweep64<kNt, true> : k_sweep64<kNt, false>;
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    f<<<W, kNt, smem, st>>>(s, wk, W, p);
+    return cudaGetLastError();
+}
+
 // The sweep of a trial function with the three-body Jastrow (kJ3).
 template <typename T, int kNt>
 static cudaError_t launch_sweep_j3(const DevSys& s, const DevWalkers& wk, int W, const SweepParams& p,
@@ -41,6 +60,7 @@ static cudaError_t launch_sweep_j3(const DevSys& s, const DevWalkers& wk, int W,
 
 template <typename T>
 size_t sweep_smem_bytes(const DevSys& s, int ainv_smem, int g_smem) {
+    if (sizeof(T) == 8 && sweep64_fits(s)) return Sweep64Layout(s, ainv_smem, g_smem).total;
     size_t a, b, c, d, e;
     return sweep_smem_layout<T>(s.N, s.n_basis, s.n_up, s.n_dn, ainv_smem, g_smem, &a, &b, &c, &d, &e);
 }
@@ -51,6 +71,8 @@ cudaError_t launch_sweep(const DevSys& s, const DevWalkers& wk, int W, const Swe
     if (W == 0 || s.N == 0) return cudaSuccess;
     const size_t smem = sweep_smem_bytes<T>(s, p.ainv_smem, p.g_smem);
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
+    if (sizeof(T) == 8 && sweep64_fits(s))
+        return nmax > 64 ? launch_sweep64<256>(s, wk, W, p, smem, st) : launch_sweep64<128>(s, wk, W, p, smem, st);
     if (s.n3 > 0)
         return nmax > 64 ? launch_sweep_j3<T, 256>(s, wk, W, p, n_live, smem, st)
                          : launch_sweep_j3<T, 128>(s, wk, W, p, n_live, smem, st);

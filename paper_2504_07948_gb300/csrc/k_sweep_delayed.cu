@@ -21,7 +21,7 @@
 // a float copy of K^-1 y.
 #include "batch.cuh"
 #include "qmc_internal.cuh"
-#include "sweep_sm.cuh"
+#include "sweep64.cuh"
 
 namespace qmc {
 
@@ -459,7 +459,7 @@ cudaError_t launch_sweep_delayed(const DevSys& s, const DevWalkers& wk, int W, c
 // which no system uses delayed updates.
 // ---------------------------------------------------------------------
 template <typename T, bool kDelayed>
-__global__ void __launch_bounds__(256, 3)
+__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 3)
     k_sweep_batch(const BatchSys* __restrict__ sys, BatchPlan* plan, const BatchCtl* __restrict__ ctl, int parity,
                   double tau, int ctr) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -480,7 +480,9 @@ __global__ void __launch_bounds__(256, 3)
         p.g_smem = 0;
         if (kDelayed && bs.delay_rank > 1)
             sweep_delayed_walker<T>(bs.s, bs.wk[parity], s_idx, p, bs.delay_rank, smem);
-        else
+        else if (sizeof(T) == 8 && sweep64_fits(bs.s)) {
+            if constexpr (sizeof(T) == 8) sweep_walker64<false>(bs.s, bs.wk[parity], s_idx, p, smem);
+        } else
             sweep_walker<T>(bs.s, bs.wk[parity], s_idx, p, smem);
         __syncthreads();
     }

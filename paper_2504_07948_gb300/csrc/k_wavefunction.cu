@@ -9,70 +9,44 @@
 
 namespace qmc {
 
-// Orbitals of electron i of walker w without lists or limbs (see
-// orbitals_item), for a basis whose lists exceed shared
-// memory (about 2500 functions): 5 n_basis doubles of it.
-template <typename T>
-__device__ __noinline__ void orbitals_item_plain(const DevSys& s, const DevWalkers& wk, int w, int i, double* bas) {
-    const int nb = s.n_basis;
-    const double* r = wk.R + ((size_t)w * s.N + i) * 3;
-    for (int sh = threadIdx.x; sh < s.n_shell; sh += blockDim.x) shell_vgl<double>(s, sh, r, bas, nb);
-    __syncthreads();
-    const int spin = i < s.n_up ? 0 : 1, n = spin ? s.n_dn : s.n_up, k = spin ? i - s.n_up : i;
-    for (int vir = 0; vir < (s.msd ? 2 : 1); ++vir) {
-        const int nj = vir ? s.n_vir[spin] : n;
-        const double* C = vir ? s.Cv[spin] : s.C[spin];
-        T* G = (T*)(vir ? wk.Gv[spin] : wk.G[spin]) + ((size_t)w * n + k) * 4 * nj;
-        for (int o = threadIdx.x; o < 5 * nj; o += blockDim.x) {
-            const int c = o / nj, j = o - c * nj;
-            double acc = 0.0;
-            for (int l = 0; l < nb; ++l) acc += C[(size_t)l * nj + j] * bas[c * nb + l];
-            if (c)
-                G[(c - 1) * nj + j] = (T)acc;
-            else if (vir)
-                ((T*)wk.Av[spin])[((size_t)w * n + k) * nj + j] = (T)acc;
-            else
-                wk.Ascr[spin][((size_t)w * n + k) * n + j] = acc;
-        }
-    }
-}
-
 // Orbitals of electron i of walker w by one CTA (body of k_orbitals_all):
 // the live basis functions at r_i in FP64 and the LCAO contraction phi_j =
 // sum_l C_l^j Phi_l (Eq. 2) in fixed point (basis64.cuh) for the occupied
-// orbitals of the electron's spin.  A goes to FP64 scratch, the gradient and
-// Laplacian rows to the walker cache in the storage type T.  sm:
-// orbitals_smem_bytes of shared memory.
+// orbitals of the electron's spin and the active virtual ones of a
+// determinant expansion.  A goes to FP64 scratch, the gradient and Laplacian
+// rows to the walker cache in the storage type T.  sm: orbitals_smem_bytes of
+// shared memory (a basis whose lists exceed it, about 2500 functions, is
+// contracted in FP64).
 template <typename T>
 __device__ __forceinline__ void orbitals_item(const DevSys& s, const DevWalkers& wk, int w, int i, unsigned char* sm) {
     const Basis64Layout L(s.n_nuc, s.n_prim, s.n_shell, s.n_basis);
-    if (L.total > kBasis64Max) {
-        orbitals_item_plain<T>(s, wk, w, i, (double*)sm);
-        return;
-    }
-    const double* r = wk.R + ((size_t)w * s.N + i) * 3;
-    const int nrow = basis64(s, L, sm, r[0], r[1], r[2]);
+    const double* rp = wk.R + ((size_t)w * s.N + i) * 3;
+    const double r[3] = {rp[0], rp[1], rp[2]};
     const int spin = i < s.n_up ? 0 : 1;
-    const int n = spin ? s.n_dn : s.n_up;
+    const int n = spin ? s.n_dn : s.n_up, nv = s.msd ? s.n_vir[spin] : 0;
     const int k = spin ? i - s.n_up : i;
     T* G = (T*)wk.G[spin] + ((size_t)w * n + k) * 4 * n;
     double* A = wk.Ascr[spin] + ((size_t)w * n + k) * n;
-    contract64(L, sm, nrow, s.Ck[spin], s.Ck_s[spin], n, [&](int c, int j, double v) {
+    T* Av = (T*)wk.Av[spin] + ((size_t)w * n + k) * nv;
+    T* Gv = (T*)wk.Gv[spin] + ((size_t)w * n + k) * 4 * nv;
+    const auto put = [&](int c, int j, double v) {
         if (c == 0)
             A[j] = v;
         else
             G[(c - 1) * n + j] = (T)v;
-    });
-    if (s.msd && s.n_vir[spin] > 0) {  // active virtual orbitals of a determinant expansion
-        const int nv = s.n_vir[spin];
-        T* Av = (T*)wk.Av[spin] + ((size_t)w * n + k) * nv;
-        T* Gv = (T*)wk.Gv[spin] + ((size_t)w * n + k) * 4 * nv;
-        contract64(L, sm, nrow, s.Cvk[spin], s.Cvk_s[spin], nv, [&](int c, int j, double v) {
-            if (c == 0)
-                Av[j] = (T)v;
-            else
-                Gv[(c - 1) * nv + j] = (T)v;
-        });
+    };
+    const auto put_v = [&](int c, int j, double v) {
+        if (c == 0)
+            Av[j] = (T)v;
+        else
+            Gv[(c - 1) * nv + j] = (T)v;
+    };
+    if (L.total <= kBasis64Max) {
+        orbitals64(s, L, sm, r[0], r[1], r[2], s.Ck[spin], s.Ck_s[spin], s.C[spin], n, put, s.Cvk[spin], s.Cvk_s[spin],
+                   s.Cv[spin], nv, put_v);
+    } else {
+        orbitals_plain(s, r, s.C[spin], n, (double*)sm, put);
+        if (nv > 0) orbitals_plain(s, r, s.Cv[spin], nv, (double*)sm, put_v);
     }
 }
 

@@ -555,20 +555,27 @@ struct qmc_ctx {
                 for (int j = 0; j < n; ++j) Cs[(size_t)l * n + j] = C[(size_t)occ[j] * n_basis + l];
             s.C[spin] = upload(sys_allocs, Cs);
             s.C_f[spin] = upload(sys_allocs, std::vector<float>(Cs.begin(), Cs.end()));
+            upload_columns(Cs, n_basis, n, &s.Ck[spin], &s.Ck_s[spin]);
             {
-                const size_t n = occ.size();
+                // the rows' limbs, every orbital in units of its column's scale
                 std::vector<int2> q(Cs.size());
-                std::vector<double> sc(n_basis);
+                std::vector<double> sc(n_basis), row(n);
+                std::vector<int> ce(n, 0);
+                for (int l = 0; l < n_basis; ++l)
+                    for (int j = 0; j < n; ++j) ce[j] = std::max(ce[j], fx_expo(Cs[(size_t)l * n + j]));
                 for (int l = 0; l < n_basis; ++l) {
                     int e = 0;
-                    for (size_t j = 0; j < n; ++j) e = std::max(e, fx_expo(Cs[l * n + j]));
-                    for (size_t j = 0; j < n; ++j) q[l * n + j] = fx_limbs(Cs[l * n + j], e);
+                    for (int j = 0; j < n; ++j) {
+                        const double u = fx_scale(ce[j]);
+                        row[j] = u != 0.0 ? Cs[(size_t)l * n + j] / u : 0.0;
+                        e = std::max(e, fx_expo(row[j]));
+                    }
+                    for (int j = 0; j < n; ++j) q[(size_t)l * n + j] = fx_limbs(row[j], e);
                     sc[l] = fx_scale(e);
                 }
                 s.Cq[spin] = upload(sys_allocs, q);
                 s.Cq_s[spin] = upload(sys_allocs, sc);
             }
-            upload_columns(Cs, n_basis, n, &s.Ck[spin], &s.Ck_s[spin]);
         }
         if (have_msd) build_multidet(s);
         ds = s;
