@@ -34,7 +34,7 @@
 namespace qmc {
 
 struct Basis64Layout {
-    size_t nuc, ev, fs, bas, plist, slist, flist, rows, cnt, total;
+    size_t nuc, ev, fs, bas, tf, plist, slist, flist, rows, cnt, total;
     int ldb;
     __host__ __device__ Basis64Layout(int n_nuc, int n_prim, int n_shell, int n_basis) {
         ldb = (n_basis + 1) & ~1;
@@ -47,6 +47,8 @@ struct Basis64Layout {
         o += sizeof(double) * 3 * (size_t)n_shell;
         bas = o;
         o += sizeof(double) * 5 * (size_t)ldb;
+        tf = o;
+        o += sizeof(float) * (size_t)n_nuc;
         plist = o;
         o += sizeof(int) * (size_t)n_prim;
         slist = o;
@@ -75,6 +77,7 @@ __device__ __forceinline__ int basis64(const DevSys& s, const Basis64Layout& L, 
     double* ev = (double*)(sm + L.ev);
     double* fs = (double*)(sm + L.fs);
     double* bas = (double*)(sm + L.bas);
+    float* tf = (float*)(sm + L.tf);
     int* plist = (int*)(sm + L.plist);
     int* slist = (int*)(sm + L.slist);
     int* flist = (int*)(sm + L.flist);   // functions by kind: s from 0, p from n_fn_s, d from n_fn_s + n_fn_p
@@ -86,13 +89,15 @@ __device__ __forceinline__ int basis64(const DevSys& s, const Basis64Layout& L, 
     for (int q = tid; q < 32; q += nt) cnt[q] = 0;
     for (int a = tid; a < s.n_nuc; a += nt) {
         const double x = r0 - s.Rn[3 * a], y = r1 - s.Rn[3 * a + 1], z = r2 - s.Rn[3 * a + 2];
-        nuc[a] = make_double4(x, y, z, x * x + y * y + z * z);
+        const double t = x * x + y * y + z * z;
+        nuc[a] = make_double4(x, y, z, t);
+        tf[a] = (float)t;   // a conversion costs the FP64 pipe as much as an addition
     }
     __syncthreads();
     const float cut = (float)kScreenExponent;
     for (int p0 = tid - lane; p0 < s.n_prim; p0 += nt) {
         const int p = p0 + lane;
-        const bool live = p < s.n_prim && !(s.alpha_f[p] * (float)nuc[s.prim_ctr[p]].w > cut);
+        const bool live = p < s.n_prim && !(s.alpha_f[p] * tf[s.prim_ctr[p]] > cut);
         const unsigned m = __ballot_sync(0xffffffffu, live);
         int base = 0;
         if (lane == 0 && m) base = atomicAdd(&cnt[0], __popc(m));
@@ -101,7 +106,7 @@ __device__ __forceinline__ int basis64(const DevSys& s, const Basis64Layout& L, 
     }
     for (int q0 = tid - lane; q0 < s.n_shell; q0 += nt) {
         const int sh = q0 + lane;
-        const bool live = sh < s.n_shell && !(s.shell_amin_f[sh] * (float)nuc[s.shell[sh].x].w > cut);
+        const bool live = sh < s.n_shell && !(s.shell_amin_f[sh] * tf[s.shell[sh].x] > cut);
         const unsigned m = __ballot_sync(0xffffffffu, live);
         int base = 0;
         if (lane == 0 && m) base = atomicAdd(&cnt[1], __popc(m));
@@ -118,10 +123,10 @@ __device__ __forceinline__ int basis64(const DevSys& s, const Basis64Layout& L, 
         const int sh = slist[k];
         const int4 d = s.shell[sh];
         const double t = nuc[d.x].w;
-        const float tf = (float)t;
+        const float tc = tf[d.x];
         double f0 = 0.0, f1 = 0.0, f2 = 0.0;
         for (int p = d.z; p < d.z + d.w; ++p) {
-            if (s.alpha_f[p] * tf > cut) continue;
+            if (s.alpha_f[p] * tc > cut) continue;
             const double a = s.alpha[p], e = ev[p], e1 = a * e;
             f0 += e;
             f1 -= e1;
@@ -160,22 +165,41 @@ __device__ __forceinline__ int basis64(const DevSys& s, const Basis64Layout& L, 
         } else if (kind == 1) {
             const double P = f == 0 ? x.x : f == 1 ? x.y : x.z, Pg = P * g1;
             v[0] = P * f0;
-            v[1] = x.x * Pg;
-            v[2] = x.y * Pg;
-            v[3] = x.z * Pg;
-            if (f == 0) v[1] += f0;
-            if (f == 1) v[2] += f0;
-            if (f == 2) v[3] += f0;
+            v[1] = fma(x.x, Pg, f == 0 ? f0 : 0.0);
+            v[2] = fma(x.y, Pg, f == 1 ? f0 : 0.0);
+            v[3] = fma(x.z, Pg, f == 2 ? f0 : 0.0);
             v[4] = P * gl;
         } else {
-            const AngPoly<double> a = angular<double>(2, d.y >> 8, f, x.x, x.y, x.z);
-            const double Pg = a.P * g1;
-            v[0] = a.P * f0;
-            v[1] = x.x * Pg + a.Px * f0;
-            v[2] = x.y * Pg + a.Py * f0;
-            v[3] = x.z * Pg + a.Pz * f0;
-            v[4] = a.P * gl;
-            if ((d.y >> 8) == 0) v[4] += (a.Hxx + a.Hyy + a.Hzz) * f0;   // pure d functions are harmonic
+            // sqrt3 u v of two coordinates, or a x^2 + b y^2 + c z^2 (gradient
+            // 2 (a x, b y, c z)); Cartesian squares are not harmonic (tr H)
+            const double s3 = 1.7320508075688772;
+            const bool pure = (d.y >> 8) != 0;
+            const int uv = pure ? (f == 0 ? 1 : f == 1 ? 6 : f == 3 ? 2 : 0)      // 3 u + v of (0, 1), (1, 2), (0, 2)
+                                : (f == 1 ? 1 : f == 2 ? 2 : f == 4 ? 6 : 0);
+            double P, gx, gy, gz, tr = 0.0;
+            if (uv) {
+                const double su = s3 * (uv == 6 ? x.y : x.x), vv = uv == 1 ? x.y : x.z, sv = s3 * vv;
+                P = su * vv;
+                gx = uv == 6 ? 0.0 : sv;
+                gy = uv == 1 ? su : uv == 6 ? sv : 0.0;
+                gz = uv == 1 ? 0.0 : su;
+            } else {
+                const double a = pure ? (f == 2 ? -1.0 : s3) : (f == 0 ? 2.0 : 0.0);
+                const double b = pure ? (f == 2 ? -1.0 : -s3) : (f == 3 ? 2.0 : 0.0);
+                const double c = pure ? (f == 2 ? 2.0 : 0.0) : (f == 5 ? 2.0 : 0.0);
+                gx = a * x.x;
+                gy = b * x.y;
+                gz = c * x.z;
+                P = 0.5 * (gx * x.x + gy * x.y + gz * x.z);
+                tr = pure ? 0.0 : 2.0;
+            }
+            const double Pg = P * g1;
+            v[0] = P * f0;
+            v[1] = x.x * Pg + gx * f0;
+            v[2] = x.y * Pg + gy * f0;
+            v[3] = x.z * Pg + gz * f0;
+            v[4] = P * gl;
+            if (!pure) v[4] += tr * f0;
         }
         const int r = q + (kind == 0 ? 0 : kind == 1 ? ns : ns + np);
         rows[r] = s.shell_fn[sh] + f;

@@ -30,9 +30,12 @@ __global__ void __launch_bounds__(kNt, sizeof(T) == 4 ? (kNt == 128 ? 7 : 3) : (
 }
 
 // The FP64 form (sweep64.cuh); k_sweep<double> is left for bases whose lists
-// exceed shared memory.
+// exceed shared memory.  256 threads above 64 electrons per spin, 64 where two
+// warps hold a move's partners (electrons and nuclei; 2048 walkers of 1, 2 and
+// 4 waters: 629 -> 529, 1299 -> 1110 and 3139 -> 2801 us a sweep against 128
+// threads, 6 waters 6.0 -> 7.1 ms), else 128.
 template <int kNt, bool kJ3>
-__global__ void __launch_bounds__(kNt, kNt == 128 ? 5 : 2) k_sweep64(DevSys s, DevWalkers wk, int W, SweepParams p) {
+__global__ void __launch_bounds__(kNt, kNt <= 64 ? 8 : kNt == 128 ? 5 : 2) k_sweep64(DevSys s, DevWalkers wk, int W, SweepParams p) {
     extern __shared__ __align__(16) unsigned char smem[];
     if ((int)blockIdx.x >= W) return;
     sweep_walker64<kJ3>(s, wk, blockIdx.x, p, smem);
@@ -72,7 +75,9 @@ cudaError_t launch_sweep(const DevSys& s, const DevWalkers& wk, int W, const Swe
     const size_t smem = sweep_smem_bytes<T>(s, p.ainv_smem, p.g_smem);
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
     if (sizeof(T) == 8 && sweep64_fits(s))
-        return nmax > 64 ? launch_sweep64<256>(s, wk, W, p, smem, st) : launch_sweep64<128>(s, wk, W, p, smem, st);
+        return nmax > 64                ? launch_sweep64<256>(s, wk, W, p, smem, st)
+               : s.N + s.n_nuc > 64 ? launch_sweep64<128>(s, wk, W, p, smem, st)
+                                    : launch_sweep64<64>(s, wk, W, p, smem, st);
     if (s.n3 > 0)
         return nmax > 64 ? launch_sweep_j3<T, 256>(s, wk, W, p, n_live, smem, st)
                          : launch_sweep_j3<T, 128>(s, wk, W, p, n_live, smem, st);

@@ -14,8 +14,9 @@
 //     ratios, once per sweep;
 //   - pair terms and determinant terms sum in separate warps (a butterfly over
 //     four values), reciprocals of values >= 1 by one refinement step.
-// 6-water cluster, 2048 walkers: 9.9 -> 6.1 ms a sweep (1345 FP64 warp
-// instructions a move before).
+//   - a move's serial part runs on three lanes, one component each.
+// 6-water cluster, 2048 walkers: 9.9 -> 5.8 ms a sweep (1345 -> about 600 FP64
+// warp instructions a move); one water, 512 walkers: 283 -> 180 us.
 #pragma once
 
 #include "basis64.cuh"
@@ -76,20 +77,28 @@ __device__ __forceinline__ double sqrt_ge1(double x) {
     return fma(t, e * fma(e, 0.375, 0.5), t);
 }
 
-// Factor of the capped drift, v * 2 / (1 + sqrt(1 + 2 v^2 tau)).
-__device__ __forceinline__ double drift_factor(double gx, double gy, double gz, double tau) {
-    const double a = 1.0 + 2.0 * (gx * gx + gy * gy + gz * gz) * tau;
+// Factor of the capped drift, 2 / (1 + sqrt(1 + 2 v^2 tau)).
+__device__ __forceinline__ double drift_factor(double v2, double tau) {
+    const double a = fma(2.0 * v2, tau, 1.0);
     if (!(a < 1e300)) return 2.0 / (1.0 + sqrt(a));   // infinite or undefined gradients
     return 2.0 * rcp_ge1(1.0 + sqrt_ge1(a));
 }
 
+// Reciprocal of a finite positive value: one refinement of the hardware's
+// approximation (see rcp_ge1) where neither it nor the error term leaves the
+// normal range, else a division.
+__device__ __forceinline__ double rcp_pos(double x) {
+    const int e = fx_expo(x);
+    return e > 64 && e < 1983 ? rcp_ge1(x) : 1.0 / x;
+}
+
 // Sums over the CTA of the pair terms v (from the low threads up) and the
 // determinant terms d (from the high threads down): per warp only what it
-// holds (pw, dw: warp-uniform).  Thread 0 gets v[0..3], d[0..3] in out after
-// the second barrier it must pass; ends synchronised.  red: 8 x 8 doubles
-// for the at most 8 warps of a sweep CTA.
-__device__ __forceinline__ void sweep64_sum(const double (&v)[4], const double (&d)[4], bool pw, bool dw, double* red,
-                                            double* out) {
+// holds (pw, dw: warp-uniform).  Returns v[lane] (lane < 4) and d[lane - 4]
+// (lane < 8) to warp 0.  red: 8 x 8 doubles for the at most 8 warps of a
+// sweep CTA.
+__device__ __forceinline__ double sweep64_sum(const double (&v)[4], const double (&d)[4], bool pw, bool dw,
+                                              double* red) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const double a = pw ? warp_fold4(v) : 0.0, b = dw ? warp_fold4(d) : 0.0;
     if ((lane & 7) == 0) {
@@ -98,12 +107,17 @@ __device__ __forceinline__ void sweep64_sum(const double (&v)[4], const double (
         red[wid * 8 + 4 + q] = b;
     }
     __syncthreads();
+    double t = 0.0;
     if (threadIdx.x < 8) {
-        double t = 0.0;
-        for (int q = 0; q < nw; ++q) t += red[q * 8 + threadIdx.x];
-        out[threadIdx.x] = t;
+        t = red[threadIdx.x];
+        for (int q = 1; q < nw; ++q) t += red[q * 8 + threadIdx.x];
     }
-    __syncwarp();
+    return t;
+}
+
+// Sum of lanes 0, 1, 2, in every lane of the warp.
+__device__ __forceinline__ double sum3(double x) {
+    return __shfl_sync(0xffffffffu, x, 0) + __shfl_sync(0xffffffffu, x, 1) + __shfl_sync(0xffffffffu, x, 2);
 }
 
 // One CTA (at most 256 threads) sweeps walker w (every electron once).
@@ -118,7 +132,7 @@ __device__ __forceinline__ void sweep_walker64(const DevSys& s, const DevWalkers
     double* sR = (double*)(smem + L.sR);
     double* chi = (double*)(smem + L.chi);      // [N][4]: three normals, ln of the acceptance uniform
     double* red = (double*)(smem + L.red);
-    double* scal = (double*)(smem + L.scal);    // [0..2] r', [3..5] drift, [6] 1 / ratio, [7] accept, [8..15] sums
+    double* scal = (double*)(smem + L.scal);    // [0..2] r', [3] 1 / ratio, [4] accept
     double* phi = (double*)(smem + L.phi);
     double* cold = (double*)(smem + L.cold);
     double* fq = cold + nmax;
@@ -158,8 +172,8 @@ __device__ __forceinline__ void sweep_walker64(const DevSys& s, const DevWalkers
         chi[4 * e + 3] = log(u01(philox4x32_10(make_uint4(p.sweep, (uint32_t)e, (uint32_t)w, 1u), p.key).x));
     const double tau = p.tau, sqt = sqrt(tau), i2t = 1.0 / (2.0 * tau);
     // product of the accepted ratios per spin, as mantissa and power of two
-    double pm[2] = {1.0, 1.0};
-    int pe[2] = {0, 0};
+    double pm0 = 1.0, pm1 = 1.0;
+    int pe0 = 0, pe1 = 0;
     unsigned long long acc = 0;
     __syncthreads();
 
@@ -208,19 +222,17 @@ __device__ __forceinline__ void sweep_walker64(const DevSys& s, const DevWalkers
                 v[3] += gg[2];
             }
         }
-        sweep64_sum(v, d, pw, dw, red, scal + 8);
-        double u_old = 0.0;
-        if (tid == 0) {
-            u_old = scal[8];
-            const double g0 = scal[9] + scal[13], g1 = scal[10] + scal[14], g2 = scal[11] + scal[15];
-            const double f = drift_factor(g0, g1, g2, tau);
-            const double vb[3] = {f * g0, f * g1, f * g2};
-            const double ro[3] = {re0, re1, re2};
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                scal[c] = ro[c] + tau * vb[c] + sqt * chi[4 * e + c];
-                scal[3 + c] = vb[c];
-            }
+        double t = sweep64_sum(v, d, pw, dw, red);
+        // the move's serial part: warp 0, its first three lanes one component each
+        const int c3 = lane < 3 ? lane : 0;
+        double u_old = 0.0, vb = 0.0, re = 0.0, rn = 0.0;
+        if (wid == 0) {
+            u_old = __shfl_sync(0xffffffffu, t, 0);
+            const double g = __shfl_sync(0xffffffffu, t, 1 + c3) + __shfl_sync(0xffffffffu, t, 5 + c3);
+            vb = drift_factor(sum3(g * g), tau) * g;
+            re = sR[3 * e + c3];
+            rn = fma(sqt, chi[4 * e + c3], fma(tau, vb, re));
+            if (lane < 3) scal[lane] = rn;
         }
         __syncthreads();
         const double rn0 = scal[0], rn1 = scal[1], rn2 = scal[2];
@@ -268,52 +280,56 @@ __device__ __forceinline__ void sweep_walker64(const DevSys& s, const DevWalkers
                 v[3] += gg[2];
             }
         }
-        sweep64_sum(v, d, pw, dw, red, scal + 8);
-        if (tid == 0) {
-            const double rho = scal[12];
+        t = sweep64_sum(v, d, pw, dw, red);
+        if (wid == 0) {
+            const double rho = __shfl_sync(0xffffffffu, t, 4);
             int accept = 0;
             double ir = 0.0;
-            if (rho > 0.0 && isfinite(rho)) {
-                ir = 1.0 / rho;
-                const double dJ = scal[8] - u_old;
-                const double g0 = scal[13] * ir + scal[9], g1 = scal[14] * ir + scal[10], g2 = scal[15] * ir + scal[11];
-                const double f = drift_factor(g0, g1, g2, tau);
-                const double dr[3] = {rn0 - re0, rn1 - re1, rn2 - re2}, gn[3] = {f * g0, f * g1, f * g2};
-                double diff = 0.0;   // |r - r' - tau v'|^2 - |r' - r - tau v|^2
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const double fw = dr[c] - tau * scal[3 + c], bk = dr[c] + tau * gn[c];
-                    diff += bk * bk - fw * fw;
-                }
+            if (rho > 0.0 && isfinite(rho)) {   // uniform in the warp
+                ir = rcp_pos(rho);
+                const double g = fma(__shfl_sync(0xffffffffu, t, 5 + c3), ir, __shfl_sync(0xffffffffu, t, 1 + c3));
+                const double dJ = __shfl_sync(0xffffffffu, t, 0) - u_old;
+                const double vn = drift_factor(sum3(g * g), tau) * g;
+                const double dr = rn - re, fw = fma(-tau, vb, dr), bk = fma(tau, vn, dr);
+                // |r - r' - tau v'|^2 - |r' - r - tau v|^2
+                const double diff = sum3(fma(bk, bk, -fw * fw));
                 // accept iff 2 ln rho + rest > ln u.  The logarithm in FP32 (an
                 // error below 2^-20 (1 + |ln rho|)) settles all but about one
                 // move in 10^5.
-                const double rest = 2.0 * dJ - diff * i2t - chi[4 * e + 3];
-                const float lr = logf((float)rho);
-                const double t = rest + 2.0 * (double)lr;
-                if (fabs(t) > 1e-5 * (1.0 + fabs((double)lr)) && rho < 1e30 && rho > 1e-30)
-                    accept = t > 0.0;
+                const double rest = fma(2.0, dJ, fma(-diff, i2t, -chi[4 * e + 3]));
+                const float lr = logf((float)rho), rf = (float)rest, tf = fmaf(2.0f, lr, rf);
+                if (fabsf(tf) > 1e-5f * (1.0f + fabsf(lr) + fabsf(rf)) && rho < 1e30 && rho > 1e-30)
+                    accept = tf > 0.0f;
                 else
                     accept = rest + 2.0 * log(rho) > 0.0;
             }
-            scal[6] = ir;
-            scal[7] = accept ? 1.0 : 0.0;
-            if (accept) {
-                const double m = pm[spin] * rho;
-                const long long b = fx_bits(m);
-                const int ex = (int)((b >> 52) & 0x7ff);
-                if (ex > 0 && ex < 2047 && fx_expo(rho) > 0) {
-                    pe[spin] += ex - 1023;   // m >= 0: leave its mantissa in [1, 2)
-                    pm[spin] = fx_double((b & 0xfffffffffffffLL) | (1023LL << 52));
-                } else {
-                    wk.logdet[2 * w + spin] += log(rho);   // a product out of range: add its logarithm
+            if (lane == 0) {
+                scal[3] = ir;
+                scal[4] = accept ? 1.0 : 0.0;
+                if (accept) {
+                    const double m = (spin ? pm1 : pm0) * rho;
+                    const long long b = fx_bits(m);
+                    const int ex = (int)((b >> 52) & 0x7ff);
+                    if (ex > 0 && ex < 2047 && fx_expo(rho) > 0) {
+                        // m > 0: leave its mantissa in [1, 2)
+                        const double mant = fx_double((b & 0xfffffffffffffLL) | (1023LL << 52));
+                        if (spin) {
+                            pm1 = mant;
+                            pe1 += ex - 1023;
+                        } else {
+                            pm0 = mant;
+                            pe0 += ex - 1023;
+                        }
+                    } else {
+                        wk.logdet[2 * w + spin] += log(rho);   // a product out of range: add its logarithm
+                    }
                 }
             }
         }
         __syncthreads();
-        if (scal[7] != 0.0) {
+        if (scal[4] != 0.0) {
             for (int j = tid; j < n; j += nt) cold[j] = A[(size_t)k * n + j];
-            const double rinv = scal[6];
+            const double rinv = scal[3];
             if (p.ainv_smem) {
                 // each row's dot product on its own thread, then the rank-1 update
                 for (int q = tid; q < n; q += nt) {
@@ -369,9 +385,9 @@ __device__ __forceinline__ void sweep_walker64(const DevSys& s, const DevWalkers
         for (int q = tid; q < 4 * nd * nd; q += nt) gG[1][q] = Gc[1][q];
     }
     if (tid == 0) {
-#pragma unroll
-        for (int sp = 0; sp < 2; ++sp)
-            wk.logdet[2 * w + sp] += log(pm[sp]) + (double)pe[sp] * 0.69314718055994530942;
+        const double ln2 = 0.69314718055994530942;
+        wk.logdet[2 * w] += log(pm0) + (double)pe0 * ln2;
+        wk.logdet[2 * w + 1] += log(pm1) + (double)pe1 * ln2;
         if (acc) atomicAdd(wk.n_acc, acc);
     }
 }
