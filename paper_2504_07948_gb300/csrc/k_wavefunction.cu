@@ -3,6 +3,8 @@
 // the Slater matrices, and the local energy.  These kernels serve the
 // parity entry point and the periodic FP64 recompute of the incremental
 // inverse.
+#include <algorithm>
+
 #include "basis64.cuh"
 #include "batch.cuh"
 #include "qmc_internal.cuh"
@@ -193,8 +195,6 @@ __global__ void k_invert(DevSys s, DevWalkers wk, int W, int store_fp32, unsigne
 // walker, one thread per electron; sums in FP64.
 //   E_L = sum_i -1/2 [lap_i D/D + lap_i J + 2 grad_i J . grad_i D/D
 //         + |grad_i J|^2] + V_ee + V_en + V_nn.
-// Local energy of walker w (body of k_eloc).  sR: 3 N doubles of shared
-// memory.
 // J3 seen from electron i: the value of the pairs (i, j > i) and the
 // gradient and Laplacian in r_i of every pair (i, j != i).
 __device__ void j3_electron(const DevSys& s, const double* sR, int i, double& val, double g[3], double& lap) {
@@ -225,165 +225,306 @@ __device__ void j3_electron(const DevSys& s, const double* sR, int i, double& va
     }
 }
 
+// Local energy of walker w (body of k_eloc).  The first half of the CTA's
+// threads takes the electron pairs, the second half the electron-nucleus
+// terms, the determinant and the assembly, a thread per electron each (strided
+// when the electrons outnumber it), so that the two parts run on different
+// warps at once.
+//   FP64 form (bound by its FP64 instructions): up to kElocSym electrons every
+// pair is formed once, by electron i for the cyclic neighbours i + 1 .. i + N/2,
+// and added to both: the partner's share goes to an array of the warp, in which
+// the lanes of a round touch distinct electrons.
+//   Mixed form (was bound by uncoalesced reads of the gradient cache, a row
+// per thread): the determinant sums of an electron are taken by a warp; pair
+// terms in FP32 with compensated sums, assembled in FP64.
+// 6-water cluster, 2048 walkers: 756 -> 415 us FP64, 143 -> 84 us mixed;
+// 32-water cluster, 1024 walkers, mixed: 1.84 -> 0.79 ms (a thread per electron
+// for everything before).
+// sm: eloc_smem_bytes.
+constexpr int kElocSym = 160;
+struct ElocLayout {
+    int H;                      // threads of each half
+    // byte offsets of [N][4] pair sums (mixed form [N][5]: the Laplacian as high and low word), and of the
+    // partners' shares [H / 32][4][N] or the determinant sums [N][8]
+    size_t part, other, total;
+    __host__ __device__ ElocLayout(int N, int nt, int elem) {
+        H = nt / 2;
+        const size_t pos = (sizeof(double) * 3 + sizeof(float) * 8) * (size_t)N;
+        part = (pos + 15) & ~(size_t)15;
+        other = (part + (size_t)elem * (elem == 4 ? 5 : 4) * N + 15) & ~(size_t)15;
+        total = other + (elem == 4 ? sizeof(float) * 8 * (size_t)N
+                                   : N <= kElocSym ? sizeof(double) * 4 * (size_t)N * (H / 32) : 0);
+        total = (total + 15) & ~(size_t)15;
+    }
+};
+size_t eloc_smem_bytes(const DevSys& s, int nt, int elem) { return ElocLayout(s.N, nt, elem).total; }
+
 template <typename T>
 __device__ __forceinline__ void eloc_walker(const DevSys& s, const DevWalkers& wk, int w, double* eloc_out, double* logpsi, double* grad,
-                                            double* lap, unsigned* err, double* sR) {
+                                            double* lap, unsigned* err, unsigned char* sm) {
     __shared__ double scratch[kMaxWarps * 2];
-    const int N = s.N, nu = s.n_up;
-    float* sRf = (float*)(sR + 3 * N);   // float copy for the pair terms of the mixed form
-    for (int q = threadIdx.x; q < 3 * N; q += blockDim.x) {
-        sR[q] = wk.R[(size_t)w * 3 * N + q];
-        sRf[q] = (float)sR[q];
-    }
+    const int N = s.N, nu = s.n_up, nn = s.n_nuc;
+    const ElocLayout L(N, blockDim.x, sizeof(T));
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, H = L.H;
+    double* sR = (double*)sm;
+    float4* sRf = (float4*)(sR + 3 * N + (N & 1));   // float positions of the mixed form's pairs
+    T* part = (T*)(sm + L.part);
+    for (int q = tid; q < 3 * N; q += blockDim.x) sR[q] = wk.R[(size_t)w * 3 * N + q];
     __syncthreads();
-    double v[2] = {0.0, 0.0};
     if constexpr (sizeof(T) == 4) {
-        // Mixed form: pair terms and dot products in FP32 with compensated
-        // per-electron sums, assembled in FP64.
-        for (int i = threadIdx.x; i < N; i += blockDim.x) {
-            const int spin = i >= nu;
-            const int n = spin ? s.n_dn : nu;
-            const int k = spin ? i - nu : i;
+        for (int i = tid; i < N; i += blockDim.x)
+            sRf[i] = make_float4((float)sR[3 * i], (float)sR[3 * i + 1], (float)sR[3 * i + 2], 0.f);
+        // determinant sums (gradient and Laplacian over the orbitals), a warp per electron
+        float* det = (float*)(sm + L.other);   // [N][8]: four (high, low) pairs
+        for (int i = wid; i < N; i += (int)blockDim.x >> 5) {
+            const int spin = i >= nu, n = spin ? s.n_dn : nu, k = spin ? i - nu : i;
             const float* Ai = (const float*)wk.Ainv[spin] + ((size_t)w * n + k) * n;
             const float* Gi = (const float*)wk.G[spin] + ((size_t)w * n + k) * 4 * n;
             Acc<float> dd[4];
-            for (int j = 0; j < n; ++j) {
+            for (int j = lane; j < n; j += 32) {
                 const float a = Ai[j];
-                dd[0].add(Gi[j] * a);
-                dd[1].add(Gi[n + j] * a);
-                dd[2].add(Gi[2 * n + j] * a);
-                dd[3].add(Gi[3 * n + j] * a);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) dd[c].add(Gi[c * n + j] * a);
             }
-            const float xi = sRf[3 * i], yi = sRf[3 * i + 1], zi = sRf[3 * i + 2];
-            const float bee = (float)s.b_ee, ben = (float)s.b_en;
-            float gx = 0.f, gy = 0.f, gz = 0.f;
-            Acc<float> lJ, Ji, V;
-            for (int j = 0; j < N; ++j) {
-                if (j == i) continue;
-                const float x = xi - sRf[3 * j], y = yi - sRf[3 * j + 1], z = zi - sRf[3 * j + 2];
-                const float r2 = x * x + y * y + z * z;
-                const float ir = rsqrtf(r2), r = r2 * ir;
-                const float a = (float)(((i < nu) == (j < nu)) ? s.a_par : s.a_anti);
-                const float q = 1.0f / (1.0f + bee * r);
-                const float du = a * q * q, g = du * ir;
-                gx += g * x;
-                gy += g * y;
-                gz += g * z;
-                lJ.add(-2.0f * bee * du * q + 2.0f * g);
-                if (j > i) {
-                    Ji.add(a * r * q);
-                    V.add(ir);
+            // transposing butterfly over the four sums: lanes 8 q hold sum q
+            const bool h4 = lane & 16, h3 = lane & 8;
+            Acc<float> r[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const Acc<float> send = h4 ? dd[q] : dd[q + 2];
+                r[q] = h4 ? dd[q + 2] : dd[q];
+                r[q].add_pair(__shfl_xor_sync(0xffffffffu, send.h, 16), __shfl_xor_sync(0xffffffffu, send.l, 16));
+            }
+            const Acc<float> send = h3 ? r[0] : r[1];
+            Acc<float> t = h3 ? r[1] : r[0];
+            t.add_pair(__shfl_xor_sync(0xffffffffu, send.h, 8), __shfl_xor_sync(0xffffffffu, send.l, 8));
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1)
+                t.add_pair(__shfl_xor_sync(0xffffffffu, t.h, o), __shfl_xor_sync(0xffffffffu, t.l, o));
+            if ((lane & 7) == 0) {
+                const int q = ((lane >> 3) & 1) + 2 * (lane >> 4);
+                det[8 * i + 2 * q] = t.h;
+                det[8 * i + 2 * q + 1] = t.l;
+            }
+        }
+        __syncthreads();
+    }
+    double v[2] = {0.0, 0.0};
+    if (tid < H) {
+        // ---- electron pairs: gradient and Laplacian of J per electron into part
+        if constexpr (sizeof(T) == 4) {
+            const float b = (float)s.b_ee;
+            for (int i = tid; i < N; i += H) {
+                const float4 ri = sRf[i];
+                float gx = 0.f, gy = 0.f, gz = 0.f;
+                Acc<float> lJ, Ji, V;
+                for (int half = 0; half < 2; ++half) {   // the pairs' own values once, from the lower electron
+                    const int j0 = half ? i + 1 : 0, j1 = half ? N : i;
+                    for (int j = j0; j < j1; ++j) {
+                        const float4 rj = sRf[j];
+                        const float x = ri.x - rj.x, y = ri.y - rj.y, z = ri.z - rj.z;
+                        const float r2 = x * x + y * y + z * z;
+                        const float ir = rsqrtf(r2), r = r2 * ir;
+                        const float a = (float)(((i < nu) == (j < nu)) ? s.a_par : s.a_anti);
+                        const float q = __fdividef(1.0f, 1.0f + b * r);
+                        const float du = a * q * q, g = du * ir;
+                        gx += g * x;
+                        gy += g * y;
+                        gz += g * z;
+                        lJ.add(-2.0f * b * du * q + 2.0f * g);
+                        if (half) {
+                            Ji.add(a * r * q);
+                            V.add(ir);
+                        }
+                    }
+                }
+                v[0] += (double)V.h + V.l;
+                v[1] += (double)Ji.h + Ji.l;
+                part[5 * i] = gx;
+                part[5 * i + 1] = gy;
+                part[5 * i + 2] = gz;
+                part[5 * i + 3] = lJ.h;
+                part[5 * i + 4] = lJ.l;
+            }
+        } else {
+            const double b = s.b_ee;
+            // u, u'/r and the Laplacian u'' + 2 u'/r with one reciprocal square
+            // root and one reciprocal: u = a r q, u' = a q^2, u'' = -2 b u' q
+            double x, y, z, ir, u, g, l;
+            auto pair = [&](int i, int j) {
+                x = sR[3 * i] - sR[3 * j];
+                y = sR[3 * i + 1] - sR[3 * j + 1];
+                z = sR[3 * i + 2] - sR[3 * j + 2];
+                const double r2 = x * x + y * y + z * z;
+                ir = rsqrt(r2);
+                const double r = r2 * ir, q = rcp_ge1(1.0 + b * r);
+                const double aq = (((i < nu) == (j < nu)) ? s.a_par : s.a_anti) * q, du = aq * q;
+                u = aq * r;
+                g = du * ir;
+                l = fma(-2.0 * b, du * q, 2.0 * g);
+            };
+            if (N <= kElocSym) {
+                double* oth = (double*)(sm + L.other) + (size_t)wid * 4 * N;
+                for (int q = lane; q < 4 * N; q += 32) oth[q] = 0.0;
+                __syncwarp();
+                for (int i0 = tid - lane; i0 < N; i0 += H) {   // whole warps
+                    const int i = i0 + lane;
+                    double gx = 0.0, gy = 0.0, gz = 0.0, lJ = 0.0;
+                    for (int k = 1; 2 * k <= N; ++k) {
+                        if (i < (2 * k == N ? k : N)) {
+                            const int j = i + k < N ? i + k : i + k - N;
+                            pair(i, j);
+                            gx += g * x;
+                            gy += g * y;
+                            gz += g * z;
+                            lJ += l;
+                            oth[j] -= g * x;
+                            oth[N + j] -= g * y;
+                            oth[2 * N + j] -= g * z;
+                            oth[3 * N + j] += l;
+                            v[1] += u;
+                            v[0] += ir;
+                        }
+                        __syncwarp();
+                    }
+                    if (i < N) {
+                        part[4 * i] = gx;
+                        part[4 * i + 1] = gy;
+                        part[4 * i + 2] = gz;
+                        part[4 * i + 3] = lJ;
+                    }
+                }
+            } else {
+                for (int i = tid; i < N; i += H) {
+                    double gx = 0.0, gy = 0.0, gz = 0.0, lJ = 0.0;
+                    for (int j = 0; j < N; ++j) {
+                        if (j == i) continue;
+                        pair(i, j);
+                        gx += g * x;
+                        gy += g * y;
+                        gz += g * z;
+                        lJ += l;
+                        if (j > i) {
+                            v[1] += u;
+                            v[0] += ir;
+                        }
+                    }
+                    part[4 * i] = gx;
+                    part[4 * i + 1] = gy;
+                    part[4 * i + 2] = gz;
+                    part[4 * i + 3] = lJ;
                 }
             }
-            for (int a = 0; a < s.n_nuc; ++a) {
-                const float x = (float)(sR[3 * i] - s.Rn[3 * a]), y = (float)(sR[3 * i + 1] - s.Rn[3 * a + 1]),
-                            z = (float)(sR[3 * i + 2] - s.Rn[3 * a + 2]);
-                const float r2 = x * x + y * y + z * z;
-                const float ir = rsqrtf(r2), r = r2 * ir;
-                const float ae = (float)s.a_en[a];
-                const float q = 1.0f / (1.0f + ben * r);
-                const float du = ae * q * q, g = du * ir;
-                gx += g * x;
-                gy += g * y;
-                gz += g * z;
-                lJ.add(-2.0f * ben * du * q + 2.0f * g);
-                Ji.add(ae * r * q);
-                V.add(-(float)s.Z[a] * ir);
-                if (s.npp) V.add(pp_local<float>(s, a, r));
+        }
+    }
+    // ---- electron-nucleus terms and determinant (second half); the barrier
+    // after the pair sums falls between these and the assembly of a thread's
+    // first electron
+    for (int i0 = 0; i0 < N; i0 += H) {
+        const int i = i0 + tid - H;
+        const bool on = tid >= H && i < N;
+        double d0 = 0.0, d1 = 0.0, d2 = 0.0, dl = 0.0, gx = 0.0, gy = 0.0, gz = 0.0, lJ = 0.0;
+        if (on) {
+            if constexpr (sizeof(T) == 4) {
+                const float* det = (const float*)(sm + L.other) + 8 * i;
+                d0 = (double)det[0] + det[1];
+                d1 = (double)det[2] + det[3];
+                d2 = (double)det[4] + det[5];
+                dl = (double)det[6] + det[7];
+                const float b = (float)s.b_en;
+                const float4 rh = sRf[i];
+                const float rl[3] = {(float)(sR[3 * i] - (double)rh.x), (float)(sR[3 * i + 1] - (double)rh.y),
+                                     (float)(sR[3 * i + 2] - (double)rh.z)};
+                float fx = 0.f, fy = 0.f, fz = 0.f;
+                Acc<float> lE, Ji, V;
+                for (int a = 0; a < nn; ++a) {
+                    const float x = diff_f2(rh.x, rl[0], s.Rn_hi[3 * a], s.Rn_lo[3 * a]);
+                    const float y = diff_f2(rh.y, rl[1], s.Rn_hi[3 * a + 1], s.Rn_lo[3 * a + 1]);
+                    const float z = diff_f2(rh.z, rl[2], s.Rn_hi[3 * a + 2], s.Rn_lo[3 * a + 2]);
+                    const float r2 = x * x + y * y + z * z;
+                    const float ir = rsqrtf(r2), r = r2 * ir;
+                    const float ae = s.a_en_f[a];
+                    const float q = __fdividef(1.0f, 1.0f + b * r);
+                    const float du = ae * q * q, g = du * ir;
+                    fx += g * x;
+                    fy += g * y;
+                    fz += g * z;
+                    lE.add(-2.0f * b * du * q + 2.0f * g);
+                    Ji.add(ae * r * q);
+                    V.add(-s.Z_f[a] * ir);
+                    if (s.npp) V.add(pp_local<float>(s, a, r));
+                }
+                gx = fx;
+                gy = fy;
+                gz = fz;
+                lJ = (double)lE.h + lE.l;
+                v[0] += (double)V.h + V.l;
+                v[1] += (double)Ji.h + Ji.l;
+            } else {
+                const int spin = i >= nu, n = spin ? s.n_dn : nu, k = spin ? i - nu : i;
+                const double* Ai = (const double*)wk.Ainv[spin] + ((size_t)w * n + k) * n;
+                const double* Gi = (const double*)wk.G[spin] + ((size_t)w * n + k) * 4 * n;
+                for (int j = 0; j < n; ++j) {
+                    const double a = Ai[j];
+                    d0 += Gi[j] * a;
+                    d1 += Gi[n + j] * a;
+                    d2 += Gi[2 * n + j] * a;
+                    dl += Gi[3 * n + j] * a;
+                }
+                const double b = s.b_en, xi = sR[3 * i], yi = sR[3 * i + 1], zi = sR[3 * i + 2];
+                double Ji = 0.0, V = 0.0;
+                for (int a = 0; a < nn; ++a) {
+                    const double x = xi - s.Rn[3 * a], y = yi - s.Rn[3 * a + 1], z = zi - s.Rn[3 * a + 2];
+                    const double r2 = x * x + y * y + z * z;
+                    const double ir = rsqrt(r2), r = r2 * ir;
+                    const double q = rcp_ge1(1.0 + b * r);
+                    const double aq = s.a_en[a] * q, du = aq * q, g = du * ir;
+                    gx += g * x;
+                    gy += g * y;
+                    gz += g * z;
+                    lJ += fma(-2.0 * b, du * q, 2.0 * g);
+                    Ji += aq * r;
+                    V -= s.Z[a] * ir;
+                    if (s.npp) V += pp_local<double>(s, a, r);
+                }
+                v[0] += V;
+                v[1] += Ji;
             }
-            const double d0 = (double)dd[0].h + dd[0].l, d1 = (double)dd[1].h + dd[1].l;
-            const double d2 = (double)dd[2].h + dd[2].l, dl = (double)dd[3].h + dd[3].l;
-            double lj = (double)lJ.h + lJ.l;
             if (s.n3 > 0) {
                 double v3, g3[3], l3;
                 j3_electron(s, sR, i, v3, g3, l3);
-                gx = (float)((double)gx + g3[0]);
-                gy = (float)((double)gy + g3[1]);
-                gz = (float)((double)gz + g3[2]);
-                lj += l3;
+                gx += g3[0];
+                gy += g3[1];
+                gz += g3[2];
+                lJ += l3;
                 v[1] += v3;
             }
-            const double Ti = -0.5 * (dl + lj + 2.0 * (gx * d0 + gy * d1 + gz * d2) + (double)gx * gx +
-                                      (double)gy * gy + (double)gz * gz);
-            v[0] += Ti + ((double)V.h + V.l);
-            v[1] += (double)Ji.h + Ji.l;
+        }
+        if (i0 == 0) __syncthreads();   // part and other are complete
+        if (on) {
+            constexpr int kP = sizeof(T) == 4 ? 5 : 4;
+            gx += (double)part[kP * i];
+            gy += (double)part[kP * i + 1];
+            gz += (double)part[kP * i + 2];
+            lJ += (double)part[kP * i + 3];
+            if (sizeof(T) == 4) lJ += (double)part[kP * i + kP - 1];
+            if (sizeof(T) == 8 && N <= kElocSym)
+                for (int q = 0; q < H / 32; ++q) {
+                    const double* oth = (const double*)(sm + L.other) + (size_t)q * 4 * N;
+                    gx += oth[i];
+                    gy += oth[N + i];
+                    gz += oth[2 * N + i];
+                    lJ += oth[3 * N + i];
+                }
+            v[0] -= 0.5 * (dl + lJ + 2.0 * (gx * d0 + gy * d1 + gz * d2) + gx * gx + gy * gy + gz * gz);
             if (grad) {
                 double* g = grad + ((size_t)w * N + i) * 3;
                 g[0] = gx + d0;
                 g[1] = gy + d1;
                 g[2] = gz + d2;
             }
-            if (lap) lap[(size_t)w * N + i] = lj + dl - (d0 * d0 + d1 * d1 + d2 * d2);
+            if (lap) lap[(size_t)w * N + i] = lJ + dl - (d0 * d0 + d1 * d1 + d2 * d2);
         }
-    } else
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        const int spin = i >= nu;
-        const int n = spin ? s.n_dn : nu;
-        const int k = spin ? i - nu : i;
-        const T* Ai = (const T*)wk.Ainv[spin] + ((size_t)w * n + k) * n;
-        const T* Gi = (const T*)wk.G[spin] + ((size_t)w * n + k) * 4 * n;
-        double d0 = 0, d1 = 0, d2 = 0, dl = 0;
-        for (int j = 0; j < n; ++j) {
-            const double a = (double)Ai[j];
-            d0 += (double)Gi[j] * a;
-            d1 += (double)Gi[n + j] * a;
-            d2 += (double)Gi[2 * n + j] * a;
-            dl += (double)Gi[3 * n + j] * a;
-        }
-        const double xi = sR[3 * i], yi = sR[3 * i + 1], zi = sR[3 * i + 2];
-        double gx = 0, gy = 0, gz = 0, lJ = 0, Ji = 0, V = 0;
-        // pair terms with one reciprocal square root and one division each:
-        // u = a r q, u' = a q^2, u'' = -2 a b q^3 with q = 1 / (1 + b r)
-        for (int j = 0; j < N; ++j) {
-            if (j == i) continue;
-            const double x = xi - sR[3 * j], y = yi - sR[3 * j + 1], z = zi - sR[3 * j + 2];
-            const double r2 = x * x + y * y + z * z;
-            const double ir = rsqrt(r2), r = r2 * ir;
-            const double a = ((i < nu) == (j < nu)) ? s.a_par : s.a_anti;
-            const double q = 1.0 / (1.0 + s.b_ee * r);
-            const double du = a * q * q, g = du * ir;
-            gx += g * x;
-            gy += g * y;
-            gz += g * z;
-            lJ += -2.0 * s.b_ee * du * q + 2.0 * g;
-            if (j > i) {
-                Ji += a * r * q;
-                V += ir;
-            }
-        }
-        for (int a = 0; a < s.n_nuc; ++a) {
-            const double x = xi - s.Rn[3 * a], y = yi - s.Rn[3 * a + 1], z = zi - s.Rn[3 * a + 2];
-            const double r2 = x * x + y * y + z * z;
-            const double ir = rsqrt(r2), r = r2 * ir;
-            const double q = 1.0 / (1.0 + s.b_en * r);
-            const double du = s.a_en[a] * q * q, g = du * ir;
-            gx += g * x;
-            gy += g * y;
-            gz += g * z;
-            lJ += -2.0 * s.b_en * du * q + 2.0 * g;
-            Ji += s.a_en[a] * r * q;
-            V -= s.Z[a] * ir;
-            if (s.npp) V += pp_local<double>(s, a, r);
-        }
-        if (s.n3 > 0) {
-            double v3, g3[3], l3;
-            j3_electron(s, sR, i, v3, g3, l3);
-            gx += g3[0];
-            gy += g3[1];
-            gz += g3[2];
-            lJ += l3;
-            Ji += v3;
-        }
-        const double Ti = -0.5 * (dl + lJ + 2.0 * (gx * d0 + gy * d1 + gz * d2) + gx * gx + gy * gy + gz * gz);
-        v[0] += Ti + V;
-        v[1] += Ji;
-        if (grad) {
-            double* g = grad + ((size_t)w * N + i) * 3;
-            g[0] = gx + d0;
-            g[1] = gy + d1;
-            g[2] = gz + d2;
-        }
-        if (lap) lap[(size_t)w * N + i] = lJ + dl - (d0 * d0 + d1 * d1 + d2 * d2);
     }
     block_sum<2>(v, scratch);
     if (threadIdx.x == 0) {
@@ -394,13 +535,14 @@ __device__ __forceinline__ void eloc_walker(const DevSys& s, const DevWalkers& w
     }
 }
 
+constexpr int kElocThreads = 640;   // at most
 template <typename T>
-__global__ void k_eloc(DevSys s, DevWalkers wk, int W, double* eloc_out, double* logpsi,
-                       double* grad, double* lap, unsigned* err) {
-    extern __shared__ double sR[];  // [N][3]
+__global__ void __launch_bounds__(kElocThreads) k_eloc(DevSys s, DevWalkers wk, int W, double* eloc_out, double* logpsi,
+                                                       double* grad, double* lap, unsigned* err) {
+    extern __shared__ __align__(16) unsigned char esm[];
     const int w = blockIdx.x;
     if (w >= W) return;
-    eloc_walker<T>(s, wk, w, eloc_out, logpsi, grad, lap, err, sR);
+    eloc_walker<T>(s, wk, w, eloc_out, logpsi, grad, lap, err, esm);
 }
 
 // Jastrow parameter derivatives of walker w (one CTA): d ln|psi| / dp is
@@ -580,12 +722,12 @@ template <typename T>
 cudaError_t launch_eloc(const DevSys& s, const DevWalkers& wk, int W, double* eloc_out, double* logpsi,
                         double* grad, double* lap, unsigned* err, cudaStream_t st) {
     if (W == 0) return cudaSuccess;
-    const size_t smem = (sizeof(double) + sizeof(float)) * 3 * s.N;
+    const int nt = std::min(kElocThreads, 2 * ((s.N + 31) & ~31));
+    const size_t smem = eloc_smem_bytes(s, nt, sizeof(T));
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_eloc<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    const int nt = s.N > 128 ? 256 : (s.N > 32 ? 128 : 32);
     k_eloc<T><<<W, nt, smem, st>>>(s, wk, W, eloc_out, logpsi, grad, lap, err);
     return cudaGetLastError();
 }
@@ -637,7 +779,7 @@ __global__ void k_invert_batch(const BatchSys* __restrict__ sys, BatchPlan* plan
 
 template <typename T>
 __global__ void k_eloc_batch(const BatchSys* __restrict__ sys, BatchPlan* plan, int parity, int into_walker, int ctr) {
-    extern __shared__ double sR[];
+    extern __shared__ __align__(16) unsigned char esm[];
     __shared__ BatchSys bs;
     __shared__ int s_sys, s_idx;
     for (;;) {
@@ -648,7 +790,7 @@ __global__ void k_eloc_batch(const BatchSys* __restrict__ sys, BatchPlan* plan, 
         batch_load(&bs, sys + q);
         __syncthreads();
         eloc_walker<T>(bs.s, bs.wk[parity], s_idx, into_walker ? bs.wk[parity].eloc : bs.eloc_new, nullptr, nullptr,
-                       nullptr, bs.err, sR);
+                       nullptr, bs.err, esm);
         __syncthreads();
     }
 }

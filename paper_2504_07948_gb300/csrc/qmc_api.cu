@@ -432,6 +432,8 @@ struct qmc_ctx {
             }
         s.vnn = vnn;
         s.Z = upload(sys_allocs, Z);
+        s.a_en_f = upload(sys_allocs, std::vector<float>(a_en.begin(), a_en.end()));
+        s.Z_f = upload(sys_allocs, std::vector<float>(Z.begin(), Z.end()));
         s.Rn = upload(sys_allocs, Rn);
         {
             std::vector<float> hi(Rn.size()), lo(Rn.size());
@@ -491,7 +493,6 @@ struct qmc_ctx {
                 s.CT[spin] = upload(sys_allocs, ct);
                 s.CT_f[spin] = upload(sys_allocs, std::vector<float>(ct.begin(), ct.end()));
             }
-            s.a_en_f = upload(sys_allocs, std::vector<float>(a_en.begin(), a_en.end()));
             std::vector<int> bytype((size_t)s.n_shell);
             for (int q = 0; q < s.n_shell; ++q) bytype[q] = q;
             std::stable_sort(bytype.begin(), bytype.end(), [&](int x, int y) {
@@ -2440,7 +2441,7 @@ struct qmc_batch {
             const int nmax = std::max(s.n_up, s.n_dn);
             orb = std::max(orb, orbitals_smem_bytes(s));
             inv = std::max(inv, sizeof(double) * ((size_t)nmax * nmax + nmax + 1));
-            el = std::max(el, (sizeof(double) + sizeof(float)) * 3 * (size_t)s.N);
+            el = std::max(el, eloc_smem_bytes(s, 128, elem()));
             fo = std::max(fo, force_batch_smem_bytes(s, elem(), warp[q]));
         }
         const bool mx = mode == QMC_MIXED;

@@ -29,6 +29,7 @@ struct DevSys {
     int n_nuc, n_up, n_dn, N;
     int n_shell, n_basis, n_prim;
     const double* Z;      // [n_nuc]
+    const float* Z_f;     // the same in float
     const double* Rn;     // [n_nuc][3]
     const float* Rn_hi;   // [n_nuc][3] float(Rn) and float(Rn - float(Rn)): with the same split
     const float* Rn_lo;   // of an electron position, FP32 offsets keep FP32 relative accuracy
@@ -1288,6 +1289,7 @@ struct SweepParams {
 };
 
 size_t orbitals_smem_bytes(const DevSys& s);
+size_t eloc_smem_bytes(const DevSys& s, int nt, int elem);
 template <typename T>
 cudaError_t launch_orbitals_all(const DevSys& s, const DevWalkers& wk, int W, cudaStream_t st,
                                 const int* only = nullptr);
