@@ -785,7 +785,8 @@ __global__ void k_force_prep(DevSys s, DevWalkers wk, int w0, int W, const doubl
 }
 
 // Third-order basis contraction with M, Y read from the GEMM outputs
-// Mw/Yw [spin][walker][n_basis][n] (type T).
+// Mw/Yw [spin][walker][n_basis][n] (type T; each spin's block starts at
+// spin W n_basis max(n_up, n_dn)).
 template <typename T, bool kE>
 __global__ void __launch_bounds__(256) k_force_contract(DevSys s, DevWalkers wk, int w0, int W, const T* Mw,
                                                         const T* Yw, const double* gJw, const double* accw,
@@ -810,8 +811,9 @@ __global__ void __launch_bounds__(256) k_force_contract(DevSys s, DevWalkers wk,
         const int n = spin ? s.n_dn : nu;
         if (n == 0) continue;
         const int i0 = spin ? nu : 0;
-        const T* M = Mw + ((size_t)(spin * W + wl)) * nb * n;
-        const T* Y = Yw + ((size_t)(spin * W + wl)) * nb * n;
+        const size_t off = (size_t)spin * W * nb * (nu > s.n_dn ? nu : s.n_dn) + (size_t)wl * nb * n;
+        const T* M = Mw + off;
+        const T* Y = Yw + off;
         // warp per run of shells on one centre, lanes over electrons: term
         // sums in T, one FP64 atomic per run and component
         for (int run = wid; run < s.n_run; run += nw) {

@@ -1192,8 +1192,8 @@ struct qmc_ctx {
                 const T* Bm = (const T*)d_fB + (size_t)spin * wc * nmax * nmax;
                 T* PT = (T*)d_fPT + (size_t)spin * wc * nmax * nmax;
                 T* Q = (T*)d_fQ + (size_t)spin * wc * nmax * nmax;
-                T* M = (T*)d_fM + (size_t)spin * wc * nb * n;
-                T* Y = (T*)d_fY + (size_t)spin * wc * nb * n;
+                T* M = (T*)d_fM + (size_t)spin * wc * nb * nmax;
+                T* Y = (T*)d_fY + (size_t)spin * wc * nb * nmax;
                 const T* Cs = sizeof(T) == 8 ? (const T*)(const void*)ds.C[spin] : (const T*)(const void*)ds.C_f[spin];
                 const long long nn2 = (long long)nmax * nmax, n2 = (long long)n * n;
                 if (sizeof(T) == 4 && !force_gemm_cublas) {

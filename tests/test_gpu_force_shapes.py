@@ -55,3 +55,20 @@ def test_fused_force_of_large_determinants_against_gemm_path(m, warp, monkeypatc
         g.close()
     scale = np.maximum(1.0, np.abs(out[0]).max(axis=(2, 3), keepdims=True))
     assert np.all(np.abs(out[1] - out[0]) <= 1e-10 * scale)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_gemm_force_path_with_fewer_down_electrons(precision, monkeypatch):
+    """The two spins' weights M and Y must not share memory when n_dn < n_up."""
+    from oracle import oracle as O
+    from paper_2504_07948_gb300 import qmc as Q
+    monkeypatch.setenv("QMC_FORCE_GEMM_MIN_N", "1")
+    s = _cut(3, 16, 8)
+    R = synth.initial_walkers(s, 3, seed=21)
+    g = Q.QMC(s, precision=precision)
+    g.set_walkers(R)
+    _, pw = g.forces()
+    g.close()
+    for got, ref in zip((pw[:, 0], pw[:, 1]), O.Oracle(s).forces(R)):
+        tol = 1e-10 if precision == "fp64" else 1e-2
+        assert np.all(np.abs(got - ref) <= tol * np.maximum(1.0, np.abs(ref).max(axis=(1, 2), keepdims=True)))
