@@ -16,6 +16,7 @@
 
 #include "batch.cuh"
 #include "fixed64.cuh"
+#include "gemm64.cuh"
 #include "qmc.h"
 #include "qmc_internal.cuh"
 #include "sweep_tiled.cuh"
@@ -315,6 +316,10 @@ struct qmc_ctx {
     int fchunk = 0;
     void *d_fB = nullptr, *d_fPT = nullptr, *d_fQ = nullptr, *d_fM = nullptr, *d_fY = nullptr;
     double *d_fgJ = nullptr, *d_faccw = nullptr;
+    // digits of the FP64 GEMM force path (k_gemm64.cu) for a chunk of walkers:
+    // A^-T over Q, B, A^-1, P^T; and of C per spin (with the system)
+    Gemm64Operand g64[4] = {}, g64C[2] = {};
+    int* d_Ce[2] = {nullptr, nullptr};   // exponent fields of the orbitals' largest coefficients
     unsigned* d_err = nullptr;
     unsigned long long* d_nacc = nullptr;
     // sharded DMC: a caller-supplied sum over ranks of each step's sums, and
@@ -561,7 +566,7 @@ struct qmc_ctx {
                 // the rows' limbs, every orbital in units of its column's scale
                 std::vector<int2> q(Cs.size());
                 std::vector<double> sc(n_basis), row(n);
-                std::vector<int> ce(n, 0);
+                std::vector<int> ce(std::max(n, 1), 0);
                 for (int l = 0; l < n_basis; ++l)
                     for (int j = 0; j < n; ++j) ce[j] = std::max(ce[j], fx_expo(Cs[(size_t)l * n + j]));
                 for (int l = 0; l < n_basis; ++l) {
@@ -576,6 +581,8 @@ struct qmc_ctx {
                 }
                 s.Cq[spin] = upload(sys_allocs, q);
                 s.Cq_s[spin] = upload(sys_allocs, sc);
+                d_Ce[spin] = upload(sys_allocs, ce);
+                g64C[spin] = Gemm64Operand{};
             }
         }
         if (have_msd) build_multidet(s);
@@ -1160,15 +1167,28 @@ struct qmc_ctx {
     void gemm_sb(cublasOperation_t ta, cublasOperation_t tb, int m, int n, int k, const T* A, int lda, long long sA,
                  const T* B, int ldb, long long sB, T* Cm, int ldc, long long sC, int batch);
 
+    // Digit buffers of one operand of the FP64 GEMM (rows a multiple of 64).
+    Gemm64Operand gemm64_operand(std::vector<void*>& list, int rows, int K, int batch) {
+        Gemm64Operand o{};
+        o.groups = rows / 8;
+        o.stride = gemm64_bytes(o.groups, K);
+        o.estride = rows;
+        o.dig = (unsigned char*)dalloc<char>(list, o.stride * batch);
+        o.expo = dalloc<int>(list, (size_t)rows * batch);
+        return o;
+    }
+
     // Adjoint forces with the dense products as batched GEMMs, in walker
     // chunks: prep (B, grad J, Jastrow terms) -> PT = AT B^T, Q = PT AT,
     // M = C AT^T, Y = C Q^T per spin -> third-order basis contraction.
     template <typename T>
     void forces_gemm(const DevWalkers& kw) {
         const int nmax = std::max(n_up, n_dn), nb = n_basis, N3 = 3 * N(), nn = n_nuc;
-        const int Wc = std::min(W, 512);
+        constexpr bool kFp64 = sizeof(T) == 8;
+        const int chunk = kFp64 ? 256 : 512;
+        const int Wc = std::min(W, chunk);
         if (fchunk < Wc) {
-            fchunk = std::max(Wc, std::min(cap, 512));
+            fchunk = std::max(Wc, std::min(cap, chunk));
             d_fB = dalloc<T>(wk_allocs, 2 * (size_t)fchunk * nmax * nmax);
             d_fPT = dalloc<T>(wk_allocs, 2 * (size_t)fchunk * nmax * nmax);
             d_fQ = dalloc<T>(wk_allocs, 2 * (size_t)fchunk * nmax * nmax);
@@ -1176,11 +1196,29 @@ struct qmc_ctx {
             d_fY = dalloc<T>(wk_allocs, 2 * (size_t)fchunk * nb * nmax);
             d_fgJ = dalloc<double>(wk_allocs, (size_t)fchunk * N3);
             d_faccw = dalloc<double>(wk_allocs, (size_t)fchunk * 6 * nn);
+            if (kFp64) {
+                // rows the tiles read: 128 of a left operand, 64 of a right one
+                const int n8 = (nmax + 7) / 8 * 8, rl = (nmax + 127) / 128 * 128, rr = (nmax + 63) / 64 * 64;
+                const int rows[4] = {std::max(rl, (n8 + nmax + 63) / 64 * 64), rr, rr, rl};
+                for (int q = 0; q < 4; ++q) g64[q] = gemm64_operand(wk_allocs, rows[q], nmax, fchunk);
+            }
         }
-        if (!blas) {
-            require(cublasCreate(&blas) == CUBLAS_STATUS_SUCCESS, QMC_ERR_CUDA, "cublasCreate failed");
+        if (kFp64) {
+            require(nmax <= kGemm64MaxK, QMC_ERR_UNSUPPORTED, "the FP64 force path takes at most 170 electrons per spin");
+            for (int spin = 0; spin < 2; ++spin) {
+                const int n = spin ? n_dn : n_up;
+                if (n == 0 || g64C[spin].dig) continue;
+                g64C[spin] = gemm64_operand(sys_allocs, (nb + 127) / 128 * 128, n, 1);
+                g64C[spin].stride = 0;
+                g64C[spin].estride = 0;
+                QMC_CK(launch_digits(1, ds.C[spin], 0, n, 0, nb, (nb + 7) / 8 * 8, n, d_Ce[spin], 0, -1, g64C[spin], 0,
+                                     stream));
+            }
         }
-        require(cublasSetStream(blas, stream) == CUBLAS_STATUS_SUCCESS, QMC_ERR_CUDA, "cublasSetStream failed");
+        if (!kFp64 && force_gemm_cublas) {
+            if (!blas) require(cublasCreate(&blas) == CUBLAS_STATUS_SUCCESS, QMC_ERR_CUDA, "cublasCreate failed");
+            require(cublasSetStream(blas, stream) == CUBLAS_STATUS_SUCCESS, QMC_ERR_CUDA, "cublasSetStream failed");
+        }
         const DevWalkers& k = kw;
         for (int w0 = 0; w0 < W; w0 += Wc) {
             const int wc = std::min(Wc, W - w0);
@@ -1211,11 +1249,30 @@ struct qmc_ctx {
                                           d_err, stream));
                     continue;
                 }
-                // column-major views of row-major matrices are their transposes
-                gemm_sb<T>(CUBLAS_OP_T, CUBLAS_OP_N, n, n, n, Bm, n, nn2, AT, n, n2, PT, n, nn2, wc);   // PT = AT B^T
-                gemm_sb<T>(CUBLAS_OP_N, CUBLAS_OP_N, n, n, n, AT, n, n2, PT, n, nn2, Q, n, nn2, wc);    // Q = PT AT
-                gemm_sb<T>(CUBLAS_OP_T, CUBLAS_OP_N, n, nb, n, AT, n, n2, Cs, n, 0, M, n, (long long)nb * n, wc);
-                gemm_sb<T>(CUBLAS_OP_T, CUBLAS_OP_N, n, nb, n, Q, n, nn2, Cs, n, 0, Y, n, (long long)nb * n, wc);
+                if constexpr (sizeof(T) == 8) {
+                    // bf16 digits on the tensor cores: X holds A^-T and below it Q;
+                    // orbitals in units of their largest coefficient, electrons in
+                    // units of their row of A^-T
+                    const Gemm64Operand &X = g64[0], &Bd = g64[1], &Ai = g64[2], &Pd = g64[3];
+                    const int n8 = (n + 7) / 8 * 8;
+                    const int* ce = d_Ce[spin];
+                    const long long es = X.estride;
+                    QMC_CK(launch_digits(wc, AT, n2, n, 0, n, n8, n, ce, 0, 1, X, 0, stream));
+                    QMC_CK(launch_digits(wc, Bm, nn2, n, 0, n, n8, n, ce, 0, -1, Bd, 0, stream));
+                    QMC_CK(launch_gemm64(X, Bd, n, n, n, wc, PT, nn2, n, n, PT, nn2, n, d_err, stream));   // PT = AT B^T
+                    QMC_CK(launch_digits(wc, AT, n2, n, 1, n, n8, n, X.expo, es, -1, Ai, 0, stream));
+                    QMC_CK(launch_digits(wc, PT, nn2, n, 0, n, n8, n, X.expo, es, 1, Pd, 0, stream));
+                    QMC_CK(launch_gemm64(Pd, Ai, n, n, n, wc, Q, nn2, n, n, Q, nn2, n, d_err, stream));    // Q = PT AT
+                    QMC_CK(launch_digits(wc, Q, nn2, n, 0, n, n8, n, ce, 0, 1, X, n8, stream));
+                    QMC_CK(launch_gemm64(g64C[spin], X, nb, n8 + n, n, wc, M, (long long)nb * n, n, n8, Y,
+                                         (long long)nb * n, n, d_err, stream));   // M = C AT^T, Y = C Q^T
+                } else {
+                    // column-major views of row-major matrices are their transposes
+                    gemm_sb<T>(CUBLAS_OP_T, CUBLAS_OP_N, n, n, n, Bm, n, nn2, AT, n, n2, PT, n, nn2, wc);   // PT = AT B^T
+                    gemm_sb<T>(CUBLAS_OP_N, CUBLAS_OP_N, n, n, n, AT, n, n2, PT, n, nn2, Q, n, nn2, wc);    // Q = PT AT
+                    gemm_sb<T>(CUBLAS_OP_T, CUBLAS_OP_N, n, nb, n, AT, n, n2, Cs, n, 0, M, n, (long long)nb * n, wc);
+                    gemm_sb<T>(CUBLAS_OP_T, CUBLAS_OP_N, n, nb, n, Q, n, nn2, Cs, n, 0, Y, n, (long long)nb * n, wc);
+                }
             }
             QMC_CK(launch_force_contract<T>(ds, k, w0, wc, d_fM, d_fY, d_fgJ, d_faccw, d_dEL, d_dlog, d_gEdet,
                                             stream));
@@ -1323,16 +1380,6 @@ struct qmc_ctx {
         ++gen;
     }
 };
-
-template <>
-void qmc_ctx::gemm_sb<double>(cublasOperation_t ta, cublasOperation_t tb, int m, int n, int k, const double* A, int lda,
-                              long long sA, const double* B, int ldb, long long sB, double* Cm, int ldc, long long sC,
-                              int batch) {
-    const double one = 1.0, zero = 0.0;
-    const cublasStatus_t st =
-        cublasDgemmStridedBatched(blas, ta, tb, m, n, k, &one, A, lda, sA, B, ldb, sB, &zero, Cm, ldc, sC, batch);
-    require(st == CUBLAS_STATUS_SUCCESS, QMC_ERR_CUDA, "cublasDgemmStridedBatched failed: " + std::to_string((int)st));
-}
 
 template <>
 void qmc_ctx::gemm_sb<float>(cublasOperation_t ta, cublasOperation_t tb, int m, int n, int k, const float* A, int lda,
