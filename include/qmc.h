@@ -63,7 +63,8 @@ enum { QMC_POP_BRANCH = 0, QMC_POP_FIXED = 1 };                    /* population
  * kernel paths (for tests and measurements; the defaults are the fast ones):
  *   QMC_SWEEP_TILED=0          no walker-tiled sweep (the fused delayed sweep)
  *   QMC_SWEEP_TILED_MIN_N=k    tiled sweep from k electrons per spin (96)
- *   QMC_SWEEP_TILED_GROUPS=g   walker groups of the tiled sweep, 1..4 (2)
+ *   QMC_SWEEP_TILED_GROUPS=g   walker groups of the tiled sweep, 1..4 (one below
+ *                              3072 walkers, else 2)
  *   QMC_FORCE_GEMM_MIN_N=k     GEMM force path from k electrons per spin (65)
  *   QMC_FORCE_GEMM_CUBLAS=1    the mixed GEMM force path's products on cuBLAS
  *   QMC_NLPP_TC=0              u_k of the non-local pass formed in the kernel

@@ -152,43 +152,107 @@ __device__ __forceinline__ float2 df_rcp(float r) {
     return df_quick(q, q * res);
 }
 
-struct ProposeSmem {
-    float y[32], tf[32], red[4 * 7], fs[6];
-    int rows[32];
-    float rad[3 * kTiledMaxShells];   // f, f', f'' of every shell at r' (zeros where screened)
-};
-struct AcceptSmem {
-    float red[4 * 8];
-    float c[32];
+// Shared memory of a walker's CTA: K^-1 (read by its loops instead of global
+// memory, where every step of their serial sums waited for L2), the move's
+// small vectors, and behind them (dynamic) the offsets from the nuclei at r'
+// and the radial sums of every shell.
+struct TiledSmem {
+    float2 KT[32][33];   // KT[q][m] = (K^-1)_{mq}
     float2 u[32], t[32];
+    float y[32], tf[32], c[32], red[4 * 8], fs[6], chi[3], uni, rho;
     int rows[32], acc;
-    float rho;
 };
+__host__ __device__ inline size_t tiled_smem_bytes(int n_nuc, int n_shell) {
+    return sizeof(TiledSmem) + sizeof(float) * (6 * (size_t)n_nuc + 3 * (size_t)n_shell);
+}
+
+// K^-1, the queue's row indices, t and the nuclei into shared memory
+// (asynchronously; tiled_wait completes them).
+__device__ __forceinline__ void tiled_fetch(const DevSys& s, const TiledState& ts, int w, int dq, TiledSmem& S,
+                                            bool with_t) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, kmax = ts.kmax;
+    const float2* KT = ts.KinvT + (size_t)w * kmax * kmax;
+    for (int q = wid; q < dq; q += kTb / 32)
+        if (lane < dq)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(&S.KT[q][lane])),
+                         "l"(KT + (size_t)q * kmax + lane));
+    asm volatile("cp.async.commit_group;");
+    float* nuc = (float*)(&S + 1);
+    for (int a = threadIdx.x; a < s.n_nuc; a += kTb)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            nuc[6 * a + c] = s.Rn_hi[3 * a + c];
+            nuc[6 * a + 3 + c] = s.Rn_lo[3 * a + c];
+        }
+    if ((int)threadIdx.x < dq) {
+        S.rows[threadIdx.x] = ts.rows[(size_t)w * kmax + threadIdx.x];
+        if (with_t) S.t[threadIdx.x] = ts.tv[(size_t)w * kmax + threadIdx.x];
+    }
+}
+__device__ __forceinline__ void tiled_wait() {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+}
+
+// out[m] = sum_j x[j] row_m[j] for m < dq (row_m = base + stride(m)), a warp
+// per m and four m in flight at a time; the terms of one m are added in the
+// order of a warp that takes it alone.
+template <typename RowOf>
+__device__ __forceinline__ void queue_dots(int dq, int n, const float* x, RowOf row_of, float* out) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    constexpr int kW = kTb / 32, kU = 4;
+    for (int m0 = wid; m0 < dq; m0 += kW * kU) {
+        const float* r[kU];
+        float a[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            r[u] = row_of(min(m0 + kW * u, dq - 1));
+            a[u] = 0.f;
+        }
+#pragma unroll 2
+        for (int j = lane; j < n; j += 32) {
+            const float xj = x[j];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) a[u] += xj * r[u][j];
+        }
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            a[u] = wsum(a[u]);
+            if (lane == 0 && m0 + kW * u < dq) out[m0 + kW * u] = a[u];
+        }
+    }
+}
+
+// The proposal's normals, drawn early by one thread of the last warp while
+// the others work (the serial part of a move holds every thread of the CTA).
+__device__ __forceinline__ void tiled_draw_normals(const SweepParams& p, int e, int w, TiledSmem& S) {
+    if (threadIdx.x == kTb - 32) {
+        float chi[3];
+        draw_normals_f(p.key, p.sweep, (uint32_t)e, (uint32_t)w, chi);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) S.chi[c] = chi[c];
+    }
+}
 
 // Column e of the current inverse, drift, proposal and the basis at r' as
-// TF32 hi / lo rows of B', for walker w (the whole CTA).
+// TF32 hi / lo rows of B', for walker w (the whole CTA).  dq: queue length;
+// S holds K^-1 and the rows (tiled_fetch, complete) and the normals.
 __device__ __forceinline__ void propose_body(const DevSys& s, const DevWalkers& wk, const TiledState& ts, int w,
-                                             int e, const SweepParams& p, ProposeSmem& S) {
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+                                             int e, const SweepParams& p, int dq, TiledSmem& S) {
+    const int tid = threadIdx.x;
     const int nu = s.n_up, N = s.N, spin = e >= nu, n = spin ? s.n_dn : nu, k = spin ? e - nu : e;
     const int kmax = ts.kmax, ldv = ts.ldv, nbp = ts.nbp;
+    float* nuc = (float*)(&S + 1);        // nuclei as hi / lo floats, [n_nuc][6] (tiled_fetch)
+    float* rad = nuc + 6 * s.n_nuc;       // f, f', f'' of every shell at r' (zeros where screened)
     const float* AT = (const float*)wk.Ainv[spin] + (size_t)w * n * n;
     const float* V = ts.V + (size_t)w * kmax * ldv;
-    const int dq = ts.dq[w];
-    if (tid < dq) S.rows[tid] = ts.rows[(size_t)w * kmax + tid];
-    // y_m = phi'_m . A0^-1[:, e] (row k of A0^-T): a warp per m
-    for (int m = wid; m < dq; m += kTb / 32) {
-        float a = 0.f;
-        for (int j = lane; j < n; j += 32) a += V[(size_t)m * ldv + j] * AT[(size_t)k * n + j];
-        a = wsum(a);
-        if (lane == 0) S.y[m] = a;
-    }
+    // y_m = phi'_m . A0^-1[:, e] (row k of A0^-T)
+    queue_dots(dq, n, AT + (size_t)k * n, [&](int m) { return V + (size_t)m * ldv; }, S.y);
     __syncthreads();
-    // t = K^-1 y in double-float (KinvT[q][m] = (K^-1)_{mq}), thread m
+    // t = K^-1 y in double-float, thread m
     if (tid < dq) {
-        const float2* KT = ts.KinvT + (size_t)w * kmax * kmax;
         float2 t = make_float2(0.f, 0.f);
-        for (int q = 0; q < dq; ++q) t = df_add(t, df_mulf(KT[(size_t)q * kmax + tid], S.y[q]));
+        for (int q = 0; q < dq; ++q) t = df_add(t, df_mulf(S.KT[q][tid], S.y[q]));
         ts.tv[(size_t)w * kmax + tid] = t;
         S.tf[tid] = t.x + t.y;
     }
@@ -199,11 +263,20 @@ __device__ __forceinline__ void propose_body(const DevSys& s, const DevWalkers& 
     float v7[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     for (int j = tid; j < n; j += kTb) {
         float a = AT[(size_t)k * n + j];
-        for (int m = 0; m < dq; ++m) a -= S.tf[m] * AT[(size_t)S.rows[m] * n + j];
+        const float g0 = Gk[j], g1 = Gk[n + j], g2 = Gk[2 * n + j];
+        int m = 0;
+        for (; m + 8 <= dq; m += 8) {   // eight rows in flight, subtracted in order
+            float r[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) r[u] = AT[(size_t)S.rows[m + u] * n + j];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) a -= S.tf[m + u] * r[u];
+        }
+        for (; m < dq; ++m) a -= S.tf[m] * AT[(size_t)S.rows[m] * n + j];
         ce[j] = a;
-        v7[0] += Gk[j] * a;
-        v7[1] += Gk[n + j] * a;
-        v7[2] += Gk[2 * n + j] * a;
+        v7[0] += g0 * a;
+        v7[1] += g1 * a;
+        v7[2] += g2 * a;
     }
     // Jastrow value and gradient at r_e
     const float2* Rp = ts.Rp + (size_t)w * 3 * N;
@@ -223,7 +296,8 @@ __device__ __forceinline__ void propose_body(const DevSys& s, const DevWalkers& 
         const double r[3] = {R[0], R[1], R[2]};
         double scal[8];
         float fs[12];
-        propose_move_mixed(g, p.tau, r, p.key, p.sweep, (uint32_t)e, (uint32_t)w, scal, fs);
+        const float chi[3] = {S.chi[0], S.chi[1], S.chi[2]};
+        propose_move_drawn(g, p.tau, r, chi, scal, fs);
         float* mv = ts.mv + (size_t)w * kTiledMv;
 #pragma unroll
         for (int c = 0; c < 12; ++c) mv[c] = fs[c];
@@ -236,41 +310,41 @@ __device__ __forceinline__ void propose_body(const DevSys& s, const DevWalkers& 
         for (int c = 0; c < 6; ++c) S.fs[c] = fs[c];
     }
     __syncthreads();
-    const float ph[3] = {S.fs[0], S.fs[1], S.fs[2]}, pl[3] = {S.fs[3], S.fs[4], S.fs[5]};
-    // basis at r': the radial sums of every shell once (thread per shell,
-    // zeros where screened) into shared memory, then the walker's five rows
-    // of B' as TF32 hi / lo halves, one thread per basis function
+    // basis at r': offsets from the nuclei once, the radial sums of every
+    // shell once (thread per shell, zeros where screened), then the walker's
+    // five rows of B' as TF32 hi / lo halves, one thread per basis function
     // (consecutive threads write consecutive columns); functions of screened
     // shells are written as zeros (the buffers are reused every move)
+    const float ph[3] = {S.fs[0], S.fs[1], S.fs[2]}, pl[3] = {S.fs[3], S.fs[4], S.fs[5]};
     float* Bh = ts.Bh + (size_t)w * 5 * nbp;
     float* Bl = ts.Bl + (size_t)w * 5 * nbp;
     const float* amin = s.shell_amin_f;
     for (int sh = tid; sh < s.n_shell; sh += kTb) {
         const int4 d = s.shell[sh];
-        const int c3 = 3 * d.x;
-        const float x = diff_f2(ph[0], pl[0], s.Rn_hi[c3], s.Rn_lo[c3]);
-        const float y = diff_f2(ph[1], pl[1], s.Rn_hi[c3 + 1], s.Rn_lo[c3 + 1]);
-        const float z = diff_f2(ph[2], pl[2], s.Rn_hi[c3 + 2], s.Rn_lo[c3 + 2]);
+        const float* c6 = nuc + 6 * d.x;
+        const float x = diff_f2(ph[0], pl[0], c6[0], c6[3]);
+        const float y = diff_f2(ph[1], pl[1], c6[1], c6[4]);
+        const float z = diff_f2(ph[2], pl[2], c6[2], c6[5]);
         const float t2 = x * x + y * y + z * z;
         float f0 = 0.f, f1 = 0.f, f2 = 0.f, f3;
         if (!(amin[sh] * t2 > (float)kScreenExponent)) radial<float, false>(s.alpha_f, s.cn_f, d.z, d.w, t2, f0, f1, f2, f3);
-        S.rad[3 * sh] = f0;
-        S.rad[3 * sh + 1] = f1;
-        S.rad[3 * sh + 2] = f2;
+        rad[3 * sh] = f0;
+        rad[3 * sh + 1] = f1;
+        rad[3 * sh + 2] = f2;
     }
     __syncthreads();
+    grid_release();   // the GEMM may set itself up; it waits for this grid's rows
     for (int fn = tid; fn < s.n_basis; fn += kTb) {
-        const int sh = ts.fn_shell[fn];
-        const int4 d = s.shell[sh];
-        const int c3 = 3 * d.x;
-        const float x = diff_f2(ph[0], pl[0], s.Rn_hi[c3], s.Rn_lo[c3]);
-        const float y = diff_f2(ph[1], pl[1], s.Rn_hi[c3 + 1], s.Rn_lo[c3 + 1]);
-        const float z = diff_f2(ph[2], pl[2], s.Rn_hi[c3 + 2], s.Rn_lo[c3 + 2]);
+        const int2 fi = ts.fn_info[fn];
+        const float* c6 = nuc + 6 * (fi.y >> 8);
+        const float x = diff_f2(ph[0], pl[0], c6[0], c6[3]);
+        const float y = diff_f2(ph[1], pl[1], c6[1], c6[4]);
+        const float z = diff_f2(ph[2], pl[2], c6[2], c6[5]);
         const float t2 = x * x + y * y + z * z;
         float out[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-        const float f0 = S.rad[3 * sh], f1 = S.rad[3 * sh + 1], f2 = S.rad[3 * sh + 2];
+        const float f0 = rad[3 * fi.x], f1 = rad[3 * fi.x + 1], f2 = rad[3 * fi.x + 2];
         if (f0 != 0.f || f1 != 0.f || f2 != 0.f) {
-            const AngPoly<float> a = angular<float>(d.y & 0xff, d.y >> 8, fn - s.shell_fn[sh], x, y, z);
+            const AngPoly<float> a = angular<float>((fi.y >> 1) & 7, fi.y & 1, (fi.y >> 4) & 15, x, y, z);
             const float Sx = 2.f * x * f1, Sy = 2.f * y * f1, Sz = 2.f * z * f1;
             const float LS = 6.f * f1 + 4.f * t2 * f2;
             out[0] = a.P * f0;
@@ -289,23 +363,21 @@ __device__ __forceinline__ void propose_body(const DevSys& s, const DevWalkers& 
 }
 
 // Ratio, drift at r', Jastrow change, Metropolis test of walker w's move of
-// electron e; an accepted move borders K^-1 and queues its orbital row.
-__device__ __forceinline__ void accept_body(const DevSys& s, const DevWalkers& wk, const TiledState& ts, int w, int e,
-                                            const SweepParams& p, AcceptSmem& S) {
+// electron e; an accepted move borders K^-1 (in S and in global memory) and
+// queues its orbital row.  dq: queue length; tiled_fetch has been started.
+// Returns the queue length after the move; ends synchronised.
+__device__ __forceinline__ int accept_body(const DevSys& s, const DevWalkers& wk, const TiledState& ts, int w, int e,
+                                           const SweepParams& p, int dq, TiledSmem& S) {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int nu = s.n_up, N = s.N, spin = e >= nu, n = spin ? s.n_dn : nu, k = spin ? e - nu : e;
     const int kmax = ts.kmax, ldv = ts.ldv;
     const float* Phi = ts.Phi + (size_t)w * 5 * n;
     const float* ce = ts.ce + (size_t)w * ldv;
     const float* mv = ts.mv + (size_t)w * kTiledMv;
+    // everything that does not need the orbitals, while the GEMM before this
+    // launch is still running (see launch_after)
+    if (tid == kTb - 64) S.uni = accept_uniform_f(p.key, p.sweep, (uint32_t)e, (uint32_t)w);
     float v8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int j = tid; j < n; j += kTb) {
-        const float a = ce[j];
-        v8[0] += Phi[j] * a;
-        v8[1] += Phi[n + j] * a;
-        v8[2] += Phi[2 * n + j] * a;
-        v8[3] += Phi[3 * n + j] * a;
-    }
     const float2* Rp = ts.Rp + (size_t)w * 3 * N;
     {
         const float rh[3] = {mv[0], mv[1], mv[2]}, rl[3] = {mv[3], mv[4], mv[5]};
@@ -315,35 +387,32 @@ __device__ __forceinline__ void accept_body(const DevSys& s, const DevWalkers& w
         v8[6] = gj[1];
         v8[7] = gj[2];
     }
+    grid_wait();
+    for (int j = tid; j < n; j += kTb) {
+        const float a = ce[j];
+        v8[0] += Phi[j] * a;
+        v8[1] += Phi[n + j] * a;
+        v8[2] += Phi[2 * n + j] * a;
+        v8[3] += Phi[3 * n + j] * a;
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");   // before the sum's barrier: K^-1 is complete after it
     cta_sum_to0<8>(v8, S.red);
     if (tid == 0) {
         float fs[12];
 #pragma unroll
         for (int c = 0; c < 12; ++c) fs[c] = mv[c];
         const float gd[3] = {v8[1], v8[2], v8[3]}, gj[3] = {v8[5], v8[6], v8[7]};
-        S.acc = accept_move_mixed(v8[0], gd, gj, v8[4] - mv[12], p.tau, fs, p.key, p.sweep, (uint32_t)e,
-                                  (uint32_t)w);
+        S.acc = accept_move_drawn(v8[0], gd, gj, v8[4] - mv[12], p.tau, fs, S.uni);
         S.rho = v8[0];
     }
     __syncthreads();
-    if (!S.acc) return;   // uniform over the CTA
+    if (!S.acc) return dq;   // uniform over the CTA
     const float rho = S.rho;
     const float* AT = (const float*)wk.Ainv[spin] + (size_t)w * n * n;
     float* V = ts.V + (size_t)w * kmax * ldv;
     float2* KT = ts.KinvT + (size_t)w * kmax * kmax;
-    const int dq = ts.dq[w];
-    if (tid < dq) {
-        S.rows[tid] = ts.rows[(size_t)w * kmax + tid];
-        S.t[tid] = ts.tv[(size_t)w * kmax + tid];
-    }
-    __syncthreads();
-    // new row of K: c_m = phi' . A0^-1[:, r_m] (a warp per m)
-    for (int m = wid; m < dq; m += kTb / 32) {
-        float a = 0.f;
-        for (int j = lane; j < n; j += 32) a += Phi[j] * AT[(size_t)S.rows[m] * n + j];
-        a = wsum(a);
-        if (lane == 0) S.c[m] = a;
-    }
+    // new row of K: c_m = phi' . A0^-1[:, r_m]
+    queue_dots(dq, n, Phi, [&](int m) { return AT + (size_t)S.rows[m] * n; }, S.c);
     for (int j = tid; j < n; j += kTb) V[(size_t)dq * ldv + j] = Phi[j];
     float* Gk = (float*)wk.G[spin] + ((size_t)w * n + k) * 4 * n;
     for (int o = tid; o < 4 * n; o += kTb) Gk[o] = Phi[n + o];
@@ -351,23 +420,29 @@ __device__ __forceinline__ void accept_body(const DevSys& s, const DevWalkers& w
     // u^T = c^T K^-1: u_m = sum_q c_q (K^-1)_{qm} = sum_q c_q KinvT[m][q]
     if (tid < dq) {
         float2 u = make_float2(0.f, 0.f);
-        for (int q = 0; q < dq; ++q) u = df_add(u, df_mulf(KT[(size_t)tid * kmax + q], S.c[q]));
+        for (int q = 0; q < dq; ++q) u = df_add(u, df_mulf(S.KT[tid][q], S.c[q]));
         S.u[tid] = u;
     }
     __syncthreads();
     // K'^-1 = [[Ki + t u^T / rho, -t / rho], [-u^T / rho, 1 / rho]]
     const float2 is = df_rcp(rho);
-    for (int q2 = tid; q2 < dq * dq; q2 += kTb) {
-        const int q = q2 / dq, m = q2 - q * dq;
-        float2* kk = KT + (size_t)q * kmax + m;                            // (Ki)_{mq}
-        *kk = df_add(*kk, df_mul(df_mul(S.t[m], S.u[q]), is));
-    }
+    if (lane < dq)
+        for (int q = wid; q < dq; q += kTb / 32) {
+            const float2 kk = df_add(S.KT[q][lane], df_mul(df_mul(S.t[lane], S.u[q]), is));   // (Ki)_{mq}, m = lane
+            S.KT[q][lane] = kk;
+            KT[(size_t)q * kmax + lane] = kk;
+        }
     if (tid < dq) {
-        KT[(size_t)dq * kmax + tid] = df_neg(df_mul(S.t[tid], is));        // (K'^-1)_{tid, dq}
-        KT[(size_t)tid * kmax + dq] = df_neg(df_mul(S.u[tid], is));        // (K'^-1)_{dq, tid}
+        const float2 a = df_neg(df_mul(S.t[tid], is)), b = df_neg(df_mul(S.u[tid], is));
+        S.KT[dq][tid] = a;                                                  // (K'^-1)_{tid, dq}
+        KT[(size_t)dq * kmax + tid] = a;
+        S.KT[tid][dq] = b;                                                  // (K'^-1)_{dq, tid}
+        KT[(size_t)tid * kmax + dq] = b;
     }
     if (tid == 0) {
+        S.KT[dq][dq] = is;
         KT[(size_t)dq * kmax + dq] = is;
+        S.rows[dq] = k;
         ts.rows[(size_t)w * kmax + dq] = k;
         ts.dq[w] = dq + 1;
         wk.logdet[2 * w + spin] += (double)logf(rho);
@@ -381,40 +456,65 @@ __device__ __forceinline__ void accept_body(const DevSys& s, const DevWalkers& w
         }
         ts.acc[w] += 1u;
     }
+    __syncthreads();
+    return dq + 1;
 }
 
+// Launches of a move's kernels follow each other programmatically: the next
+// grid starts once every CTA of this one has passed grid_release, and reads
+// what this grid writes only after its grid_wait.  The GEMM releases after its
+// own wait, so an accept launch that has started finds everything the previous
+// accept / propose launch wrote and can form the Jastrow sums, fetch K^-1 and
+// draw its random numbers while the GEMM runs.  Used where one chain of launches
+// has the GPU (32 waters, 256 walkers: 49 -> 42 us an electron); with several
+// groups a GEMM that waits for its rows would hold SMs the other group could
+// use (4096 walkers, two groups: 206 -> 217), and launches are plain.
+//
 // Walkers w0 + blockIdx.x < W of the launch's walker group.
 __global__ void __launch_bounds__(kTb, 8) k_tiled_propose(DevSys s, DevWalkers wk, TiledState ts, int w0, int W,
                                                           int e, SweepParams p) {
-    __shared__ ProposeSmem S;
+    extern __shared__ __align__(16) unsigned char tsm[];
+    TiledSmem& S = *reinterpret_cast<TiledSmem*>(tsm);
     const int w = w0 + (int)blockIdx.x;
     if (w >= W) return;
-    propose_body(s, wk, ts, w, e, p, S);
+    const int dq = ts.dq[w];
+    tiled_fetch(s, ts, w, dq, S, false);
+    tiled_draw_normals(p, e, w, S);
+    tiled_wait();
+    propose_body(s, wk, ts, w, e, p, dq, S);
 }
 
 __global__ void __launch_bounds__(kTb, 8) k_tiled_accept(DevSys s, DevWalkers wk, TiledState ts, int w0, int W,
                                                          int e, SweepParams p) {
-    __shared__ AcceptSmem S;
+    extern __shared__ __align__(16) unsigned char tsm[];
+    TiledSmem& S = *reinterpret_cast<TiledSmem*>(tsm);
     const int w = w0 + (int)blockIdx.x;
     if (w >= W) return;
-    accept_body(s, wk, ts, w, e, p, S);
+    const int dq = ts.dq[w];
+    tiled_fetch(s, ts, w, dq, S, true);
+    accept_body(s, wk, ts, w, e, p, dq, S);
 }
 
 // The accept step of electron e and the proposal of electron e + 1 of the
-// same walker in one launch (no flush between them): the walker's queue,
-// inverse and positions written by the accept step are read back by the
-// same CTA after a barrier.  Bound by the latency of its dependent loads:
-// twelve CTAs per SM (40 registers, 36 bytes of spills) hide more of it than
-// eight (64 registers): the 32-water step 100.9 -> 95.3 ms at 4096 walkers.
-__global__ void __launch_bounds__(kTb, 12) k_tiled_accept_propose(DevSys s, DevWalkers wk, TiledState ts, int w0,
-                                                                 int W, int e, SweepParams p) {
-    __shared__ AcceptSmem Sa;
-    __shared__ ProposeSmem Sp;
+// same walker in one launch (no flush between them): the walker's inverse and
+// positions written by the accept step are read back by the same CTA after a
+// barrier, K^-1 stays in shared memory.  Bound by the latency of its
+// dependent loads (512 walkers of the 32-water cluster: 33.4 us with the serial
+// loops over K^-1 reading global memory and one queued row in flight per warp,
+// 26.2 us now).  Eight CTAs per SM with 64 registers, for loads ahead of their
+// use, against twelve with 40: 2048 walkers in one chain of launches 119 against
+// 127 us an electron, 4096 in two groups 209 against 206.
+__global__ void __launch_bounds__(kTb, 8) k_tiled_accept_propose(DevSys s, DevWalkers wk, TiledState ts, int w0,
+                                                                   int W, int e, SweepParams p) {
+    extern __shared__ __align__(16) unsigned char tsm[];
+    TiledSmem& S = *reinterpret_cast<TiledSmem*>(tsm);
     const int w = w0 + (int)blockIdx.x;
     if (w >= W) return;
-    accept_body(s, wk, ts, w, e, p, Sa);
-    __syncthreads();
-    propose_body(s, wk, ts, w, e + 1, p, Sp);
+    const int dq = ts.dq[w];
+    tiled_fetch(s, ts, w, dq, S, true);
+    tiled_draw_normals(p, e + 1, w, S);
+    const int dq1 = accept_body(s, wk, ts, w, e, p, dq, S);
+    propose_body(s, wk, ts, w, e + 1, p, dq1, S);
 }
 
 // P[m] = row r_m of A0^-T for m < dq, zero rows beyond.
@@ -501,22 +601,22 @@ cudaError_t tiled_begin(const DevWalkers& wk, int W, int N, const TiledState& ts
 cudaError_t tiled_propose(const DevSys& s, const DevWalkers& wk, const TiledState& ts, int w0, int nw, int e,
                           const SweepParams& p, cudaStream_t st) {
     if (nw <= 0) return cudaSuccess;
-    k_tiled_propose<<<nw, kTb, 0, st>>>(s, wk, ts, w0, w0 + nw, e, p);
+    k_tiled_propose<<<nw, kTb, tiled_smem_bytes(s.n_nuc, s.n_shell), st>>>(s, wk, ts, w0, w0 + nw, e, p);
     return cudaGetLastError();
 }
 
 cudaError_t tiled_accept(const DevSys& s, const DevWalkers& wk, const TiledState& ts, int w0, int nw, int e,
-                         const SweepParams& p, cudaStream_t st) {
+                         const SweepParams& p, bool alone, cudaStream_t st) {
     if (nw <= 0) return cudaSuccess;
-    k_tiled_accept<<<nw, kTb, 0, st>>>(s, wk, ts, w0, w0 + nw, e, p);
-    return cudaGetLastError();
+    return launch_after(k_tiled_accept, dim3(nw), kTb, tiled_smem_bytes(s.n_nuc, s.n_shell), st, alone, s, wk, ts, w0,
+                        w0 + nw, e, p);
 }
 
 cudaError_t tiled_accept_propose(const DevSys& s, const DevWalkers& wk, const TiledState& ts, int w0, int nw, int e,
-                                 const SweepParams& p, cudaStream_t st) {
+                                 const SweepParams& p, bool alone, cudaStream_t st) {
     if (nw <= 0) return cudaSuccess;
-    k_tiled_accept_propose<<<nw, kTb, 0, st>>>(s, wk, ts, w0, w0 + nw, e, p);
-    return cudaGetLastError();
+    return launch_after(k_tiled_accept_propose, dim3(nw), kTb,
+                        tiled_smem_bytes(s.n_nuc, s.n_shell), st, alone, s, wk, ts, w0, w0 + nw, e, p);
 }
 
 // The queues of walkers [w0, w0 + nw) into A0^-T of one spin (four

@@ -717,19 +717,18 @@ __host__ __device__ inline SplitSmem split_layout(int Np) {
 __global__ void __launch_bounds__(192, 1)
     k_tc_gemm_split(const __grid_constant__ CUtensorMap tAh, const __grid_constant__ CUtensorMap tAl,
                     const __grid_constant__ CUtensorMap tBh, const __grid_constant__ CUtensorMap tBl, int M, int N,
-                    int K, float* __restrict__ D, int ldd, unsigned* err) {
+                    int Np, int K, float* __restrict__ D, int ldd, unsigned* err) {
     extern __shared__ unsigned char ssm_raw[];
     __shared__ __align__(8) uint64_t bar_full[kSStages], bar_empty[kSStages], bar_acc, bar_drain;
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
-    const int Np = (N + 15) & ~15;
     uint32_t ncol = 32;
     while ((int)ncol < Np) ncol <<= 1;
     const SplitSmem L = split_layout(Np);
     const uint32_t sraw = smem_u32(ssm_raw);
     const uint32_t sbase = (sraw + 1023u) & ~1023u;      // 1024-byte aligned stages
     unsigned char* ssm = ssm_raw + (sbase - sraw);
-    const int m0 = blockIdx.x * kTcM;
+    const int m0 = blockIdx.x * kTcM, n0 = blockIdx.y * Np;   // Np: columns of a tile
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_stage = (K + kSK - 1) / kSK;
     volatile int* abort_flag = &s_abort;
@@ -756,6 +755,8 @@ __global__ void __launch_bounds__(192, 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = s_tmem;
+    grid_wait();      // A's rows come from the launch before this one
+    grid_release();   // the next launch reads D only after its own wait
     if (warp == 0) {
         if (lane == 0) {
             int issued = 0;
@@ -770,8 +771,8 @@ __global__ void __launch_bounds__(192, 1)
                 const int k0 = s * kSK;
                 tma_load_2d(st, &tAh, k0, m0, full);
                 tma_load_2d(st + L.a_bytes, &tAl, k0, m0, full);
-                tma_load_2d(st + 2 * L.a_bytes, &tBh, k0, 0, full);
-                tma_load_2d(st + 2 * L.a_bytes + L.b_bytes, &tBl, k0, 0, full);
+                tma_load_2d(st + 2 * L.a_bytes, &tBh, k0, n0, full);
+                tma_load_2d(st + 2 * L.a_bytes + L.b_bytes, &tBl, k0, n0, full);
                 ++issued;
             }
             for (int s = (issued > (int)L.slots ? issued - (int)L.slots : 0); s < issued; ++s)
@@ -833,10 +834,10 @@ __global__ void __launch_bounds__(192, 1)
 #pragma unroll
                 for (int j = 0; j < 32; ++j) buf[lane * 33 + j] = __uint_as_float(r[j]);
                 __syncwarp();
-                const int col = c0 + lane;
+                const int col = n0 + c0 + lane;
                 for (int rr = 0; rr < 32; ++rr) {
                     const int row = m0 + q4 * 32 + rr;
-                    if (row < M && col < N) D[(size_t)row * ldd + col] = buf[rr * 33 + lane];
+                    if (row < M && c0 + lane < Np && col < N) D[(size_t)row * ldd + col] = buf[rr * 33 + lane];
                 }
                 __syncwarp();
             }
@@ -929,28 +930,36 @@ bool tc_split_plan(TcSplitPlan* p, int M, int N, int K, const float* Ah, const f
     if (M <= 0 || N <= 0 || N > kTcMaxN || K <= 0 || lda % 4 || ldb % 4 || !al16(Ah) || !al16(Al) || !al16(Bh) ||
         !al16(Bl))
         return false;
-    const int Np = (N + 15) & ~15;
+    // tile columns: all N where the row tiles fill the chip, else as few (32 at
+    // least: below, reading A's tile from shared memory bounds the MMAs) as keep
+    // the launch within one wave.  The products of an output are added in the
+    // same order either way.  32-water sweep, 512 walkers a launch (20 row
+    // tiles): 22.4 -> 19.0 us, then bound by the row tiles' reads from L2.
+    int dev = 0, n_sm = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    const int mt = (M + kTcM - 1) / kTcM;
+    int Np = 32;
+    while (Np < N && (long long)mt * ((N + Np - 1) / Np) > n_sm) Np += 16;
+    if (Np > ((N + 15) & ~15)) Np = (N + 15) & ~15;
     p->M = M;
     p->N = N;
     p->K = K;
+    p->Np = Np;
     return make_map_sw128(reinterpret_cast<CUtensorMap*>(p->map[0]), Ah, K, M, lda, kTcM) &&
            make_map_sw128(reinterpret_cast<CUtensorMap*>(p->map[1]), Al, K, M, lda, kTcM) &&
            make_map_sw128(reinterpret_cast<CUtensorMap*>(p->map[2]), Bh, K, N, ldb, Np) &&
            make_map_sw128(reinterpret_cast<CUtensorMap*>(p->map[3]), Bl, K, N, ldb, Np);
 }
 
-size_t tc_split_smem_bytes(int N) { return split_layout((N + 15) & ~15).total; }
-
-cudaError_t tc_split_prepare(int N) {
-    return cudaFuncSetAttribute(k_tc_gemm_split, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)tc_split_smem_bytes(N));
+cudaError_t tc_split_prepare() {
+    return cudaFuncSetAttribute(k_tc_gemm_split, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448 - 2048);
 }
 
-cudaError_t launch_tc_gemm_split(const TcSplitPlan& p, float* D, int ldd, unsigned* err, cudaStream_t st) {
+cudaError_t launch_tc_gemm_split(const TcSplitPlan& p, float* D, int ldd, unsigned* err, cudaStream_t st, bool after) {
     const CUtensorMap* m = reinterpret_cast<const CUtensorMap*>(p.map[0]);
-    k_tc_gemm_split<<<(p.M + kTcM - 1) / kTcM, 192, tc_split_smem_bytes(p.N), st>>>(m[0], m[1], m[2], m[3], p.M, p.N,
-                                                                                     p.K, D, ldd, err);
-    return cudaGetLastError();
+    const dim3 grid((p.M + kTcM - 1) / kTcM, (p.N + p.Np - 1) / p.Np);
+    return launch_after(k_tc_gemm_split, grid, 192, split_layout(p.Np).total, st, after, m[0], m[1], m[2], m[3], p.M, p.N,
+                        p.Np, p.K, D, ldd, err);
 }
 
 }  // namespace qmc

@@ -60,6 +60,85 @@ __global__ void k_orbitals_all(DevSys s, DevWalkers wk, int W, const int* only) 
     orbitals_item<T>(s, wk, w, i, (unsigned char*)sh_bas);
 }
 
+// The same orbitals as FP64 sums over the basis functions in index order
+// (3 x slower on the 32-water cluster: bound by the FP64 pipe).  New walkers of
+// the mixed form are built with it, and walkers a determinant expansion rebuilds
+// inside a sweep: the last bit of an FP64 sum decides how an FP32 inverse rounds,
+// and a mixed trajectory amplifies one such bit until an accept decision turns,
+// so a seeded mixed run repeats earlier ones only from the same bits.  Also for
+// a basis whose lists exceed shared memory.  sh_bas: 5 n_basis doubles of
+// shared memory.  live (n_shell bytes of shared memory): shells whose values
+// and derivatives are all exactly zero (screened) are left out of the
+// occupied-orbital contraction; the terms that remain are added in the same
+// order.
+template <typename T>
+__device__ __forceinline__ void orbitals_sums_item(const DevSys& s, const DevWalkers& wk, int w, int i, double* sh_bas,
+                                              unsigned char* live = nullptr) {
+    const int nb = s.n_basis;
+    double r[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) r[c] = wk.R[((size_t)w * s.N + i) * 3 + c];
+    for (int sh = threadIdx.x; sh < s.n_shell; sh += blockDim.x) shell_vgl<double>(s, sh, r, sh_bas, nb);
+    __syncthreads();
+    if (live) {
+        for (int sh = threadIdx.x; sh < s.n_shell; sh += blockDim.x) {
+            const int f0 = s.shell_fn[sh], f1 = s.shell_fn[sh + 1];
+            bool nz = false;
+            for (int c = 0; c < 5 && !nz; ++c)
+                for (int f = f0; f < f1 && !nz; ++f) nz = sh_bas[c * nb + f] != 0.0;
+            live[sh] = nz ? 1 : 0;
+        }
+        __syncthreads();
+    }
+    const int spin = i < s.n_up ? 0 : 1;
+    const int n = spin ? s.n_dn : s.n_up;
+    const int k = spin ? i - s.n_up : i;
+    const double* C = s.C[spin];
+    T* G = (T*)wk.G[spin] + ((size_t)w * n + k) * 4 * n;
+    double* A = wk.Ascr[spin] + ((size_t)w * n + k) * n;
+    for (int o = threadIdx.x; o < 5 * n; o += blockDim.x) {
+        const int c = o / n, j = o - c * n;
+        const double* b = sh_bas + c * nb;
+        double acc = 0.0;
+        if (live) {
+            for (int sh = 0; sh < s.n_shell; ++sh) {
+                if (!live[sh]) continue;
+                for (int l = s.shell_fn[sh]; l < s.shell_fn[sh + 1]; ++l) acc += C[(size_t)l * n + j] * b[l];
+            }
+        } else {
+            for (int l = 0; l < nb; ++l) acc += C[(size_t)l * n + j] * b[l];
+        }
+        if (c == 0)
+            A[j] = acc;
+        else
+            G[(c - 1) * n + j] = (T)acc;
+    }
+    if (s.msd) {  // active virtual orbitals of a determinant expansion
+        const int nv = s.n_vir[spin];
+        const double* Cv = s.Cv[spin];
+        T* Av = (T*)wk.Av[spin] + ((size_t)w * n + k) * nv;
+        T* Gv = (T*)wk.Gv[spin] + ((size_t)w * n + k) * 4 * nv;
+        for (int o = threadIdx.x; o < 5 * nv; o += blockDim.x) {
+            const int c = o / nv, p = o - c * nv;
+            const double* b = sh_bas + c * nb;
+            double acc = 0.0;
+            for (int l = 0; l < nb; ++l) acc += Cv[(size_t)l * nv + p] * b[l];
+            if (c == 0)
+                Av[p] = (T)acc;
+            else
+                Gv[(c - 1) * nv + p] = (T)acc;
+        }
+    }
+}
+
+template <typename T>
+__global__ void k_orbitals_sums(DevSys s, DevWalkers wk, int W, const int* only) {
+    extern __shared__ double sh_bas[];  // [5][n_basis], then one live flag per shell
+    const int w = blockIdx.x, i = blockIdx.y;
+    if (w >= W || (only && !only[w])) return;
+    orbitals_sums_item<T>(s, wk, w, i, sh_bas, reinterpret_cast<unsigned char*>(sh_bas + 5 * s.n_basis));
+}
+
 // In-place Gauss-Jordan inversion with partial (row) pivoting, FP64, one
 // CTA per (walker, spin), the n x n matrix in shared memory.  Produces
 // ln|det A|, sign(det A) and the transposed inverse in the storage type.
@@ -692,8 +771,19 @@ size_t orbitals_smem_bytes(const DevSys& s) {
 }
 
 template <typename T>
-cudaError_t launch_orbitals_all(const DevSys& s, const DevWalkers& wk, int W, cudaStream_t st, const int* only) {
+cudaError_t launch_orbitals_all(const DevSys& s, const DevWalkers& wk, int W, cudaStream_t st, const int* only,
+                                bool sums) {
     if (W == 0 || s.N == 0) return cudaSuccess;
+    if (sums || Basis64Layout(s.n_nuc, s.n_prim, s.n_shell, s.n_basis).total > kBasis64Max) {
+        const size_t smem = sizeof(double) * 5 * s.n_basis + (size_t)s.n_shell;
+        if (smem > 48 * 1024) {
+            cudaError_t e = cudaFuncSetAttribute(k_orbitals_sums<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        k_orbitals_sums<T><<<dim3(W, s.N), s.n_up > 32 ? 256 : 128, smem, st>>>(s, wk, W, only);
+        return cudaGetLastError();
+    }
     const size_t smem = orbitals_smem_bytes(s);
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
     const int nt = nmax > 128 ? (nmax > 256 ? 256 : (nmax + 31) & ~31) : 128;   // a thread per orbital
@@ -843,8 +933,8 @@ template cudaError_t launch_eloc_batch<double>(const BatchSys*, BatchPlan*, int,
                                                cudaStream_t);
 template cudaError_t launch_eloc_batch<float>(const BatchSys*, BatchPlan*, int, int, int, int, size_t, cudaStream_t);
 
-template cudaError_t launch_orbitals_all<double>(const DevSys&, const DevWalkers&, int, cudaStream_t, const int*);
-template cudaError_t launch_orbitals_all<float>(const DevSys&, const DevWalkers&, int, cudaStream_t, const int*);
+template cudaError_t launch_orbitals_all<double>(const DevSys&, const DevWalkers&, int, cudaStream_t, const int*, bool);
+template cudaError_t launch_orbitals_all<float>(const DevSys&, const DevWalkers&, int, cudaStream_t, const int*, bool);
 template cudaError_t launch_eloc<double>(const DevSys&, const DevWalkers&, int, double*, double*, double*,
                                          double*, unsigned*, cudaStream_t);
 template cudaError_t launch_eloc<float>(const DevSys&, const DevWalkers&, int, double*, double*, double*,

@@ -337,6 +337,7 @@ struct qmc_ctx {
     // walker groups of the tiled sweep: group 0 on the handle's stream, the
     // others on streams of their own, forked from it and joined back
     int tiled_groups = 2;
+    bool tiled_groups_set = false;   // by the environment
     cudaStream_t tiled_side[kTiledMaxGroups - 1] = {};
     cudaEvent_t tiled_ev[kTiledMaxGroups] = {};   // the fork, then one join per side stream
 
@@ -824,11 +825,12 @@ struct qmc_ctx {
 
     // FP64 recompute of every walker's inverse, log-determinant and
     // orbital-gradient cache from its positions.
-    void recompute(int which) {
+    // fresh: walkers that were just set (see k_orbitals_sums).
+    void recompute(int which, bool fresh = false) {
         const DevWalkers& k = wk[which];
         tm.begin(stream);
         if (mode == QMC_MIXED) {
-            QMC_CK(launch_orbitals_all<float>(ds, k, W, stream));
+            QMC_CK(launch_orbitals_all<float>(ds, k, W, stream, nullptr, fresh));
         } else {
             QMC_CK(launch_orbitals_all<double>(ds, k, W, stream));
         }
@@ -970,12 +972,13 @@ struct qmc_ctx {
         t.rn = dalloc<double>(tiled_allocs, (size_t)Wt * 3);
         t.Rp = dalloc<float2>(tiled_allocs, (size_t)Wt * 3 * N());
         {
-            std::vector<int> fs;
+            std::vector<int2> fi;
             for (int q = 0; q < (int)sh_l.size(); ++q) {
                 const int nf = sh_l[q] == 0 ? 1 : sh_l[q] == 1 ? 3 : (sh_pure[q] ? 5 : 6);
-                for (int f = 0; f < nf; ++f) fs.push_back(q);
+                for (int f = 0; f < nf; ++f)
+                    fi.push_back(make_int2(q, (sh_center[q] << 8) | (f << 4) | (sh_l[q] << 1) | (sh_pure[q] ? 1 : 0)));
             }
-            t.fn_shell = upload(tiled_allocs, fs);
+            t.fn_info = upload(tiled_allocs, fi);
         }
         // the padding columns of B' and the queue rows are read by the GEMMs
         // before anything is written there: start from zeros
@@ -999,7 +1002,12 @@ struct qmc_ctx {
     void sweep_tiled(const SweepParams& p) {
         ensure_tiled();
         const DevWalkers& k = wk[cur];
-        const int groups_max = std::max(1, std::min(tiled_groups, W / 256));
+        // one chain below kTiledSplitW walkers unless the environment asks
+        // for groups: 32 waters, 1024 / 2048 walkers 67 / 119 us an electron in
+        // one chain and 78 / 125 in two, 4096 walkers 230 and 206
+        constexpr int kTiledSplitW = 3072;
+        const int groups_max =
+            tiled_groups_set || W >= kTiledSplitW ? std::max(1, std::min(tiled_groups, W / 256)) : 1;
         const int per = ((W + groups_max - 1) / groups_max + 127) / 128 * 128;
         const int ng = std::max(1, (W + per - 1) / per);
         int gw0[kTiledMaxGroups + 1];
@@ -1022,8 +1030,7 @@ struct qmc_ctx {
                                       tiled.Bl + off, tiled.nbp, tiled.Cth[spin], tiled.Ctl[spin], tiled.nbp),
                         QMC_ERR_UNSUPPORTED, "tensor maps of the tiled sweep's orbital GEMM could not be encoded");
             }
-        for (int spin = 0; spin < 2; ++spin)
-            if ((spin ? n_dn : n_up) > 0) QMC_CK(tc_split_prepare(spin ? n_dn : n_up));
+        QMC_CK(tc_split_prepare());
         cudaEvent_t t0 = tm.mark(stream);
         int launches = 1;
         QMC_CK(tiled_begin(k, W, N(), tiled, stream));
@@ -1041,17 +1048,18 @@ struct qmc_ctx {
                 for (int g = 0; g < ng; ++g) {
                     const int w0 = gw0[g], nw = gw0[g + 1] - gw0[g];
                     cudaEvent_t a = tm.mark(st[g]);
-                    QMC_CK(launch_tc_gemm_split(plan[g][spin], tiled.Phi + (size_t)w0 * 5 * n, n, d_err, st[g]));
+                    QMC_CK(launch_tc_gemm_split(plan[g][spin], tiled.Phi + (size_t)w0 * 5 * n, n, d_err, st[g],
+                                                ng == 1));
                     tm.span(F_SWEEP_GEMM, 1, a, st[g]);
                     if (flush) {
                         // accept, flush the queues, then (unless it was the
                         // last electron) propose the next electron's move
-                        QMC_CK(tiled_accept(ds, k, tiled, w0, nw, e, p, st[g]));
+                        QMC_CK(tiled_accept(ds, k, tiled, w0, nw, e, p, ng == 1, st[g]));
                         QMC_CK(tiled_flush(k, tiled, w0, nw, spin, n, d_err, st[g]));
                         if (e + 1 < N()) QMC_CK(tiled_propose(ds, k, tiled, w0, nw, e + 1, p, st[g]));
                         launches += e + 1 < N() ? 6 : 5;
                     } else {
-                        QMC_CK(tiled_accept_propose(ds, k, tiled, w0, nw, e, p, st[g]));
+                        QMC_CK(tiled_accept_propose(ds, k, tiled, w0, nw, e, p, ng == 1, st[g]));
                         launches += 1;
                     }
                 }
@@ -1102,7 +1110,7 @@ struct qmc_ctx {
             tm.begin(stream);
             const DevWalkers& k = wk[cur];
             if (mode == QMC_MIXED) {
-                QMC_CK(launch_orbitals_all<float>(ds, k, W, stream, d_refresh));
+                QMC_CK(launch_orbitals_all<float>(ds, k, W, stream, d_refresh, true));
             } else {
                 QMC_CK(launch_orbitals_all<double>(ds, k, W, stream, d_refresh));
             }
@@ -1452,8 +1460,10 @@ int qmc_create(qmc_t* out, int device, void* cuda_stream) {
     if (const char* env = std::getenv("QMC_SWEEP_TILED_MIN_N")) h->tiled_min_n = std::max(4, std::atoi(env));
     if (const char* env = std::getenv("QMC_NLPP_TC")) h->nlpp_tc = std::atoi(env) != 0;
     if (const char* env = std::getenv("QMC_NLPP_TC_MIN_N")) h->nlpp_tc_min_n = std::max(1, std::atoi(env));
-    if (const char* env = std::getenv("QMC_SWEEP_TILED_GROUPS"))
+    if (const char* env = std::getenv("QMC_SWEEP_TILED_GROUPS")) {
+        h->tiled_groups_set = true;
         h->tiled_groups = std::max(1, std::min(kTiledMaxGroups, std::atoi(env)));
+    }
     if (cudaSetDevice(device) != cudaSuccess) {
         g_create_error = "cudaSetDevice failed";
         delete h;
@@ -1794,7 +1804,7 @@ int qmc_set_walkers(qmc_t h, int n_walkers, const double* R, int on_device) {
                                on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->stream));
         k_fill<<<(n_walkers + 255) / 256, 256, 0, h->stream>>>(h->wk[0].weight, n_walkers, 1.0);
         QMC_CK(cudaGetLastError());
-        h->recompute(0);
+        h->recompute(0, true);
         h->eloc(0, h->wk[0].eloc, nullptr, nullptr, nullptr);
         h->check_device_errors();
         h->walkers_valid = true;
@@ -1843,7 +1853,7 @@ int qmc_init_walkers(qmc_t h, int n_walkers, uint64_t seed) {
         QMC_CK(cudaGetLastError());
         k_fill<<<(n_walkers + 255) / 256, 256, 0, h->stream>>>(h->wk[0].weight, n_walkers, 1.0);
         QMC_CK(cudaGetLastError());
-        h->recompute(0);
+        h->recompute(0, true);
         h->eloc(0, h->wk[0].eloc, nullptr, nullptr, nullptr);
         h->check_device_errors();
         h->walkers_valid = true;
@@ -3049,7 +3059,7 @@ int qmc_tc_gemm_split(int M, int N, int K, const float* A_hi, const float* A_lo,
     TcSplitPlan plan;
     if (!tc_split_plan(&plan, M, N, K, A_hi, A_lo, lda, B_hi, B_lo, ldb)) return QMC_ERR_UNSUPPORTED;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    if (tc_split_prepare(N) != cudaSuccess || launch_tc_gemm_split(plan, D, ldd, d_flag[dev], st) != cudaSuccess)
+    if (tc_split_prepare() != cudaSuccess || launch_tc_gemm_split(plan, D, ldd, d_flag[dev], st) != cudaSuccess)
         return QMC_ERR_CUDA;
     unsigned f = 0;
     if (cudaMemcpyAsync(&f, d_flag[dev], sizeof(unsigned), cudaMemcpyDeviceToHost, st) != cudaSuccess ||

@@ -372,14 +372,13 @@ __device__ __forceinline__ int accept_move(T rho, const T gd[3], const T gj[3], 
 // [6..8] and the drift at r [9..11].  The acceptance test reads the step and
 // drift back instead of forming r' - r in FP64 (the step is the float that
 // was added to r, so both agree).
-__device__ __forceinline__ void propose_move_mixed(const float g[3], double tau, const double r[3], uint2 key,
-                                                   uint32_t sweep, uint32_t e, uint32_t slot, double* scal,
-                                                   float* fs) {
+// propose_move_drawn and accept_move_drawn take the random numbers drawn
+// beforehand (draw_normals_f, accept_uniform_f).
+__device__ __forceinline__ void propose_move_drawn(const float g[3], double tau, const double r[3],
+                                                   const float chi[3], double* scal, float* fs) {
     const float tf = (float)tau;
     const float v2 = g[0] * g[0] + g[1] * g[1] + g[2] * g[2];
     const float f = 2.0f / (1.0f + sqrtf(1.0f + 2.0f * v2 * tf));
-    float chi[3];
-    draw_normals_f(key, sweep, e, slot, chi);
     const float sq = sqrtf(tf);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -394,10 +393,21 @@ __device__ __forceinline__ void propose_move_mixed(const float g[3], double tau,
         fs[9 + c] = vb;
     }
 }
+__device__ __forceinline__ void propose_move_mixed(const float g[3], double tau, const double r[3], uint2 key,
+                                                   uint32_t sweep, uint32_t e, uint32_t slot, double* scal,
+                                                   float* fs) {
+    float chi[3];
+    draw_normals_f(key, sweep, e, slot, chi);
+    propose_move_drawn(g, tau, r, chi, scal, fs);
+}
 
-__device__ __forceinline__ int accept_move_mixed(float rho, const float gd[3], const float gj[3], float dJ,
-                                                 double tau, const float* fs, uint2 key, uint32_t sweep, uint32_t e,
-                                                 uint32_t slot) {
+__device__ __forceinline__ float accept_uniform_f(uint2 key, uint32_t sweep, uint32_t e, uint32_t slot) {
+    const uint4 x = philox4x32_10(make_uint4(sweep, e, slot, 1u), key);
+    return ((float)x.x + 0.5f) * 2.3283064365386963e-10f;
+}
+
+__device__ __forceinline__ int accept_move_drawn(float rho, const float gd[3], const float gj[3], float dJ,
+                                                 double tau, const float* fs, float u) {
     if (!(rho > 0.0f && isfinite(rho))) return 0;
     const float ir = 1.0f / rho;
     float g[3];
@@ -416,9 +426,12 @@ __device__ __forceinline__ int accept_move_mixed(float rho, const float gd[3], c
         bwd += bk * bk;
     }
     const float lnp = 2.0f * logf(rho) + 2.0f * dJ - (bwd - fwd) / (2.0f * tf);
-    const uint4 x = philox4x32_10(make_uint4(sweep, e, slot, 1u), key);
-    const float u = ((float)x.x + 0.5f) * 2.3283064365386963e-10f;
     return (lnp >= 0.0f) || (u < expf(lnp));
+}
+__device__ __forceinline__ int accept_move_mixed(float rho, const float gd[3], const float gj[3], float dJ,
+                                                 double tau, const float* fs, uint2 key, uint32_t sweep, uint32_t e,
+                                                 uint32_t slot) {
+    return accept_move_drawn(rho, gd, gj, dJ, tau, fs, accept_uniform_f(key, sweep, e, slot));
 }
 
 // ---------------------------------------------------------------------
@@ -1278,6 +1291,35 @@ __device__ __forceinline__ float warp_sum(float v) {
 
 
 // ---------------------------------------------------------------------
+// Programmatic dependent launch: a kernel launched with launch_after may start
+// when every CTA of the kernel before it in the stream has called
+// grid_release (or ended); grid_wait returns when that kernel has completed and
+// its writes are visible.  Without the launch attribute (after false) both do
+// nothing.
+// ---------------------------------------------------------------------
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+inline cudaError_t launch_after(void (*f)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, bool after,
+                                A&&... args) {
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = after ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, f, P(args)...);
+}
+
+// ---------------------------------------------------------------------
 // Launchers (defined in the kernel translation units).
 // ---------------------------------------------------------------------
 struct SweepParams {
@@ -1292,8 +1334,9 @@ size_t orbitals_smem_bytes(const DevSys& s);
 size_t eloc_smem_bytes(const DevSys& s, int nt, int elem);
 template <typename T>
 cudaError_t launch_orbitals_all(const DevSys& s, const DevWalkers& wk, int W, cudaStream_t st,
-                                const int* only = nullptr);
+                                const int* only = nullptr, bool sums = false);
 // only (optional, [W]): rebuild just the walkers whose flag is nonzero.
+// launch_orbitals_all, sums: FP64 sums in index order (see k_orbitals_sums).
 cudaError_t launch_invert(const DevSys& s, const DevWalkers& wk, int W, int store_fp32, unsigned* err,
                           cudaStream_t st, const int* only = nullptr);
 // Jastrow parameter derivatives (k_wavefunction.cu): for P = 4 + n_nuc +
@@ -1384,12 +1427,14 @@ cudaError_t launch_tc_gemm(int batch, int M, int N, int K, const float* A, long 
 // (call it outside any stream capture).
 struct alignas(64) TcSplitPlan {
     unsigned char map[4][128];   // CUtensorMap of A_hi, A_lo, B_hi, B_lo
-    int M, N, K;
+    int M, N, K, Np;             // Np: columns of a tile
 };
 bool tc_split_plan(TcSplitPlan* p, int M, int N, int K, const float* Ah, const float* Al, int lda, const float* Bh,
                    const float* Bl, int ldb);
-cudaError_t tc_split_prepare(int N);
-cudaError_t launch_tc_gemm_split(const TcSplitPlan& p, float* D, int ldd, unsigned* err, cudaStream_t st);
+cudaError_t tc_split_prepare();
+// after: the launch may start before the kernel ahead of it ends (launch_after)
+cudaError_t launch_tc_gemm_split(const TcSplitPlan& p, float* D, int ldd, unsigned* err, cudaStream_t st,
+                                 bool after = false);
 cudaError_t launch_tc_gemm_ab(int batch, int M, int N, int K, float alpha, const float* A, long long sA, int lda,
                               const float* B, long long sB, int ldb, int b_trans, float beta, float* D, long long sD,
                               int ldd, unsigned* err, cudaStream_t st);

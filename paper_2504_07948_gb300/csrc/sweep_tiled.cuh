@@ -31,7 +31,7 @@ struct TiledState {
     float* mv;       // [W][kTiledMv] r' hi/lo, step, drift at r, Jastrow at r
     double* rn;      // [W][3]        r' in double
     float2* Rp;      // [W][N][3]     positions as hi/lo floats
-    const int* fn_shell;   // [n_basis]  shell of each basis function
+    const int2* fn_info;   // [n_basis]  (shell, centre << 8 | function of the shell << 4 | l << 1 | pure)
 };
 
 // Pieces of one sweep of every walker (mixed form only; k_sweep_tiled.cu):
@@ -44,11 +44,12 @@ struct TiledState {
 cudaError_t tiled_begin(const DevWalkers& wk, int W, int N, const TiledState& ts, cudaStream_t st);
 cudaError_t tiled_propose(const DevSys& s, const DevWalkers& wk, const TiledState& ts, int w0, int nw, int e,
                           const SweepParams& p, cudaStream_t st);
+// alone: the group's launches have the GPU to themselves.
 cudaError_t tiled_accept(const DevSys& s, const DevWalkers& wk, const TiledState& ts, int w0, int nw, int e,
-                         const SweepParams& p, cudaStream_t st);
+                         const SweepParams& p, bool alone, cudaStream_t st);
 // tiled_accept of electron e and tiled_propose of e + 1 in one launch.
 cudaError_t tiled_accept_propose(const DevSys& s, const DevWalkers& wk, const TiledState& ts, int w0, int nw, int e,
-                                 const SweepParams& p, cudaStream_t st);
+                                 const SweepParams& p, bool alone, cudaStream_t st);
 cudaError_t tiled_flush(const DevWalkers& wk, const TiledState& ts, int w0, int nw, int spin, int n, unsigned* err,
                         cudaStream_t st);
 cudaError_t tiled_end(const TiledState& ts, int W, unsigned long long* n_acc, cudaStream_t st);
