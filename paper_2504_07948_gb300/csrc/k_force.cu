@@ -162,27 +162,6 @@ __device__ __forceinline__ void warp_radial3(const DevSys& s, int p0, int np, do
     }
 }
 
-// Sum over a warp of 8 values per lane by a transposing butterfly: 9 adds
-// per lane instead of 40; v[0] of the lanes with (lane & 3) == 0 becomes the
-// total of value fold8_index(lane).
-__device__ __forceinline__ int fold8_index(int lane) {
-    return ((lane >> 2) & 1) | (((lane >> 3) & 1) << 1) | (((lane >> 4) & 1) << 2);
-}
-template <typename A>
-__device__ __forceinline__ A warp_fold8(const A (&v)[8]) {
-    const int lane = threadIdx.x & 31;
-    A a[4];
-    const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) a[i] = (h4 ? v[i + 4] : v[i]) + __shfl_xor_sync(0xffffffffu, h4 ? v[i] : v[i + 4], 16);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) a[i] = (h3 ? a[i + 2] : a[i]) + __shfl_xor_sync(0xffffffffu, h3 ? a[i] : a[i + 2], 8);
-    A r = (h2 ? a[1] : a[0]) + __shfl_xor_sync(0xffffffffu, h2 ? a[0] : a[1], 4);
-    r += __shfl_xor_sync(0xffffffffu, r, 2);
-    r += __shfl_xor_sync(0xffffffffu, r, 1);
-    return r;
-}
-
 // Terms of the shells [sh0, sh1) of one centre at one electron per lane (the
 // whole warp calls; `on`: the lane holds an electron): derivatives v, w with
 // respect to the electron coordinate (see RunTerms).  M, Y: weights of the

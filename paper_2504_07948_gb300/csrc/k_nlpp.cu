@@ -24,8 +24,9 @@
 //   4. per pass of at most kPtCap points: pair data (direction, distance,
 //      channel potentials) once per pair and point data (position, weight)
 //      once per point, by one thread each, into shared memory;
-//   5. one warp per quadrature point: lanes over shells for chi(r') . u_k,
-//      then over electrons and nuclei for the Jastrow change;
+//   5. one warp per pair, its points in registers: lanes over the nucleus's
+//      live primitives for chi(r') . u_k, then over electrons and nuclei for
+//      the Jastrow change;
 //   6. the walker total, summed in a fixed order, added to E_L.
 // The mixed form runs the basis, dot products and pair terms in FP32
 // (offsets from hi/lo split positions) and keeps FP64 to the per-pair and
@@ -117,73 +118,82 @@ __device__ __forceinline__ double legendre_dx(int l, double x) {
     return l == 0 ? 0.0 : l == 1 ? 1.0 : l == 2 ? 3.0 * x : 0.5 * (15.0 * x * x - 3.0);
 }
 
-// Value-only contracted shell at offset (x, y, z): sum_p c_p exp(-a_p t).
-template <typename T>
-__device__ __forceinline__ T radial0(const DevSys& s, int p0, int np, T t) {
-    const T* al = sys_alpha<T>(s);
-    const T* cn = sys_cn<T>(s);
-    T f = T(0);
-    for (int p = p0; p < p0 + np; ++p) {
-        const T a = al[p];
-        if (a * t > T(kScreenExponent)) continue;
-        f += cn[p] * dexp<T>(-a * t);
-    }
-    return f;
-}
-
 // Quadrature points of one pair processed together in registers.
 constexpr int kQ = 12;
 
-// Sum over a shell's functions of P_f(x, y, z) u_f (values only; the angular
-// forms and their order as in `angular`).
-template <typename T>
-__device__ __forceinline__ T shell_dot(int l, int pure, T x, T y, T z, const T (&uf)[6]) {
-    const T s3 = T(1.7320508075688772);
-    if (l == 0) return uf[0];
-    if (l == 1) return x * uf[0] + y * uf[1] + z * uf[2];
-    if (pure)
-        return s3 * (x * y * uf[0] + y * z * uf[1] + x * z * uf[3]) + (z * z - T(0.5) * (x * x + y * y)) * uf[2] +
-               T(0.5) * s3 * (x * x - y * y) * uf[4];
-    return x * x * uf[0] + y * y * uf[3] + z * z * uf[5] + s3 * (x * y * uf[1] + x * z * uf[2] + y * z * uf[4]);
-}
-
 // Lane's share of chi(R_a + r d_q) . u at the batch's points q < nqb of one
-// pair (nucleus a, distance r; dq[q] = r d_q): each lane takes shells in
-// (l, pure) order (neighbouring lanes mostly of one type), loads a shell's
-// data once and evaluates it at every point of the batch, so the loads are
-// shared by the points and the points give independent work.  A shell is
-// skipped when even the sphere's nearest point is screened.
+// pair (nucleus a = ecp_nuc[k], distance r; dq[q] = r d_q).  The nucleus's
+// primitives (those alive within its cutoff) are sorted by the distance at which they come alive on the
+// sphere of the points (|R_a - R_c| - sqrt(kScreenExponent / alpha)), so the
+// live ones are the first cnt, found by bisection, and consecutive lanes take
+// consecutive live primitives.  A lane loads a primitive and its shell's
+// combined polynomial c sum_f P_f u_f (1 + 3 + 6 coefficients, so s, p and d
+// primitives run the same instructions) once for all points.  (A lane per
+// shell, its primitives tested point by point, ran 120 instructions per shell
+// and point with half the lanes idle: 32 valence waters, 304 walkers 2.8 ms,
+// now 1.4 ms.)
 template <typename T>
-__device__ __forceinline__ void pair_basis_lane(const DevSys& s, int a, T r, const T (&dq)[kQ][3], int nqb,
+__device__ __forceinline__ void pair_basis_lane(const DevSys& s, int k, T r, const T (&dq)[kQ][3], int nqb,
                                                 const T* __restrict__ u, T (&dr)[kQ], int lane) {
-    for (int k = lane; k < s.n_shell; k += 32) {
-        const int sh = s.shell_by_type[k];
-        const int4 d = s.shell[sh];
-        const int c = 3 * d.x;
-        T cx, cy, cz;   // R_a - R_c
+    const int o = s.ecp_off[k];
+    int lo = 0, cnt = s.ecp_off[k + 1] - o;   // to the first primitive that is dead at r
+    while (lo < cnt) {
+        const int mid = (lo + cnt) >> 1;
+        if (s.ecp_live[o + mid] <= (float)r)
+            lo = mid + 1;
+        else
+            cnt = mid;
+    }
+    const T s3 = T(1.7320508075688772);
+    for (int p = lane; p < cnt; p += 32) {
+        T cx, cy, cz, al, cn;   // R_a - R_c, exponent, coefficient
         if constexpr (sizeof(T) == 8) {
-            cx = s.Rn[3 * a] - s.Rn[c];
-            cy = s.Rn[3 * a + 1] - s.Rn[c + 1];
-            cz = s.Rn[3 * a + 2] - s.Rn[c + 2];
+            const double4 g = s.ecp_geo[o + p];
+            cx = g.x;
+            cy = g.y;
+            cz = g.z;
+            al = g.w;
+            cn = s.ecp_cn[o + p];
         } else {
-            cx = diff_f2(s.Rn_hi[3 * a], s.Rn_lo[3 * a], s.Rn_hi[c], s.Rn_lo[c]);
-            cy = diff_f2(s.Rn_hi[3 * a + 1], s.Rn_lo[3 * a + 1], s.Rn_hi[c + 1], s.Rn_lo[c + 1]);
-            cz = diff_f2(s.Rn_hi[3 * a + 2], s.Rn_lo[3 * a + 2], s.Rn_hi[c + 2], s.Rn_lo[c + 2]);
+            const float4 g = s.ecp_geo_f[o + p];
+            cx = g.x;
+            cy = g.y;
+            cz = g.z;
+            al = g.w;
+            cn = s.ecp_cn_f[o + p];
         }
-        const T amin = sys_amin<T>(s)[sh];
-        const T gap = sqrt(cx * cx + cy * cy + cz * cz) - r;
-        if (gap > T(0) && amin * gap * gap > T(kScreenExponent)) continue;
-        const int l = d.y & 0xff, pure = d.y >> 8, fn0 = s.shell_fn[sh];
-        const int nf = shell_nfn(l, pure);
-        T uf[6];
-#pragma unroll
-        for (int f = 0; f < 6; ++f) uf[f] = f < nf ? u[fn0 + f] : T(0);
+        const int fn = s.ecp_fn[o + p], kind = fn & 7;
+        const T* uf = u + (fn >> 3);
+        T k0 = T(0), kx = T(0), ky = T(0), kz = T(0), xx = T(0), xy = T(0), xz = T(0), yy = T(0), yz = T(0), zz = T(0);
+        if (kind == 0) {
+            k0 = cn * uf[0];
+        } else if (kind == 2) {   // l << 1 | pure
+            kx = cn * uf[0];
+            ky = cn * uf[1];
+            kz = cn * uf[2];
+        } else if (kind == 5) {
+            const T a = T(-0.5) * cn * uf[2], b = T(0.5) * s3 * cn * uf[4];
+            xy = s3 * cn * uf[0];
+            yz = s3 * cn * uf[1];
+            xz = s3 * cn * uf[3];
+            xx = a + b;
+            yy = a - b;
+            zz = cn * uf[2];
+        } else {
+            xx = cn * uf[0];
+            xy = s3 * cn * uf[1];
+            xz = s3 * cn * uf[2];
+            yy = cn * uf[3];
+            yz = s3 * cn * uf[4];
+            zz = cn * uf[5];
+        }
 #pragma unroll
         for (int q = 0; q < kQ; ++q) {
             if (q < nqb) {
                 const T x = cx + dq[q][0], y = cy + dq[q][1], z = cz + dq[q][2];
                 const T t = x * x + y * y + z * z;
-                if (amin * t <= T(kScreenExponent)) dr[q] += radial0<T>(s, d.z, d.w, t) * shell_dot<T>(l, pure, x, y, z, uf);
+                const T P = k0 + x * (kx + xx * x + xy * y + xz * z) + y * (ky + yy * y + yz * z) + z * (kz + zz * z);
+                dr[q] += P * dexp<T>(-al * t);
             }
         }
     }
@@ -604,7 +614,7 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
     }
     const int M = s_count;
     const int gsize = kPtCap / nq;   // pairs per pass (the setter keeps nq <= kPtCap)
-    double part = 0.0;               // this warp's points (lane 0)
+    double part = 0.0;               // this lane's points
 
     for (int c0 = 0; c0 < M;) {
         // chunk: up to kChunk listed electrons of the spin of el[c0]
@@ -785,7 +795,7 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
                             else dq[q][c] = q < nqb ? ptf[3 * (p0 + q) + c] : 0.f;
                         }
                     }
-                    pair_basis_lane<T>(s, a, r, dq, nqb, U + ce * ldu, dr, lane);
+                    pair_basis_lane<T>(s, pk.y, r, dq, nqb, U + ce * ldu, dr, lane);
                     if constexpr (sizeof(T) == 8) pair_jastrow_lane_d(s, sR, i, a, dq, nqb, dj, lane);
                     else pair_jastrow_lane_f(s, sRf, i, a, dq, nqb, dj, lane);
                     if (s.n3 > 0) {
@@ -800,6 +810,23 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
                             for (int qq = 0; qq < kQ; ++qq)
                                 if (qq == q) dj[qq] += (T)d3;
                         }
+                    }
+                    if constexpr (kMode == kNlEnergy) {
+                        // warp totals by folds of eight; lane q then takes point q
+                        const T f0[8] = {dr[0], dr[1], dr[2], dr[3], dr[4], dr[5], dr[6], dr[7]};
+                        const T f1[8] = {dr[8], dr[9], dr[10], dr[11], dj[8], dj[9], dj[10], dj[11]};
+                        const T f2[8] = {dj[0], dj[1], dj[2], dj[3], dj[4], dj[5], dj[6], dj[7]};
+                        const T t0 = warp_fold8(f0), t1 = warp_fold8(f1), t2 = warp_fold8(f2);
+                        const int q = lane < kQ ? lane : 0;
+                        const int s8 = fold8_lane(q & 7), s4 = fold8_lane((q & 3) + 4);   // lanes that hold value q
+                        const T r0 = __shfl_sync(0xffffffffu, t0, s8), r1 = __shfl_sync(0xffffffffu, t1, fold8_lane(q & 3));
+                        const T j0 = __shfl_sync(0xffffffffu, t2, s8), j1 = __shfl_sync(0xffffffffu, t1, s4);
+                        if (lane < nqb) {
+                            const T d = q < 8 ? r0 : r1, j = q < 8 ? j0 : j1;
+                            if constexpr (sizeof(T) == 8) part += pt[8 * (p0 + q) + 3] * d * exp(j - jold[ce]);
+                            else part += pt[8 * (p0 + q) + 3] * (double)(d * expf(j));
+                        }
+                        continue;
                     }
 #pragma unroll
                     for (int q = 0; q < kQ; ++q)
@@ -842,14 +869,6 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
                             }
                         }
                         param_lane(s, sR, i, a, pt, p0, fq, nqb, pacc, dvw + wid * P, lane);
-                    } else if (lane == 0) {
-#pragma unroll
-                        for (int q = 0; q < kQ; ++q) {
-                            if (q < nqb) {
-                                if constexpr (sizeof(T) == 8) part += pt[8 * (p0 + q) + 3] * dr[q] * exp(dj[q] - jold[ce]);
-                                else part += pt[8 * (p0 + q) + 3] * (double)(dr[q] * expf(dj[q]));
-                            }
-                        }
                     }
                 }
             }
@@ -891,6 +910,7 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
         }
         return;
     }
+    part = warp_sum(part);
     if (lane == 0) s_part[wid] = part;
     __syncthreads();
     if (tid == 0) {

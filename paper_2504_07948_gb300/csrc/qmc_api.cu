@@ -542,6 +542,54 @@ struct qmc_ctx {
             s.shell_amin = upload(sys_allocs, am);
             s.shell_amin_f = upload(sys_allocs, amf);
         }
+        if (n_pp && s.n_ecp) {
+            struct Prim {
+                double live, x[3];
+                int p, sh;
+            };
+            std::vector<int> off(1, 0), fnk;
+            std::vector<float> live;
+            std::vector<double4> geo;
+            std::vector<double> ecn;
+            for (int a = 0; a < n_nuc; ++a) {
+                bool nl = false;
+                for (int t = 0; t < n_pp; ++t) nl |= pp_nuc[t] == a && pp_l[t] >= 0;
+                if (!nl || !(pp_rcut[a] > 0.0)) continue;
+                std::vector<Prim> pr;
+                for (int q = 0; q < s.n_shell; ++q) {
+                    double x[3], d2 = 0.0;
+                    for (int c = 0; c < 3; ++c) {
+                        x[c] = Rn[3 * a + c] - Rn[3 * sh[q].x + c];
+                        d2 += x[c] * x[c];
+                    }
+                    const double d = std::sqrt(d2);
+                    for (int p = sh[q].z; p < sh[q].z + sh[q].w; ++p) {
+                        // the margin covers the float comparison in the kernel
+                        const double reach = alpha[p] > 0.0 ? std::sqrt(kScreenExponent / alpha[p]) : 1e30;
+                        const double lv = d - reach - 1e-5 * (1.0 + d);
+                        if (lv <= pp_rcut[a]) pr.push_back(Prim{lv, {x[0], x[1], x[2]}, p, q});
+                    }
+                }
+                std::stable_sort(pr.begin(), pr.end(), [](const Prim& u, const Prim& v) { return u.live < v.live; });
+                for (const Prim& v : pr) {
+                    live.push_back((float)v.live);
+                    geo.push_back(make_double4(v.x[0], v.x[1], v.x[2], alpha[v.p]));
+                    ecn.push_back(cn[v.p]);
+                    fnk.push_back(fn[v.sh] << 3 | sh_l[v.sh] << 1 | (sh_l[v.sh] == 2 && sh_pure[v.sh] ? 1 : 0));
+                }
+                off.push_back((int)live.size());
+            }
+            std::vector<float4> gf(geo.size());
+            for (size_t i = 0; i < geo.size(); ++i)
+                gf[i] = make_float4((float)geo[i].x, (float)geo[i].y, (float)geo[i].z, (float)geo[i].w);
+            s.ecp_off = upload(sys_allocs, off);
+            s.ecp_live = upload(sys_allocs, live);
+            s.ecp_fn = upload(sys_allocs, fnk);
+            s.ecp_geo = upload(sys_allocs, geo);
+            s.ecp_cn = upload(sys_allocs, ecn);
+            s.ecp_geo_f = upload(sys_allocs, gf);
+            s.ecp_cn_f = upload(sys_allocs, std::vector<float>(ecn.begin(), ecn.end()));
+        }
         {
             std::vector<int> pc(alpha.size());
             s.n_fn_s = s.n_fn_p = 0;

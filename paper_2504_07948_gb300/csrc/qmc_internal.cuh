@@ -93,10 +93,22 @@ struct DevSys {
     const double* pp_rcut;   // [n_nuc]
     int n_ecp;               // nuclei with a non-local channel
     const int* ecp_nuc;      // [n_ecp]
+    // primitives seen from each such nucleus k, [ecp_off[k], ecp_off[k + 1]):
+    // those unscreened somewhere within its cutoff, sorted by the distance r
+    // at which they first are on the sphere of radius r about it; that
+    // distance, R_a - R_c and the exponent, the coefficient, first
+    // function << 3 | l << 1 | pure
+    const int* ecp_off;      // [n_ecp + 1]
+    const float* ecp_live;
+    const double4* ecp_geo;   // FP64 form
+    const double* ecp_cn;
+    const float4* ecp_geo_f;  // mixed form
+    const float* ecp_cn_f;
+    const int* ecp_fn;
     const double* CT[2];     // [n_s][n_basis] occupied coefficients, orbital-major (coalesced over the basis)
     const float* CT_f[2];
     const float* a_en_f;     // [n_nuc]
-    const int* shell_by_type;  // [n_shell] shells sorted by (l, pure), stable
+    const int* shell_by_type;  // [n_shell] shells sorted by (l, pure), stable (the force pass)
     int pp_nq, pp_rotate;
     const double* pp_quad;   // [pp_nq][3] unit vectors
     const double* pp_qw;     // [pp_nq] weights (sum 1)
@@ -1278,6 +1290,29 @@ __device__ __forceinline__ void block_sum8_to0(A (&v)[8], A* scratch) {
 #pragma unroll
         for (int k = 0; k < 8; ++k) v[k] = __shfl_sync(0xffffffffu, a, k);
     }
+}
+
+// Sum over a warp of 8 values per lane by a transposing butterfly: 9 adds
+// per lane instead of 40; v[0] of the lanes with (lane & 3) == 0 becomes the
+// total of value fold8_index(lane).
+__device__ __forceinline__ int fold8_index(int lane) {
+    return ((lane >> 2) & 1) | (((lane >> 3) & 1) << 1) | (((lane >> 4) & 1) << 2);
+}
+// A lane that holds value k (k < 8).
+__device__ __forceinline__ int fold8_lane(int k) { return ((k & 1) << 2) | ((k & 2) << 2) | ((k & 4) << 2); }
+template <typename A>
+__device__ __forceinline__ A warp_fold8(const A (&v)[8]) {
+    const int lane = threadIdx.x & 31;
+    A a[4];
+    const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) a[i] = (h4 ? v[i + 4] : v[i]) + __shfl_xor_sync(0xffffffffu, h4 ? v[i] : v[i + 4], 16);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) a[i] = (h3 ? a[i + 2] : a[i]) + __shfl_xor_sync(0xffffffffu, h3 ? a[i] : a[i + 2], 8);
+    A r = (h2 ? a[1] : a[0]) + __shfl_xor_sync(0xffffffffu, h2 ? a[0] : a[1], 4);
+    r += __shfl_xor_sync(0xffffffffu, r, 2);
+    r += __shfl_xor_sync(0xffffffffu, r, 1);
+    return r;
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
