@@ -28,6 +28,10 @@
 //      live primitives for chi(r') . u_k, then over electrons and nuclei for
 //      the Jastrow change;
 //   6. the walker total, summed in a fixed order, added to E_L.
+// The energy pass runs a walker as a cluster of up to kMaxSlices CTAs when the
+// walkers alone are few waves of CTAs: CTA c of S takes electrons c, c + S, ...
+// and the first sums the cluster's totals in order through distributed shared
+// memory.
 // The mixed form runs the basis, dot products and pair terms in FP32
 // (offsets from hi/lo split positions) and keeps FP64 to the per-pair and
 // per-point set-up (one thread each, not one warp) and the walker total:
@@ -35,9 +39,13 @@
 // across the lanes of every point would dominate.  The FP64 form takes the
 // Jastrow terms of each chunk electron at its old position once and only
 // the new terms per point.
+#include <cooperative_groups.h>
+
 #include "qmc_internal.cuh"
 
 namespace qmc {
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -47,6 +55,17 @@ constexpr int kChunk = 8;
 
 // Points of one pass: at most kPtCap quadrature points (pairs x rule).
 constexpr int kPtCap = 192;
+
+// Energy pass with the rows u_k at hand: the rows are read where they lie, so
+// a chunk costs only its pair list and holds up to kUgChunk electrons, a pass
+// up to kUgPtCap points; up to kUgMaxEcp pseudopotential nuclei (the pair list
+// grows as chunk x nuclei: 16 KB there), kChunk beyond.
+constexpr int kUgChunk = 32;
+constexpr int kUgPtCap = 576;
+constexpr int kUgMaxEcp = 64;
+__host__ __device__ inline int nl_chunk(bool ug, int n_ecp) { return ug && n_ecp <= kUgMaxEcp ? kUgChunk : kChunk; }
+__host__ __device__ constexpr int nl_pts(bool ug) { return ug ? kUgPtCap : kPtCap; }
+constexpr int kMaxSlices = 8;   // CTAs per walker of the energy pass (a portable cluster)
 
 struct NlLayout {
     size_t sR, sRf, rot, el, Ak, U, pairs, pg, pt, ptf, jold, beta, Fd, dvw, total;
@@ -58,7 +77,8 @@ enum NlMode { kNlEnergy = 0, kNlForce = 1, kNlParam = 2 };
 
 template <typename T>
 __host__ __device__ inline NlLayout nl_layout(int N, int nmax, int nb, int n_ecp, int n_shell, int n_nuc,
-                                              int mode, int n_par) {
+                                              int mode, int n_par, bool ug, int nq) {
+    const int chunk = nl_chunk(ug, n_ecp), pts = nl_pts(ug);
     const bool force = mode == kNlForce;
     NlLayout L;
     size_t o = 0;
@@ -71,13 +91,13 @@ __host__ __device__ inline NlLayout nl_layout(int N, int nmax, int nb, int n_ecp
     L.sRf = take(sizeof(float) * 3 * N);
     L.rot = take(sizeof(double) * 9 * (n_ecp > 0 ? n_ecp : 1));
     L.el = take(sizeof(int) * (N + 1));
-    L.Ak = take(sizeof(T) * kChunk * ((nmax + 3) & ~3));
-    L.U = take(sizeof(T) * kChunk * ((nb + 3) & ~3));
-    L.pairs = take(sizeof(int2) * kChunk * (n_ecp > 0 ? n_ecp : 1));
-    L.pg = take(sizeof(double) * 12 * kPtCap);   // per pair: x_hat[3], r, v_l[4], dv_l/dr[4]
-    L.pt = take(sizeof(double) * 8 * kPtCap);    // per point: r d_q [3], weight, dW/dR_a [3]
-    L.ptf = take(sizeof(float) * 3 * kPtCap);    // per point: r d_q in FP32
-    L.jold = take(sizeof(double) * kChunk);      // FP64 form: J terms of each chunk electron
+    L.Ak = take(ug ? 0 : sizeof(T) * chunk * ((nmax + 3) & ~3));
+    L.U = take(ug ? 0 : sizeof(T) * chunk * ((nb + 3) & ~3));
+    L.pairs = take(sizeof(int2) * chunk * (n_ecp > 0 ? n_ecp : 1));
+    L.pg = take(sizeof(double) * 12 * (pts / nq));   // per pair: x_hat[3], r, v_l[4], dv_l/dr[4]
+    L.pt = take(sizeof(double) * 8 * pts);       // per point: r d_q [3], weight, dW/dR_a [3]
+    L.ptf = take(sizeof(float) * 3 * pts);       // per point: r d_q in FP32
+    L.jold = take(sizeof(double) * chunk);      // FP64 form: J terms of each chunk electron
     // force pass: sum_p c_p chi(r'_p) per chunk electron, direct terms per nucleus
     L.beta = take(force ? sizeof(T) * kChunk * ((nb + 3) & ~3) : 0);
     L.Fd = take(force ? sizeof(double) * 3 * n_nuc : 0);
@@ -532,10 +552,25 @@ __device__ void param_lane(const DevSys& s, const double* sR, int i, int a, cons
     }
 }
 
+// Electron i within the cutoff of nucleus a (FP64 distance).  Distances that
+// FP32 shows to be beyond it, by more than its error for coordinates of this
+// size, take no FP64 (nearly all of the N x nuclei pairs).
+__device__ __forceinline__ int within_cutoff(const DevSys& s, const double* sR, const float* sRf, int i, int a) {
+    const double rc = s.pp_rcut[a];
+    const float ex = sRf[3 * i], ey = sRf[3 * i + 1], ez = sRf[3 * i + 2];
+    const float ax = s.Rn_hi[3 * a], ay = s.Rn_hi[3 * a + 1], az = s.Rn_hi[3 * a + 2];
+    const float fx = ex - ax, fy = ey - ay, fz = ez - az;
+    const float m = (float)rc + 1e-6f * (fabsf(ex) + fabsf(ey) + fabsf(ez) + fabsf(ax) + fabsf(ay) + fabsf(az) + 1.f);
+    if (fx * fx + fy * fy + fz * fz > m * m * (1.f + 1e-6f)) return 0;
+    const double x = sR[3 * i] - s.Rn[3 * a], y = sR[3 * i + 1] - s.Rn[3 * a + 1], z = sR[3 * i + 2] - s.Rn[3 * a + 2];
+    return sqrt(x * x + y * y + z * z) < rc;
+}
+
 // Walkers w0 + blockIdx.x < W.  Ug0 / Ug1: u_k of every electron of the
 // launch's walkers per spin, [w - w0][k][ldu] (formed on the tensor cores
 // beforehand), or nullptr: formed here.
-template <typename T, int kMode>
+// kUg (energy pass only): Ug0 / Ug1 are given and read in place.
+template <typename T, int kMode, bool kUg = false>
 __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, int w0, int W, double* eloc, uint2 key,
                                                       uint32_t sweep, const T* __restrict__ Ug0,
                                                       const T* __restrict__ Ug1, T* nlB0, T* nlB1, double* nlF) {
@@ -543,11 +578,15 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
     // parameter pass: eloc is deloc [W][P], P = 4 + n_nuc (1 + n3)
     const int P = 4 + s.n_nuc * (1 + s.n3);
     extern __shared__ __align__(16) unsigned char smem[];
-    const int w = w0 + (int)blockIdx.x;
+    // slice c of nsl: electrons c, c + nsl, ... of walker w
+    const int nsl = kMode == kNlEnergy ? (int)cg::this_cluster().num_blocks() : 1;
+    const int slice = kMode == kNlEnergy ? (int)cg::this_cluster().block_rank() : 0;
+    const int w = w0 + (int)blockIdx.x / nsl;
     if (w >= W) return;
     const int N = s.N, nu = s.n_up, nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
     const int nb = s.n_basis, ldu = (nb + 3) & ~3, nq = s.pp_nq;
-    const NlLayout L = nl_layout<T>(N, nmax, nb, s.n_ecp, s.n_shell, s.n_nuc, kMode, P);
+    const NlLayout L = nl_layout<T>(N, nmax, nb, s.n_ecp, s.n_shell, s.n_nuc, kMode, P, kUg, nq);
+    const int chunk = nl_chunk(kUg, s.n_ecp);
     double* sR = (double*)(smem + L.sR);
     float* sRf = (float*)(smem + L.sRf);
     double* rot = (double*)(smem + L.rot);
@@ -588,16 +627,11 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
     if (tid == 0) s_count = 0;
     __syncthreads();
     // electrons within some cutoff, ascending (warp-ordered ballots)
-    for (int base = 0; base < N; base += blockDim.x) {
-        const int i = base + tid;
+    for (int base = 0; base < N; base += nsl * blockDim.x) {
+        const int i = base + nsl * tid + slice;
         int in = 0;
         if (i < N)
-            for (int k = 0; k < s.n_ecp && !in; ++k) {
-                const int a = s.ecp_nuc[k];
-                const double x = sR[3 * i] - s.Rn[3 * a], y = sR[3 * i + 1] - s.Rn[3 * a + 1],
-                             z = sR[3 * i + 2] - s.Rn[3 * a + 2];
-                in = sqrt(x * x + y * y + z * z) < s.pp_rcut[a];
-            }
+            for (int k = 0; k < s.n_ecp && !in; ++k) in = within_cutoff(s, sR, sRf, i, s.ecp_nuc[k]);
         const unsigned bal = __ballot_sync(0xffffffffu, in);
         if (lane == 0) s_wcnt[wid] = __popc(bal);
         __syncthreads();
@@ -613,20 +647,22 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
         __syncthreads();
     }
     const int M = s_count;
-    const int gsize = kPtCap / nq;   // pairs per pass (the setter keeps nq <= kPtCap)
+    const int gsize = nl_pts(kUg) / nq;   // pairs per pass (the setter keeps nq <= kPtCap)
     double part = 0.0;               // this lane's points
 
     for (int c0 = 0; c0 < M;) {
         // chunk: up to kChunk listed electrons of the spin of el[c0]
         const int spin = el[c0] >= nu;
         int c1 = c0;
-        while (c1 < M && c1 - c0 < kChunk && (el[c1] >= nu) == spin) ++c1;
+        while (c1 < M && c1 - c0 < chunk && (el[c1] >= nu) == spin) ++c1;
         const int nc = c1 - c0;
         const int n = spin ? s.n_dn : nu;
         const T* Ainv = (const T*)wk.Ainv[spin];
         const T* Ug = spin ? Ug1 : Ug0;
         const int n4 = (n + 3) & ~3;
-        if (Ug) {
+        if constexpr (kUg) {
+            // the pairs read the precomputed rows in place
+        } else if (Ug) {
             // u_k precomputed: the chunk's rows into shared memory
             for (int q = tid; q < nc * ldu; q += blockDim.x) {
                 const int ce = q / ldu, b = q - ce * ldu;
@@ -650,12 +686,7 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
                 for (int k0 = 0; k0 < s.n_ecp; k0 += 32) {
                     const int k = k0 + lane;
                     int in = 0;
-                    if (k < s.n_ecp) {
-                        const int a = s.ecp_nuc[k];
-                        const double x = sR[3 * i] - s.Rn[3 * a], y = sR[3 * i + 1] - s.Rn[3 * a + 1],
-                                     z = sR[3 * i + 2] - s.Rn[3 * a + 2];
-                        in = sqrt(x * x + y * y + z * z) < s.pp_rcut[a];
-                    }
+                    if (k < s.n_ecp) in = within_cutoff(s, sR, sRf, i, s.ecp_nuc[k]);
                     const unsigned bal = __ballot_sync(0xffffffffu, in);
                     if (in) pairs[np + __popc(bal & ((1u << lane) - 1u))] = make_int2(ce, k);
                     np += __popc(bal);
@@ -666,7 +697,7 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
         __syncthreads();
         // u_ce = C_spin A^-1 e_k over the basis (orbital-major coefficients:
         // consecutive threads read consecutive basis functions)
-        if (!Ug) {
+        if (!kUg && !Ug) {
             const T* Cs;
             if constexpr (sizeof(T) == 8) Cs = s.CT[spin];
             else Cs = s.CT_f[spin];
@@ -795,7 +826,9 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
                             else dq[q][c] = q < nqb ? ptf[3 * (p0 + q) + c] : 0.f;
                         }
                     }
-                    pair_basis_lane<T>(s, pk.y, r, dq, nqb, U + ce * ldu, dr, lane);
+                    const T* u = U + ce * ldu;
+                    if constexpr (kUg) u = Ug + ((size_t)(w - w0) * n + (i - (spin ? nu : 0))) * ldu;
+                    pair_basis_lane<T>(s, pk.y, r, dq, nqb, u, dr, lane);
                     if constexpr (sizeof(T) == 8) pair_jastrow_lane_d(s, sR, i, a, dq, nqb, dj, lane);
                     else pair_jastrow_lane_f(s, sRf, i, a, dq, nqb, dj, lane);
                     if (s.n3 > 0) {
@@ -916,9 +949,16 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
     if (tid == 0) {
         double v = 0.0;
         for (int q = 0; q < kNlWarps; ++q) v += s_part[q];
+        s_part[0] = v;
+    }
+    if (nsl > 1) cg::this_cluster().sync();
+    if (tid == 0 && slice == 0) {
+        double v = s_part[0];
+        for (int c = 1; c < nsl; ++c) v += *cg::this_cluster().map_shared_rank(s_part, c);
         eloc[w] += v;
         if (!isfinite(eloc[w]) && wk.err) atomicOr(wk.err, kErrNonFinite);
     }
+    if (nsl > 1) cg::this_cluster().sync();   // the slices' totals have been read
 }
 
 }  // namespace
@@ -929,14 +969,33 @@ cudaError_t launch_nlpp(const DevSys& s, const DevWalkers& wk, int w0, int W, do
     if (W <= w0 || s.npp == 0 || s.n_ecp == 0) return cudaSuccess;
     if (s.pp_nq < 1 || s.pp_nq > kPtCap) return cudaErrorInvalidValue;
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
-    const size_t smem = nl_layout<T>(s.N, nmax, s.n_basis, s.n_ecp, s.n_shell, s.n_nuc, kNlEnergy, 0).total;
+    bool ug = U0 && U1;
+    size_t smem = nl_layout<T>(s.N, nmax, s.n_basis, s.n_ecp, s.n_shell, s.n_nuc, kNlEnergy, 0, ug, s.pp_nq).total;
+    if (ug && smem > 112 * 1024) {   // two CTAs per SM no longer fit
+        ug = false;
+        smem = nl_layout<T>(s.N, nmax, s.n_basis, s.n_ecp, s.n_shell, s.n_nuc, kNlEnergy, 0, ug, s.pp_nq).total;
+    }
     if (smem > 227 * 1024) return cudaErrorNotSupported;   // the host reports QMC_ERR_UNSUPPORTED
-    cudaError_t e =
-        cudaFuncSetAttribute(k_nlpp<T, kNlEnergy>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto f = ug ? k_nlpp<T, kNlEnergy, true> : k_nlpp<T, kNlEnergy, false>;
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_nlpp<T, kNlEnergy><<<W - w0, kNlThreads, smem, st>>>(s, wk, w0, W, eloc, key, sweep, (const T*)U0,
-                                                          (const T*)U1, nullptr, nullptr, nullptr);
-    return cudaGetLastError();
+    // slices until there are six waves of CTAs, while each still has a warp's
+    // worth of electrons (a slice repeats the rotations and positions)
+    int nsl = 1;
+    while (nsl < kMaxSlices && (long long)(W - w0) * nsl < 6 * 304 && s.N / (2 * nsl) >= 32) nsl *= 2;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = nsl;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(W - w0) * nsl);
+    cfg.blockDim = dim3(kNlThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, f, s, wk, w0, W, eloc, key, sweep, (const T*)U0, (const T*)U1, (T*)nullptr,
+                              (T*)nullptr, (double*)nullptr);
 }
 
 template <typename T>
@@ -945,7 +1004,7 @@ cudaError_t launch_nlpp_param(const DevSys& s, const DevWalkers& wk, int w0, int
     if (W <= w0 || s.npp == 0 || s.n_ecp == 0) return cudaSuccess;
     if (s.pp_nq < 1 || s.pp_nq > kPtCap) return cudaErrorInvalidValue;
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn, P = 4 + s.n_nuc * (1 + s.n3);
-    const size_t smem = nl_layout<T>(s.N, nmax, s.n_basis, s.n_ecp, s.n_shell, s.n_nuc, kNlParam, P).total;
+    const size_t smem = nl_layout<T>(s.N, nmax, s.n_basis, s.n_ecp, s.n_shell, s.n_nuc, kNlParam, P, false, s.pp_nq).total;
     if (smem > 227 * 1024) return cudaErrorNotSupported;   // the host reports QMC_ERR_UNSUPPORTED
     cudaError_t e = cudaFuncSetAttribute(k_nlpp<T, kNlParam>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -961,7 +1020,7 @@ cudaError_t launch_nlpp_force(const DevSys& s, const DevWalkers& wk, int w0, int
     if (W <= w0 || s.npp == 0 || s.n_ecp == 0) return cudaSuccess;
     if (s.pp_nq < 1 || s.pp_nq > kPtCap) return cudaErrorInvalidValue;
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
-    const size_t smem = nl_layout<T>(s.N, nmax, s.n_basis, s.n_ecp, s.n_shell, s.n_nuc, kNlForce, 0).total;
+    const size_t smem = nl_layout<T>(s.N, nmax, s.n_basis, s.n_ecp, s.n_shell, s.n_nuc, kNlForce, 0, false, s.pp_nq).total;
     if (smem > 227 * 1024) return cudaErrorNotSupported;   // the host reports QMC_ERR_UNSUPPORTED
     cudaError_t e = cudaFuncSetAttribute(k_nlpp<T, kNlForce>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

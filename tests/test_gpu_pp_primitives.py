@@ -78,3 +78,20 @@ def test_water_mixed(Q, monkeypatch, m, nq, tc):
     ref = O.Oracle(s).evaluate(R, pp_seed=9, pp_sweep=2)["eloc"]
     assert rel(e, ref) <= 1e-5, rel(e, ref)
     g.close()
+
+
+@pytest.mark.parametrize("m,W", [(9, 5), (17, 3), (32, 2)])
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-10), ("mixed", 1e-5)])
+def test_walkers_in_slices(Q, m, W, prec, tol):
+    """Few walkers of many electrons (the energy pass runs 2, 4 and 8 CTAs per
+    walker), and the same result a second time."""
+    s = synth.with_pseudopotential(synth.water_system(m))
+    R = walkers_at_edges(s, W, 11)
+    g = Q.QMC(s, precision=prec, seed=9)
+    Q.qmc_set_rng(g.h, 9, 2)
+    g.set_walkers(R)
+    e = g.eval_cached()["eloc"]
+    ref = O.Oracle(s).evaluate(R, pp_seed=9, pp_sweep=2)["eloc"]
+    assert rel(e, ref) <= tol, rel(e, ref)
+    assert np.array_equal(e, g.eval_cached()["eloc"])
+    g.close()
