@@ -29,9 +29,13 @@
 //      the Jastrow change;
 //   6. the walker total, summed in a fixed order, added to E_L.
 // The energy pass runs a walker as a cluster of up to kMaxSlices CTAs when the
-// walkers alone are few waves of CTAs: CTA c of S takes electrons c, c + S, ...
-// and the first sums the cluster's totals in order through distributed shared
-// memory.
+// walkers alone are few waves of CTAs: each takes a run of electrons (runs of
+// whole molecules; with every S-th electron the molecules' pattern of electrons
+// near and far from such nuclei left a slice of four at a third of the others'
+// work) and the first sums the cluster's totals in order through distributed
+// shared memory.  Barriers are few (a chunk and a pass each cover a slice of
+// the usual size): 32 valence waters, 512 walkers, 2.6 ms with a CTA per walker
+// and chunks of eight, now 1.8 ms.
 // The mixed form runs the basis, dot products and pair terms in FP32
 // (offsets from hi/lo split positions) and keeps FP64 to the per-pair and
 // per-point set-up (one thread each, not one warp) and the walker total:
@@ -59,9 +63,9 @@ constexpr int kPtCap = 192;
 // Energy pass with the rows u_k at hand: the rows are read where they lie, so
 // a chunk costs only its pair list and holds up to kUgChunk electrons, a pass
 // up to kUgPtCap points; up to kUgMaxEcp pseudopotential nuclei (the pair list
-// grows as chunk x nuclei: 16 KB there), kChunk beyond.
-constexpr int kUgChunk = 32;
-constexpr int kUgPtCap = 576;
+// grows as chunk x nuclei: 32 KB there), kChunk beyond.
+constexpr int kUgChunk = 64;
+constexpr int kUgPtCap = 768;
 constexpr int kUgMaxEcp = 64;
 __host__ __device__ inline int nl_chunk(bool ug, int n_ecp) { return ug && n_ecp <= kUgMaxEcp ? kUgChunk : kChunk; }
 __host__ __device__ constexpr int nl_pts(bool ug) { return ug ? kUgPtCap : kPtCap; }
@@ -578,7 +582,7 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
     // parameter pass: eloc is deloc [W][P], P = 4 + n_nuc (1 + n3)
     const int P = 4 + s.n_nuc * (1 + s.n3);
     extern __shared__ __align__(16) unsigned char smem[];
-    // slice c of nsl: electrons c, c + nsl, ... of walker w
+    // slice c of nsl: electrons [c N / nsl, (c + 1) N / nsl) of walker w
     const int nsl = kMode == kNlEnergy ? (int)cg::this_cluster().num_blocks() : 1;
     const int slice = kMode == kNlEnergy ? (int)cg::this_cluster().block_rank() : 0;
     const int w = w0 + (int)blockIdx.x / nsl;
@@ -627,10 +631,11 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
     if (tid == 0) s_count = 0;
     __syncthreads();
     // electrons within some cutoff, ascending (warp-ordered ballots)
-    for (int base = 0; base < N; base += nsl * blockDim.x) {
-        const int i = base + nsl * tid + slice;
+    const int e1 = (slice + 1) * N / nsl;
+    for (int base = slice * N / nsl; base < e1; base += blockDim.x) {
+        const int i = base + tid;
         int in = 0;
-        if (i < N)
+        if (i < e1)
             for (int k = 0; k < s.n_ecp && !in; ++k) in = within_cutoff(s, sR, sRf, i, s.ecp_nuc[k]);
         const unsigned bal = __ballot_sync(0xffffffffu, in);
         if (lane == 0) s_wcnt[wid] = __popc(bal);
