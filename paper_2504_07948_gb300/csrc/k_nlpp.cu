@@ -35,7 +35,7 @@
 // work) and the first sums the cluster's totals in order through distributed
 // shared memory.  Barriers are few (a chunk and a pass each cover a slice of
 // the usual size): 32 valence waters, 512 walkers, 2.6 ms with a CTA per walker
-// and chunks of eight, now 1.8 ms.
+// and chunks of eight, 1.8 ms with slices of 256-thread CTAs, now 1.6 ms.
 // The mixed form runs the basis, dot products and pair terms in FP32
 // (offsets from hi/lo split positions) and keeps FP64 to the per-pair and
 // per-point set-up (one thread each, not one warp) and the walker total:
@@ -53,8 +53,13 @@ namespace cg = cooperative_groups;
 
 namespace {
 
+enum NlMode { kNlEnergy = 0, kNlForce = 1, kNlParam = 2 };
+
 constexpr int kNlThreads = 256;
 constexpr int kNlWarps = kNlThreads / 32;
+// energy pass with the rows u_k at hand: small CTAs, so that one's serial
+// set-up runs under the others' points
+constexpr int kUgThreads = 128;
 constexpr int kChunk = 8;
 
 // Points of one pass: at most kPtCap quadrature points (pairs x rule).
@@ -63,11 +68,13 @@ constexpr int kPtCap = 192;
 // Energy pass with the rows u_k at hand: the rows are read where they lie, so
 // a chunk costs only its pair list and holds up to kUgChunk electrons, a pass
 // up to kUgPtCap points; up to kUgMaxEcp pseudopotential nuclei (the pair list
-// grows as chunk x nuclei: 32 KB there), kChunk beyond.
-constexpr int kUgChunk = 64;
-constexpr int kUgPtCap = 768;
+// grows as chunk x nuclei: 16 KB there), kChunk beyond.
+constexpr int kUgChunk = 32;
+constexpr int kUgPtCap = 384;
 constexpr int kUgMaxEcp = 64;
 __host__ __device__ inline int nl_chunk(bool ug, int n_ecp) { return ug && n_ecp <= kUgMaxEcp ? kUgChunk : kChunk; }
+__host__ __device__ constexpr int nl_pg(int mode) { return mode == kNlEnergy ? 8 : 12; }   // doubles per pair
+__host__ __device__ constexpr int nl_pt(int mode) { return mode == kNlEnergy ? 4 : 8; }    // and per point
 __host__ __device__ constexpr int nl_pts(bool ug) { return ug ? kUgPtCap : kPtCap; }
 constexpr int kMaxSlices = 8;   // CTAs per walker of the energy pass (a portable cluster)
 
@@ -77,7 +84,6 @@ struct NlLayout {
 
 // Passes of the kernel: the energy, the ionic-derivative terms, the Jastrow
 // parameter derivatives.
-enum NlMode { kNlEnergy = 0, kNlForce = 1, kNlParam = 2 };
 
 template <typename T>
 __host__ __device__ inline NlLayout nl_layout(int N, int nmax, int nb, int n_ecp, int n_shell, int n_nuc,
@@ -98,8 +104,8 @@ __host__ __device__ inline NlLayout nl_layout(int N, int nmax, int nb, int n_ecp
     L.Ak = take(ug ? 0 : sizeof(T) * chunk * ((nmax + 3) & ~3));
     L.U = take(ug ? 0 : sizeof(T) * chunk * ((nb + 3) & ~3));
     L.pairs = take(sizeof(int2) * chunk * (n_ecp > 0 ? n_ecp : 1));
-    L.pg = take(sizeof(double) * 12 * (pts / nq));   // per pair: x_hat[3], r, v_l[4], dv_l/dr[4]
-    L.pt = take(sizeof(double) * 8 * pts);       // per point: r d_q [3], weight, dW/dR_a [3]
+    L.pg = take(sizeof(double) * nl_pg(mode) * (pts / nq));   // per pair: x_hat[3], r, v_l[4], force: dv_l/dr[4]
+    L.pt = take(sizeof(double) * nl_pt(mode) * pts);   // per point: r d_q [3], weight, force: dW/dR_a [3]
     L.ptf = take(sizeof(float) * 3 * pts);       // per point: r d_q in FP32
     L.jold = take(sizeof(double) * chunk);      // FP64 form: J terms of each chunk electron
     // force pass: sum_p c_p chi(r'_p) per chunk electron, direct terms per nucleus
@@ -575,10 +581,12 @@ __device__ __forceinline__ int within_cutoff(const DevSys& s, const double* sR, 
 // beforehand), or nullptr: formed here.
 // kUg (energy pass only): Ug0 / Ug1 are given and read in place.
 template <typename T, int kMode, bool kUg = false>
-__global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, int w0, int W, double* eloc, uint2 key,
+__global__ void __launch_bounds__(kUg ? kUgThreads : kNlThreads) k_nlpp(DevSys s, DevWalkers wk, int w0, int W, double* eloc, uint2 key,
                                                       uint32_t sweep, const T* __restrict__ Ug0,
                                                       const T* __restrict__ Ug1, T* nlB0, T* nlB1, double* nlF) {
     constexpr bool kForce = kMode == kNlForce;
+    constexpr int kWarps = (kUg ? kUgThreads : kNlThreads) / 32;
+    constexpr int kPg = nl_pg(kMode), kPt = nl_pt(kMode);
     // parameter pass: eloc is deloc [W][P], P = 4 + n_nuc (1 + n3)
     const int P = 4 + s.n_nuc * (1 + s.n3);
     extern __shared__ __align__(16) unsigned char smem[];
@@ -608,12 +616,12 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
     if constexpr (kForce)
         for (int q = threadIdx.x; q < 3 * s.n_nuc; q += blockDim.x) Fd[q] = 0.0;
     if constexpr (kMode == kNlParam)
-        for (int q = threadIdx.x; q < kNlWarps * P; q += blockDim.x) dvw[q] = 0.0;
+        for (int q = threadIdx.x; q < kWarps * P; q += blockDim.x) dvw[q] = 0.0;
     double pacc[4] = {0.0, 0.0, 0.0, 0.0};   // parameter pass: this lane's a_anti, a_par, b_ee, b_en parts
     const int nmax4 = (nmax + 3) & ~3;
     __shared__ int s_count, s_npair;
-    __shared__ int s_wcnt[kNlWarps];
-    __shared__ double s_part[kNlWarps];
+    __shared__ int s_wcnt[kWarps];
+    __shared__ double s_part[kWarps];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 
     for (int q = tid; q < 3 * N; q += blockDim.x) {
@@ -646,7 +654,7 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
         __syncthreads();
         if (tid == 0) {
             int t = 0;
-            for (int q = 0; q < kNlWarps; ++q) t += s_wcnt[q];
+            for (int q = 0; q < kWarps; ++q) t += s_wcnt[q];
             s_count = s_count + t;
         }
         __syncthreads();
@@ -737,7 +745,7 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
         }
         if constexpr (sizeof(T) == 8) {
             // Jastrow terms of each chunk electron at its old position (one warp each)
-            for (int ce = wid; ce < nc; ce += kNlWarps) {
+            for (int ce = wid; ce < nc; ce += kWarps) {
                 const int i = el[c0 + ce];
                 double J = jastrow_terms_lane(s, sR, i, sR + 3 * i, lane);
                 for (int o = 16; o > 0; o >>= 1) J += __shfl_xor_sync(0xffffffffu, J, o);
@@ -759,7 +767,7 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
                     r2 += x[c] * x[c];
                 }
                 const double r = sqrt(r2);
-                double* d = pg + 12 * t;
+                double* d = pg + kPg * t;
 #pragma unroll
                 for (int c = 0; c < 3; ++c) d[c] = x[c] / r;
                 d[3] = r;
@@ -774,7 +782,7 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
 #pragma unroll
                 for (int l = 0; l < 4; ++l) {
                     d[4 + l] = v[l];
-                    d[8 + l] = dv[l];
+                    if constexpr (kForce) d[8 + l] = dv[l];
                 }
             }
             __syncthreads();
@@ -784,14 +792,14 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
                 const int2 pk = pairs[g0 + pr];
                 const double* m = rot + 9 * pk.y;
                 const double* o = s.pp_quad + 3 * q;
-                const double* d = pg + 12 * pr;
+                const double* d = pg + kPg * pr;
                 double cth = 0.0, dqv[3];
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
                     const double dq = m[3 * c] * o[0] + m[3 * c + 1] * o[1] + m[3 * c + 2] * o[2];
                     dqv[c] = dq;
                     cth += dq * d[c];
-                    pt[8 * t + c] = d[3] * dq;
+                    pt[kPt * t + c] = d[3] * dq;
                     ptf[3 * t + c] = (float)(d[3] * dq);
                 }
                 double wq = 0.0, dw[3] = {0.0, 0.0, 0.0};
@@ -808,16 +816,17 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
                                               d[4 + l] * legendre_dx(l, cth) * (-(dqv[c] - cth * d[c]) / d[3]));
                         }
                     }
-                pt[8 * t + 3] = wq * s.pp_qw[q];
+                pt[kPt * t + 3] = wq * s.pp_qw[q];
 #pragma unroll
-                for (int c = 0; c < 3; ++c) pt[8 * t + 4 + c] = dw[c] * s.pp_qw[q];
+                for (int c = 0; c < 3; ++c)
+                    if constexpr (kForce) pt[kPt * t + 4 + c] = dw[c] * s.pp_qw[q];
             }
             __syncthreads();
             // one warp per pair, its points in register batches of kQ
-            for (int pr = wid; pr < ng; pr += kNlWarps) {
+            for (int pr = wid; pr < ng; pr += kWarps) {
                 const int2 pk = pairs[g0 + pr];
                 const int ce = pk.x, i = el[c0 + ce], a = s.ecp_nuc[pk.y];
-                const T r = (T)pg[12 * pr + 3];
+                const T r = (T)pg[kPg * pr + 3];
                 for (int q0 = 0; q0 < nq; q0 += kQ) {
                     const int nqb = min(kQ, nq - q0);
                     const int p0 = pr * nq + q0;
@@ -827,7 +836,7 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
                         dr[q] = dj[q] = T(0);
 #pragma unroll
                         for (int c = 0; c < 3; ++c) {
-                            if constexpr (sizeof(T) == 8) dq[q][c] = q < nqb ? pt[8 * (p0 + q) + c] : 0.0;
+                            if constexpr (sizeof(T) == 8) dq[q][c] = q < nqb ? pt[kPt * (p0 + q) + c] : 0.0;
                             else dq[q][c] = q < nqb ? ptf[3 * (p0 + q) + c] : 0.f;
                         }
                     }
@@ -841,8 +850,8 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
                         const double re[3] = {sR[3 * i], sR[3 * i + 1], sR[3 * i + 2]};
                         const double J3o = jastrow3_lane(s, sR, i, re, lane);
                         for (int q = 0; q < nqb; ++q) {
-                            const double rp[3] = {s.Rn[3 * a] + pt[8 * (p0 + q)], s.Rn[3 * a + 1] + pt[8 * (p0 + q) + 1],
-                                                  s.Rn[3 * a + 2] + pt[8 * (p0 + q) + 2]};
+                            const double rp[3] = {s.Rn[3 * a] + pt[kPt * (p0 + q)], s.Rn[3 * a + 1] + pt[kPt * (p0 + q) + 1],
+                                                  s.Rn[3 * a + 2] + pt[kPt * (p0 + q) + 2]};
                             const double d3 = jastrow3_lane(s, sR, i, rp, lane) - (sizeof(T) == 8 ? 0.0 : J3o);
 #pragma unroll
                             for (int qq = 0; qq < kQ; ++qq)
@@ -861,8 +870,8 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
                         const T j0 = __shfl_sync(0xffffffffu, t2, s8), j1 = __shfl_sync(0xffffffffu, t1, s4);
                         if (lane < nqb) {
                             const T d = q < 8 ? r0 : r1, j = q < 8 ? j0 : j1;
-                            if constexpr (sizeof(T) == 8) part += pt[8 * (p0 + q) + 3] * d * exp(j - jold[ce]);
-                            else part += pt[8 * (p0 + q) + 3] * (double)(d * expf(j));
+                            if constexpr (sizeof(T) == 8) part += pt[kPt * (p0 + q) + 3] * d * exp(j - jold[ce]);
+                            else part += pt[kPt * (p0 + q) + 3] * (double)(d * expf(j));
                         }
                         continue;
                     }
@@ -878,9 +887,9 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
                         for (int q = 0; q < kQ; ++q) {
                             if constexpr (sizeof(T) == 8) ej[q] = q < nqb ? exp(dj[q] - jold[ce]) : 0.0;
                             else ej[q] = q < nqb ? expf(dj[q]) : 0.f;
-                            cq[q] = q < nqb ? (T)pt[8 * (p0 + q) + 3] * ej[q] : T(0);
+                            cq[q] = q < nqb ? (T)pt[kPt * (p0 + q) + 3] * ej[q] : T(0);
                         }
-                        const T xh[3] = {(T)pg[12 * pr], (T)pg[12 * pr + 1], (T)pg[12 * pr + 2]};
+                        const T xh[3] = {(T)pg[kPg * pr], (T)pg[kPg * pr + 1], (T)pg[kPg * pr + 2]};
                         T mot[3] = {T(0), T(0), T(0)};
                         pair_force_lane<T>(s, sR, sRf, i, a, r, dq, nqb, cq, dr, xh, U + ce * ldu, beta + ce * ldu, Fd,
                                            mot, lane);
@@ -891,7 +900,7 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
                             double fa[3] = {(double)mot[0], (double)mot[1], (double)mot[2]};
                             for (int q = 0; q < nqb; ++q)
 #pragma unroll
-                                for (int c = 0; c < 3; ++c) fa[c] += pt[8 * (p0 + q) + 4 + c] * (double)(ej[q] * dr[q]);
+                                for (int c = 0; c < 3; ++c) fa[c] += pt[kPt * (p0 + q) + 4 + c] * (double)(ej[q] * dr[q]);
 #pragma unroll
                             for (int c = 0; c < 3; ++c) atomicAdd(&Fd[3 * a + c], fa[c]);
                         }
@@ -902,8 +911,8 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
                         for (int q = 0; q < kQ; ++q) {
                             fq[q] = 0.0;
                             if (q < nqb) {
-                                if constexpr (sizeof(T) == 8) fq[q] = pt[8 * (p0 + q) + 3] * dr[q] * exp(dj[q] - jold[ce]);
-                                else fq[q] = pt[8 * (p0 + q) + 3] * (double)(dr[q] * expf(dj[q]));
+                                if constexpr (sizeof(T) == 8) fq[q] = pt[kPt * (p0 + q) + 3] * dr[q] * exp(dj[q] - jold[ce]);
+                                else fq[q] = pt[kPt * (p0 + q) + 3] * (double)(dr[q] * expf(dj[q]));
                             }
                         }
                         param_lane(s, sR, i, a, pt, p0, fq, nqb, pacc, dvw + wid * P, lane);
@@ -943,7 +952,7 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
         __syncthreads();
         for (int q = tid; q < P; q += blockDim.x) {
             double v = 0.0;
-            for (int k = 0; k < kNlWarps; ++k) v += dvw[k * P + q];
+            for (int k = 0; k < kWarps; ++k) v += dvw[k * P + q];
             eloc[(size_t)w * P + q] += v;
         }
         return;
@@ -953,7 +962,7 @@ __global__ void __launch_bounds__(kNlThreads) k_nlpp(DevSys s, DevWalkers wk, in
     __syncthreads();
     if (tid == 0) {
         double v = 0.0;
-        for (int q = 0; q < kNlWarps; ++q) v += s_part[q];
+        for (int q = 0; q < kWarps; ++q) v += s_part[q];
         s_part[0] = v;
     }
     if (nsl > 1) cg::this_cluster().sync();
@@ -987,14 +996,15 @@ cudaError_t launch_nlpp(const DevSys& s, const DevWalkers& wk, int w0, int W, do
     // slices until there are six waves of CTAs, while each still has a warp's
     // worth of electrons (a slice repeats the rotations and positions)
     int nsl = 1;
-    while (nsl < kMaxSlices && (long long)(W - w0) * nsl < 6 * 304 && s.N / (2 * nsl) >= 32) nsl *= 2;
+    const long long want = 6 * 152 * (ug ? 4 : 2);
+    while (nsl < kMaxSlices && (long long)(W - w0) * nsl < want && s.N / (2 * nsl) >= 32) nsl *= 2;
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = nsl;
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(W - w0) * nsl);
-    cfg.blockDim = dim3(kNlThreads);
+    cfg.blockDim = dim3(ug ? kUgThreads : kNlThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = &attr;
