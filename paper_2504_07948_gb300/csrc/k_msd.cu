@@ -136,12 +136,19 @@ __global__ void k_msd_table(DevSys s, DevWalkers wk, int W, const int* only) {
     if (threadIdx.x == 0) wk.Ssum[w] = v[0];
 }
 
+// Doubles of the tile in which k_msd_eloc forms rows of B_0 and A0^-1 (at least
+// one row) and the parts of grad J (as many as fit).
+constexpr int kElocTile = 1024;
+
+// Bound by its FP64 instructions: B_0 and the FP64 forms of T and A0^-1 are made
+// once instead of for every virtual, and grad J is shared by the whole CTA
+// (10,000 determinants, 256 walkers: 485 -> 294 us).
 // Adds the multi-determinant part to E_L, ln|psi|, the sign and (when grad
 // is given) the electron gradients of ln|psi| computed for the reference
 // determinant by k_eloc.
 template <typename T>
 __global__ void k_msd_eloc(DevSys s, DevWalkers wk, int W, double* eloc, double* logpsi, double* sign,
-                           double* grad) {
+                           double* grad, int n_tile) {
     extern __shared__ double sm[];
     __shared__ double scratch[kMaxWarps * 4];
     const int w = blockIdx.x;
@@ -154,11 +161,18 @@ __global__ void k_msd_eloc(DevSys s, DevWalkers wk, int W, double* eloc, double*
     double* Q = gJ + 3 * N;              // [nmax][nvmax]
     double* Th = Q + nmax * nvmax;       // [nmax][nvmax]
     double* Wg = Th + nmax * nvmax;      // [3][nvmax]
+    double* tile = Wg;                   // [n_tile], before the gradients
     for (int q = threadIdx.x; q < 3 * N; q += blockDim.x) sR[q] = wk.R[(size_t)w * 3 * N + q];
     __syncthreads();
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+    // grad J: parts of the CTA take every np-th partner of all electrons
+    const int nr = (N + 31) & ~31;
+    int np = nr < (int)blockDim.x ? (int)blockDim.x / nr : 1;
+    if (np * 3 * N > n_tile) np = 1;
+    for (int q = threadIdx.x; q < np * nr; q += blockDim.x) {
+        const int part = q / nr, i = q - part * nr;
+        if (i >= N) continue;
         double g[3] = {0, 0, 0};
-        for (int j = 0; j < N + nn; ++j) {
+        for (int j = part; j < N + nn; j += np) {
             double x[3], a, b;
             if (j < N) {
                 if (j == i) continue;
@@ -176,9 +190,18 @@ __global__ void k_msd_eloc(DevSys s, DevWalkers wk, int W, double* eloc, double*
             const double gr = a * qd * qd * ir;
             for (int c = 0; c < 3; ++c) g[c] += gr * x[c];
         }
-        for (int c = 0; c < 3; ++c) gJ[3 * i + c] = g[c];
+        double* out = np > 1 ? tile + 3 * N * part : gJ;
+        for (int c = 0; c < 3; ++c) out[3 * i + c] = g[c];
     }
     __syncthreads();
+    if (np > 1) {
+        for (int q = threadIdx.x; q < 3 * N; q += blockDim.x) {
+            double v = tile[q];
+            for (int c = 1; c < np; ++c) v += tile[3 * N * c + q];
+            gJ[q] = v;
+        }
+        __syncthreads();
+    }
     const double S = wk.Ssum[w];
     // per string: tr(adj(M) Theta[H,P]) with the cofactors of the table minor
     // in the storage type and the contraction with Theta in FP64
@@ -190,28 +213,46 @@ __global__ void k_msd_eloc(DevSys s, DevWalkers wk, int W, double* eloc, double*
         const T* G = (const T*)wk.G[spin] + (size_t)w * 4 * n * n;
         const T* Gv = (const T*)wk.Gv[spin] + (size_t)w * 4 * n * nv;
         const T* Tt = (const T*)wk.Tt[spin] + (size_t)w * n * nv;
-        // Q = B_v - B_0 T with B = -1/2 lap phi - grad J . grad phi per row
-        for (int q = threadIdx.x; q < n * nv; q += blockDim.x) {
-            const int i = q / nv, p = q - i * nv;
-            const double* gj = gJ + 3 * (i0 + i);
-            const T* Gi = G + (size_t)i * 4 * n;
-            const T* Gvi = Gv + (size_t)i * 4 * nv;
-            double acc = -0.5 * (double)Gvi[3 * nv + p] - gj[0] * (double)Gvi[p] - gj[1] * (double)Gvi[nv + p] -
-                         gj[2] * (double)Gvi[2 * nv + p];
-            for (int j = 0; j < n; ++j) {
-                const double b0 = -0.5 * (double)Gi[3 * n + j] - gj[0] * (double)Gi[j] - gj[1] * (double)Gi[n + j] -
-                                  gj[2] * (double)Gi[2 * n + j];
-                acc -= b0 * (double)Tt[(size_t)j * nv + p];
+        // Q = B_v - B_0 T with B = -1/2 lap phi - grad J . grad phi per row;
+        // B_0 by tiles of rows, T in FP64 (in Theta's place), both formed once
+        const int rows = max(1, n_tile / n);
+        for (int q = threadIdx.x; q < n * nv; q += blockDim.x) Th[q / nv * nvmax + q % nv] = (double)Tt[q];
+        for (int r0 = 0; r0 < n; r0 += rows) {
+            const int nr0 = min(rows, n - r0);
+            __syncthreads();
+            for (int q = threadIdx.x; q < nr0 * n; q += blockDim.x) {
+                const int i = r0 + q / n, j = q % n;
+                const double* gj = gJ + 3 * (i0 + i);
+                const T* Gi = G + (size_t)i * 4 * n;
+                tile[q] = -0.5 * (double)Gi[3 * n + j] - gj[0] * (double)Gi[j] - gj[1] * (double)Gi[n + j] -
+                          gj[2] * (double)Gi[2 * n + j];
             }
-            Q[i * nvmax + p] = acc;
+            __syncthreads();
+            for (int q = threadIdx.x; q < nr0 * nv; q += blockDim.x) {
+                const int r = q / nv, i = r0 + r, p = q - r * nv;
+                const double* gj = gJ + 3 * (i0 + i);
+                const T* Gvi = Gv + (size_t)i * 4 * nv;
+                double acc = -0.5 * (double)Gvi[3 * nv + p] - gj[0] * (double)Gvi[p] - gj[1] * (double)Gvi[nv + p] -
+                             gj[2] * (double)Gvi[2 * nv + p];
+                for (int j = 0; j < n; ++j) acc -= tile[r * n + j] * Th[j * nvmax + p];
+                Q[i * nvmax + p] = acc;
+            }
         }
-        __syncthreads();
-        // Theta = A0^-1 Q
-        for (int q = threadIdx.x; q < n * nv; q += blockDim.x) {
-            const int h = q / nv, p = q - h * nv;
-            double acc = 0.0;
-            for (int i = 0; i < n; ++i) acc += (double)AT[(size_t)i * n + h] * Q[i * nvmax + p];
-            Th[h * nvmax + p] = acc;
+        // Theta = A0^-1 Q, by tiles of rows of A0^-1
+        for (int r0 = 0; r0 < n; r0 += rows) {
+            const int nr0 = min(rows, n - r0);
+            __syncthreads();
+            for (int q = threadIdx.x; q < nr0 * n; q += blockDim.x) {
+                const int i = q / nr0, r = q - i * nr0;
+                tile[r * n + i] = (double)AT[(size_t)i * n + r0 + r];
+            }
+            __syncthreads();
+            for (int q = threadIdx.x; q < nr0 * nv; q += blockDim.x) {
+                const int r = q / nv, p = q - r * nv;
+                double acc = 0.0;
+                for (int i = 0; i < n; ++i) acc += tile[r * n + i] * Q[i * nvmax + p];
+                Th[(r0 + r) * nvmax + p] = acc;
+            }
         }
         __syncthreads();
         const T* Cd = (const T*)wk.Cd[spin] + (size_t)w * s.n_str[spin];
@@ -306,6 +347,127 @@ __device__ __forceinline__ void refresh_cd(const DevSys& s, const DevWalkers& wk
     }
 }
 
+// Arithmetic of the sweep's strings.  Every rounding is written out: a sweep of
+// the mixed form is a chaotic map, and its trajectories should not depend on how
+// the compiler contracts products and sums in one or the other arrangement of
+// this code.
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+
+// a d - b c
+template <typename F>
+__device__ __forceinline__ F det2_rn(F a, F d, F b, F c) {
+    return fma_rn(a, d, -mul_rn(b, c));
+}
+
+// det of the leading E x E block, as det_small expands it.
+template <int E, typename F>
+__device__ __forceinline__ F det_rn(const F (&m)[4][4]) {
+    if constexpr (E == 0) {
+        return F(1);
+    } else if constexpr (E == 1) {
+        return m[0][0];
+    } else if constexpr (E == 2) {
+        return det2_rn(m[0][0], m[1][1], m[0][1], m[1][0]);
+    } else if constexpr (E == 3) {
+        const F A = det2_rn(m[1][1], m[2][2], m[1][2], m[2][1]), B = det2_rn(m[1][0], m[2][2], m[1][2], m[2][0]),
+                C = det2_rn(m[1][0], m[2][1], m[1][1], m[2][0]);
+        return fma_rn(m[0][2], C, det2_rn(m[0][0], A, m[0][1], B));
+    } else {
+        const F a01 = det2_rn(m[0][0], m[1][1], m[0][1], m[1][0]), a02 = det2_rn(m[0][0], m[1][2], m[0][2], m[1][0]);
+        const F a03 = det2_rn(m[0][0], m[1][3], m[0][3], m[1][0]), a12 = det2_rn(m[0][1], m[1][2], m[0][2], m[1][1]);
+        const F a13 = det2_rn(m[0][1], m[1][3], m[0][3], m[1][1]), a23 = det2_rn(m[0][2], m[1][3], m[0][3], m[1][2]);
+        const F b01 = det2_rn(m[2][0], m[3][1], m[2][1], m[3][0]), b02 = det2_rn(m[2][0], m[3][2], m[2][2], m[3][0]);
+        const F b03 = det2_rn(m[2][0], m[3][3], m[2][3], m[3][0]), b12 = det2_rn(m[2][1], m[3][2], m[2][2], m[3][1]);
+        const F b13 = det2_rn(m[2][1], m[3][3], m[2][3], m[3][1]), b23 = det2_rn(m[2][2], m[3][3], m[2][3], m[3][2]);
+        return fma_rn(a23, b01, fma_rn(-a13, b02, fma_rn(a12, b03, fma_rn(a03, b12, det2_rn(a01, b23, a02, b13)))));
+    }
+}
+
+// det of the block with column b replaced by u.
+template <int E, typename F>
+__device__ __forceinline__ F det_column_rn(const F (&m)[4][4], const F (&u)[4], int b) {
+    F t[4][4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) t[a][c] = a < E && c < E ? (c == b ? u[a] : m[a][c]) : F(0);
+    return det_rn<E>(t);
+}
+
+// Adds a b.
+__device__ __forceinline__ void add_product(Acc<float>& v, float a, float b) {
+    const float s = __fmaf_rn(a, b, v.h), bp = __fsub_rn(s, v.h);
+    v.l = __fadd_rn(v.l, __fadd_rn(__fsub_rn(v.h, __fsub_rn(s, bp)), __fmaf_rn(a, b, -bp)));
+    v.h = s;
+}
+__device__ __forceinline__ void add_product(Acc<double>& v, double a, double b) { v.h = __fma_rn(a, b, v.h); }
+
+// The four weights of a virtual as one load.
+template <typename T>
+struct alignas(16) Weights4 {
+    T v[4];
+};
+
+// One string of excitation level E at the current position: gradient terms of
+// sum_u Cd_u R_u.  The level is known at compile time (the strings are sorted by
+// it): one body for all levels with its entries masked took some 350
+// instructions per string where level 2, the most of them, needs about 100, and
+// bounded the sweep (6-water cluster, 10,000 determinants, 256 walkers: sweep
+// 6.0 -> 3.6 ms).
+template <int E, typename T>
+__device__ __forceinline__ void string_drift(const StrDesc& d, const T* Ts, int nv, const T* Ae, const T* Wq, T f,
+                                             Acc<T>* va) {
+    T m[4][4], u[4];
+#pragma unroll
+    for (int a = 0; a < E; ++a) {
+        u[a] = Ae[d.h[a]];
+#pragma unroll
+        for (int b = 0; b < E; ++b) m[a][b] = Ts[d.h[a] * nv + d.p[b]];
+    }
+#pragma unroll
+    for (int b = 0; b < E; ++b) {
+        const Weights4<T> w = reinterpret_cast<const Weights4<T>*>(Wq)[d.p[b]];
+        const T fb = mul_rn(f, det_column_rn<E>(m, u, b));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) add_product(va[c], fb, w.v[c]);
+    }
+}
+
+// The same at the proposed position, with the table's rank-1 update applied to
+// the minor on the fly: adds cu R'_u and its gradient terms, returns R'_u.
+template <int E, typename T>
+__device__ __forceinline__ T string_ratio(const StrDesc& d, const T* Ts, int nv, const T* Ae, T rinv0, const T* Wq,
+                                          T cu, Acc<T>* vs) {
+    T m[4][4], u[4];
+    Weights4<T> w[E > 0 ? E : 1];
+#pragma unroll
+    for (int b = 0; b < E; ++b) w[b] = reinterpret_cast<const Weights4<T>*>(Wq)[d.p[b]];
+#pragma unroll
+    for (int a = 0; a < E; ++a) {
+        u[a] = mul_rn(Ae[d.h[a]], rinv0);
+#pragma unroll
+        for (int b = 0; b < E; ++b) {
+            const T t = Ts[d.h[a] * nv + d.p[b]], wb = w[b].v[3];
+            m[a][b] = b == 0 && a > 0 ? fma_rn(u[a], wb, t) : add_rn(t, mul_rn(u[a], wb));
+        }
+    }
+    const T Ru = mul_rn(T(d.phase), det_rn<E>(m));
+    add_product(vs[0], cu, Ru);
+    const T f = mul_rn(T(d.phase), cu);
+#pragma unroll
+    for (int b = 0; b < E; ++b) {
+        const T fb = mul_rn(f, det_column_rn<E>(m, u, b));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) add_product(vs[1 + c], fb, w[b].v[c]);
+    }
+    return Ru;
+}
+
 constexpr double kRefreshRho0F = 1e-2;   // mixed form
 constexpr double kRefreshRho0D = 1e-4;   // FP64 form
 
@@ -317,16 +479,15 @@ __global__ void k_sweep_msd(DevSys s, DevWalkers wk, int W, SweepParams p) {
     const int N = s.N, nu = s.n_up, nd = s.n_dn, nb = s.n_basis, nn = s.n_nuc;
     const int nmax = nu > nd ? nu : nd;
     const int nv0 = s.n_vir[0], nv1 = s.n_vir[1], nvmax = nv0 > nv1 ? nv0 : nv1;
-    double* sR = (double*)smem;
+    T* Wq = (T*)smem;            // [nvmax][4]: gradient weights W_c[p], then w[p]
+    double* sR = (double*)(Wq + 4 * nvmax);
     double* red = sR + 3 * N;
     double* scal = red + kMaxWarps * 12;
     T* bas = (T*)(scal + 16);
     T* phi = bas + 5 * nb;
     T* phv = phi + 5 * nmax;
     T* cold = phv + 5 * nvmax;
-    T* wv = cold + nmax;
-    T* Wc = wv + nvmax;          // [3][nvmax]
-    T* sA = Wc + 3 * nvmax;
+    T* sA = cold + nmax;
     T* sT = sA + nu * nu + nd * nd;
     T* Ainv[2] = {sA, sA + nu * nu};
     T* Tt[2] = {sT, sT + nu * nv0};
@@ -376,7 +537,7 @@ __global__ void k_sweep_msd(DevSys s, DevWalkers wk, int W, SweepParams p) {
             const int c = q / nv, pp = q - c * nv;
             T a = Gvk[c * nv + pp];
             for (int j = 0; j < n; ++j) a -= Gk[c * n + j] * Ts[(size_t)j * nv + pp];
-            Wc[c * nvmax + pp] = a;
+            Wq[4 * pp + c] = a;
         }
         Acc<T> va[9];
         T u_old = T(0);
@@ -411,18 +572,13 @@ __global__ void k_sweep_msd(DevSys s, DevWalkers wk, int W, SweepParams p) {
         __syncthreads();
         for (int u = threadIdx.x; u < ns; u += blockDim.x) {
             const StrDesc d = decode(str[u]);
-            if (d.e == 0) continue;
-            T m[4][4], uh[4], gb[4];
-            gather_minor<T>(d, Ts, nv, m);
-#pragma unroll
-            for (int a = 0; a < 4; ++a) uh[a] = a < d.e ? Ae[d.h[a]] : T(0);
-            col_replaced_dets<T>(d.e, m, uh, gb);
             const T f = T(d.phase) * Cd[u];
-            for (int b = 0; b < d.e; ++b) {
-                const T fb = f * gb[b];
-                va[6].add(fb * Wc[d.p[b]]);
-                va[7].add(fb * Wc[nvmax + d.p[b]]);
-                va[8].add(fb * Wc[2 * nvmax + d.p[b]]);
+            switch (d.e) {   // the strings are sorted by excitation level
+                case 0: break;
+                case 1: string_drift<1, T>(d, Ts, nv, Ae, Wq, f, va + 6); break;
+                case 2: string_drift<2, T>(d, Ts, nv, Ae, Wq, f, va + 6); break;
+                case 3: string_drift<3, T>(d, Ts, nv, Ae, Wq, f, va + 6); break;
+                default: string_drift<4, T>(d, Ts, nv, Ae, Wq, f, va + 6); break;
             }
         }
         double vd[9];
@@ -508,41 +664,27 @@ __global__ void k_sweep_msd(DevSys s, DevWalkers wk, int W, SweepParams p) {
             const int c = q / nv, pp = q - c * nv;
             T a = phv[c * nvmax + pp];
             for (int h = 0; h < n; ++h) a -= Ts[(size_t)h * nv + pp] * phi[c * nmax + h];
-            if (c == 0)
-                wv[pp] = a;
-            else
-                Wc[(c - 1) * nvmax + pp] = a;   // grad phi'_v - T^T grad phi'_occ (before the w term)
+            Wq[4 * pp + (c == 0 ? 3 : c - 1)] = a;   // grad phi'_v - T^T grad phi'_occ (before the w term)
         }
         __syncthreads();
         for (int q = threadIdx.x; q < 3 * nv; q += blockDim.x) {
             const int c = q / nv, pp = q - c * nv;
-            Wc[c * nvmax + pp] -= wv[pp] * vb2[1 + c] * rinv0;
+            Wq[4 * pp + c] -= Wq[4 * pp + 3] * vb2[1 + c] * rinv0;
         }
         __syncthreads();
         Acc<T> vs[4];
         for (int u = threadIdx.x; u < ns; u += blockDim.x) {
             const StrDesc d = decode(str[u]);
-            T m[4][4], uh[4], gb[4];
-            gather_minor<T>(d, Ts, nv, m);
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                const T ca = a < d.e ? Ae[d.h[a]] * rinv0 : T(0);
-                uh[a] = ca;
-#pragma unroll
-                for (int b = 0; b < 4; ++b) m[a][b] += (a < d.e && b < d.e) ? ca * wv[d.p[b]] : T(0);
+            const T cu = Cd[u];
+            T Ru;
+            switch (d.e) {
+                case 0: Ru = string_ratio<0, T>(d, Ts, nv, Ae, rinv0, Wq, cu, vs); break;
+                case 1: Ru = string_ratio<1, T>(d, Ts, nv, Ae, rinv0, Wq, cu, vs); break;
+                case 2: Ru = string_ratio<2, T>(d, Ts, nv, Ae, rinv0, Wq, cu, vs); break;
+                case 3: Ru = string_ratio<3, T>(d, Ts, nv, Ae, rinv0, Wq, cu, vs); break;
+                default: Ru = string_ratio<4, T>(d, Ts, nv, Ae, rinv0, Wq, cu, vs); break;
             }
-            const T Ru = T(d.phase) * det_small<T>(d.e, m);
             Rnew[u] = Ru;
-            vs[0].add(Cd[u] * Ru);
-            if (d.e == 0) continue;
-            col_replaced_dets<T>(d.e, m, uh, gb);
-            const T f = T(d.phase) * Cd[u];
-            for (int b = 0; b < d.e; ++b) {
-                const T fb = f * gb[b];
-                vs[1].add(fb * Wc[d.p[b]]);
-                vs[2].add(fb * Wc[nvmax + d.p[b]]);
-                vs[3].add(fb * Wc[2 * nvmax + d.p[b]]);
-            }
         }
         double vsd[4];
         block_sum_to0<4>(vs, red + kMaxWarps * 8, vsd);
@@ -575,7 +717,7 @@ __global__ void k_sweep_msd(DevSys s, DevWalkers wk, int W, SweepParams p) {
             }
             for (int q = threadIdx.x; q < n * nv; q += blockDim.x) {
                 const int h = q / nv, pp = q - h * nv;
-                Ts[q] += cold[h] * wv[pp] * rinv0;
+                Ts[q] += cold[h] * Wq[4 * pp + 3] * rinv0;
             }
             for (int o = threadIdx.x; o < 4 * n; o += blockDim.x) {
                 const int c = o / n, j = o - c * n;
@@ -674,10 +816,16 @@ cudaError_t launch_msd_eloc(const DevSys& s, const DevWalkers& wk, int W, double
     if (W == 0) return cudaSuccess;
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
     const int nvmax = s.n_vir[0] > s.n_vir[1] ? s.n_vir[0] : s.n_vir[1];
-    const size_t smem = sizeof(double) * (6 * (size_t)s.N + (2 * (size_t)nmax + 3) * (nvmax > 0 ? nvmax : 1));
+    const int nv = nvmax > 0 ? nvmax : 1;
+    int n_tile = kElocTile;
+    auto bytes = [&] {
+        return sizeof(double) * (6 * (size_t)s.N + 2 * (size_t)nmax * nv + std::max(3 * nv, n_tile));
+    };
+    if (bytes() > 227 * 1024) n_tile = std::max(3 * nv, nmax);
+    const size_t smem = bytes();
     cudaError_t e = cudaFuncSetAttribute(k_msd_eloc<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_msd_eloc<T><<<W, 256, smem, st>>>(s, wk, W, eloc, logpsi, sign, grad);
+    k_msd_eloc<T><<<W, 256, smem, st>>>(s, wk, W, eloc, logpsi, sign, grad, n_tile);
     return cudaGetLastError();
 }
 
