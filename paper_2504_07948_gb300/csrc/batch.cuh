@@ -128,12 +128,14 @@ cudaError_t launch_invert_batch(const BatchSys* sys, BatchPlan* plan, int parity
 template <typename T>
 cudaError_t launch_eloc_batch(const BatchSys* sys, BatchPlan* plan, int parity, int into_walker, int ctr, int grid,
                               size_t smem, cudaStream_t st);
-size_t force_batch_smem_bytes(const DevSys& s, int elem, int space_warp);
+// nw: warps of a CTA, the largest any system asks for (force_batch_warps)
+int force_batch_warps(const DevSys& s, int elem, int space_warp);
+size_t force_batch_smem_bytes(const DevSys& s, int elem, int space_warp, int nw);
 template <typename T>
-int force_batch_prepare(size_t smem, int any_warp);
+int force_batch_prepare(size_t smem, int any_warp, int nw);
 template <typename T>
 cudaError_t launch_force_batch(const BatchSys* sys, BatchPlan* plan, int parity, int ctr, int grid, size_t smem,
-                               int any_warp, cudaStream_t st);
+                               int any_warp, int nw, cudaStream_t st);
 // Space warp of the ionic derivatives of the systems that have it on (the
 // others' walker items are skipped).
 size_t space_warp_batch_smem_bytes(const DevSys& s, int elem);

@@ -458,12 +458,19 @@ __host__ __device__ inline int force_row_groups(int n) {
 // cluster, 2048 walkers: 8.10 -> 3.38 ms FP64 and 0.81 -> 0.45 ms mixed
 // against one derivative evaluation per basis function, FP64 products and a
 // masked exponential per primitive.
+// Where only one CTA fits an SM (above kForceTwo bytes: determinants above about
+// 55), it takes the whole SM: sixteen warps instead of eight, each with its
+// scratch, and tiles of as many basis functions as fit, so that a tile has centres
+// enough for the warps (a batch of 16 clusters of up to 130 electrons, 64 walkers
+// each: 5.2 -> 4.4 ms; sixteen warps with the smallest tiles 6.0, eight with
+// large ones 4.8).
+constexpr size_t kForceTwo = 113 * 1024;
 template <typename T>
 struct ForceShape {
     bool stg;
     int ld, F, scr;                                      // scr: bytes of scratch per warp
     size_t AT, PT, sA, scratch, M, Y, gE, total;         // byte offsets
-    __host__ __device__ ForceShape(int N, int nn, int nmax, int nb, bool kE) {
+    __host__ __device__ ForceShape(int N, int nn, int nmax, int nb, bool kE, int nw = 8) {
         const size_t head = (force_head_bytes<T>(N, nn) + 15) & ~(size_t)15;
         const size_t e_bytes = kE ? sizeof(double) * 3 * (size_t)N : 0;
         ld = nmax | 1;
@@ -485,9 +492,10 @@ struct ForceShape {
         PT = AT + (stg ? mat : 0);
         sA = PT + (stg ? mat : 0);
         scratch = (sA + (stg ? 2 * sizeof(T) * (size_t)nmax : 0) + 15) & ~(size_t)15;
-        M = scratch + 8 * (size_t)scr;
-        const size_t budget = (sizeof(T) == 8 ? 112 : 74) * 1024;
+        M = scratch + nw * (size_t)scr;
+        size_t budget = (sizeof(T) == 8 ? 112 : 74) * 1024;
         F = fmin;
+        if (M + e_bytes + row * fmin > kForceTwo) budget = 220 * 1024;   // one CTA per SM: all there is
         if (stg && budget > M + e_bytes + row * fmin) {
             const size_t fit = (budget - M - e_bytes) / row;
             F = fit < (size_t)nb ? (int)fit : nb;
@@ -497,10 +505,14 @@ struct ForceShape {
         gE = (Y + sizeof(T) * (size_t)F * nmax + 15) & ~(size_t)15;
         total = gE + e_bytes;
     }
+    // warps of a CTA: sixteen where only one CTA fits an SM
+    static int warps(int N, int nn, int nmax, int nb, bool kE) {
+        return ForceShape(N, nn, nmax, nb, kE).total > kForceTwo ? 16 : 8;
+    }
 };
 
 // Adjoint ionic derivatives of walker w (body of k_force).  sm: the
-// dynamic shared memory of launch_force (ForceShape), 256 threads.  kE: also
+// dynamic shared memory of launch_force (ForceShape), 256 or 512 threads.  kE: also
 // the determinant part of dE_L/dr_i (the same basis-space terms, every basis
 // function moving with the electron, d/dr_i = -d/dR) into gEdet [W][N][3]
 // and grad_i ln|psi| into gtot [W][N][3], for the space warp.
@@ -512,7 +524,7 @@ __device__ __forceinline__ void force_walker(const DevSys& s, const DevWalkers& 
     const int nmax = nu > s.n_dn ? nu : s.n_dn;
     constexpr bool kFx = sizeof(T) == 8;
     using Q = std::conditional_t<kFx, int2, float>;   // staged operands
-    const ForceShape<T> fs(N, nn, nmax, s.n_basis, kE);
+    const ForceShape<T> fs(N, nn, nmax, s.n_basis, kE, blockDim.x >> 5);
     unsigned char* smb = (unsigned char*)sm;
     const ForceHead<T> h(sm, N, nn);
     double* acc = h.acc;
@@ -710,10 +722,10 @@ __device__ __forceinline__ void force_walker(const DevSys& s, const DevWalkers& 
 
 // Three CTAs per SM in the FP32 form (80 registers, no spills); the FP64
 // form keeps two (at three it spills).
-template <typename T, bool kE>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_force(DevSys s, DevWalkers wk, int W, const double* dvnn,
-                                                  double* Bscr, double* Pscr, double* dEL, double* dlog,
-                                                  double* gEdet, double* gtot) {
+template <typename T, bool kE, int kNt>
+__global__ void __launch_bounds__(kNt, kNt == 512 ? 1 : sizeof(T) == 4 ? 3 : 2)
+    k_force(DevSys s, DevWalkers wk, int W, const double* dvnn, double* Bscr, double* Pscr, double* dEL, double* dlog,
+            double* gEdet, double* gtot) {
     extern __shared__ double sm[];
     const int w = blockIdx.x;
     if (w >= W) return;
@@ -907,17 +919,14 @@ cudaError_t launch_force(const DevSys& s, const DevWalkers& wk, int W, const dou
                          double* Pscr, double* dEL, double* dlog, double* gEdet, double* gtot, cudaStream_t st) {
     if (W == 0) return cudaSuccess;
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
-    if (gEdet) {
-        const size_t smem = ForceShape<T>(s.N, s.n_nuc, nmax, s.n_basis, true).total;
-        cudaError_t e = cudaFuncSetAttribute(k_force<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        k_force<T, true><<<W, 256, smem, st>>>(s, wk, W, dvnn, Bscr, Pscr, dEL, dlog, gEdet, gtot);
-        return cudaGetLastError();
-    }
-    const size_t smem = ForceShape<T>(s.N, s.n_nuc, nmax, s.n_basis, false).total;
-    cudaError_t e = cudaFuncSetAttribute(k_force<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const bool kE = gEdet != nullptr;
+    const int nw = ForceShape<T>::warps(s.N, s.n_nuc, nmax, s.n_basis, kE);
+    const size_t smem = ForceShape<T>(s.N, s.n_nuc, nmax, s.n_basis, kE, nw).total;
+    const auto f = nw == 16 ? (kE ? k_force<T, true, 512> : k_force<T, false, 512>)
+                            : (kE ? k_force<T, true, 256> : k_force<T, false, 256>);
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_force<T, false><<<W, 256, smem, st>>>(s, wk, W, dvnn, Bscr, Pscr, dEL, dlog, nullptr, nullptr);
+    f<<<W, 32 * nw, smem, st>>>(s, wk, W, dvnn, Bscr, Pscr, dEL, dlog, gEdet, kE ? gtot : nullptr);
     return cudaGetLastError();
 }
 
@@ -1094,9 +1103,9 @@ template cudaError_t launch_space_warp<float>(const DevSys&, const DevWalkers&, 
 // Batched form: persistent CTAs over the walkers of every system.
 // kWarp: some member of the batch has the space warp on (its walkers also
 // get the per-electron outputs); batches without it run the plain body.
-template <typename T, bool kWarp>
-__global__ void __launch_bounds__(256, 2) k_force_batch(const BatchSys* __restrict__ sys, BatchPlan* plan,
-                                                        int parity, int ctr) {
+template <typename T, bool kWarp, int kNt>
+__global__ void __launch_bounds__(kNt, kNt == 512 ? 1 : 2) k_force_batch(const BatchSys* __restrict__ sys,
+                                                                         BatchPlan* plan, int parity, int ctr) {
     extern __shared__ double sm[];
     __shared__ BatchSys bs;
     __shared__ int s_sys, s_idx;
@@ -1120,10 +1129,22 @@ __global__ void __launch_bounds__(256, 2) k_force_batch(const BatchSys* __restri
     }
 }
 
-size_t force_batch_smem_bytes(const DevSys& s, int elem, int space_warp) {
+int force_batch_warps(const DevSys& s, int elem, int space_warp) {
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
-    return elem == 4 ? ForceShape<float>(s.N, s.n_nuc, nmax, s.n_basis, space_warp != 0).total
-                     : ForceShape<double>(s.N, s.n_nuc, nmax, s.n_basis, space_warp != 0).total;
+    return elem == 4 ? ForceShape<float>::warps(s.N, s.n_nuc, nmax, s.n_basis, space_warp != 0)
+                     : ForceShape<double>::warps(s.N, s.n_nuc, nmax, s.n_basis, space_warp != 0);
+}
+
+size_t force_batch_smem_bytes(const DevSys& s, int elem, int space_warp, int nw) {
+    const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
+    return elem == 4 ? ForceShape<float>(s.N, s.n_nuc, nmax, s.n_basis, space_warp != 0, nw).total
+                     : ForceShape<double>(s.N, s.n_nuc, nmax, s.n_basis, space_warp != 0, nw).total;
+}
+
+template <typename T>
+static auto force_batch_kernel(int any_warp, int nw) {
+    return nw == 16 ? (any_warp ? k_force_batch<T, true, 512> : k_force_batch<T, false, 512>)
+                    : (any_warp ? k_force_batch<T, true, 256> : k_force_batch<T, false, 256>);
 }
 
 // Batched space warp: persistent CTAs over the walkers of every system; the
@@ -1177,11 +1198,11 @@ template cudaError_t launch_space_warp_batch<double>(const BatchSys*, BatchPlan*
 template cudaError_t launch_space_warp_batch<float>(const BatchSys*, BatchPlan*, int, int, int, size_t, cudaStream_t);
 
 template <typename T>
-int force_batch_prepare(size_t smem, int any_warp) {
+int force_batch_prepare(size_t smem, int any_warp, int nw) {
     int nb = 0;
-    const void* f = any_warp ? (const void*)k_force_batch<T, true> : (const void*)k_force_batch<T, false>;
+    const void* f = (const void*)force_batch_kernel<T>(any_warp, nw);
     if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, 256, smem) != cudaSuccess) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, 32 * nw, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -1190,19 +1211,17 @@ int force_batch_prepare(size_t smem, int any_warp) {
 
 template <typename T>
 cudaError_t launch_force_batch(const BatchSys* sys, BatchPlan* plan, int parity, int ctr, int grid, size_t smem,
-                               int any_warp, cudaStream_t st) {
-    if (any_warp)
-        k_force_batch<T, true><<<grid, 256, smem, st>>>(sys, plan, parity, ctr);
-    else
-        k_force_batch<T, false><<<grid, 256, smem, st>>>(sys, plan, parity, ctr);
+                               int any_warp, int nw, cudaStream_t st) {
+    force_batch_kernel<T>(any_warp, nw)<<<grid, 32 * nw, smem, st>>>(sys, plan, parity, ctr);
     return cudaGetLastError();
 }
 
-template int force_batch_prepare<double>(size_t, int);
-template int force_batch_prepare<float>(size_t, int);
-template cudaError_t launch_force_batch<double>(const BatchSys*, BatchPlan*, int, int, int, size_t, int,
+template int force_batch_prepare<double>(size_t, int, int);
+template int force_batch_prepare<float>(size_t, int, int);
+template cudaError_t launch_force_batch<double>(const BatchSys*, BatchPlan*, int, int, int, size_t, int, int,
                                                 cudaStream_t);
-template cudaError_t launch_force_batch<float>(const BatchSys*, BatchPlan*, int, int, int, size_t, int, cudaStream_t);
+template cudaError_t launch_force_batch<float>(const BatchSys*, BatchPlan*, int, int, int, size_t, int, int,
+                                               cudaStream_t);
 
 template cudaError_t launch_force<double>(const DevSys&, const DevWalkers&, int, const double*, double*, double*,
                                           double*, double*, double*, double*, cudaStream_t);

@@ -2432,6 +2432,7 @@ struct qmc_batch {
     int any_delay = 0;             // some member uses delayed updates
     std::vector<int> delay, ainv;  // per descriptor
     size_t orb_smem = 0, inv_smem = 0, eloc_smem = 0, force_smem = 0;
+    int force_warps = 8;
     int orb_grid = 0, inv_grid = 0, eloc_grid = 0, force_grid = 0, copy_grid = 0;
     std::vector<int> warp;         // per descriptor: space warp on (read at creation)
     int any_warp = 0;
@@ -2541,21 +2542,24 @@ struct qmc_batch {
 
     void configure_other() {
         size_t orb = 0, inv = 0, el = 0, fo = 0;
+        force_warps = 8;
         for (int q = 0; q < n; ++q) {
             const DevSys& s = sys[q]->ds;
             const int nmax = std::max(s.n_up, s.n_dn);
             orb = std::max(orb, orbitals_smem_bytes(s));
             inv = std::max(inv, sizeof(double) * ((size_t)nmax * nmax + nmax + 1));
             el = std::max(el, eloc_smem_bytes(s, 128, elem()));
-            fo = std::max(fo, force_batch_smem_bytes(s, elem(), warp[q]));
+            force_warps = std::max(force_warps, force_batch_warps(s, elem(), warp[q]));
         }
+        for (int q = 0; q < n; ++q) fo = std::max(fo, force_batch_smem_bytes(sys[q]->ds, elem(), warp[q], force_warps));
         const bool mx = mode == QMC_MIXED;
         const int o_orb = wf_batch_prepare(mx ? 3 : 0, 128, orb);
         const int o_inv = wf_batch_prepare(1, 256, inv);
         const int o_el = wf_batch_prepare(mx ? 4 : 2, 128, el);
         int aw = 0;
         for (int q = 0; q < n; ++q) aw |= warp[q];
-        const int o_fo = mx ? force_batch_prepare<float>(fo, aw) : force_batch_prepare<double>(fo, aw);
+        const int o_fo = mx ? force_batch_prepare<float>(fo, aw, force_warps)
+                            : force_batch_prepare<double>(fo, aw, force_warps);
         require(o_orb > 0 && o_inv > 0 && o_el > 0 && o_fo > 0, QMC_ERR_UNSUPPORTED,
                 "a batched kernel does not fit the largest system");
         orb_smem = orb;
@@ -2624,9 +2628,11 @@ struct qmc_batch {
         if (forces) {
             tm.begin(stream);
             if (mx)
-                QMC_CK(launch_force_batch<float>(d_sys, d_plan, parity, 4, force_grid, force_smem, any_warp, stream));
+                QMC_CK(launch_force_batch<float>(d_sys, d_plan, parity, 4, force_grid, force_smem, any_warp, force_warps,
+                                                 stream));
             else
-                QMC_CK(launch_force_batch<double>(d_sys, d_plan, parity, 4, force_grid, force_smem, any_warp, stream));
+                QMC_CK(launch_force_batch<double>(d_sys, d_plan, parity, 4, force_grid, force_smem, any_warp, force_warps,
+                                                  stream));
             ++launches;
             if (any_warp) {
                 if (mx)
@@ -2823,9 +2829,22 @@ int qmc_batch_create(qmc_batch_t* out, int n_systems, qmc_t const* systems) {
         alloc((void**)&b->d_ctl, sizeof(BatchCtl) * n_systems);
         alloc((void**)&b->d_hist, sizeof(double) * (size_t)b->chunk * n_systems * b->hist_stride);
         QMC_CK(cudaMemsetAsync(b->d_plan, 0, sizeof(BatchPlan), b->stream));
-        // default configuration: Sherman-Morrison everywhere, A^-1 in shared
-        // memory for every system that fits 100 KB
-        b->configure(128, 100 * 1024, 1, 0);
+        // default configuration: Sherman-Morrison everywhere.  Mixed: A^-1 in
+        // shared memory for every system that fits 100 KB.  FP64: with few walkers
+        // per SM the largest systems' walkers, one after the other, set the time:
+        // eight warps each and A^-1 in shared memory wherever it fits; with many
+        // the instruction rate does: four CTAs of four warps per SM.  Clusters of
+        // 1 to 16 waters, sweep of the batch, four / eight warps: 1024 walkers 9.0 /
+        // 6.1 ms, 4096 walkers 21.3 / 24.9 and 37.9 / 43.4 ms (16 and 64 systems;
+        // 30.7 and 59.6 ms with four warps and A^-1 in up to 100 KB).
+        long long walkers = 0;
+        for (int q = 0; q < n_systems; ++q) walkers += systems[q]->W;
+        if (b->mode == QMC_MIXED)
+            b->configure(128, 100 * 1024, 1, 0);
+        else if (walkers < 16LL * b->n_sm)
+            b->configure(256, 220 * 1024, 1, 0);
+        else
+            b->configure(128, 45 * 1024, 1, 0);
         b->configure_other();
         b->sync();
     });

@@ -285,3 +285,27 @@ def test_batch_large_members_follow_oracle(Q, precision):
     batch.close()
     for m in members:
         m.close()
+
+
+def test_batch_default_of_many_walkers(Q):
+    """A batch of many walkers per SM takes a narrower sweep CTA and less shared
+    memory by default than one of few; both give the same run (populations
+    equal, step energies to 1e-10 relative)."""
+    systems = [(synth.water_system(1), 2000, 31, -76.0), (synth.water_system(3), 500, 32, -228.0)]
+    runs = []
+    for block, budget in ((None, None), (256, 220 * 1024)):
+        members = []
+        for s, W, seed, _ in systems:
+            m = Q.QMC(s, precision="fp64", seed=seed, cap_factor=2)
+            m.set_walkers(synth.initial_walkers(s, W, seed=seed))
+            members.append(m)
+        b = Q.Batch(members)
+        if block:
+            b.set_options(sweep_block=block, smem_budget=budget)
+        runs.append(b.dmc(2, TAU, [e for *_, e in systems]))
+        b.close()
+        for m in members:
+            m.close()
+    assert np.array_equal(runs[0]["pop"], runs[1]["pop"])
+    e0, e1 = runs[0]["e_step"], runs[1]["e_step"]
+    assert (np.abs(e0 - e1) / np.abs(e1)).max() <= 1e-10
