@@ -203,6 +203,11 @@ __device__ __forceinline__ void capped_drift(const double g[3], double tau, doub
 __device__ __forceinline__ double rsqrt_t(double v) { return rsqrt(v); }
 __device__ __forceinline__ float rsqrt_t(float v) { return rsqrtf(v); }
 
+// Keeps a converted constant in a register: without it a selection between two
+// of them becomes a selection in FP64 and a conversion each time.
+__device__ __forceinline__ void hold(float& v) { asm("" : "+f"(v)); }
+__device__ __forceinline__ void hold(double&) {}
+
 // Reciprocal of a value known to be finite and at least 1: the FP64 form
 // refines the hardware's 20-bit approximation y by 1/x = y (1 + e + e^2 +
 // ...), e = 1 - x y, to the last bit or two (3 FP64 instructions instead of a
