@@ -315,10 +315,14 @@ namespace {
 //             (A: 128 rows x 16 k; B: N rows x 16 k, or 16 k x N when B is
 //             given [K][N]) into kRaw raw buffers, completion counted on an
 //             mbarrier by bytes;
-//   warps 4-7 split each raw tile into TF32 hi / lo tiles (lo rounded to
-//             nearest) in the no-swizzle K-major core-matrix layout of
-//             tcgen05 (kConv buffers), release the raw buffer and mark the
-//             converted one full;
+//   warps 4-7 and 12-15 split each raw tile into TF32 hi / lo tiles (lo
+//             rounded to nearest) in the no-swizzle K-major core-matrix layout
+//             of tcgen05 (kConv buffers, one per group of four warps), release
+//             the raw buffer and mark the converted one full.  A thread loads
+//             all its 16-byte pieces of a stage before it converts and stores
+//             any: taken one by one (a store might alias the next load) a stage
+//             took a chain of some 2000 cycles, four times its MMAs, and bounded
+//             the kernel;
 //   warp 1    one thread issues the 2 K-steps x 3 MMAs (lo*hi, hi*lo, hi*hi)
 //             of a converted stage into the tile's accumulator (two 128 x N
 //             FP32 blocks of tensor memory, alternating by tile) and
@@ -329,13 +333,16 @@ namespace {
 //             beta D and write rows through a padded shared-memory
 //             transpose (every warp store covers 128 contiguous bytes),
 //             while the other roles already work on the next tile.
+// 512 products of 768 x 160 by 160 x 160 (40 GFLOP as three TF32 products, 252 MB
+// of results): 253 -> 161 us, now within 1.4 of the shared memory's bandwidth (raw
+// and split tiles in and out, and each split tile read by two of the products).
 // Every mbarrier wait is bounded.  A role that gives up sets kErrTimeout
 // and a shared abort flag that makes the other roles skip their remaining
 // waits; before the CTA frees its tensor memory the MMA thread waits
 // (bounded) for the MMAs it issued and the load thread for its loads.
 // ---------------------------------------------------------------------
 constexpr int kPK = 16;       // K per stage
-constexpr int kRaw = 3;       // raw (TMA) buffers
+constexpr int kRaw = 4;       // raw (TMA) buffers
 constexpr int kConv = 2;      // converted (hi / lo) buffers
 
 __device__ __forceinline__ int ptile_off(int r, int k) {   // [rows][kPK] core-matrix layout, floats
@@ -349,8 +356,14 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
+// Nearest TF32 value, ties away from zero, by integers (two instructions; the
+// conversion takes several).  A NaN may lose its payload here and become a zero;
+// the remainder then still is a NaN.
+__device__ __forceinline__ float tf32_near(float x) {
+    return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u);
+}
 __device__ __forceinline__ float4 split_hi4(float4 x) {
-    return make_float4(tf32_hi(x.x), tf32_hi(x.y), tf32_hi(x.z), tf32_hi(x.w));
+    return make_float4(tf32_near(x.x), tf32_near(x.y), tf32_near(x.z), tf32_near(x.w));
 }
 // lo = round_tf32(x - hi): the tensor core reads only the TF32 bits of an
 // operand, so the remainder is rounded to nearest here instead of being cut
@@ -378,7 +391,7 @@ __host__ __device__ inline PipeSmem pipe_layout(int Np) {
 
 // D_b = alpha A_b B_b^T + beta D_b: A through tmA (dims K, M, batch), B
 // through tmB (dims K, N, batch; or N, K, batch when b_trans).
-__global__ void __launch_bounds__(384, 1)
+__global__ void __launch_bounds__(512, 1)
     k_tc_gemm_pipe(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M, int N, int K,
                    int batch, int b_trans, int a_batched, int b_batched, float alpha, float beta,
                    float* __restrict__ D, long long sD, int ldd, unsigned* err) {
@@ -497,14 +510,24 @@ __global__ void __launch_bounds__(384, 1)
                 smem_u32(&bar_drain)));
             pdrain(smem_u32(&bar_drain), 0);
         }
-    } else if (warp >= 4 && warp < 8) {
-        // ---- split into hi / lo -----------------------------------------
-        const int t = threadIdx.x - 128;      // 0..127
-        const int q = t & 7;                  // lane within a quarter warp
+    } else if ((warp >= 4 && warp < 8) || warp >= 12) {
+        // ---- split into hi / lo: every other stage -----------------------
+        const int grp = warp >= 12;
+        const int t = threadIdx.x & 127;      // 0..127
+        // pieces (row, 4 k): a quarter warp takes the eight rows of a core matrix,
+        // at a k that differs by row pair, so its reads and its writes fall on
+        // distinct banks
+        // (offsets of a thread's pieces: these plus 512 floats per 32 rows)
+        const int ra0 = 8 * (t >> 5) + (t & 7), ka = (((t >> 3) & 3) + ((t & 7) >> 1)) & 3;
+        const int rawa = ra0 * kPK + 4 * ka, cona = ptile_off(ra0, 4 * ka);
+        // B's likewise, or, from [kPK][Np] (n contiguous), lanes over n and a warp per k
+        const int rb0 = b_trans ? lane : ra0, conb = b_trans ? ptile_off(lane, 4 * (warp & 3)) : cona;
+        const int rawb = b_trans ? 4 * (warp & 3) * Np + lane : rawa;
         int g = 0;
         bool ok = true;
         for (int i = 0; i < my_tiles && ok; ++i) {
             for (int s = 0; s < n_stage; ++s, ++g) {
+                if ((g & 1) != grp) continue;
                 const int rs = g % kRaw, cs = g % kConv;
                 ok = pwait(smem_u32(&bar_raw_full[rs]), (g / kRaw) & 1, abort_flag, err);
                 if (ok && g >= kConv) ok = pwait(smem_u32(&bar_conv_empty[cs]), ((g / kConv) - 1) & 1, abort_flag, err);
@@ -515,41 +538,29 @@ __global__ void __launch_bounds__(384, 1)
                 float* aL = aH + kTcM * kPK;
                 float* bH = reinterpret_cast<float*>(psm + L.convB + cs * L.conv_bytes);
                 float* bL = bH + Np * kPK;
-                // A: thread t owns row t; its four 16-byte chunks are visited
-                // in a rotated order so a quarter warp's reads spread over the banks
-#pragma unroll
-                for (int j = 0; j < kPK / 4; ++j) {
-                    const int kq = (q + j) & 3;
-                    const float4 x = *reinterpret_cast<const float4*>(rA + t * kPK + 4 * kq);
+                auto put = [](float* H, float* Lo, float4 x) {
                     const float4 h = split_hi4(x);
-                    const int o = ptile_off(t, 4 * kq);
-                    *reinterpret_cast<float4*>(aH + o) = h;
-                    *reinterpret_cast<float4*>(aL + o) = split_lo4(x, h);
-                }
-                if (!b_trans) {
-                    for (int r = t; r < Np; r += 128)
+                    *reinterpret_cast<float4*>(H) = h;
+                    *reinterpret_cast<float4*>(Lo) = split_lo4(x, h);
+                };
+                float4 xa[4], xb[kTcMaxN / 32];
 #pragma unroll
-                        for (int j = 0; j < kPK / 4; ++j) {
-                            const int kq = (q + j) & 3;
-                            const float4 x = *reinterpret_cast<const float4*>(rB + r * kPK + 4 * kq);
-                            const float4 h = split_hi4(x);
-                            const int o = ptile_off(r, 4 * kq);
-                            *reinterpret_cast<float4*>(bH + o) = h;
-                            *reinterpret_cast<float4*>(bL + o) = split_lo4(x, h);
-                        }
-                } else {
-                    // raw B is [kPK][Np] (n contiguous): thread -> n
-                    for (int r = t; r < Np; r += 128)
+                for (int j = 0; j < 4; ++j) xa[j] = *reinterpret_cast<const float4*>(rA + rawa + 512 * j);
 #pragma unroll
-                        for (int kq = 0; kq < kPK / 4; ++kq) {
-                            const float4 x = make_float4(rB[(4 * kq) * Np + r], rB[(4 * kq + 1) * Np + r],
-                                                         rB[(4 * kq + 2) * Np + r], rB[(4 * kq + 3) * Np + r]);
-                            const float4 h = split_hi4(x);
-                            const int o = ptile_off(r, 4 * kq);
-                            *reinterpret_cast<float4*>(bH + o) = h;
-                            *reinterpret_cast<float4*>(bL + o) = split_lo4(x, h);
+                for (int j = 0; j < kTcMaxN / 32; ++j)
+                    if (rb0 + 32 * j < Np) {
+                        if (!b_trans) {
+                            xb[j] = *reinterpret_cast<const float4*>(rB + rawb + 512 * j);
+                        } else {
+                            const float* x = rB + rawb + 32 * j;
+                            xb[j] = make_float4(x[0], x[Np], x[2 * Np], x[3 * Np]);
                         }
-                }
+                    }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) put(aH + cona + 512 * j, aL + cona + 512 * j, xa[j]);
+#pragma unroll
+                for (int j = 0; j < kTcMaxN / 32; ++j)
+                    if (rb0 + 32 * j < Np) put(bH + conb + 512 * j, bL + conb + 512 * j, xb[j]);
                 // generic-proxy stores -> visible to the tensor core's reads
                 asm volatile("fence.proxy.async.shared::cta;");
                 __syncwarp();
@@ -559,7 +570,7 @@ __global__ void __launch_bounds__(384, 1)
                 }
             }
         }
-    } else if (warp >= 8) {
+    } else if (warp >= 8 && warp < 12) {
         // ---- epilogue ---------------------------------------------------
         const int q4 = warp & 3;
         float* buf = reinterpret_cast<float*>(psm + L.epi) + q4 * (32 * 33);
@@ -612,10 +623,15 @@ __global__ void __launch_bounds__(384, 1)
                             Db[(size_t)row * ldd + col] = alpha * buf[rr * 33 + lane] + beta * old[rr];
                     }
                 } else {
-                    for (int rr = 0; rr < 32; ++rr) {
-                        const int row = m0 + q4 * 32 + rr;
-                        if (row < M && col < N) Db[(size_t)row * ldd + col] = alpha * buf[rr * 33 + lane];
-                    }
+                    // (read before any store, as above)
+                    float v[32];
+#pragma unroll
+                    for (int rr = 0; rr < 32; ++rr) v[rr] = buf[rr * 33 + lane];
+                    float* Dc = Db + (size_t)(m0 + q4 * 32) * ldd + col;
+                    const int nr = col < N ? min(32, M - m0 - q4 * 32) : 0;
+#pragma unroll
+                    for (int rr = 0; rr < 32; ++rr)
+                        if (rr < nr) Dc[(size_t)rr * ldd] = alpha * v[rr];
                 }
                 __syncwarp();
             }
@@ -896,7 +912,7 @@ cudaError_t launch_tc_gemm_ab(int batch, int M, int N, int K, float alpha, const
     if (!n_sm[dev] && cudaDeviceGetAttribute(&n_sm[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return cudaErrorInvalidDevice;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tc_gemm_pipe, 384, L.total);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tc_gemm_pipe, 512, L.total);
     if (e != cudaSuccess) return e;
     uint32_t ncol = 32;
     while ((int)ncol < Np) ncol <<= 1;
@@ -905,7 +921,7 @@ cudaError_t launch_tc_gemm_ab(int batch, int M, int N, int K, float alpha, const
     if (per_sm < 1) per_sm = 1;
     const long long tiles = (long long)((M + kTcM - 1) / kTcM) * batch;
     const int grid = (int)(tiles < (long long)n_sm[dev] * per_sm ? tiles : (long long)n_sm[dev] * per_sm);
-    k_tc_gemm_pipe<<<grid, 384, L.total, st>>>(ta, tb, M, N, K, batch, b_trans, sA != 0, sB != 0, alpha, beta, D, sD,
+    k_tc_gemm_pipe<<<grid, 512, L.total, st>>>(ta, tb, M, N, K, batch, b_trans, sA != 0, sB != 0, alpha, beta, D, sD,
                                              ldd, err);
     return cudaGetLastError();
 }
