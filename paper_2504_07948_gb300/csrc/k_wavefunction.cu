@@ -142,13 +142,56 @@ __global__ void k_orbitals_sums(DevSys s, DevWalkers wk, int W, const int* only)
 // In-place Gauss-Jordan inversion with partial (row) pivoting, FP64, one
 // CTA per (walker, spin), the n x n matrix in shared memory.  Produces
 // ln|det A|, sign(det A) and the transposed inverse in the storage type.
+//
+// Bound by the FP64 pipe for large n (n^3 multiply-adds: 12,500 of some 15,500
+// cycles a pivot at n = 160), by the chain from pivot to pivot for small ones.
+// So no FP64 instruction is spent on the rest: magnitudes are compared as
+// integers, one lane takes the reciprocal, the logarithms wait for the end, and
+// a warp walks a row without divisions.  While the other warps eliminate column
+// k, warp 0 first brings column k + 1 up to date and picks its pivot: two
+// barriers a pivot.  Row interchanges are collected as one permutation of the
+// result's columns.  2 x 77 matrices of 15: 50 -> 27 us; 512 of 160: 6.9 -> 6.0 ms
+// (serial pivot search and logarithm, five barriers, a reciprocal per thread).
+
+// Pivot of column k from row k on (warp 0): row, reciprocal and, into piv[k], the
+// pivot itself.
+__device__ __forceinline__ void find_pivot(const double* M, int n, int k, double* piv, int* s_piv, double* s_pinv,
+                                           int* s_sing) {
+    const int lane = threadIdx.x & 31;
+    long long best = -1;
+    int bi = k;
+    for (int i = k + lane; i < n; i += 32) {
+        long long v = fx_bits(M[i * n + k]) & 0x7fffffffffffffffLL;   // |.| in the order of its value
+        if (v > 0x7ff0000000000000LL) v = -1;                         // never a NaN
+        if (v > best) {
+            best = v;
+            bi = i;
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (ob > best || (ob == best && oi < bi)) {
+            best = ob;
+            bi = oi;
+        }
+    }
+    if (lane == 0) {
+        const double v = M[bi * n + k];
+        const int e = fx_expo(v);
+        *s_piv = bi;
+        *s_pinv = 1.0 / v;
+        piv[k] = v;
+        if (e == 2047 || (fx_bits(v) & 0x7fffffffffffffffLL) == 0) *s_sing = 1;
+    }
+}
+
 // Inversion of one (walker, spin) matrix (body of k_invert).  M: n^2 + n
-// doubles of shared memory.
+// doubles of shared memory; at least n threads.
 __device__ __forceinline__ void invert_item(const DevSys& s, const DevWalkers& wk, int w, int spin, int store_fp32, unsigned* err, double* M) {
-    __shared__ int s_piv;
-    __shared__ int s_ipiv[256];
-    __shared__ double s_ld, s_sg;
-    __shared__ int s_sing;
+    __shared__ int s_perm[256];
+    __shared__ double s_pinv;
+    __shared__ int s_piv, s_sing, s_row[2];
     const int n = spin ? s.n_dn : s.n_up;
     if (n == 0) {
         if (threadIdx.x == 0) {
@@ -158,71 +201,61 @@ __device__ __forceinline__ void invert_item(const DevSys& s, const DevWalkers& w
         return;
     }
     double* fcol = M + n * n;
-    const double* A = wk.Ascr[spin] + (size_t)w * n * n;
+    double* A = wk.Ascr[spin] + (size_t)w * n * n;   // its first row receives the pivots
     for (int q = threadIdx.x; q < n * n; q += blockDim.x) M[q] = A[q];
     if (threadIdx.x == 0) {
-        s_ld = 0.0;
-        s_sg = 1.0;
         s_sing = 0;
+        s_row[0] = s_row[1] = 0;
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // rows of an elimination step of a warp, and this lane's row and first column of them
+    const int sub = n <= 8 ? 8 : n <= 16 ? 16 : 32, nrow = 32 / sub, lr = lane / sub, lc = lane % sub;
+    if (wid == 0) find_pivot(M, n, 0, A, &s_piv, &s_pinv, &s_sing);
+    __syncthreads();
+    int cur = threadIdx.x, swaps = 0;   // where this thread's column ends up; interchanges so far
     for (int k = 0; k < n; ++k) {
-        if (wid == 0) {
-            double best = -1.0;
-            int bi = k;
-            for (int i = k + lane; i < n; i += 32) {
-                const double v = fabs(M[i * n + k]);
-                if (v > best) {
-                    best = v;
-                    bi = i;
-                }
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-                if (ob > best || (ob == best && oi < bi)) {
-                    best = ob;
-                    bi = oi;
-                }
-            }
-            if (lane == 0) s_piv = bi;
-        }
-        __syncthreads();
+        if (s_sing) break;   // uniform: written before the last barrier
         const int p = s_piv;
-        if (p != k)
-            for (int j = threadIdx.x; j < n; j += blockDim.x) {
-                const double t = M[k * n + j];
-                M[k * n + j] = M[p * n + j];
-                M[p * n + j] = t;
-            }
-        __syncthreads();
-        const double piv = M[k * n + k];
-        if (piv == 0.0 || !isfinite(piv)) {
-            if (threadIdx.x == 0) s_sing = 1;
-            break;  // uniform: every thread read the same pivot
-        }
-        if (threadIdx.x == 0) {
-            s_ipiv[k] = p;
-            s_ld += log(fabs(piv));
-            s_sg *= (piv < 0.0 ? -1.0 : 1.0) * (p != k ? -1.0 : 1.0);
-        }
-        const double pinv = 1.0 / piv;
-        __syncthreads();
+        const double pinv = s_pinv;
+        // interchange rows k and p, scale the pivot row, keep the column
         for (int j = threadIdx.x; j < n; j += blockDim.x) {
-            fcol[j] = (j == k) ? 0.0 : M[j * n + k];
-            M[k * n + j] = (j == k) ? pinv : M[k * n + j] * pinv;
+            const double t = M[k * n + j], u = M[p * n + j];
+            if (p != k) M[p * n + j] = t;
+            M[k * n + j] = (j == k) ? pinv : u * pinv;
+            if (j == k) {
+                if (p != k) fcol[p] = t;
+                fcol[k] = 0.0;
+            }
+            if (j != k && j != p) fcol[j] = M[j * n + k];
         }
+        if (threadIdx.x == 0) s_row[(k + 1) & 1] = 0;
+        swaps += p != k;
+        cur = cur == k ? p : cur == p ? k : cur;
         __syncthreads();
-        for (int q = threadIdx.x; q < n * n; q += blockDim.x) {
-            const int i = q / n, j = q - i * n;
-            if (i == k) continue;
-            const double base = (j == k) ? 0.0 : M[q];
-            M[q] = base - fcol[i] * M[k * n + j];
+        const int ahead = k + 1 < n ? k + 1 : -1;   // the column that warp 0 takes
+        if (wid == 0 && ahead > 0) {
+            for (int i = lane; i < n; i += 32)
+                if (i != k) M[i * n + ahead] = M[i * n + ahead] - fcol[i] * M[k * n + ahead];
+            __syncwarp();
+            find_pivot(M, n, ahead, A, &s_piv, &s_pinv, &s_sing);
+        }
+        for (;;) {   // the other columns, rows to whichever warp is free
+            int i = 0;
+            if (lane == 0) i = atomicAdd(&s_row[k & 1], nrow);
+            i = __shfl_sync(0xffffffffu, i, 0);
+            if (i >= n) break;
+            i += lr;
+            if (i == k || i >= n) continue;
+            const double f = fcol[i];
+            for (int j = lc; j < n; j += sub) {
+                if (j == ahead) continue;
+                const double base = (j == k) ? 0.0 : M[i * n + j];
+                M[i * n + j] = base - f * M[k * n + j];
+            }
         }
         __syncthreads();
     }
-    __syncthreads();
     if (s_sing) {
         if (threadIdx.x == 0) {
             wk.logdet[2 * w + spin] = -INFINITY;
@@ -231,34 +264,33 @@ __device__ __forceinline__ void invert_item(const DevSys& s, const DevWalkers& w
         }
         return;
     }
-    // undo the row interchanges as column interchanges, last first
-    for (int k = n - 1; k >= 0; --k) {
-        const int p = s_ipiv[k];
-        if (p != k)
-            for (int i = threadIdx.x; i < n; i += blockDim.x) {
-                const double t = M[i * n + k];
-                M[i * n + k] = M[i * n + p];
-                M[i * n + p] = t;
-            }
-        __syncthreads();
+    int neg = 0;
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+        s_perm[k] = cur;
+        const double v = A[k];
+        neg = v < 0.0;
+        fcol[k] = log(fabs(v));
     }
-    // AinvT[e][j] = (A^-1)[j][e]
+    neg = __syncthreads_count(neg);
+    // AinvT[e][j] = (A^-1)[j][e], the interchanges undone as interchanges of its columns, last first
     if (store_fp32) {
         float* out = (float*)wk.Ainv[spin] + (size_t)w * n * n;
         for (int q = threadIdx.x; q < n * n; q += blockDim.x) {
             const int e = q / n, j = q - e * n;
-            out[q] = (float)M[j * n + e];
+            out[q] = (float)M[j * n + s_perm[e]];
         }
     } else {
         double* out = (double*)wk.Ainv[spin] + (size_t)w * n * n;
         for (int q = threadIdx.x; q < n * n; q += blockDim.x) {
             const int e = q / n, j = q - e * n;
-            out[q] = M[j * n + e];
+            out[q] = M[j * n + s_perm[e]];
         }
     }
     if (threadIdx.x == 0) {
-        wk.logdet[2 * w + spin] = s_ld;
-        wk.sgn[2 * w + spin] = s_sg;
+        double ld = 0.0;
+        for (int k = 0; k < n; ++k) ld += fcol[k];
+        wk.logdet[2 * w + spin] = ld;
+        wk.sgn[2 * w + spin] = (neg + swaps) & 1 ? -1.0 : 1.0;
     }
 }
 
@@ -803,7 +835,7 @@ cudaError_t launch_invert(const DevSys& s, const DevWalkers& wk, int W, int stor
     const size_t smem = sizeof(double) * ((size_t)nmax * nmax + nmax + 1);
     cudaError_t e = cudaFuncSetAttribute(k_invert, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const int nt = nmax > 64 ? 512 : (nmax > 16 ? 256 : 64);
+    const int nt = nmax > 64 ? 512 : (nmax > 16 ? 256 : 128);
     k_invert<<<dim3(W, 2), nt, smem, st>>>(s, wk, W, store_fp32, err, only);
     return cudaGetLastError();
 }
