@@ -118,6 +118,11 @@ __global__ void k_moments(const double* x, int W, double* out /*[2]*/) {
         out[1] = v[1];
     }
 }
+// Sign of the determinant product of every walker.
+__global__ void k_sign(double* out, const double* sgn, int W) {
+    const int w = blockIdx.x * blockDim.x + threadIdx.x;
+    if (w < W) out[w] = sgn[2 * w] * sgn[2 * w + 1];
+}
 __global__ void k_fill(double* x, int n, double v) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) x[i] = v;
@@ -1958,20 +1963,16 @@ static void evaluate_impl(qmc_t h, double* logpsi, double* sign, double* eloc, d
         if (logpsi && !on_device) copy_out(h, logpsi, d_lp2, sizeof(double) * W, 0);
         if (grad && !on_device) copy_out(h, grad, d_g, sizeof(double) * W * N * 3, 0);
         if (sign) {
-            std::vector<double> sg(2 * (size_t)W);
-            QMC_CK(cudaMemcpyAsync(sg.data(), h->wk[h->cur].sgn, sizeof(double) * 2 * W, cudaMemcpyDeviceToHost,
-                                   h->stream));
-            h->sync();
-            std::vector<double> s1(W);
-            for (int w = 0; w < W; ++w) s1[w] = sg[2 * w] * sg[2 * w + 1];
+            double* d_s = on_device ? sign : h->dalloc<double>(tmp, W);
             if (h->ds.msd) {
-                QMC_CK(cudaMemcpyAsync(s1.data(), h->d_sign, sizeof(double) * W, cudaMemcpyDeviceToHost, h->stream));
-                h->sync();
+                QMC_CK(cudaMemcpyAsync(d_s, h->d_sign, sizeof(double) * W, cudaMemcpyDeviceToDevice, h->stream));
+            } else {
+                k_sign<<<(W + 255) / 256, 256, 0, h->stream>>>(d_s, h->wk[h->cur].sgn, W);
+                QMC_CK(cudaGetLastError());
             }
-            QMC_CK(cudaMemcpyAsync(sign, s1.data(), sizeof(double) * W,
-                                   on_device ? cudaMemcpyHostToDevice : cudaMemcpyHostToHost, h->stream));
+            if (!on_device) copy_out(h, sign, d_s, sizeof(double) * W, 0);
         }
-        h->sync();
+        if (!tmp.empty()) h->sync();   // else the check below waits
         h->free_list(tmp);
         h->check_device_errors();
     }
