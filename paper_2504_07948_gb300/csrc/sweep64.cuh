@@ -199,7 +199,7 @@ __device__ __forceinline__ void sweep_walker64(const DevSys& s, const DevWalkers
         }
         auto pair = [&](double x, double y, double z, double r2, double a, double b) {
             const double ir = rsqrt(r2), q = rcp_ge1(1.0 + b * (r2 * ir));
-            const double aq = a * q, g = aq * q * ir;   // u'(r) / r
+            const double aq = a * q, g = aq * (q * ir);   // u'(r) / r, its two products side by side
             v[0] += aq * (r2 * ir);
             v[1] += g * x;
             v[2] += g * y;
