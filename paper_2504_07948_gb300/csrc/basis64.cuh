@@ -13,10 +13,16 @@
 //   5. value, gradient and Laplacian of the listed functions, split into
 //      limbs with one scale per component;
 //   6. phi[c][j] = sum_r C[row_r][j] bas[c][r], three 32-bit multiply-adds per
-//      term, slices of the rows on neighbouring lanes.
-// Bound by instruction issue (30 %, with the barriers between the steps) and
-// by the FP64 pipe (50 % at 30 orbitals).  Rebuild of the 32-water cluster, 256
-// walkers: 51 -> 17 ms against a masked basis and FP64 chains; 6-water cluster, 512 walkers: 1.64 -> 0.86 ms.
+//      term, slices of the rows on neighbouring lanes; rows without high limbs
+//      (below 2^-28 of the component's largest) take one, rows of zeros none: on
+//      the 32-water cluster 157 of an electron's 340 listed functions have high
+//      limbs and 60 are zero.
+// Bound by instruction issue (45 % with 15 to 20 warps on an SM: registers and
+// shared memory allow four CTAs of five warps, so the primitives' arrays share
+// their place with the functions') and by the FP64 pipe (50 % at 30 orbitals).
+// Rebuild of the 32-water cluster, 256 walkers: 51 -> 9.3 ms against a masked
+// basis and FP64 chains (17 ms with every listed row in three products and two
+// CTAs per SM); 6-water cluster, 512 walkers: 1.64 -> 0.85 ms.
 // The lists are filled in any order: every sum over them is exact integer
 // arithmetic, so the result does not depend on it.
 //
@@ -41,24 +47,23 @@ struct Basis64Layout {
         size_t o = 0;
         nuc = o;
         o += sizeof(double) * 4 * (size_t)n_nuc;
-        ev = o;
-        o += sizeof(double) * (size_t)n_prim;
         fs = o;
         o += sizeof(double) * 3 * (size_t)n_shell;
-        bas = o;
-        o += sizeof(double) * 5 * (size_t)ldb;
-        tf = o;
-        o += sizeof(float) * (size_t)n_nuc;
-        plist = o;
-        o += sizeof(int) * (size_t)n_prim;
-        slist = o;
-        o += sizeof(int) * (size_t)n_shell;
         flist = o;
         o += sizeof(int) * (size_t)n_basis;
         rows = o;
         o += sizeof(int) * (size_t)n_basis;
         cnt = o;
         o += sizeof(int) * 32;
+        o = (o + 15) & ~(size_t)15;
+        // the primitives' lists and exponentials end before the functions begin
+        bas = o;
+        ev = o;
+        tf = ev + sizeof(double) * (size_t)n_prim;
+        plist = tf + sizeof(float) * (size_t)n_nuc;
+        slist = plist + sizeof(int) * (size_t)n_prim;
+        const size_t prim = slist + sizeof(int) * (size_t)n_shell, fns = bas + sizeof(double) * 5 * (size_t)ldb;
+        o = prim > fns ? prim : fns;
         total = (o + 15) & ~(size_t)15;
     }
 };
@@ -68,10 +73,11 @@ struct Basis64Layout {
 constexpr size_t kBasis64Max = 224 * 1024;
 
 // Steps 1 to 5 at position (r0, r1, r2).  Leaves the limbs in bas [5][ldb]
-// (int2), the functions' indices in rows and returns their number; the
-// components' scales are fx_scale(cnt[8 + c]).  All threads call; ends
-// synchronised.  nuc: the nuclear offsets (x, y, z, r^2) stay valid after it.
-__device__ __forceinline__ int basis64(const DevSys& s, const Basis64Layout& L, unsigned char* sm, double r0, double r1,
+// (int2) and their entries (function << 16 | row) in flist: cnt[5] rows with some
+// high limb from its front, cnt[6] with low limbs only from its back; rows of
+// zeros are left out.  The components' scales are fx_scale(cnt[8 + c]).  All
+// threads call; ends synchronised.  nuc: the nuclear offsets (x, y, z, r^2) stay valid after it.
+__device__ __forceinline__ void basis64(const DevSys& s, const Basis64Layout& L, unsigned char* sm, double r0, double r1,
                                        double r2) {
     double4* nuc = (double4*)(sm + L.nuc);
     double* ev = (double*)(sm + L.ev);
@@ -82,7 +88,8 @@ __device__ __forceinline__ int basis64(const DevSys& s, const Basis64Layout& L, 
     int* slist = (int*)(sm + L.slist);
     int* flist = (int*)(sm + L.flist);   // functions by kind: s from 0, p from n_fn_s, d from n_fn_s + n_fn_p
     int* rows = (int*)(sm + L.rows);
-    int* cnt = (int*)(sm + L.cnt);       // [0] primitives, [1] shells, [2..4] functions by kind, [8..12] exponents,
+    int* cnt = (int*)(sm + L.cnt);       // [0] primitives, [1] shells, [2..4] functions by kind, [5], [6] rows,
+                                         // [8..12] exponents,
                                          // [16..20], [24..28] exponents of the sums (orbitals64)
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, ldb = L.ldb;
     const unsigned below = (1u << lane) - 1u;
@@ -219,13 +226,32 @@ __device__ __forceinline__ int basis64(const DevSys& s, const Basis64Layout& L, 
     int em[5];
 #pragma unroll
     for (int c = 0; c < 5; ++c) em[c] = cnt[8 + c];
-    for (int o = tid; o < 5 * nrow; o += nt) {
-        const int c = o / nrow, q = c * ldb + o - c * nrow;
-        const int e = c == 0 ? em[0] : c == 1 ? em[1] : c == 2 ? em[2] : c == 3 ? em[3] : em[4];
-        ((int2*)bas)[q] = fx_limbs(bas[q], e);
+    for (int r0 = tid - lane; r0 < nrow; r0 += nt) {
+        const int r = r0 + lane;
+        int hi = 0, lo = 0;
+        if (r < nrow)
+#pragma unroll
+            for (int c = 0; c < 5; ++c) {
+                const int2 v = fx_limbs(bas[c * ldb + r], em[c]);
+                ((int2*)bas)[c * ldb + r] = v;
+                hi |= v.x;
+                lo |= v.y;
+            }
+        // (the function lists are used up: their place takes the entries)
+        const unsigned mh = __ballot_sync(0xffffffffu, hi != 0), ml = __ballot_sync(0xffffffffu, hi == 0 && lo != 0);
+        int bh = 0, bl = 0;
+        if (lane == 0) {
+            bh = mh ? atomicAdd(&cnt[5], __popc(mh)) : 0;
+            bl = ml ? atomicAdd(&cnt[6], __popc(ml)) : 0;
+        }
+        bh = __shfl_sync(0xffffffffu, bh, 0) + __popc(mh & below);
+        bl = __shfl_sync(0xffffffffu, bl, 0) + __popc(ml & below);
+        if (hi)
+            flist[bh] = rows[r] << 16 | r;
+        else if (lo)
+            flist[s.n_basis - 1 - bl] = rows[r] << 16 | r;
     }
     __syncthreads();
-    return nrow;
 }
 
 // Step 6: put(c, j, phi_cj) for c < 5 and every orbital j < n of a
@@ -234,13 +260,13 @@ __device__ __forceinline__ int basis64(const DevSys& s, const Basis64Layout& L, 
 // keep n S within the CTA.  big: five counters (zero before the call) that
 // receive the largest exponent of the integer sums per component.
 template <typename Put>
-__device__ __forceinline__ void contract64(const Basis64Layout& L, const unsigned char* sm, int nrow,
+__device__ __forceinline__ void contract64(const Basis64Layout& L, const unsigned char* sm, int nb,
                                            const int2* __restrict__ Ck, const double* __restrict__ sC, int n, int* big,
                                            Put put) {
     const int2* bas = (const int2*)(sm + L.bas);
-    const int* rows = (const int*)(sm + L.rows);
+    const int* list = (const int*)(sm + L.flist);
     const int* cnt = (const int*)(sm + L.cnt);
-    const int ldb = L.ldb;
+    const int ldb = L.ldb, nh = cnt[5], nl = cnt[6];
     int lg = 4;
     while (lg > 0 && (n << lg) > (int)blockDim.x) --lg;
     const int S = 1 << lg, items = (n << lg);
@@ -249,14 +275,31 @@ __device__ __forceinline__ void contract64(const Basis64Layout& L, const unsigne
         const int o = o0 + (threadIdx.x & 31), sl = o & (S - 1);
         const int j = min(o >> lg, n - 1);
         FxSum sum[5];
-        for (int r0 = sl; r0 < nrow; r0 += kFxBlock * S) {
+        for (int r0 = sl; r0 < nh; r0 += kFxBlock * S) {
             FxDot d[5];
-            const int r1 = min(nrow, r0 + kFxBlock * S);
+            const int r1 = min(nh, r0 + kFxBlock * S);
 #pragma unroll 4
             for (int r = r0; r < r1; r += S) {
-                const int2 cv = Ck[(size_t)rows[r] * n + j];
+                const int e = list[r];
+                const int2 cv = Ck[(e >> 16) * n + j];
+                const int2* b = bas + (e & 0xffff);
 #pragma unroll
-                for (int c = 0; c < 5; ++c) d[c].add(cv, bas[c * ldb + r]);
+                for (int c = 0; c < 5; ++c) d[c].add(cv, b[c * ldb]);
+            }
+#pragma unroll
+            for (int c = 0; c < 5; ++c) sum[c].fold(d[c]);
+        }
+        // without high limbs one product of the three is left
+        for (int r0 = sl; r0 < nl; r0 += kFxBlock * S) {
+            FxDot d[5];
+            const int r1 = min(nl, r0 + kFxBlock * S);
+#pragma unroll 4
+            for (int r = r0; r < r1; r += S) {
+                const int e = list[nb - 1 - r];
+                const int ch = Ck[(e >> 16) * n + j].x;
+                const int2* b = bas + (e & 0xffff);
+#pragma unroll
+                for (int c = 0; c < 5; ++c) d[c].mid += (long long)ch * b[c * ldb].y;
             }
 #pragma unroll
             for (int c = 0; c < 5; ++c) sum[c].fold(d[c]);
@@ -312,9 +355,9 @@ __device__ __forceinline__ void orbitals64(const DevSys& s, const Basis64Layout&
                                            int n, Put put, const int2* Ck2, const double* sC2, const double* C2, int n2,
                                            Put2 put2) {
     int* cnt = (int*)(sm + L.cnt);
-    const int nrow = basis64(s, L, sm, r0, r1, r2);
-    contract64(L, sm, nrow, Ck, sC, n, cnt + 16, put);
-    if (n2 > 0) contract64(L, sm, nrow, Ck2, sC2, n2, cnt + 24, put2);
+    basis64(s, L, sm, r0, r1, r2);
+    contract64(L, sm, s.n_basis, Ck, sC, n, cnt + 16, put);
+    if (n2 > 0) contract64(L, sm, s.n_basis, Ck2, sC2, n2, cnt + 24, put2);
     __syncthreads();
     // integer sums of the largest possible product: 2^56 (biased 1079)
     bool low = false, low2 = false;

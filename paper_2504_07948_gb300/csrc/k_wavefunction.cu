@@ -53,7 +53,7 @@ __device__ __forceinline__ void orbitals_item(const DevSys& s, const DevWalkers&
 }
 
 template <typename T>
-__global__ void k_orbitals_all(DevSys s, DevWalkers wk, int W, const int* only) {
+__global__ void __launch_bounds__(320, 2) k_orbitals_all(DevSys s, DevWalkers wk, int W, const int* only) {
     extern __shared__ double sh_bas[];
     const int w = blockIdx.x, i = blockIdx.y;
     if (w >= W || (only && !only[w])) return;
