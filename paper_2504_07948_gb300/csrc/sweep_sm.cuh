@@ -76,6 +76,11 @@ __device__ __forceinline__ void sweep_walker(const DevSys& s, const DevWalkers& 
     // step r' - r, [9..11] the drift at r, [12] ratio, [13] accept (int).
     float* fs = (float*)(scal + 8);
     constexpr bool kMixed = sizeof(T) == 4;
+    // Mixed form: random numbers of 32 moves (three normals, the acceptance
+    // uniform), drawn by the lanes of one warp together; one by one they were a
+    // sixth of the serial part of a move.  In the reductions' scratch, of which
+    // the mixed form uses the first half.
+    float* drawn = (float*)(red + kMaxWarps * 4);
     // positions in the precision of the pair terms
     T* sRt = sizeof(T) == 8 ? (T*)(void*)sR : (T*)(void*)sRf;
     T* bas = (T*)(smem + ob);
@@ -130,6 +135,12 @@ __device__ __forceinline__ void sweep_walker(const DevSys& s, const DevWalkers& 
         const T* Ae = A + (size_t)k * n;
         const T* Ge = Gs + (size_t)k * 4 * n;
         const double re0 = sR[3 * e], re1 = sR[3 * e + 1], re2 = sR[3 * e + 2];
+        if constexpr (kMixed) {
+            if ((e & 31) == 0 && wid == nw - 1 && e + lane < N) {
+                draw_normals_f(p.key, p.sweep, (uint32_t)(e + lane), (uint32_t)w, drawn + 4 * lane);
+                drawn[4 * lane + 3] = accept_uniform_f(p.key, p.sweep, (uint32_t)(e + lane), (uint32_t)w);
+            }
+        }
         const T et0 = sRt[3 * e], et1 = sRt[3 * e + 1], et2 = sRt[3 * e + 2];
 
         // -- drift at the current position: grad_e ln|D| + grad_e J --------
@@ -187,7 +198,7 @@ __device__ __forceinline__ void sweep_walker(const DevSys& s, const DevWalkers& 
             const T g[3] = {va[0] + va[3], va[1] + va[4], va[2] + va[5]};
             const double r[3] = {re0, re1, re2};
             if constexpr (kMixed) {
-                if (threadIdx.x == 0) propose_move_mixed(g, tau, r, p.key, p.sweep, (uint32_t)e, (uint32_t)w, scal, fs);
+                if (threadIdx.x == 0) propose_move_drawn(g, tau, r, drawn + 4 * (e & 31), scal, fs);
             } else {
                 const double gd[3] = {g[0], g[1], g[2]};
                 propose_move_fp64_pair(gd, tau, r, p.key, p.sweep, (uint32_t)e, (uint32_t)w, scal);
@@ -266,8 +277,8 @@ __device__ __forceinline__ void sweep_walker(const DevSys& s, const DevWalkers& 
         if (threadIdx.x == 0) {
             const T gd[3] = {vb2[1], vb2[2], vb2[3]}, gj[3] = {vb2[5], vb2[6], vb2[7]};
             if constexpr (kMixed) {
-                const int accept = accept_move_mixed(vb2[0], gd, gj, vb2[4], tau, fs, p.key, p.sweep, (uint32_t)e,
-                                                     (uint32_t)w);
+                const int accept =
+                    accept_move_drawn(vb2[0], gd, gj, vb2[4], tau, fs, drawn[4 * (e & 31) + 3]);
                 fs[12] = vb2[0];
                 ((int*)fs)[13] = accept;
             } else {
