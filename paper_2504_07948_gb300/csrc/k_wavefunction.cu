@@ -818,7 +818,10 @@ cudaError_t launch_orbitals_all(const DevSys& s, const DevWalkers& wk, int W, cu
     }
     const size_t smem = orbitals_smem_bytes(s);
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
-    const int nt = nmax > 128 ? (nmax > 256 ? 256 : (nmax + 31) & ~31) : 128;   // a thread per orbital
+    // a thread per orbital; few orbitals share their rows among lanes anyway, and
+    // two warps per electron leave room for twice the electrons (3 waters, 77
+    // walkers: three waves of CTAs become two, evaluation 164 -> 144 us)
+    const int nt = nmax > 128 ? (nmax > 256 ? 256 : (nmax + 31) & ~31) : nmax > 16 ? 128 : 64;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_orbitals_all<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem);
