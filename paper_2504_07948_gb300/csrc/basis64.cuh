@@ -22,7 +22,8 @@
 // their place with the functions') and by the FP64 pipe (50 % at 30 orbitals).
 // Rebuild of the 32-water cluster, 256 walkers: 51 -> 9.3 ms against a masked
 // basis and FP64 chains (17 ms with every listed row in three products and two
-// CTAs per SM); 6-water cluster, 512 walkers: 1.64 -> 0.85 ms.
+// CTAs per SM); 6-water cluster, 512 walkers: 1.64 -> 0.86 ms (before
+// the split by limbs).
 // The lists are filled in any order: every sum over them is exact integer
 // arithmetic, so the result does not depend on it.
 //
