@@ -166,17 +166,8 @@ __host__ __device__ inline size_t tiled_smem_bytes(int n_nuc, int n_shell) {
     return sizeof(TiledSmem) + sizeof(float) * (6 * (size_t)n_nuc + 3 * (size_t)n_shell);
 }
 
-// K^-1, the queue's row indices, t and the nuclei into shared memory
-// (asynchronously; tiled_wait completes them).
-__device__ __forceinline__ void tiled_fetch(const DevSys& s, const TiledState& ts, int w, int dq, TiledSmem& S,
-                                            bool with_t) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, kmax = ts.kmax;
-    const float2* KT = ts.KinvT + (size_t)w * kmax * kmax;
-    for (int q = wid; q < dq; q += kTb / 32)
-        if (lane < dq)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(&S.KT[q][lane])),
-                         "l"(KT + (size_t)q * kmax + lane));
-    asm volatile("cp.async.commit_group;");
+// The nuclei into shared memory.
+__device__ __forceinline__ void tiled_nuclei(const DevSys& s, TiledSmem& S) {
     float* nuc = (float*)(&S + 1);
     for (int a = threadIdx.x; a < s.n_nuc; a += kTb)
 #pragma unroll
@@ -184,6 +175,18 @@ __device__ __forceinline__ void tiled_fetch(const DevSys& s, const TiledState& t
             nuc[6 * a + c] = s.Rn_hi[3 * a + c];
             nuc[6 * a + 3 + c] = s.Rn_lo[3 * a + c];
         }
+}
+
+// K^-1, the queue's row indices and t into shared memory (asynchronously;
+// tiled_wait completes them).
+__device__ __forceinline__ void tiled_fetch(const TiledState& ts, int w, int dq, TiledSmem& S, bool with_t) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, kmax = ts.kmax;
+    const float2* KT = ts.KinvT + (size_t)w * kmax * kmax;
+    for (int q = wid; q < dq; q += kTb / 32)
+        if (lane < dq)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(&S.KT[q][lane])),
+                         "l"(KT + (size_t)q * kmax + lane));
+    asm volatile("cp.async.commit_group;");
     if ((int)threadIdx.x < dq) {
         S.rows[threadIdx.x] = ts.rows[(size_t)w * kmax + threadIdx.x];
         if (with_t) S.t[threadIdx.x] = ts.tv[(size_t)w * kmax + threadIdx.x];
@@ -233,10 +236,14 @@ __device__ __forceinline__ void tiled_draw_normals(const SweepParams& p, int e, 
         for (int c = 0; c < 3; ++c) S.chi[c] = chi[c];
     }
 }
+// The acceptance uniform of electron e's move, by a thread of another warp.
+__device__ __forceinline__ void tiled_draw_uniform(const SweepParams& p, int e, int w, TiledSmem& S) {
+    if (threadIdx.x == kTb - 64) S.uni = accept_uniform_f(p.key, p.sweep, (uint32_t)e, (uint32_t)w);
+}
 
 // Column e of the current inverse, drift, proposal and the basis at r' as
 // TF32 hi / lo rows of B', for walker w (the whole CTA).  dq: queue length;
-// S holds K^-1 and the rows (tiled_fetch, complete) and the normals.
+// S holds the nuclei, K^-1 and the rows (tiled_fetch, complete) and the normals.
 __device__ __forceinline__ void propose_body(const DevSys& s, const DevWalkers& wk, const TiledState& ts, int w,
                                              int e, const SweepParams& p, int dq, TiledSmem& S) {
     const int tid = threadIdx.x;
@@ -364,8 +371,9 @@ __device__ __forceinline__ void propose_body(const DevSys& s, const DevWalkers& 
 
 // Ratio, drift at r', Jastrow change, Metropolis test of walker w's move of
 // electron e; an accepted move borders K^-1 (in S and in global memory) and
-// queues its orbital row.  dq: queue length; tiled_fetch has been started.
-// Returns the queue length after the move; ends synchronised.
+// queues its orbital row.  dq: queue length; tiled_fetch has been started, S
+// holds the uniform.  Returns the queue length after the move; ends
+// synchronised.
 __device__ __forceinline__ int accept_body(const DevSys& s, const DevWalkers& wk, const TiledState& ts, int w, int e,
                                            const SweepParams& p, int dq, TiledSmem& S) {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -374,10 +382,14 @@ __device__ __forceinline__ int accept_body(const DevSys& s, const DevWalkers& wk
     const float* Phi = ts.Phi + (size_t)w * 5 * n;
     const float* ce = ts.ce + (size_t)w * ldv;
     const float* mv = ts.mv + (size_t)w * kTiledMv;
-    // everything that does not need the orbitals, while the GEMM before this
-    // launch is still running (see launch_after)
-    if (tid == kTb - 64) S.uni = accept_uniform_f(p.key, p.sweep, (uint32_t)e, (uint32_t)w);
     float v8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int j = tid; j < n; j += kTb) {
+        const float a = ce[j];
+        v8[0] += Phi[j] * a;
+        v8[1] += Phi[n + j] * a;
+        v8[2] += Phi[2 * n + j] * a;
+        v8[3] += Phi[3 * n + j] * a;
+    }
     const float2* Rp = ts.Rp + (size_t)w * 3 * N;
     {
         const float rh[3] = {mv[0], mv[1], mv[2]}, rl[3] = {mv[3], mv[4], mv[5]};
@@ -386,14 +398,6 @@ __device__ __forceinline__ int accept_body(const DevSys& s, const DevWalkers& wk
         v8[5] = gj[0];
         v8[6] = gj[1];
         v8[7] = gj[2];
-    }
-    grid_wait();
-    for (int j = tid; j < n; j += kTb) {
-        const float a = ce[j];
-        v8[0] += Phi[j] * a;
-        v8[1] += Phi[n + j] * a;
-        v8[2] += Phi[2 * n + j] * a;
-        v8[3] += Phi[3 * n + j] * a;
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");   // before the sum's barrier: K^-1 is complete after it
     cta_sum_to0<8>(v8, S.red);
@@ -461,11 +465,11 @@ __device__ __forceinline__ int accept_body(const DevSys& s, const DevWalkers& wk
 }
 
 // Launches of a move's kernels follow each other programmatically: the next
-// grid starts once every CTA of this one has passed grid_release, and reads
-// what this grid writes only after its grid_wait.  The GEMM releases after its
-// own wait, so an accept launch that has started finds everything the previous
-// accept / propose launch wrote and can form the Jastrow sums, fetch K^-1 and
-// draw its random numbers while the GEMM runs.  Used where one chain of launches
+// grid starts once every CTA of this one has passed grid_release, and touches
+// what any launch of the sweep writes only after its grid_wait: a release
+// promises the next grid no memory, neither this grid's nor that of the grids
+// before it.  Ahead of its wait an accept launch takes the constants (nuclei)
+// and draws its random numbers, while the GEMM runs.  Used where one chain of launches
 // has the GPU (32 waters, 256 walkers: 49 -> 42 us an electron); with several
 // groups a GEMM that waits for its rows would hold SMs the other group could
 // use (4096 walkers, two groups: 206 -> 217), and launches are plain.
@@ -478,7 +482,8 @@ __global__ void __launch_bounds__(kTb, 8) k_tiled_propose(DevSys s, DevWalkers w
     const int w = w0 + (int)blockIdx.x;
     if (w >= W) return;
     const int dq = ts.dq[w];
-    tiled_fetch(s, ts, w, dq, S, false);
+    tiled_fetch(ts, w, dq, S, false);
+    tiled_nuclei(s, S);
     tiled_draw_normals(p, e, w, S);
     tiled_wait();
     propose_body(s, wk, ts, w, e, p, dq, S);
@@ -490,8 +495,10 @@ __global__ void __launch_bounds__(kTb, 8) k_tiled_accept(DevSys s, DevWalkers wk
     TiledSmem& S = *reinterpret_cast<TiledSmem*>(tsm);
     const int w = w0 + (int)blockIdx.x;
     if (w >= W) return;
+    tiled_draw_uniform(p, e, w, S);
+    grid_wait();
     const int dq = ts.dq[w];
-    tiled_fetch(s, ts, w, dq, S, true);
+    tiled_fetch(ts, w, dq, S, true);
     accept_body(s, wk, ts, w, e, p, dq, S);
 }
 
@@ -510,9 +517,12 @@ __global__ void __launch_bounds__(kTb, 8) k_tiled_accept_propose(DevSys s, DevWa
     TiledSmem& S = *reinterpret_cast<TiledSmem*>(tsm);
     const int w = w0 + (int)blockIdx.x;
     if (w >= W) return;
-    const int dq = ts.dq[w];
-    tiled_fetch(s, ts, w, dq, S, true);
+    tiled_nuclei(s, S);
+    tiled_draw_uniform(p, e, w, S);
     tiled_draw_normals(p, e + 1, w, S);
+    grid_wait();
+    const int dq = ts.dq[w];
+    tiled_fetch(ts, w, dq, S, true);
     const int dq1 = accept_body(s, wk, ts, w, e, p, dq, S);
     propose_body(s, wk, ts, w, e + 1, p, dq1, S);
 }
