@@ -19,6 +19,7 @@
 // is O(n^2 n_basis + n^3 + N n_basis) per walker, independent of N_atom.
 // Basis derivatives to third order are recomputed per walker rather than
 // stored.  The e-n Jastrow, V_en and V_nn terms are added directly.
+#include <algorithm>
 #include <type_traits>
 
 #include "batch.cuh"
@@ -795,12 +796,18 @@ __global__ void k_force_prep(DevSys s, DevWalkers wk, int w0, int W, const doubl
 // the last one is not most of the time; one where the per-electron sums of the
 // space warp are wanted, which run over all nuclei.  32-water cluster, 512
 // walkers, mixed: 855 -> 509 us, with the runs shared out as warps come free.
+// Each spin adds to sums of its own: both on the nucleus's one made the last
+// bits depend on which warp came first (one warp taking both spins of a run,
+// which also fixes the order, was 3 % slower on the whole pass).
 static int contract_parts(int W, int nn, bool kE) {
     if (kE) return 1;
     int p = 1;
     while ((long long)W * p < 6 * 152 * 3 && nn / (2 * p) >= 24) p *= 2;
     return p;
 }
+// Nuclei of a part up to which spin down has sums of its own: thousands of
+// nuclei (point charges) would not leave them room.
+constexpr int kContractOwn = 1024;
 
 // Third-order basis contraction with M, Y read from the GEMM outputs
 // Mw/Yw [spin][walker][n_basis][n] (type T; each spin's block starts at
@@ -818,13 +825,19 @@ __global__ void __launch_bounds__(256) k_force_contract(DevSys s, DevWalkers wk,
     const ForceHead<T> h(sm, N, nn);
     double* acc = h.acc;
     unsigned char* scr = (unsigned char*)sm + ((force_head_bytes<T>(N, nn) + 15) & ~(size_t)15);
-    double* gEs = (double*)(scr + (sizeof(T) == 8 ? 8 * kRadialScratch : 0));
+    // spin down's sums [6 (nz - na)], acc: spin up's (or both)
+    const bool own = nz - na <= kContractOwn;
+    double* acc_dn = (double*)(scr + (sizeof(T) == 8 ? 8 * kRadialScratch : 0));
+    double* gEs = acc_dn + (own ? 6 * (nz - na) : 0);
     scr += (threadIdx.x >> 5) * kRadialScratch;   // the warp's radial scratch (FP64 form)
     force_load_positions(h, wk.R + (size_t)w * 3 * N, N);
     if constexpr (kE)
         for (int q = threadIdx.x; q < 3 * N; q += blockDim.x) gEs[q] = 0.0;
     for (int q = threadIdx.x; q < 3 * N; q += blockDim.x) h.gJ[q] = T(gJw[(size_t)wl * 3 * N + q]);
-    for (int q = 6 * na + threadIdx.x; q < 6 * nz; q += blockDim.x) acc[q] = accw[(size_t)wl * 6 * nn + q];
+    for (int q = 6 * na + threadIdx.x; q < 6 * nz; q += blockDim.x) {
+        acc[q] = accw[(size_t)wl * 6 * nn + q];
+        if (own) acc_dn[q - 6 * na] = 0.0;
+    }
     __syncthreads();
     // both spins' runs in turn to whichever warp is free (functions per run differ)
     __shared__ int s_next;
@@ -868,14 +881,16 @@ __global__ void __launch_bounds__(256) k_force_contract(DevSys s, DevWalkers wk,
             }
             const T sum = warp_fold8(v);
             const int q = fold8_index(lane);
-            if ((lane & 3) == 0 && q < 6) atomicAdd(&acc[6 * ctr + q], q < 3 ? double(sum) : -double(sum));
+            double* to = spin && own ? acc_dn + 6 * (ctr - na) : acc + 6 * ctr;
+            if ((lane & 3) == 0 && q < 6) atomicAdd(&to[q], q < 3 ? double(sum) : -double(sum));
         }
     }
     __syncthreads();
     for (int q = 3 * na + threadIdx.x; q < 3 * nz; q += blockDim.x) {
         const int a = q / 3, c = q - 3 * a;
-        dEL[(size_t)w * 3 * nn + q] = acc[6 * a + c] + (wk.nlF ? wk.nlF[(size_t)w * 3 * nn + q] : 0.0);
-        dlog[(size_t)w * 3 * nn + q] = acc[6 * a + 3 + c];
+        const double dT = own ? acc_dn[6 * (a - na) + c] : 0.0, dJ = own ? acc_dn[6 * (a - na) + 3 + c] : 0.0;
+        dEL[(size_t)w * 3 * nn + q] = acc[6 * a + c] + dT + (wk.nlF ? wk.nlF[(size_t)w * 3 * nn + q] : 0.0);
+        dlog[(size_t)w * 3 * nn + q] = acc[6 * a + 3 + c] + dJ;
     }
     if constexpr (kE)
         for (int q = threadIdx.x; q < 3 * N; q += blockDim.x) gEdet[(size_t)w * 3 * N + q] = gEs[q];
@@ -906,9 +921,10 @@ cudaError_t launch_force_prep(const DevSys& s, const DevWalkers& wk, int w0, int
 }
 
 template <typename T>
-static size_t contract_smem(int N, int nn, bool kE) {
+static size_t contract_smem(int N, int nn, int parts, bool kE) {
+    const int part = (nn + parts - 1) / parts;   // of the largest part
     return ((force_head_bytes<T>(N, nn) + 15) & ~(size_t)15) + (sizeof(T) == 8 ? 8 * kRadialScratch : 0) +
-           (kE ? sizeof(double) * 3 * (size_t)N : 0);
+           sizeof(double) * 6 * (size_t)std::min(part, kContractOwn) + (kE ? sizeof(double) * 3 * (size_t)N : 0);
 }
 
 // gEdet (may be null): determinant part of dE_L/dr_i [W][N][3] (walker
@@ -919,24 +935,26 @@ cudaError_t launch_force_contract(const DevSys& s, const DevWalkers& wk, int w0,
                                   cudaStream_t st) {
     if (W == 0) return cudaSuccess;
     if (gEdet) {
-        const size_t smem = contract_smem<T>(s.N, s.n_nuc, true);
+        const int parts = contract_parts(W, s.n_nuc, true);
+        const size_t smem = contract_smem<T>(s.N, s.n_nuc, parts, true);
         if (smem > 48 * 1024) {
             cudaError_t e = cudaFuncSetAttribute(k_force_contract<T, true>,
                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        k_force_contract<T, true><<<dim3(W, contract_parts(W, s.n_nuc, true)), 256, smem, st>>>(s, wk, w0, W, (const T*)Mw, (const T*)Yw, gJw, accw, dEL,
-                                                         dlog, gEdet);
+        k_force_contract<T, true><<<dim3(W, parts), 256, smem, st>>>(s, wk, w0, W, (const T*)Mw, (const T*)Yw, gJw, accw,
+                                                                     dEL, dlog, gEdet);
         return cudaGetLastError();
     }
-    const size_t smem = contract_smem<T>(s.N, s.n_nuc, false);
+    const int parts = contract_parts(W, s.n_nuc, false);
+    const size_t smem = contract_smem<T>(s.N, s.n_nuc, parts, false);
     if (smem > 48 * 1024) {
         cudaError_t e =
             cudaFuncSetAttribute(k_force_contract<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    k_force_contract<T, false><<<dim3(W, contract_parts(W, s.n_nuc, false)), 256, smem, st>>>(s, wk, w0, W, (const T*)Mw, (const T*)Yw, gJw, accw, dEL, dlog,
-                                                      nullptr);
+    k_force_contract<T, false><<<dim3(W, parts), 256, smem, st>>>(s, wk, w0, W, (const T*)Mw, (const T*)Yw, gJw, accw, dEL,
+                                                                  dlog, nullptr);
     return cudaGetLastError();
 }
 
