@@ -437,7 +437,7 @@ __device__ __forceinline__ void eloc_walker(const DevSys& s, const DevWalkers& w
                         const float r2 = x * x + y * y + z * z;
                         const float ir = rsqrtf(r2), r = r2 * ir;
                         const float a = (float)(((i < nu) == (j < nu)) ? s.a_par : s.a_anti);
-                        const float q = __fdividef(1.0f, 1.0f + b * r);
+                        const float q = 1.0f / (1.0f + b * r);
                         const float du = a * q * q, g = du * ir;
                         gx += g * x;
                         gy += g * y;
@@ -555,7 +555,7 @@ __device__ __forceinline__ void eloc_walker(const DevSys& s, const DevWalkers& w
                     const float r2 = x * x + y * y + z * z;
                     const float ir = rsqrtf(r2), r = r2 * ir;
                     const float ae = s.a_en_f[a];
-                    const float q = __fdividef(1.0f, 1.0f + b * r);
+                    const float q = 1.0f / (1.0f + b * r);
                     const float du = ae * q * q, g = du * ir;
                     fx += g * x;
                     fy += g * y;
