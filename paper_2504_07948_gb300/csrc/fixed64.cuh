@@ -25,6 +25,12 @@ constexpr int kFxQ = 57;
 constexpr int kFxLimb = 29;
 constexpr int kFxBlock = 32;
 
+// Bits by which the product of two rows' largest entries may exceed the largest
+// product of their entries before a fixed-point dot product of them gives way to
+// FP64: its error is some 2^-59 sqrt(k) of the former, that of an FP64 chain some
+// 2^-54 sqrt(k) of the latter (k_wavefunction.cu, sweep64.cuh, k_force.cu).
+constexpr int kFxSlack = 6;
+
 // Biased exponent of x (2047: infinity or NaN).
 __host__ __device__ __forceinline__ long long fx_bits(double x) {
     long long b;

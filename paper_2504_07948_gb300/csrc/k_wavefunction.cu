@@ -11,6 +11,11 @@
 
 namespace qmc {
 
+// Whether the orbitals of this basis are taken in fixed point.
+__host__ __device__ static inline bool orbitals_fx(const DevSys& s) {
+    return Basis64Layout(s.n_nuc, s.n_prim, s.n_shell, s.n_basis).total <= kBasis64Max;
+}
+
 // Orbitals of electron i of walker w by one CTA (body of k_orbitals_all):
 // the live basis functions at r_i in FP64 and the LCAO contraction phi_j =
 // sum_l C_l^j Phi_l (Eq. 2) in fixed point (basis64.cuh) for the occupied
@@ -43,7 +48,7 @@ __device__ __forceinline__ void orbitals_item(const DevSys& s, const DevWalkers&
         else
             Gv[(c - 1) * nv + j] = (T)v;
     };
-    if (L.total <= kBasis64Max) {
+    if (orbitals_fx(s)) {
         orbitals64(s, L, sm, r[0], r[1], r[2], s.Ck[spin], s.Ck_s[spin], s.C[spin], n, put, s.Cvk[spin], s.Cvk_s[spin],
                    s.Cv[spin], nv, put_v);
     } else {
@@ -152,10 +157,22 @@ __global__ void k_orbitals_sums(DevSys s, DevWalkers wk, int W, const int* only)
 // barriers a pivot.  Row interchanges are collected as one permutation of the
 // result's columns.  2 x 77 matrices of 15: 50 -> 27 us; 512 of 160: 6.9 -> 6.0 ms
 // (serial pivot search and logarithm, five barriers, a reciprocal per thread).
+//
+// Rows of A taken in fixed point carry an error of about 2^-59 sqrt(rows) of the
+// row's largest entry, in units of the orbitals' largest coefficients, where
+// FP64 sums keep every entry's own bits.  That matters where the inverse weighs
+// a row's small entries up: electrons shared out unevenly over distant fragments
+// with orbitals of their own.  So the inverse is held against its rows:
+// with x = A^-1 e_i, a row whose max|x_j| c_j max|A_ij / c_j| exceeds max|x_j
+// A_ij| by more than kFxSlack bits would lose accuracy against FP64 sums (their
+// error is some 2^-54 sqrt(rows) of the latter), and the orbitals of the spin's
+// electrons are taken again that way, as they are for a singular matrix.  On water
+// clusters with dense orbitals (1 to 32 waters) no row comes above 4 bits; with two
+// waters 11 bohr apart, six electrons of a spin on one of them, the rows
+// concerned stand at 8 to 20.
 
-// Pivot of column k from row k on (warp 0): row, reciprocal and, into piv[k], the
-// pivot itself.
-__device__ __forceinline__ void find_pivot(const double* M, int n, int k, double* piv, int* s_piv, double* s_pinv,
+// Pivot of column k from row k on (warp 0): row, value and reciprocal.
+__device__ __forceinline__ void find_pivot(const double* M, int n, int k, int* s_piv, double* s_val, double* s_pinv,
                                            int* s_sing) {
     const int lane = threadIdx.x & 31;
     long long best = -1;
@@ -181,16 +198,47 @@ __device__ __forceinline__ void find_pivot(const double* M, int n, int k, double
         const int e = fx_expo(v);
         *s_piv = bi;
         *s_pinv = 1.0 / v;
-        piv[k] = v;
+        *s_val = v;
         if (e == 2047 || (fx_bits(v) & 0x7fffffffffffffffLL) == 0) *s_sing = 1;
     }
 }
 
+// The orbitals of the electrons of one spin as FP64 sums, by the whole CTA; ends
+// synchronised.  sm: 5 n_basis doubles and n_shell bytes of shared memory.
+__device__ __noinline__ void orbitals_again(const DevSys& s, const DevWalkers& wk, int w, int spin, int fp32, double* sm) {
+    const int i0 = spin ? s.n_up : 0, n = spin ? s.n_dn : s.n_up;
+    unsigned char* live = reinterpret_cast<unsigned char*>(sm + 5 * s.n_basis);
+    for (int k = 0; k < n; ++k) {
+        if (fp32)
+            orbitals_sums_item<float>(s, wk, w, i0 + k, sm, live);
+        else
+            orbitals_sums_item<double>(s, wk, w, i0 + k, sm, live);
+        __syncthreads();
+    }
+}
+
+// Whether row i of A (global memory) leaves the inverse x[j] = M[j n + c] short
+// of bits if taken in fixed point (see above).
+__device__ __forceinline__ bool row_short(const double* A, const double* M, const double* __restrict__ sC, int n, int i,
+                                          int c) {
+    int am = 0, rs = -0x10000, rf = 0;   // biased exponents: max|x_j| c_j, max|A_ij| / c_j, max|x_j A_ij|
+#pragma unroll 8
+    for (int j = 0; j < n; ++j) {
+        const int ea = fx_expo(A[(size_t)i * n + j]), ex = fx_expo(M[j * n + c]), ec = fx_expo(sC[j]);
+        am = max(am, ex + ec);
+        if (ea) rs = max(rs, ea - ec);
+        if (ea && ex) rf = max(rf, ea + ex);
+    }
+    return am + rs - rf > kFxSlack;
+}
+
 // Inversion of one (walker, spin) matrix (body of k_invert).  M: n^2 + n
-// doubles of shared memory; at least n threads.
-__device__ __forceinline__ void invert_item(const DevSys& s, const DevWalkers& wk, int w, int spin, int store_fp32, unsigned* err, double* M) {
+// doubles of shared memory (invert_smem_bytes); at least n threads.  fx: A was
+// taken in fixed point.
+__device__ __forceinline__ void invert_item(const DevSys& s, const DevWalkers& wk, int w, int spin, int store_fp32, int fx,
+                                            unsigned* err, double* M) {
     __shared__ int s_perm[256];
-    __shared__ double s_pinv;
+    __shared__ double s_val, s_pinv;
     __shared__ int s_piv, s_sing, s_row[2];
     const int n = spin ? s.n_dn : s.n_up;
     if (n == 0) {
@@ -201,60 +249,80 @@ __device__ __forceinline__ void invert_item(const DevSys& s, const DevWalkers& w
         return;
     }
     double* fcol = M + n * n;
-    double* A = wk.Ascr[spin] + (size_t)w * n * n;   // its first row receives the pivots
-    for (int q = threadIdx.x; q < n * n; q += blockDim.x) M[q] = A[q];
-    if (threadIdx.x == 0) {
-        s_sing = 0;
-        s_row[0] = s_row[1] = 0;
-    }
-    __syncthreads();
+    const double* A = wk.Ascr[spin] + (size_t)w * n * n;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     // rows of an elimination step of a warp, and this lane's row and first column of them
     const int sub = n <= 8 ? 8 : n <= 16 ? 16 : 32, nrow = 32 / sub, lr = lane / sub, lc = lane % sub;
-    if (wid == 0) find_pivot(M, n, 0, A, &s_piv, &s_pinv, &s_sing);
-    __syncthreads();
-    int cur = threadIdx.x, swaps = 0;   // where this thread's column ends up; interchanges so far
-    for (int k = 0; k < n; ++k) {
-        if (s_sing) break;   // uniform: written before the last barrier
-        const int p = s_piv;
-        const double pinv = s_pinv;
-        // interchange rows k and p, scale the pivot row, keep the column
-        for (int j = threadIdx.x; j < n; j += blockDim.x) {
-            const double t = M[k * n + j], u = M[p * n + j];
-            if (p != k) M[p * n + j] = t;
-            M[k * n + j] = (j == k) ? pinv : u * pinv;
-            if (j == k) {
-                if (p != k) fcol[p] = t;
-                fcol[k] = 0.0;
-            }
-            if (j != k && j != p) fcol[j] = M[j * n + k];
+    int cur = 0, swaps = 0, neg = 0;   // where this thread's column ends up; interchanges; negative pivots
+    double piv = 0.0;                  // this thread's pivot
+    for (;;) {
+        if (threadIdx.x == 0) {
+            s_sing = 0;
+            s_row[0] = s_row[1] = 0;
         }
-        if (threadIdx.x == 0) s_row[(k + 1) & 1] = 0;
-        swaps += p != k;
-        cur = cur == k ? p : cur == p ? k : cur;
+        for (int q = threadIdx.x; q < n * n; q += blockDim.x) M[q] = A[q];
         __syncthreads();
-        const int ahead = k + 1 < n ? k + 1 : -1;   // the column that warp 0 takes
-        if (wid == 0 && ahead > 0) {
-            for (int i = lane; i < n; i += 32)
-                if (i != k) M[i * n + ahead] = M[i * n + ahead] - fcol[i] * M[k * n + ahead];
-            __syncwarp();
-            find_pivot(M, n, ahead, A, &s_piv, &s_pinv, &s_sing);
-        }
-        for (;;) {   // the other columns, rows to whichever warp is free
-            int i = 0;
-            if (lane == 0) i = atomicAdd(&s_row[k & 1], nrow);
-            i = __shfl_sync(0xffffffffu, i, 0);
-            if (i >= n) break;
-            i += lr;
-            if (i == k || i >= n) continue;
-            const double f = fcol[i];
-            for (int j = lc; j < n; j += sub) {
-                if (j == ahead) continue;
-                const double base = (j == k) ? 0.0 : M[i * n + j];
-                M[i * n + j] = base - f * M[k * n + j];
-            }
-        }
+        if (wid == 0) find_pivot(M, n, 0, &s_piv, &s_val, &s_pinv, &s_sing);
         __syncthreads();
+        cur = threadIdx.x;
+        swaps = 0;
+        for (int k = 0; k < n; ++k) {
+            if (s_sing) break;   // uniform: written before the last barrier
+            const int p = s_piv;
+            const double pinv = s_pinv;
+            if (threadIdx.x == k) piv = s_val;
+            // interchange rows k and p, scale the pivot row, keep the column
+            for (int j = threadIdx.x; j < n; j += blockDim.x) {
+                const double t = M[k * n + j], u = M[p * n + j];
+                if (p != k) M[p * n + j] = t;
+                M[k * n + j] = (j == k) ? pinv : u * pinv;
+                if (j == k) {
+                    if (p != k) fcol[p] = t;
+                    fcol[k] = 0.0;
+                }
+                if (j != k && j != p) fcol[j] = M[j * n + k];
+            }
+            if (threadIdx.x == 0) s_row[(k + 1) & 1] = 0;
+            swaps += p != k;
+            cur = cur == k ? p : cur == p ? k : cur;
+            __syncthreads();
+            const int ahead = k + 1 < n ? k + 1 : -1;   // the column that warp 0 takes
+            if (wid == 0 && ahead > 0) {
+                for (int i = lane; i < n; i += 32)
+                    if (i != k) M[i * n + ahead] = M[i * n + ahead] - fcol[i] * M[k * n + ahead];
+                __syncwarp();
+                find_pivot(M, n, ahead, &s_piv, &s_val, &s_pinv, &s_sing);
+            }
+            for (;;) {   // the other columns, rows to whichever warp is free
+                int i = 0;
+                if (lane == 0) i = atomicAdd(&s_row[k & 1], nrow);
+                i = __shfl_sync(0xffffffffu, i, 0);
+                if (i >= n) break;
+                i += lr;
+                if (i == k || i >= n) continue;
+                const double f = fcol[i];
+                for (int j = lc; j < n; j += sub) {
+                    if (j == ahead) continue;
+                    const double base = (j == k) ? 0.0 : M[i * n + j];
+                    M[i * n + j] = base - f * M[k * n + j];
+                }
+            }
+            __syncthreads();
+        }
+        neg = 0;
+        if (!s_sing)
+            for (int k = threadIdx.x; k < n; k += blockDim.x) {
+                s_perm[k] = cur;
+                neg = piv < 0.0;
+                fcol[k] = log(fabs(piv));
+            }
+        neg = __syncthreads_count(neg);
+        if (!fx) break;
+        fx = 0;
+        int again = s_sing;
+        for (int i = threadIdx.x; !again && i < n; i += blockDim.x) again = row_short(A, M, s.Ck_s[spin], n, i, s_perm[i]);
+        if (!__syncthreads_or(again)) break;
+        orbitals_again(s, wk, w, spin, store_fp32, M);
     }
     if (s_sing) {
         if (threadIdx.x == 0) {
@@ -264,14 +332,6 @@ __device__ __forceinline__ void invert_item(const DevSys& s, const DevWalkers& w
         }
         return;
     }
-    int neg = 0;
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        s_perm[k] = cur;
-        const double v = A[k];
-        neg = v < 0.0;
-        fcol[k] = log(fabs(v));
-    }
-    neg = __syncthreads_count(neg);
     // AinvT[e][j] = (A^-1)[j][e], the interchanges undone as interchanges of its columns, last first
     if (store_fp32) {
         float* out = (float*)wk.Ainv[spin] + (size_t)w * n * n;
@@ -294,11 +354,11 @@ __device__ __forceinline__ void invert_item(const DevSys& s, const DevWalkers& w
     }
 }
 
-__global__ void k_invert(DevSys s, DevWalkers wk, int W, int store_fp32, unsigned* err, const int* only) {
+__global__ void k_invert(DevSys s, DevWalkers wk, int W, int store_fp32, int fx, unsigned* err, const int* only) {
     extern __shared__ double M[];  // [n][n], then fcol[n]
     const int w = blockIdx.x, spin = blockIdx.y;
     if (w >= W || (only && !only[w])) return;
-    invert_item(s, wk, w, spin, store_fp32, err, M);
+    invert_item(s, wk, w, spin, store_fp32, fx, err, M);
 }
 
 // Local energy, ln|psi| and (optionally) grad / Laplacian of ln|psi| from
@@ -798,15 +858,22 @@ __global__ void k_weighted_sum(const double* x, const double* g, int W, int K, d
 }
 
 size_t orbitals_smem_bytes(const DevSys& s) {
-    const size_t b = Basis64Layout(s.n_nuc, s.n_prim, s.n_shell, s.n_basis).total;
-    return b <= kBasis64Max ? b : sizeof(double) * 5 * (size_t)s.n_basis;
+    return orbitals_fx(s) ? Basis64Layout(s.n_nuc, s.n_prim, s.n_shell, s.n_basis).total
+                          : sizeof(double) * 5 * (size_t)s.n_basis;
+}
+
+// The matrix and its column; with fx also the basis at a point (orbitals_again).
+size_t invert_smem_bytes(const DevSys& s, bool fx) {
+    const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
+    const size_t m = sizeof(double) * ((size_t)nmax * nmax + nmax + 1);
+    return fx && orbitals_fx(s) ? std::max(m, sizeof(double) * 5 * (size_t)s.n_basis + s.n_shell) : m;
 }
 
 template <typename T>
 cudaError_t launch_orbitals_all(const DevSys& s, const DevWalkers& wk, int W, cudaStream_t st, const int* only,
                                 bool sums) {
     if (W == 0 || s.N == 0) return cudaSuccess;
-    if (sums || Basis64Layout(s.n_nuc, s.n_prim, s.n_shell, s.n_basis).total > kBasis64Max) {
+    if (sums || !orbitals_fx(s)) {
         const size_t smem = sizeof(double) * 5 * s.n_basis + (size_t)s.n_shell;
         if (smem > 48 * 1024) {
             cudaError_t e = cudaFuncSetAttribute(k_orbitals_sums<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -831,15 +898,15 @@ cudaError_t launch_orbitals_all(const DevSys& s, const DevWalkers& wk, int W, cu
     return cudaGetLastError();
 }
 
-cudaError_t launch_invert(const DevSys& s, const DevWalkers& wk, int W, int store_fp32, unsigned* err,
+cudaError_t launch_invert(const DevSys& s, const DevWalkers& wk, int W, int store_fp32, bool sums, unsigned* err,
                           cudaStream_t st, const int* only) {
     if (W == 0) return cudaSuccess;
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
-    const size_t smem = sizeof(double) * ((size_t)nmax * nmax + nmax + 1);
+    const size_t smem = invert_smem_bytes(s, !sums);
     cudaError_t e = cudaFuncSetAttribute(k_invert, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int nt = nmax > 64 ? 512 : (nmax > 16 ? 256 : 128);
-    k_invert<<<dim3(W, 2), nt, smem, st>>>(s, wk, W, store_fp32, err, only);
+    k_invert<<<dim3(W, 2), nt, smem, st>>>(s, wk, W, store_fp32, !sums && orbitals_fx(s), err, only);
     return cudaGetLastError();
 }
 
@@ -897,7 +964,7 @@ __global__ void k_invert_batch(const BatchSys* __restrict__ sys, BatchPlan* plan
         if (q < 0) break;
         batch_load(&bs, sys + q);
         __syncthreads();
-        invert_item(bs.s, bs.wk[parity], s_idx >> 1, s_idx & 1, store_fp32, bs.err, M);
+        invert_item(bs.s, bs.wk[parity], s_idx >> 1, s_idx & 1, store_fp32, orbitals_fx(bs.s), bs.err, M);
         __syncthreads();
     }
 }

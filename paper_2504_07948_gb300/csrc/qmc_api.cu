@@ -887,7 +887,7 @@ struct qmc_ctx {
         } else {
             QMC_CK(launch_orbitals_all<double>(ds, k, W, stream));
         }
-        QMC_CK(launch_invert(ds, k, W, mode == QMC_MIXED, d_err, stream));
+        QMC_CK(launch_invert(ds, k, W, mode == QMC_MIXED, mode == QMC_MIXED && fresh, d_err, stream));
         int nk = 2;
         if (ds.msd) {
             if (mode == QMC_MIXED) {
@@ -1167,7 +1167,7 @@ struct qmc_ctx {
             } else {
                 QMC_CK(launch_orbitals_all<double>(ds, k, W, stream, d_refresh));
             }
-            QMC_CK(launch_invert(ds, k, W, mode == QMC_MIXED, d_err, stream, d_refresh));
+            QMC_CK(launch_invert(ds, k, W, mode == QMC_MIXED, mode == QMC_MIXED, d_err, stream, d_refresh));
             if (mode == QMC_MIXED) {
                 QMC_CK(launch_msd_table<float>(ds, k, W, stream, d_refresh));
             } else {
@@ -2546,9 +2546,8 @@ struct qmc_batch {
         force_warps = 8;
         for (int q = 0; q < n; ++q) {
             const DevSys& s = sys[q]->ds;
-            const int nmax = std::max(s.n_up, s.n_dn);
             orb = std::max(orb, orbitals_smem_bytes(s));
-            inv = std::max(inv, sizeof(double) * ((size_t)nmax * nmax + nmax + 1));
+            inv = std::max(inv, invert_smem_bytes(s, true));
             el = std::max(el, eloc_smem_bytes(s, 128, elem()));
             force_warps = std::max(force_warps, force_batch_warps(s, elem(), warp[q]));
         }

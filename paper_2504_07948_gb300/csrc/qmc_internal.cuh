@@ -1371,13 +1371,15 @@ struct SweepParams {
 };
 
 size_t orbitals_smem_bytes(const DevSys& s);
+size_t invert_smem_bytes(const DevSys& s, bool fx);
 size_t eloc_smem_bytes(const DevSys& s, int nt, int elem);
 template <typename T>
 cudaError_t launch_orbitals_all(const DevSys& s, const DevWalkers& wk, int W, cudaStream_t st,
                                 const int* only = nullptr, bool sums = false);
 // only (optional, [W]): rebuild just the walkers whose flag is nonzero.
 // launch_orbitals_all, sums: FP64 sums in index order (see k_orbitals_sums).
-cudaError_t launch_invert(const DevSys& s, const DevWalkers& wk, int W, int store_fp32, unsigned* err,
+// (launch_invert: the orbitals came from it)
+cudaError_t launch_invert(const DevSys& s, const DevWalkers& wk, int W, int store_fp32, bool sums, unsigned* err,
                           cudaStream_t st, const int* only = nullptr);
 // Jastrow parameter derivatives (k_wavefunction.cu): for P = 4 + n_nuc +
 // n_nuc n3 parameters (a_anti, a_par, b_ee, b_en, a_en[], c3[][]),
