@@ -91,7 +91,8 @@ __device__ __forceinline__ void basis64(const DevSys& s, const Basis64Layout& L,
     int* rows = (int*)(sm + L.rows);
     int* cnt = (int*)(sm + L.cnt);       // [0] primitives, [1] shells, [2..4] functions by kind, [5], [6] rows,
                                          // [8..12] exponents,
-                                         // [16..20], [24..28] exponents of the sums (orbitals64)
+                                         // [16..20], [24..28] exponents of the sums (orbitals64),
+                                         // [29], [30] of the ratio's factors and terms (sweep64.cuh)
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, ldb = L.ldb;
     const unsigned below = (1u << lane) - 1u;
     for (int q = tid; q < 32; q += nt) cnt[q] = 0;
@@ -349,9 +350,9 @@ __device__ __noinline__ void orbitals_plain(const DevSys& s, const double r[3], 
 
 // Basis and orbitals at (r0, r1, r2) of one or two (C2, n2 > 0) coefficient
 // blocks, all threads; ends synchronised.  The first block's nuclear offsets
-// stay in nuc (basis64).
+// stay in nuc (basis64).  Returns whether the orbitals are FP64 sums (uniform).
 template <typename Put, typename Put2>
-__device__ __forceinline__ void orbitals64(const DevSys& s, const Basis64Layout& L, unsigned char* sm, double r0,
+__device__ __forceinline__ bool orbitals64(const DevSys& s, const Basis64Layout& L, unsigned char* sm, double r0,
                                            double r1, double r2, const int2* Ck, const double* sC, const double* C,
                                            int n, Put put, const int2* Ck2, const double* sC2, const double* C2, int n2,
                                            Put2 put2) {
@@ -369,11 +370,13 @@ __device__ __forceinline__ void orbitals64(const DevSys& s, const Basis64Layout&
         low |= cnt[16 + c] < 1079 - 4;
         low2 |= cnt[24 + c] < 1079 - 4;
     }
-    if (low || (low2 && n2 > 0)) {
+    low |= low2 && n2 > 0;
+    if (low) {
         const double r[3] = {r0, r1, r2};
         orbitals_plain(s, r, C, n, (double*)(sm + L.bas), put);
         if (n2 > 0) orbitals_plain(s, r, C2, n2, (double*)(sm + L.bas), put2);
     }
+    return low;
 }
 
 }  // namespace qmc

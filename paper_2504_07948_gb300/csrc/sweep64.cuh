@@ -15,6 +15,10 @@
 //   - pair terms and determinant terms sum in separate warps (a butterfly over
 //     four values), reciprocals of values >= 1 by one refinement step.
 //   - a move's serial part runs on three lanes, one component each.
+// The fixed-point orbitals of a proposal are held against the column of the
+// inverse that they meet, as those of a rebuild are (kFxSlack, k_wavefunction.cu):
+// where the column weighs small orbitals up, the move's orbitals are taken
+// again as FP64 sums.
 // 6-water cluster, 2048 walkers: 9.9 -> 5.8 ms a sweep (1345 -> about 600 FP64
 // warp instructions a move); one water, 512 walkers: 283 -> 180 us.
 #pragma once
@@ -138,6 +142,7 @@ __device__ __forceinline__ void sweep_walker64(const DevSys& s, const DevWalkers
     double* fq = cold + nmax;
     const double4* nuc = (const double4*)(smem + LB.nuc);
     unsigned char* sb = smem + L.basis;
+    int* cnt = (int*)(sb + LB.cnt);
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
 
     double* gA[2] = {(double*)wk.Ainv[0] + (size_t)w * nu * nu, (double*)wk.Ainv[1] + (size_t)w * nd * nd};
@@ -238,20 +243,13 @@ __device__ __forceinline__ void sweep_walker64(const DevSys& s, const DevWalkers
         const double rn0 = scal[0], rn1 = scal[1], rn2 = scal[2];
 
         // -- basis and orbitals at the proposed position ---------------------
-        orbitals64(s, LB, sb, rn0, rn1, rn2, s.Ck[spin], s.Ck_s[spin], s.C[spin], n,
-                   [phi, nmax](int c, int j, double x) { phi[c * nmax + j] = x; }, nullptr, nullptr, nullptr, 0,
-                   [](int, int, double) {});
+        const auto put = [phi, nmax](int c, int j, double x) { phi[c * nmax + j] = x; };
+        bool plain = orbitals64(s, LB, sb, rn0, rn1, rn2, s.Ck[spin], s.Ck_s[spin], s.C[spin], n, put, nullptr, nullptr,
+                                nullptr, 0, [](int, int, double) {});
 
         // -- ratio, new determinant gradient, Jastrow change ----------------
 #pragma unroll
-        for (int c = 0; c < 4; ++c) v[c] = d[c] = 0.0;
-        for (int j = nt - 1 - tid; j < n; j += nt) {
-            const double a = Ae[j];
-            d[0] += phi[j] * a;
-            d[1] += phi[nmax + j] * a;
-            d[2] += phi[2 * nmax + j] * a;
-            d[3] += phi[3 * nmax + j] * a;
-        }
+        for (int c = 0; c < 4; ++c) v[c] = 0.0;
         for (int q = tid; q < N + nn; q += nt) {
             if (q == e) continue;
             double x, y, z, r2;
@@ -280,7 +278,34 @@ __device__ __forceinline__ void sweep_walker64(const DevSys& s, const DevWalkers
                 v[3] += gg[2];
             }
         }
-        t = sweep64_sum(v, d, pw, dw, red);
+        for (;; plain = true) {
+            int fac = 0, term = 0;   // exponents: max|x_j| c_j, max|x_j phi_j|
+#pragma unroll
+            for (int c = 0; c < 4; ++c) d[c] = 0.0;
+            for (int j = nt - 1 - tid; j < n; j += nt) {
+                const double a = Ae[j], f = phi[j];
+                d[0] += f * a;
+                d[1] += phi[nmax + j] * a;
+                d[2] += phi[2 * nmax + j] * a;
+                d[3] += phi[3 * nmax + j] * a;
+                const int ea = fx_expo(a), ef = fx_expo(f);
+                fac = max(fac, ea + fx_expo(s.Ck_s[spin][j]));
+                if (ef) term = max(term, ea + ef);
+            }
+            if (dw && !plain) {
+                fac = warp_max_u(fac);
+                term = warp_max_u(term);
+                if (lane == 0) {
+                    atomicMax(&cnt[29], fac);
+                    atomicMax(&cnt[30], term);
+                }
+            }
+            t = sweep64_sum(v, d, pw, dw, red);
+            // (an orbital's scale is 2^-27 of its largest coefficient's power of two)
+            if (plain || cnt[29] + 27 + cnt[8] - 1023 - cnt[30] <= kFxSlack) break;
+            const double r[3] = {rn0, rn1, rn2};
+            orbitals_plain(s, r, s.C[spin], n, (double*)(sb + LB.bas), put);
+        }
         if (wid == 0) {
             const double rho = __shfl_sync(0xffffffffu, t, 4);
             int accept = 0;

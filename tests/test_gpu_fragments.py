@@ -56,3 +56,20 @@ def test_rebuild(m, D):
     for k in ("logpsi", "eloc", "grad"):
         close(ev[k], ref[k], 1e-10)
     assert np.array_equal(ev["sign"], ref["sign"])
+
+
+@pytest.mark.parametrize("m,D", CASES)
+def test_sweeps(m, D):
+    """Two sweeps: the oracle's moves, and a propagated state that its evaluation confirms."""
+    from paper_2504_07948_gb300 import qmc as Q
+    s, R = fragments(m, D), walkers(m, D, 16)
+    g = Q.QMC(s, precision="fp64", seed=5)
+    g.set_walkers(R)
+    g.vmc(2, 0.02)
+    Rg, ev = g.get_walkers()[0], g.eval_cached()
+    g.close()
+    Ro, _, _ = O.Oracle(s).vmc(R, 2, 0.02, seed=5, step0=0, trace=False)
+    assert np.abs(Rg - Ro).max() <= 1e-8
+    ref = O.Oracle(s).evaluate(Rg)
+    for k in ("logpsi", "eloc", "grad"):
+        close(ev[k], ref[k], 1e-8)
