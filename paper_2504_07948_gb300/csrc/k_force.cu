@@ -443,6 +443,21 @@ __device__ __forceinline__ double warp_limbs(const double* x, int2* q, int n) {
     return fx_scale(e);
 }
 
+// Whether the fixed-point products of an electron's row a of A^-T would lose
+// bits against FP64 sums: the largest entries of it and of the electron's row b of
+// B, in units of the orbitals' largest coefficients, against the largest product
+// a_q b_q.  row_range takes a lane's entries (a times, b over the orbital's scale
+// c) into its exponents ea, eb, eab.
+__device__ __forceinline__ void row_range(double a, double b, double c, int& ea, int& eb, int& eab) {
+    const int ec = fx_expo(c), x = fx_expo(a) ? fx_expo(a) + ec : 0, y = fx_expo(b) ? fx_expo(b) - ec + 2046 : 0;
+    ea = max(ea, x);
+    eb = max(eb, y);
+    if (x && y) eab = max(eab, x + y);
+}
+__device__ __forceinline__ bool row_short(int ea, int eb, int eab) {
+    return warp_max_u(ea) + warp_max_u(eb) - warp_max_u(eab) > kFxSlack;
+}
+
 // Reciprocal of a scale (a power of two from fx_scale; NaN and 0 to NaN).
 __device__ __forceinline__ double fx_inverse(double scale) {
     const int e = fx_expo(scale);
@@ -479,6 +494,9 @@ __host__ __device__ inline int force_row_groups(int n) {
 // enough for the warps (a batch of 16 clusters of up to 130 electrons, 64 walkers
 // each: 5.2 -> 4.4 ms; sixteen warps with the smallest tiles 6.0, eight with
 // large ones 4.8).
+// FP64 form: a spin in which some electron's row of A^-T weighs small entries
+// of B up (row_short; electrons shared out unevenly over distant fragments with
+// orbitals of their own) is taken as a determinant too large to stage is, in FP64 sums.
 constexpr size_t kForceTwo = 113 * 1024;
 template <typename T>
 struct ForceShape {
@@ -581,20 +599,26 @@ __device__ __forceinline__ void force_walker(const DevSys& s, const DevWalkers& 
             if (nlB) b += nlB[(size_t)pp * n + qq];
             return b;
         };
-        if (fs.stg) {
+        bool stg = fs.stg;
+        if (stg) {
+            int lossy = 0;
             for (int r = wid; r < n; r += nw) {
                 T* at = (T*)(sAT + (size_t)r * ld);
                 T* bt = (T*)(sB + (size_t)r * ld);
+                int ea = 0, eb = 0, eab = 0;
                 for (int q = lane; q < n; q += 32) {
                     T a = ATg[(size_t)r * n + q], b = b_of(r, q);
                     if constexpr (kFx) {   // orbital q in units of its largest coefficient
-                        a *= s.Ck_s[spin][q];
-                        b *= fx_inverse(s.Ck_s[spin][q]);
+                        const double c = s.Ck_s[spin][q];
+                        row_range(a, b, c, ea, eb, eab);
+                        a *= c;
+                        b *= fx_inverse(c);
                     }
                     at[q] = a;
                     bt[q] = b;
                 }
                 if constexpr (kFx) {
+                    lossy |= row_short(ea, eb, eab);
                     const double a = warp_limbs(at, (int2*)at, n), b = warp_limbs(bt, (int2*)bt, n);
                     if (lane == 0) {
                         sA[r] = a;
@@ -602,7 +626,9 @@ __device__ __forceinline__ void force_walker(const DevSys& s, const DevWalkers& 
                     }
                 }
             }
-            __syncthreads();
+            stg = !__syncthreads_or(lossy);
+        }
+        if (stg) {
             // PT[i][p] = (B A^-1)_{p i} = sum_q AT[i][q] B_pq
             const int rows = kForceRows * force_row_groups(n);
             for (int r0 = wid * rows; r0 < n; r0 += nw * rows) {
@@ -641,7 +667,7 @@ __device__ __forceinline__ void force_walker(const DevSys& s, const DevWalkers& 
             while (sh1 < s.n_shell && s.shell_fn[sh1 + 1] - fl0 <= fs.F) ++sh1;
             const int nfl = s.shell_fn[sh1] - fl0;
             // M[l][i] = sum_j C[l][j] AT[i][j],  Y[l][i] = sum_p M[l][p] PT[i][p]
-            if (fs.stg) {
+            if (stg) {
                 const int rows = kForceRows * force_row_groups(n);
                 for (int r0 = wid * rows; r0 < nfl; r0 += nw * rows) {
                     const int nl = min(rows, nfl - r0), l0 = fl0 + r0;
@@ -739,11 +765,11 @@ __device__ __forceinline__ void force_walker(const DevSys& s, const DevWalkers& 
 // form keeps two (at three it spills).
 template <typename T, bool kE, int kNt>
 __global__ void __launch_bounds__(kNt, kNt == 512 ? 1 : sizeof(T) == 4 ? 3 : 2)
-    k_force(DevSys s, DevWalkers wk, int W, const double* dvnn, double* Bscr, double* Pscr, double* dEL, double* dlog,
-            double* gEdet, double* gtot) {
+    k_force(DevSys s, DevWalkers wk, int w0, int W, const int* only, const double* dvnn, double* Bscr, double* Pscr,
+            double* dEL, double* dlog, double* gEdet, double* gtot) {
     extern __shared__ double sm[];
-    const int w = blockIdx.x;
-    if (w >= W) return;
+    if ((int)blockIdx.x >= W || (only && !only[blockIdx.x])) return;
+    const int w = w0 + blockIdx.x;
     force_walker<T, kE>(s, wk, w, dvnn, Bscr, Pscr, dEL, dlog, sm, gEdet, gtot);
 }
 
@@ -762,9 +788,11 @@ __global__ void __launch_bounds__(kNt, kNt == 512 ? 1 : sizeof(T) == 4 ? 3 : 2)
 // its electron's row of B as soon as that electron's grad J is summed, so the
 // gradient cache is read from memory once (32-water cluster, 512 walkers, mixed:
 // 495 -> 398 us).
+// lossy (FP64 form): [W], whether some electron's row of A^-T weighs small entries
+// of B up (row_short): the walker's products are not left to bf16 digits then.
 template <typename T, bool kE>
 __global__ void k_force_prep(DevSys s, DevWalkers wk, int w0, int W, const double* dvnn, T* Bw, double* gJw,
-                             double* accw, double* gtot) {
+                             double* accw, double* gtot, int* lossy) {
     extern __shared__ double sm[];
     const int wl = blockIdx.x, w = w0 + wl;
     if (wl >= W) return;
@@ -774,17 +802,26 @@ __global__ void k_force_prep(DevSys s, DevWalkers wk, int w0, int W, const doubl
     force_load_positions(h, wk.R + (size_t)w * 3 * N, N);
     __syncthreads();
     const int lane = threadIdx.x & 31;
+    int low = 0;
     force_gradients_en<T>(s, wk, w, dvnn, h, [&](int spin, int k, const T* g, const T* G) {
         const int n = spin ? s.n_dn : nu;
         T* B = Bw + ((size_t)(spin * W + wl)) * nmax * nmax + (size_t)k * n;
         const T* nlB = (const T*)wk.nlB[spin];
         if (nlB) nlB += (size_t)w * n * n + (size_t)k * n;
+        const T* Ai = (const T*)wk.Ainv[spin] + ((size_t)w * n + k) * n;
+        int ea = 0, eb = 0, eab = 0;
         for (int q = lane; q < n; q += 32) {
             T b = T(-0.5) * G[3 * n + q] - g[0] * G[q] - g[1] * G[n + q] - g[2] * G[2 * n + q];
             if (nlB) b += nlB[q];   // non-local pseudopotential rows
             B[q] = b;
+            if constexpr (sizeof(T) == 8) row_range(Ai[q], b, s.Ck_s[spin][q], ea, eb, eab);
         }
+        if constexpr (sizeof(T) == 8) low |= row_short(ea, eb, eab);
     });
+    if constexpr (sizeof(T) == 8) {
+        low = __syncthreads_or(low);
+        if (threadIdx.x == 0) lossy[wl] = low;
+    }
     for (int q = threadIdx.x; q < 3 * N; q += blockDim.x) gJw[(size_t)wl * 3 * N + q] = double(h.gJ[q]);
     for (int q = threadIdx.x; q < 6 * nn; q += blockDim.x) accw[(size_t)wl * 6 * nn + q] = h.acc[q];
     if constexpr (kE)
@@ -899,7 +936,7 @@ __global__ void __launch_bounds__(256) k_force_contract(DevSys s, DevWalkers wk,
 // gtot (may be null): grad_i ln|psi| [W][N][3] of the space-warp form.
 template <typename T>
 cudaError_t launch_force_prep(const DevSys& s, const DevWalkers& wk, int w0, int W, const double* dvnn, void* Bw,
-                              double* gJw, double* accw, double* gtot, cudaStream_t st) {
+                              double* gJw, double* accw, double* gtot, int* lossy, cudaStream_t st) {
     if (W == 0) return cudaSuccess;
     const size_t smem = force_head_bytes<T>(s.N, s.n_nuc);
     if (gtot) {
@@ -908,7 +945,7 @@ cudaError_t launch_force_prep(const DevSys& s, const DevWalkers& wk, int w0, int
                 cudaFuncSetAttribute(k_force_prep<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        k_force_prep<T, true><<<W, 256, smem, st>>>(s, wk, w0, W, dvnn, (T*)Bw, gJw, accw, gtot);
+        k_force_prep<T, true><<<W, 256, smem, st>>>(s, wk, w0, W, dvnn, (T*)Bw, gJw, accw, gtot, lossy);
         return cudaGetLastError();
     }
     if (smem > 48 * 1024) {
@@ -916,7 +953,7 @@ cudaError_t launch_force_prep(const DevSys& s, const DevWalkers& wk, int w0, int
             cudaFuncSetAttribute(k_force_prep<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    k_force_prep<T, false><<<W, 256, smem, st>>>(s, wk, w0, W, dvnn, (T*)Bw, gJw, accw, nullptr);
+    k_force_prep<T, false><<<W, 256, smem, st>>>(s, wk, w0, W, dvnn, (T*)Bw, gJw, accw, nullptr, lossy);
     return cudaGetLastError();
 }
 
@@ -959,9 +996,9 @@ cudaError_t launch_force_contract(const DevSys& s, const DevWalkers& wk, int w0,
 }
 
 template cudaError_t launch_force_prep<double>(const DevSys&, const DevWalkers&, int, int, const double*, void*,
-                                               double*, double*, double*, cudaStream_t);
+                                               double*, double*, double*, int*, cudaStream_t);
 template cudaError_t launch_force_prep<float>(const DevSys&, const DevWalkers&, int, int, const double*, void*,
-                                              double*, double*, double*, cudaStream_t);
+                                              double*, double*, double*, int*, cudaStream_t);
 template cudaError_t launch_force_contract<double>(const DevSys&, const DevWalkers&, int, int, const void*,
                                                    const void*, const double*, const double*, double*, double*,
                                                    double*, cudaStream_t);
@@ -969,11 +1006,12 @@ template cudaError_t launch_force_contract<float>(const DevSys&, const DevWalker
                                                   const double*, const double*, double*, double*, double*,
                                                   cudaStream_t);
 
-// gEdet, gtot (both null, or both [W][N][3]): the space-warp form's
+// Walkers w0 .. w0 + W - 1, with only ([W]) those whose flag is set.
+// gEdet, gtot (both null, or both [.][N][3]): the space-warp form's
 // per-electron outputs (see force_walker).
 template <typename T>
-cudaError_t launch_force(const DevSys& s, const DevWalkers& wk, int W, const double* dvnn, double* Bscr,
-                         double* Pscr, double* dEL, double* dlog, double* gEdet, double* gtot, cudaStream_t st) {
+cudaError_t launch_force(const DevSys& s, const DevWalkers& wk, int w0, int W, const int* only, const double* dvnn,
+                         double* Bscr, double* Pscr, double* dEL, double* dlog, double* gEdet, double* gtot, cudaStream_t st) {
     if (W == 0) return cudaSuccess;
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
     const bool kE = gEdet != nullptr;
@@ -983,7 +1021,7 @@ cudaError_t launch_force(const DevSys& s, const DevWalkers& wk, int W, const dou
                             : (kE ? k_force<T, true, 256> : k_force<T, false, 256>);
     cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    f<<<W, 32 * nw, smem, st>>>(s, wk, W, dvnn, Bscr, Pscr, dEL, dlog, gEdet, kE ? gtot : nullptr);
+    f<<<W, 32 * nw, smem, st>>>(s, wk, w0, W, only, dvnn, Bscr, Pscr, dEL, dlog, gEdet, kE ? gtot : nullptr);
     return cudaGetLastError();
 }
 
@@ -1280,9 +1318,9 @@ template cudaError_t launch_force_batch<double>(const BatchSys*, BatchPlan*, int
 template cudaError_t launch_force_batch<float>(const BatchSys*, BatchPlan*, int, int, int, size_t, int, int,
                                                cudaStream_t);
 
-template cudaError_t launch_force<double>(const DevSys&, const DevWalkers&, int, const double*, double*, double*,
+template cudaError_t launch_force<double>(const DevSys&, const DevWalkers&, int, int, const int*, const double*, double*, double*,
                                           double*, double*, double*, double*, cudaStream_t);
-template cudaError_t launch_force<float>(const DevSys&, const DevWalkers&, int, const double*, double*, double*,
+template cudaError_t launch_force<float>(const DevSys&, const DevWalkers&, int, int, const int*, const double*, double*, double*,
                                          double*, double*, double*, double*, cudaStream_t);
 
 }  // namespace qmc

@@ -321,6 +321,7 @@ struct qmc_ctx {
     int fchunk = 0;
     void *d_fB = nullptr, *d_fPT = nullptr, *d_fQ = nullptr, *d_fM = nullptr, *d_fY = nullptr;
     double *d_fgJ = nullptr, *d_faccw = nullptr;
+    int* d_flossy = nullptr;
     // digits of the FP64 GEMM force path (k_gemm64.cu) for a chunk of walkers:
     // A^-T over Q, B, A^-1, P^T; and of C per spin (with the system)
     Gemm64Operand g64[4] = {}, g64C[2] = {};
@@ -1257,6 +1258,7 @@ struct qmc_ctx {
             d_fY = dalloc<T>(wk_allocs, 2 * (size_t)fchunk * nb * nmax);
             d_fgJ = dalloc<double>(wk_allocs, (size_t)fchunk * N3);
             d_faccw = dalloc<double>(wk_allocs, (size_t)fchunk * 6 * nn);
+            d_flossy = dalloc<int>(wk_allocs, fchunk);
             if (kFp64) {
                 // rows the tiles read: 128 of a left operand, 64 of a right one
                 const int n8 = (nmax + 7) / 8 * 8, rl = (nmax + 127) / 128 * 128, rr = (nmax + 63) / 64 * 64;
@@ -1283,7 +1285,7 @@ struct qmc_ctx {
         const DevWalkers& k = kw;
         for (int w0 = 0; w0 < W; w0 += Wc) {
             const int wc = std::min(Wc, W - w0);
-            QMC_CK(launch_force_prep<T>(ds, k, w0, wc, d_dvnn, d_fB, d_fgJ, d_faccw, d_gtot, stream));
+            QMC_CK(launch_force_prep<T>(ds, k, w0, wc, d_dvnn, d_fB, d_fgJ, d_faccw, d_gtot, d_flossy, stream));
             for (int spin = 0; spin < 2; ++spin) {
                 const int n = spin ? n_dn : n_up;
                 if (n == 0) continue;
@@ -1337,6 +1339,10 @@ struct qmc_ctx {
             }
             QMC_CK(launch_force_contract<T>(ds, k, w0, wc, d_fM, d_fY, d_fgJ, d_faccw, d_dEL, d_dlog, d_gEdet,
                                             stream));
+            // walkers that fixed-point products would cost bits
+            if (kFp64)
+                QMC_CK(launch_force<T>(ds, k, w0, wc, d_flossy, d_dvnn, d_Bscr, d_Pscr, d_dEL, d_dlog, d_gEdet, d_gtot,
+                                       stream));
         }
     }
 
@@ -1398,9 +1404,9 @@ struct qmc_ctx {
         } else {
             tm.begin(stream);
             if (mode == QMC_MIXED) {
-                QMC_CK(launch_force<float>(ds, k, W, d_dvnn, d_Bscr, d_Pscr, d_dEL, d_dlog, gE, gt, stream));
+                QMC_CK(launch_force<float>(ds, k, 0, W, nullptr, d_dvnn, d_Bscr, d_Pscr, d_dEL, d_dlog, gE, gt, stream));
             } else {
-                QMC_CK(launch_force<double>(ds, k, W, d_dvnn, d_Bscr, d_Pscr, d_dEL, d_dlog, gE, gt, stream));
+                QMC_CK(launch_force<double>(ds, k, 0, W, nullptr, d_dvnn, d_Bscr, d_Pscr, d_dEL, d_dlog, gE, gt, stream));
             }
             tm.end(F_FORCE, 1, stream);
         }

@@ -73,3 +73,17 @@ def test_sweeps(m, D):
     ref = O.Oracle(s).evaluate(Rg)
     for k in ("logpsi", "eloc", "grad"):
         close(ev[k], ref[k], 1e-8)
+
+
+@pytest.mark.parametrize("path", ["fused", "gemm"])
+@pytest.mark.parametrize("m,D", CASES)
+def test_forces(m, D, path, monkeypatch):
+    from paper_2504_07948_gb300 import qmc as Q
+    monkeypatch.setenv("QMC_FORCE_GEMM_MIN_N", "1" if path == "gemm" else "1000")
+    s, R = fragments(m, D), walkers(m, D, 16)
+    g = Q.QMC(s, precision="fp64")
+    g.set_walkers(R)
+    pw = g.forces()[1]
+    g.close()
+    for c, ref in enumerate(O.Oracle(s).forces(R)):   # E_L, ln|psi|
+        close(pw[:, c], ref, 1e-10)
