@@ -302,7 +302,7 @@ __device__ __forceinline__ void force_gradients_en(const DevSys& s, const DevWal
             }
             const T r2 = x[0] * x[0] + x[1] * x[1] + x[2] * x[2];
             const T ir = rsqrt_t(r2);
-            const T qd = rcp_ge1(T(1) + b * r2 * ir);
+            const T qd = T(1) / (T(1) + b * r2 * ir);
             const T gr = a * qd * qd * ir;  // u'(r) / r
 #pragma unroll
             for (int c = 0; c < 3; ++c) v[3 + c] += gr * x[c];

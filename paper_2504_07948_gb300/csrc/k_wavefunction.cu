@@ -528,7 +528,7 @@ __device__ __forceinline__ void eloc_walker(const DevSys& s, const DevWalkers& w
                 z = sR[3 * i + 2] - sR[3 * j + 2];
                 const double r2 = x * x + y * y + z * z;
                 ir = rsqrt(r2);
-                const double r = r2 * ir, q = rcp_ge1(1.0 + b * r);
+                const double r = r2 * ir, q = 1.0 / (1.0 + b * r);
                 const double aq = (((i < nu) == (j < nu)) ? s.a_par : s.a_anti) * q, du = aq * q;
                 u = aq * r;
                 g = du * ir;
@@ -648,7 +648,7 @@ __device__ __forceinline__ void eloc_walker(const DevSys& s, const DevWalkers& w
                     const double x = xi - s.Rn[3 * a], y = yi - s.Rn[3 * a + 1], z = zi - s.Rn[3 * a + 2];
                     const double r2 = x * x + y * y + z * z;
                     const double ir = rsqrt(r2), r = r2 * ir;
-                    const double q = rcp_ge1(1.0 + b * r);
+                    const double q = 1.0 / (1.0 + b * r);
                     const double aq = s.a_en[a] * q, du = aq * q, g = du * ir;
                     gx += g * x;
                     gy += g * y;

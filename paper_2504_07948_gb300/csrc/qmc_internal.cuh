@@ -208,18 +208,6 @@ __device__ __forceinline__ float rsqrt_t(float v) { return rsqrtf(v); }
 __device__ __forceinline__ void hold(float& v) { asm("" : "+f"(v)); }
 __device__ __forceinline__ void hold(double&) {}
 
-// Reciprocal of a value known to be finite and at least 1: the FP64 form
-// refines the hardware's 20-bit approximation y by 1/x = y (1 + e + e^2 +
-// ...), e = 1 - x y, to the last bit or two (3 FP64 instructions instead of a
-// division's 7).
-__device__ __forceinline__ double rcp_ge1(double x) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
-__device__ __forceinline__ float rcp_ge1(float x) { return 1.0f / x; }
-
 // Proposal normals in the precision of the form: FP64 (the stream both the
 // FP64 form and the oracle use) or FP32 Box-Muller from the same words.
 template <typename T>

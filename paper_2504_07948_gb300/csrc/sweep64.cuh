@@ -13,7 +13,7 @@
 //     the determinant's logarithm is taken of the product of the accepted
 //     ratios, once per sweep;
 //   - pair terms and determinant terms sum in separate warps (a butterfly over
-//     four values), reciprocals of values >= 1 by one refinement step.
+//     four values);
 //   - a move's serial part runs on three lanes, one component each.
 // The fixed-point orbitals of a proposal are held against the column of the
 // inverse that they meet, as those of a rebuild are (kFxSlack, k_wavefunction.cu):
@@ -70,30 +70,9 @@ __device__ __forceinline__ double warp_fold4(const double (&v)[4]) {
     return r;
 }
 
-// Square root of a value known to be finite and at least 1: x y with y =
-// x^-1/2 refined from the hardware's 20-bit approximation by the series
-// y (1 + e/2 + 3 e^2/8), e = 1 - x y^2.
-__device__ __forceinline__ double sqrt_ge1(double x) {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double t = x * y;
-    const double e = fma(-t, y, 1.0);
-    return fma(t, e * fma(e, 0.375, 0.5), t);
-}
-
 // Factor of the capped drift, 2 / (1 + sqrt(1 + 2 v^2 tau)).
 __device__ __forceinline__ double drift_factor(double v2, double tau) {
-    const double a = fma(2.0 * v2, tau, 1.0);
-    if (!(a < 1e300)) return 2.0 / (1.0 + sqrt(a));   // infinite or undefined gradients
-    return 2.0 * rcp_ge1(1.0 + sqrt_ge1(a));
-}
-
-// Reciprocal of a finite positive value: one refinement of the hardware's
-// approximation (see rcp_ge1) where neither it nor the error term leaves the
-// normal range, else a division.
-__device__ __forceinline__ double rcp_pos(double x) {
-    const int e = fx_expo(x);
-    return e > 64 && e < 1983 ? rcp_ge1(x) : 1.0 / x;
+    return 2.0 / (1.0 + sqrt(fma(2.0 * v2, tau, 1.0)));
 }
 
 // Sums over the CTA of the pair terms v (from the low threads up) and the
@@ -203,7 +182,7 @@ __device__ __forceinline__ void sweep_walker64(const DevSys& s, const DevWalkers
             d[3] += Ge[2 * n + j] * a;
         }
         auto pair = [&](double x, double y, double z, double r2, double a, double b) {
-            const double ir = rsqrt(r2), q = rcp_ge1(1.0 + b * (r2 * ir));
+            const double ir = rsqrt(r2), q = 1.0 / (1.0 + b * (r2 * ir));
             const double aq = a * q, g = aq * (q * ir);   // u'(r) / r, its two products side by side
             v[0] += aq * (r2 * ir);
             v[1] += g * x;
@@ -311,7 +290,7 @@ __device__ __forceinline__ void sweep_walker64(const DevSys& s, const DevWalkers
             int accept = 0;
             double ir = 0.0;
             if (rho > 0.0 && isfinite(rho)) {   // uniform in the warp
-                ir = rcp_pos(rho);
+                ir = 1.0 / rho;
                 const double g = fma(__shfl_sync(0xffffffffu, t, 5 + c3), ir, __shfl_sync(0xffffffffu, t, 1 + c3));
                 const double dJ = __shfl_sync(0xffffffffu, t, 0) - u_old;
                 const double vn = drift_factor(sum3(g * g), tau) * g;
