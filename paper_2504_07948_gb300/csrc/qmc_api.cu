@@ -375,6 +375,17 @@ struct qmc_ctx {
         if (!v.empty()) QMC_CK(cudaMemcpyAsync(p, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice, stream));
         return p;
     }
+    // Allocations that belong together: when one fails, those of f before it go too.
+    template <class F>
+    void alloc_all(std::vector<void*>& list, F f) {
+        const size_t n0 = list.size();
+        try {
+            f();
+        } catch (...) {
+            for (; list.size() > n0; list.pop_back()) cudaFree(list.back());
+            throw;
+        }
+    }
     void free_list(std::vector<void*>& list) {
         for (void* p : list) cudaFree(p);
         list.clear();
@@ -924,9 +935,10 @@ struct qmc_ctx {
         const size_t per_w = (size_t)(n_up + n_dn) * ldu * sizeof(float);
         if (nlU_W == 0) {
             // sized once for the capacity (no regrowth as the population moves)
-            nlU_W = (int)std::max<size_t>(1, std::min<size_t>((size_t)cap, kNlUBytes / per_w));
-            d_nlU = dalloc<float>(wk_allocs, (size_t)nlU_W * (n_up + n_dn) * ldu);
-            QMC_CK(cudaMemsetAsync(d_nlU, 0, (size_t)nlU_W * per_w, stream));
+            const int Wu = (int)std::max<size_t>(1, std::min<size_t>((size_t)cap, kNlUBytes / per_w));
+            d_nlU = dalloc<float>(wk_allocs, (size_t)Wu * (n_up + n_dn) * ldu);
+            QMC_CK(cudaMemsetAsync(d_nlU, 0, (size_t)Wu * per_w, stream));
+            nlU_W = Wu;
         }
         const int smax = std::min(W, nlU_W);
         const int ns = (W + smax - 1) / smax, S = (W + ns - 1) / ns;
@@ -998,6 +1010,7 @@ struct qmc_ctx {
 
     void ensure_tiled() {
         if (tiled_W >= W && tiled_W > 0) return;
+        tiled_W = 0;   // until all of it is there
         free_list(tiled_allocs);
         const int Wt = std::max(W, 1);
         const int nmax = std::max(n_up, n_dn), kmax = delay_rank;
@@ -1250,32 +1263,37 @@ struct qmc_ctx {
         const int chunk = kFp64 ? 256 : 512;
         const int Wc = std::min(W, chunk);
         if (fchunk < Wc) {
-            fchunk = std::max(Wc, std::min(cap, chunk));
-            d_fB = dalloc<T>(wk_allocs, 2 * (size_t)fchunk * nmax * nmax);
-            d_fPT = dalloc<T>(wk_allocs, 2 * (size_t)fchunk * nmax * nmax);
-            d_fQ = dalloc<T>(wk_allocs, 2 * (size_t)fchunk * nmax * nmax);
-            d_fM = dalloc<T>(wk_allocs, 2 * (size_t)fchunk * nb * nmax);
-            d_fY = dalloc<T>(wk_allocs, 2 * (size_t)fchunk * nb * nmax);
-            d_fgJ = dalloc<double>(wk_allocs, (size_t)fchunk * N3);
-            d_faccw = dalloc<double>(wk_allocs, (size_t)fchunk * 6 * nn);
-            d_flossy = dalloc<int>(wk_allocs, fchunk);
-            if (kFp64) {
-                // rows the tiles read: 128 of a left operand, 64 of a right one
-                const int n8 = (nmax + 7) / 8 * 8, rl = (nmax + 127) / 128 * 128, rr = (nmax + 63) / 64 * 64;
-                const int rows[4] = {std::max(rl, (n8 + nmax + 63) / 64 * 64), rr, rr, rl};
-                for (int q = 0; q < 4; ++q) g64[q] = gemm64_operand(wk_allocs, rows[q], nmax, fchunk);
-            }
+            const int fc = std::max(Wc, std::min(cap, chunk));
+            alloc_all(wk_allocs, [&] {
+                d_fB = dalloc<T>(wk_allocs, 2 * (size_t)fc * nmax * nmax);
+                d_fPT = dalloc<T>(wk_allocs, 2 * (size_t)fc * nmax * nmax);
+                d_fQ = dalloc<T>(wk_allocs, 2 * (size_t)fc * nmax * nmax);
+                d_fM = dalloc<T>(wk_allocs, 2 * (size_t)fc * nb * nmax);
+                d_fY = dalloc<T>(wk_allocs, 2 * (size_t)fc * nb * nmax);
+                d_fgJ = dalloc<double>(wk_allocs, (size_t)fc * N3);
+                d_faccw = dalloc<double>(wk_allocs, (size_t)fc * 6 * nn);
+                d_flossy = dalloc<int>(wk_allocs, fc);
+                if (kFp64) {
+                    // rows the tiles read: 128 of a left operand, 64 of a right one
+                    const int n8 = (nmax + 7) / 8 * 8, rl = (nmax + 127) / 128 * 128, rr = (nmax + 63) / 64 * 64;
+                    const int rows[4] = {std::max(rl, (n8 + nmax + 63) / 64 * 64), rr, rr, rl};
+                    for (int q = 0; q < 4; ++q) g64[q] = gemm64_operand(wk_allocs, rows[q], nmax, fc);
+                }
+            });
+            fchunk = fc;   // only now: a failed allocation leaves no half of it behind
         }
         if (kFp64) {
             require(nmax <= kGemm64MaxK, QMC_ERR_UNSUPPORTED, "the FP64 force path takes at most 170 electrons per spin");
             for (int spin = 0; spin < 2; ++spin) {
                 const int n = spin ? n_dn : n_up;
                 if (n == 0 || g64C[spin].dig) continue;
-                g64C[spin] = gemm64_operand(sys_allocs, (nb + 127) / 128 * 128, n, 1);
-                g64C[spin].stride = 0;
-                g64C[spin].estride = 0;
-                QMC_CK(launch_digits(1, ds.C[spin], 0, n, 0, nb, (nb + 7) / 8 * 8, n, d_Ce[spin], 0, -1, g64C[spin], 0,
-                                     stream));
+                alloc_all(sys_allocs, [&] {
+                    Gemm64Operand o = gemm64_operand(sys_allocs, (nb + 127) / 128 * 128, n, 1);
+                    o.stride = 0;
+                    o.estride = 0;
+                    QMC_CK(launch_digits(1, ds.C[spin], 0, n, 0, nb, (nb + 7) / 8 * 8, n, d_Ce[spin], 0, -1, o, 0, stream));
+                    g64C[spin] = o;
+                });
             }
         }
         if (!kFp64 && force_gemm_cublas) {
@@ -1346,14 +1364,21 @@ struct qmc_ctx {
         }
     }
 
+    // Per-electron outputs of the space warp.
+    void ensure_warp() {
+        if (d_gtot) return;
+        alloc_all(wk_allocs, [&] {
+            double* e = dalloc<double>(wk_allocs, (size_t)cap * 3 * N());
+            d_gtot = dalloc<double>(wk_allocs, (size_t)cap * 3 * N());
+            d_gEdet = e;
+        });
+    }
+
     void forces_per_walker(int which) {
         require(n3 == 0, QMC_ERR_UNSUPPORTED, "no ionic derivatives of the three-body Jastrow");
         require(n_pp == 0 || (!ds.msd && !space_warp), QMC_ERR_UNSUPPORTED,
                 "the pseudopotential's ionic derivatives are carried for single determinants without space warp");
-        if (space_warp && !d_gEdet) {
-            d_gEdet = dalloc<double>(wk_allocs, (size_t)cap * 3 * N());
-            d_gtot = dalloc<double>(wk_allocs, (size_t)cap * 3 * N());
-        }
+        if (space_warp) ensure_warp();
         double* gE = space_warp ? d_gEdet : nullptr;
         double* gt = space_warp ? d_gtot : nullptr;
         // non-local pseudopotential: its rows of the B matrix (so that
@@ -1362,10 +1387,11 @@ struct qmc_ctx {
         DevWalkers k = wk[which];
         if (ds.npp && ds.n_ecp) {
             const size_t nB = (size_t)n_up * n_up + (size_t)n_dn * n_dn;
-            if (!d_nlB) {
-                d_nlB = dalloc<double>(wk_allocs, (size_t)cap * nB);
-                d_nlF = dalloc<double>(wk_allocs, (size_t)cap * 3 * n_nuc);
-            }
+            if (!d_nlF)
+                alloc_all(wk_allocs, [&] {
+                    d_nlB = dalloc<double>(wk_allocs, (size_t)cap * nB);
+                    d_nlF = dalloc<double>(wk_allocs, (size_t)cap * 3 * n_nuc);
+                });
             void* b0 = d_nlB;
             void* b1 = (unsigned char*)d_nlB + (size_t)cap * n_up * n_up * elem();
             tm.begin(stream);
@@ -2501,10 +2527,7 @@ struct qmc_batch {
             require(h->space_warp == warp[q], QMC_ERR_STATE,
                     "a system's space-warp setting changed after qmc_batch_create; create the batch again");
             b.space_warp = warp[q];
-            if (warp[q] && !h->d_gEdet) {
-                h->d_gEdet = h->template dalloc<double>(h->wk_allocs, (size_t)h->cap * 3 * h->N());
-                h->d_gtot = h->template dalloc<double>(h->wk_allocs, (size_t)h->cap * 3 * h->N());
-            }
+            if (warp[q]) h->ensure_warp();
             b.gEdet = warp[q] ? h->d_gEdet : nullptr;
             b.gtot = warp[q] ? h->d_gtot : nullptr;
         }
