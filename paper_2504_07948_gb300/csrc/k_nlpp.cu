@@ -32,8 +32,10 @@
 // walkers alone are few waves of CTAs: each takes a run of electrons (runs of
 // whole molecules; with every S-th electron the molecules' pattern of electrons
 // near and far from such nuclei left a slice of four at a third of the others'
-// work) and the first sums the cluster's totals in order through distributed
-// shared memory.  Barriers are few (a chunk and a pass each cover a slice of
+// work).  Pairs are added in order to the sums of kMaxSlices fixed runs of
+// electrons, whichever CTAs take them, and the first CTA adds these in order
+// through distributed shared memory, so a walker's energy does not depend on the
+// number of walkers beside it.  Barriers are few (a chunk and a pass each cover a slice of
 // the usual size): 32 valence waters, 512 walkers, 2.6 ms with a CTA per walker
 // and chunks of eight, 1.8 ms with slices of 256-thread CTAs, now 1.6 ms.
 // The mixed form runs the basis, dot products and pair terms in FP32
@@ -76,7 +78,7 @@ __host__ __device__ inline int nl_chunk(bool ug, int n_ecp) { return ug && n_ecp
 __host__ __device__ constexpr int nl_pg(int mode) { return mode == kNlEnergy ? 8 : 12; }   // doubles per pair
 __host__ __device__ constexpr int nl_pt(int mode) { return mode == kNlEnergy ? 4 : 8; }    // and per point
 __host__ __device__ constexpr int nl_pts(bool ug) { return ug ? kUgPtCap : kPtCap; }
-constexpr int kMaxSlices = 8;   // CTAs per walker of the energy pass (a portable cluster)
+constexpr int kMaxSlices = 8;   // CTAs per walker of the energy pass (a portable cluster), a power of two
 
 struct NlLayout {
     size_t sR, sRf, rot, el, Ak, U, pairs, pg, pt, ptf, jold, beta, Fd, dvw, total;
@@ -621,7 +623,7 @@ __global__ void __launch_bounds__(kUg ? kUgThreads : kNlThreads) k_nlpp(DevSys s
     const int nmax4 = (nmax + 3) & ~3;
     __shared__ int s_count, s_npair;
     __shared__ int s_wcnt[kWarps];
-    __shared__ double s_part[kWarps];
+    __shared__ double s_part[kMaxSlices];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 
     for (int q = tid; q < 3 * N; q += blockDim.x) {
@@ -661,7 +663,7 @@ __global__ void __launch_bounds__(kUg ? kUgThreads : kNlThreads) k_nlpp(DevSys s
     }
     const int M = s_count;
     const int gsize = nl_pts(kUg) / nq;   // pairs per pass (the setter keeps nq <= kPtCap)
-    double part = 0.0;               // this lane's points
+    double tot = 0.0;                // thread q < kMaxSlices: the pairs of run q of the electrons
 
     for (int c0 = 0; c0 < M;) {
         // chunk: up to kChunk listed electrons of the spin of el[c0]
@@ -827,6 +829,7 @@ __global__ void __launch_bounds__(kUg ? kUgThreads : kNlThreads) k_nlpp(DevSys s
                 const int2 pk = pairs[g0 + pr];
                 const int ce = pk.x, i = el[c0 + ce], a = s.ecp_nuc[pk.y];
                 const T r = (T)pg[kPg * pr + 3];
+                double part = 0.0;   // this lane's points
                 for (int q0 = 0; q0 < nq; q0 += kQ) {
                     const int nqb = min(kQ, nq - q0);
                     const int p0 = pr * nq + q0;
@@ -918,8 +921,20 @@ __global__ void __launch_bounds__(kUg ? kUgThreads : kNlThreads) k_nlpp(DevSys s
                         param_lane(s, sR, i, a, pt, p0, fq, nqb, pacc, dvw + wid * P, lane);
                     }
                 }
+                if constexpr (kMode == kNlEnergy) {
+                    part = warp_sum(part);
+                    if (lane == 0) pg[kPg * pr] = part;   // (the unit vector has been used)
+                }
             }
             __syncthreads();
+            if constexpr (kMode == kNlEnergy) {
+                if (tid < kMaxSlices)
+                    for (int t = 0; t < ng; ++t) {
+                        const int i = el[c0 + pairs[g0 + t].x];
+                        if (i >= tid * N / kMaxSlices && i < (tid + 1) * N / kMaxSlices) tot += pg[kPg * t];
+                    }
+                if (g0 + gsize < npair) __syncthreads();   // (after the last pass the next chunk's barriers do)
+            }
         }
         if constexpr (kForce) {
             // rows of B_NL for the chunk's electrons: sum_l C[l][j] beta[l]
@@ -957,18 +972,15 @@ __global__ void __launch_bounds__(kUg ? kUgThreads : kNlThreads) k_nlpp(DevSys s
         }
         return;
     }
-    part = warp_sum(part);
-    if (lane == 0) s_part[wid] = part;
-    __syncthreads();
-    if (tid == 0) {
-        double v = 0.0;
-        for (int q = 0; q < kWarps; ++q) v += s_part[q];
-        s_part[0] = v;
-    }
+    if (tid < kMaxSlices) s_part[tid] = tot;
     if (nsl > 1) cg::this_cluster().sync();
+    else __syncthreads();
     if (tid == 0 && slice == 0) {
-        double v = s_part[0];
-        for (int c = 1; c < nsl; ++c) v += *cg::this_cluster().map_shared_rank(s_part, c);
+        double v = 0.0;
+        for (int q = 0; q < kMaxSlices; ++q) {   // from the slice that holds run q
+            const int c = q * nsl / kMaxSlices;
+            v += c ? cg::this_cluster().map_shared_rank(s_part, c)[q] : s_part[q];
+        }
         eloc[w] += v;
         if (!isfinite(eloc[w]) && wk.err) atomicOr(wk.err, kErrNonFinite);
     }
