@@ -611,8 +611,8 @@ cudaError_t tiled_begin(const DevWalkers& wk, int W, int N, const TiledState& ts
 cudaError_t tiled_propose(const DevSys& s, const DevWalkers& wk, const TiledState& ts, int w0, int nw, int e,
                           const SweepParams& p, cudaStream_t st) {
     if (nw <= 0) return cudaSuccess;
-    k_tiled_propose<<<nw, kTb, tiled_smem_bytes(s.n_nuc, s.n_shell), st>>>(s, wk, ts, w0, w0 + nw, e, p);
-    return cudaGetLastError();
+    return launch_after(k_tiled_propose, dim3(nw), kTb, tiled_smem_bytes(s.n_nuc, s.n_shell), st, false, s, wk, ts, w0,
+                        w0 + nw, e, p);
 }
 
 cudaError_t tiled_accept(const DevSys& s, const DevWalkers& wk, const TiledState& ts, int w0, int nw, int e,
