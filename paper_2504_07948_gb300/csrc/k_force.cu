@@ -839,7 +839,7 @@ __global__ void k_force_prep(DevSys s, DevWalkers wk, int w0, int W, const doubl
 static int contract_parts(int W, int nn, bool kE) {
     if (kE) return 1;
     int p = 1;
-    while ((long long)W * p < 6 * 152 * 3 && nn / (2 * p) >= 24) p *= 2;
+    while ((long long)W * p < 6LL * 3 * device_sms() && nn / (2 * p) >= 24) p *= 2;
     return p;
 }
 // Nuclei of a part up to which spin down has sums of its own: thousands of

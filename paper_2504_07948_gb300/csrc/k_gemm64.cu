@@ -306,9 +306,7 @@ cudaError_t launch_gemm64(const Gemm64Operand& A, const Gemm64Operand& B, int M,
     const size_t smem = kGSlots * kStageBytes;
     cudaError_t e = cudaFuncSetAttribute(k_gemm64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    int dev = 0, n_sm = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    const int n_sm = device_sms();
     const long long tiles = (long long)((M + kGm - 1) / kGm) * ((N + kGn - 1) / kGn) * batch;
     k_gemm64<<<(int)(tiles < n_sm ? tiles : n_sm), kGThreads, smem, st>>>(A, B, M, N, K, batch, D1, sD1, n1, n2,
                                                                           D2, sD2, ldd, err);

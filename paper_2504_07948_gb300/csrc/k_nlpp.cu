@@ -1008,7 +1008,7 @@ cudaError_t launch_nlpp(const DevSys& s, const DevWalkers& wk, int w0, int W, do
     // slices until there are six waves of CTAs, while each still has a warp's
     // worth of electrons (a slice repeats the rotations and positions)
     int nsl = 1;
-    const long long want = 6 * 152 * (ug ? 4 : 2);
+    const long long want = 6LL * device_sms() * (ug ? 4 : 2);
     while (nsl < kMaxSlices && (long long)(W - w0) * nsl < want && s.N / (2 * nsl) >= 32) nsl *= 2;
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeClusterDimension;

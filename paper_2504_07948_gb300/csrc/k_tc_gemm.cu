@@ -951,8 +951,7 @@ bool tc_split_plan(TcSplitPlan* p, int M, int N, int K, const float* Ah, const f
     // the launch within one wave.  The products of an output are added in the
     // same order either way.  32-water sweep, 512 walkers a launch (20 row
     // tiles): 22.4 -> 19.0 us, then bound by the row tiles' reads from L2.
-    int dev = 0, n_sm = 152;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    const int n_sm = device_sms();
     const int mt = (M + kTcM - 1) / kTcM;
     int Np = 32;
     while (Np < N && (long long)mt * ((N + Np - 1) / Np) > n_sm) Np += 16;

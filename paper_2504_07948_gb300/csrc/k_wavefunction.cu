@@ -78,23 +78,21 @@ __global__ void __launch_bounds__(320, 2) k_orbitals_all(DevSys s, DevWalkers wk
 // order.
 template <typename T>
 __device__ __forceinline__ void orbitals_sums_item(const DevSys& s, const DevWalkers& wk, int w, int i, double* sh_bas,
-                                              unsigned char* live = nullptr) {
+                                                   unsigned char* live) {
     const int nb = s.n_basis;
     double r[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) r[c] = wk.R[((size_t)w * s.N + i) * 3 + c];
     for (int sh = threadIdx.x; sh < s.n_shell; sh += blockDim.x) shell_vgl<double>(s, sh, r, sh_bas, nb);
     __syncthreads();
-    if (live) {
-        for (int sh = threadIdx.x; sh < s.n_shell; sh += blockDim.x) {
-            const int f0 = s.shell_fn[sh], f1 = s.shell_fn[sh + 1];
-            bool nz = false;
-            for (int c = 0; c < 5 && !nz; ++c)
-                for (int f = f0; f < f1 && !nz; ++f) nz = sh_bas[c * nb + f] != 0.0;
-            live[sh] = nz ? 1 : 0;
-        }
-        __syncthreads();
+    for (int sh = threadIdx.x; sh < s.n_shell; sh += blockDim.x) {
+        const int f0 = s.shell_fn[sh], f1 = s.shell_fn[sh + 1];
+        bool nz = false;
+        for (int c = 0; c < 5 && !nz; ++c)
+            for (int f = f0; f < f1 && !nz; ++f) nz = sh_bas[c * nb + f] != 0.0;
+        live[sh] = nz ? 1 : 0;
     }
+    __syncthreads();
     const int spin = i < s.n_up ? 0 : 1;
     const int n = spin ? s.n_dn : s.n_up;
     const int k = spin ? i - s.n_up : i;
@@ -105,13 +103,9 @@ __device__ __forceinline__ void orbitals_sums_item(const DevSys& s, const DevWal
         const int c = o / n, j = o - c * n;
         const double* b = sh_bas + c * nb;
         double acc = 0.0;
-        if (live) {
-            for (int sh = 0; sh < s.n_shell; ++sh) {
-                if (!live[sh]) continue;
-                for (int l = s.shell_fn[sh]; l < s.shell_fn[sh + 1]; ++l) acc += C[(size_t)l * n + j] * b[l];
-            }
-        } else {
-            for (int l = 0; l < nb; ++l) acc += C[(size_t)l * n + j] * b[l];
+        for (int sh = 0; sh < s.n_shell; ++sh) {
+            if (!live[sh]) continue;
+            for (int l = s.shell_fn[sh]; l < s.shell_fn[sh + 1]; ++l) acc += C[(size_t)l * n + j] * b[l];
         }
         if (c == 0)
             A[j] = acc;

@@ -1318,6 +1318,13 @@ __device__ __forceinline__ float warp_sum(float v) {
 }
 
 
+// Streaming multiprocessors of the current device.
+inline int device_sms() {
+    int dev = 0, n = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n;
+}
+
 // ---------------------------------------------------------------------
 // Programmatic dependent launch: a kernel launched with launch_after may start
 // when every CTA of the kernel before it in the stream has called
