@@ -971,6 +971,48 @@ def run_workloads(args, rank, ws, dist):
     return out
 
 
+HEADLINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                 "vs_baseline", "dtype", "data", "config", "force_evals_per_s", "gpu_launches", "clocks", "e2e")
+HEADLINE_BYTES = 2800
+
+
+def headline(line):
+    """The record of a run as one short line: every key that names the
+    workload and its rates, the roofline's figures, the oracle's rate, and of
+    the mixed form and of the other workloads their rates alone.  Readers that
+    keep the end of the output get it whole (at most HEADLINE_BYTES); the full
+    record goes to stderr."""
+    def short(x):
+        if isinstance(x, float):
+            return float(f"{x:.6g}")
+        return {k: short(v) for k, v in x.items()} if isinstance(x, dict) else x
+
+    def rates(d):
+        return {k: short(d[k]) for k in ("value", "unit", "ms_per_step", "force_evals_per_s") if d.get(k) is not None}
+
+    out = {k: line[k] for k in HEADLINE_KEYS if k in line}
+    for key, fields in (("roofline", ("kernel", "bound", "achieved", "peak", "unit", "frac")),
+                        ("cpu_baseline", ("value", "unit", "cores", "kind"))):
+        if line.get(key):
+            out[key] = {k: short(line[key][k]) for k in fields if k in line[key]}
+    if line.get("kernel_ms_per_step"):
+        out["kernel_ms_per_step"] = short(line["kernel_ms_per_step"])
+    if line.get("mixed"):
+        out["mixed"] = rates(line["mixed"])
+    if line.get("workloads"):
+        out["workloads"] = {n: rates(w) for n, w in line["workloads"].items()}
+    for drop in ("workloads", "mixed", "kernel_ms_per_step", "cpu_baseline", "roofline"):
+        if len(json.dumps(out)) <= HEADLINE_BYTES:
+            break
+        out.pop(drop, None)
+    return out
+
+
+def emit(line):
+    print(json.dumps(line), file=sys.stderr, flush=True)
+    print(json.dumps(headline(line)), flush=True)
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -1034,7 +1076,7 @@ def main():
     if args.workload == BATCH_WORKLOAD:
         line = run_batch(args, rank, dist)
         if rank == 0:
-            print(json.dumps(line))
+            emit(line)
         return
     if args.workload in (PP_WORKLOAD, PP_FORCE_WORKLOAD):
         r = run_pp_workload(args, rank, dist, args.workload)
@@ -1043,7 +1085,7 @@ def main():
                     "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32+f64",
                     "data": "synthetic", **r}
             line["config"] = {"workload": args.workload, **r["config"]}
-            print(json.dumps(line))
+            emit(line)
         return
     s, wl, W, primary, result, e2e, cpu, peaks, warp = run_gpu(args, rank, ws, dist)
     workloads = None
@@ -1086,7 +1128,7 @@ def main():
                          "kernel_ms_per_step": m["kernel_ms"],
                          "error_vs_oracle": m.get("error_vs_oracle"), "recompute": m.get("recompute"),
                          "clocks": m["clocks"]}
-    print(json.dumps(line))
+    emit(line)
 
 
 if __name__ == "__main__":
