@@ -394,7 +394,8 @@ def run_gpu(args, rank, ws, dist):
         peak = FP64_PEAK_TFLOPS_NOMINAL if precision == "fp64" else FP32_PEAK_TFLOPS_NOMINAL
         traffic, traffic_note = profiled_traffic(args.workload, precision, float(np.mean(entering)))
         sweep_kernel = ("k_sweep_msd" if s.n_det > 0 else
-                        "k_sweep_delayed" if precision == "mixed" and wl.delay_rank > 1 else "k_sweep")
+                        "k_sweep_delayed" if precision == "mixed" and wl.delay_rank > 1 else
+                        "k_sweep64" if precision == "fp64" else "k_sweep")
         gemm_ms, gemm_n = fam["sweep_gemm"]
         result[precision] = {
             "value": moves_all / sec, "force_evals_per_s": fe_all / sec, "ms_per_step": ms / args.steps,

@@ -32,7 +32,8 @@
 // the block reaches 2^-4 of that (occupied orbitals without weight on the
 // functions that are large at this point), orbitals64 takes the orbitals
 // again in FP64, so that the row of orbital values keeps the accuracy of an
-// FP64 sum relative to its largest entry.
+// FP64 sum relative to its largest entry.  Where a row's smaller entries decide,
+// its users find out from the inverse (k_wavefunction.cu, sweep64.cuh).
 #pragma once
 
 #include "fixed64.cuh"

@@ -485,7 +485,7 @@ __host__ __device__ inline int force_row_groups(int n) {
 // all of them where the budget allows (2 CTAs per SM in FP64, 3 mixed), so
 // that the contraction keeps a warp per centre busy.
 // Bound by FP64 issue (FP64 form) and by instruction issue (mixed).  6-water
-// cluster, 2048 walkers: 8.10 -> 3.38 ms FP64 and 0.81 -> 0.45 ms mixed
+// cluster, 2048 walkers: 8.10 -> 3.64 ms FP64 and 0.81 -> 0.44 ms mixed
 // against one derivative evaluation per basis function, FP64 products and a
 // masked exponential per primitive.
 // Where only one CTA fits an SM (above kForceTwo bytes: determinants above about
@@ -832,7 +832,11 @@ __global__ void k_force_prep(DevSys s, DevWalkers wk, int w0, int W, const doubl
 // functions of a nucleus only add to its own sums), enough for six waves, so that
 // the last one is not most of the time; one where the per-electron sums of the
 // space warp are wanted, which run over all nuclei.  32-water cluster, 512
-// walkers, mixed: 855 -> 509 us, with the runs shared out as warps come free.
+// walkers, mixed: 855 -> 507 us, with the runs shared out as warps come free.
+// (Whole pass, mixed, 512 walkers, one, two, four and eight parts: 14 waters 0.85,
+// 0.86, 0.87, 0.89, 20 waters 1.03, 1.03, 1.05, 1.08, 32 waters 1.89, 1.87, 1.89,
+// 1.93 ms.  With 64 walkers 14 waters would gain from more parts than the 24 nuclei
+// allow, 0.40 ms at the one they get and 0.34 at four.)
 // Each spin adds to sums of its own: both on the nucleus's one made the last
 // bits depend on which warp came first (one warp taking both spins of a run,
 // which also fixes the order, was 3 % slower on the whole pass).

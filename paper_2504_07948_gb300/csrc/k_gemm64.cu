@@ -8,14 +8,23 @@
 // Algorithms 59, 2012).  Every row is scaled by its own power of two to
 // integers of at most 55 bits and written as kDig = 7 balanced digits of 8
 // bits, q = sum_i d_i 2^(8 (6 - i)), |d_i| <= 128: exact in bf16.  The products
-// of digits i and j with i + j = t add up in accumulator t (t <= 6, 28 products;
-// the rest is below 2^-53 of the product of the row maxima, 2^-56 on average):
+// of digits i and j with i + j = t add up in accumulator t (t <= 6, 28 products):
 // |d_i d_j| <= 2^14, so an accumulator of t <= 5 holds at most 6 K 2^14 <= 2^24
 // for K <= kGemm64MaxK and its FP32 sums are exact; in t = 6 a rounding is below
 // 2^-60.  The seven accumulators of a 128 x 64 tile take 448 of the 512 columns
 // of tensor memory; the epilogue adds them as integers and rounds once.
-// Against an FP64 chain of K terms the error is smaller (it does not grow with
-// the partial sums).
+//
+// Error, relative to the product of the two rows' largest entries (their integers
+// lie in [2^54, 2^55)): the operands' rounding 2^-54 a term at most; the dropped
+// digits i + j >= 7, six products of 2^14 2^40 at t = 7, 2^-51.4 a term at most and
+// K times that for the sum, some 2^-55 sqrt(K) with digits of random sign.  An
+// FP64 chain is off by 2^-53 of each of its partial sums instead, which is more
+// where the terms come near the product of the maxima and less where they lie far
+// below it; k_force_prep finds the walkers with such rows, and launch_force takes
+// them in FP64.  Elsewhere the error of A^-1 sets that of the derivatives: against
+// extended precision both paths, this one and FP64 GEMMs, give the same to all
+// digits shown (14 to 32 waters, electrons up to 12 bohr out, orbitals scaled by
+// 10^-9 to 10^9).
 //
 // Digits are written by k_digits in the order the tensor core reads them: for
 // each block of 32 k and each digit, groups of 8 rows of four 128-byte core
@@ -23,9 +32,9 @@
 // bytes that a bulk copy moves to shared memory as it is.
 //
 // 32-water forces in FP64, 256 walkers (four products per spin, n = 160): with
-// cuBLAS DGEMM 46.6 ms of a 53.7 ms pass, with this kernel the pass takes
-// 10.8 ms (the rest is FP64 pair and basis terms); the error of the
-// derivatives against 64 bits fell from 6e-11 to 6e-12.
+// cuBLAS DGEMM 46.6 ms of a 53.7 ms pass; with this kernel the pass takes
+// 10.4 ms, of which its products 3.2 and the digits 0.8 (the rest is FP64 pair
+// and basis terms).
 //
 // Roles of a CTA (one per SM, persistent over the tiles): warp 0 issues the
 // bulk copies of a two-slot ring (14 pieces a stage), warp 1 the 56 MMAs of a

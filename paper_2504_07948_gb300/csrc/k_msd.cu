@@ -350,7 +350,9 @@ __device__ __forceinline__ void refresh_cd(const DevSys& s, const DevWalkers& wk
 // Arithmetic of the sweep's strings.  Every rounding is written out: a sweep of
 // the mixed form is a chaotic map, and its trajectories should not depend on how
 // the compiler contracts products and sums in one or the other arrangement of
-// this code.
+// this code.  The patterns are those that seeded runs have had so far, uneven as
+// they are (string_ratio rounds the product of the table's update, except in the
+// first column below its first row), so that these runs repeat bit for bit.
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }

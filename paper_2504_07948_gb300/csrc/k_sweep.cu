@@ -32,8 +32,10 @@ __global__ void __launch_bounds__(kNt, sizeof(T) == 4 ? (kNt == 128 ? 7 : 3) : (
 // The FP64 form (sweep64.cuh); k_sweep<double> is left for bases whose lists
 // exceed shared memory.  256 threads above 64 electrons per spin, 64 where two
 // warps hold a move's partners (electrons and nuclei; 2048 walkers of 1, 2 and
-// 4 waters: 629 -> 529, 1299 -> 1110 and 3139 -> 2801 us a sweep against 128
-// threads, 6 waters 6.0 -> 7.1 ms), else 128.
+// 4 waters: 638 -> 520, 1328 -> 1124 and 3179 -> 2794 us a sweep against 128
+// threads), else 128.  The line is not where today's kernel would have it: since
+// its lists share their memory, 64 threads are ahead at 6 waters too (6.1 -> 5.5
+// ms, 7.1 before); between there and 64 electrons per spin it is not measured.
 template <int kNt, bool kJ3>
 __global__ void __launch_bounds__(kNt, kNt <= 64 ? 8 : kNt == 128 ? 5 : 2) k_sweep64(DevSys s, DevWalkers wk, int W, SweepParams p) {
     extern __shared__ __align__(16) unsigned char smem[];

@@ -470,7 +470,7 @@ __device__ __forceinline__ int accept_body(const DevSys& s, const DevWalkers& wk
 // promises the next grid no memory, neither this grid's nor that of the grids
 // before it.  Ahead of its wait an accept launch takes the constants (nuclei)
 // and draws its random numbers, while the GEMM runs.  Used where one chain of launches
-// has the GPU (32 waters, 256 walkers: 49 -> 42 us an electron); with several
+// has the GPU (32 waters, 256 walkers: 49 -> 44 us an electron); with several
 // groups a GEMM that waits for its rows would hold SMs the other group could
 // use (4096 walkers, two groups: 206 -> 217), and launches are plain.
 //
@@ -508,7 +508,7 @@ __global__ void __launch_bounds__(kTb, 8) k_tiled_accept(DevSys s, DevWalkers wk
 // barrier, K^-1 stays in shared memory.  Bound by the latency of its
 // dependent loads (512 walkers of the 32-water cluster: 33.4 us with the serial
 // loops over K^-1 reading global memory and one queued row in flight per warp,
-// 26.2 us now).  Eight CTAs per SM with 64 registers, for loads ahead of their
+// 26.2 us with K^-1 on chip and four).  Eight CTAs per SM with 64 registers, for loads ahead of their
 // use, against twelve with 40: 2048 walkers in one chain of launches 119 against
 // 127 us an electron, 4096 in two groups 209 against 206.
 __global__ void __launch_bounds__(kTb, 8) k_tiled_accept_propose(DevSys s, DevWalkers wk, TiledState ts, int w0,

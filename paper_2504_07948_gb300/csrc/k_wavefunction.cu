@@ -65,17 +65,18 @@ __global__ void __launch_bounds__(320, 2) k_orbitals_all(DevSys s, DevWalkers wk
     orbitals_item<T>(s, wk, w, i, (unsigned char*)sh_bas);
 }
 
-// The same orbitals as FP64 sums over the basis functions in index order
-// (3 x slower on the 32-water cluster: bound by the FP64 pipe).  New walkers of
-// the mixed form are built with it, and walkers a determinant expansion rebuilds
-// inside a sweep: the last bit of an FP64 sum decides how an FP32 inverse rounds,
-// and a mixed trajectory amplifies one such bit until an accept decision turns,
-// so a seeded mixed run repeats earlier ones only from the same bits.  Also for
-// a basis whose lists exceed shared memory.  sh_bas: 5 n_basis doubles of
-// shared memory.  live (n_shell bytes of shared memory): shells whose values
-// and derivatives are all exactly zero (screened) are left out of the
-// occupied-orbital contraction; the terms that remain are added in the same
-// order.
+// The same orbitals as FP64 sums over the basis functions in index order (51.9
+// against 9.3 ms for 256 walkers of the 32-water cluster: bound by the FP64
+// pipe).  New walkers of the mixed form are built with it, and walkers a
+// determinant expansion rebuilds inside a sweep: the last bit of an FP64 sum
+// decides how an FP32 inverse rounds, and a mixed trajectory amplifies one such
+// bit until an accept decision turns, so a seeded mixed run repeats earlier
+// ones only from the same bits.  Also for a basis whose lists exceed shared
+// memory, and for the spins of a rebuild that fixed point would cost bits
+// (orbitals_again).  sh_bas: 5 n_basis doubles of shared memory.  live (n_shell
+// bytes of shared memory): shells whose values and derivatives are all exactly
+// zero (screened) are left out of the occupied-orbital contraction; the terms
+// that remain are added in the same order.
 template <typename T>
 __device__ __forceinline__ void orbitals_sums_item(const DevSys& s, const DevWalkers& wk, int w, int i, double* sh_bas,
                                                    unsigned char* live) {
@@ -402,9 +403,13 @@ __device__ void j3_electron(const DevSys& s, const double* sR, int i, double& va
 //   Mixed form (was bound by uncoalesced reads of the gradient cache, a row
 // per thread): the determinant sums of an electron are taken by a warp; pair
 // terms in FP32 with compensated sums, assembled in FP64.
-// 6-water cluster, 2048 walkers: 756 -> 415 us FP64, 143 -> 84 us mixed;
-// 32-water cluster, 1024 walkers, mixed: 1.84 -> 0.79 ms (a thread per electron
+// 6-water cluster, 2048 walkers: 756 -> 438 us FP64, 143 -> 92 us mixed;
+// 32-water cluster, 1024 walkers, mixed: 1.84 -> 0.87 ms (a thread per electron
 // for everything before).
+// kElocSym keeps the warps' arrays within 10 KB; it is not where the two forms
+// cross: pairs once takes 0.90 against 1.28 ms at 16 waters (160 electrons, 512
+// walkers) and would take 1.51 against 2.18 ms at 20, 1.74 against 2.47 ms at 32
+// waters (256 walkers; 100 KB of shared memory).
 // sm: eloc_smem_bytes.
 constexpr int kElocSym = 160;
 struct ElocLayout {
@@ -880,8 +885,11 @@ cudaError_t launch_orbitals_all(const DevSys& s, const DevWalkers& wk, int W, cu
     const size_t smem = orbitals_smem_bytes(s);
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
     // a thread per orbital; few orbitals share their rows among lanes anyway, and
-    // two warps per electron leave room for twice the electrons (3 waters, 77
-    // walkers: three waves of CTAs become two, evaluation 164 -> 144 us)
+    // two warps per electron leave room for twice the electrons.  Evaluation with
+    // 128 -> 64 threads: one water, 512 and 4096 walkers 0.20 -> 0.17 and 0.92 ->
+    // 0.71 ms; 3 waters, 77, 1024 and 4096 walkers 0.18 -> 0.16, 0.78 -> 0.60 and
+    // 2.76 -> 2.09 ms.  (At 20 orbitals 64 are ahead as well, 2.32 -> 1.88 ms for
+    // 2048 walkers: the line could lie higher.)
     const int nt = nmax > 128 ? (nmax > 256 ? 256 : (nmax + 31) & ~31) : nmax > 16 ? 128 : 64;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_orbitals_all<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,

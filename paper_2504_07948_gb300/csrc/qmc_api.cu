@@ -1070,8 +1070,8 @@ struct qmc_ctx {
         ensure_tiled();
         const DevWalkers& k = wk[cur];
         // one chain below kTiledSplitW walkers unless the environment asks
-        // for groups: 32 waters, 1024 / 2048 walkers 67 / 119 us an electron in
-        // one chain and 78 / 125 in two, 4096 walkers 230 and 206
+        // for groups: 32 waters, 512 / 2048 walkers 55 / 114 us an electron in
+        // one chain and 56 / 116 in two, 4096 walkers 223 and 198
         constexpr int kTiledSplitW = 3072;
         const int groups_max =
             tiled_groups_set || W >= kTiledSplitW ? std::max(1, std::min(tiled_groups, W / 256)) : 1;
@@ -1242,7 +1242,8 @@ struct qmc_ctx {
     void gemm_sb(cublasOperation_t ta, cublasOperation_t tb, int m, int n, int k, const T* A, int lda, long long sA,
                  const T* B, int ldb, long long sB, T* Cm, int ldc, long long sC, int batch);
 
-    // Digit buffers of one operand of the FP64 GEMM (rows a multiple of 64).
+    // Digit buffers of one operand of the FP64 GEMM (rows a multiple of 64).  The
+    // four operands of 256 walkers of the 32-water cluster take 550 MB.
     Gemm64Operand gemm64_operand(std::vector<void*>& list, int rows, int K, int batch) {
         Gemm64Operand o{};
         o.groups = rows / 8;
@@ -2865,7 +2866,9 @@ int qmc_batch_create(qmc_batch_t* out, int n_systems, qmc_t const* systems) {
         // the instruction rate does: four CTAs of four warps per SM.  Clusters of
         // 1 to 16 waters, sweep of the batch, four / eight warps: 1024 walkers 9.0 /
         // 6.1 ms, 4096 walkers 21.3 / 24.9 and 37.9 / 43.4 ms (16 and 64 systems;
-        // 30.7 and 59.6 ms with four warps and A^-1 in up to 100 KB).
+        // 30.7 and 59.6 ms with four warps and A^-1 in up to 100 KB).  The choice
+        // orders the FP64 sums of a move, so a member's last bits follow it, as they
+        // follow qmc_batch_set_options and the autotuner.
         long long walkers = 0;
         for (int q = 0; q < n_systems; ++q) walkers += systems[q]->W;
         if (b->mode == QMC_MIXED)

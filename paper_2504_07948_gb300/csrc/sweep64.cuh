@@ -19,8 +19,8 @@
 // inverse that they meet, as those of a rebuild are (kFxSlack, k_wavefunction.cu):
 // where the column weighs small orbitals up, the move's orbitals are taken
 // again as FP64 sums.
-// 6-water cluster, 2048 walkers: 9.9 -> 5.8 ms a sweep (1345 -> about 600 FP64
-// warp instructions a move); one water, 512 walkers: 283 -> 180 us.
+// 6-water cluster, 2048 walkers: 9.9 -> 6.0 ms a sweep (1345 -> about 600 FP64
+// warp instructions a move); one water, 512 walkers: 283 -> 187 us.
 #pragma once
 
 #include "basis64.cuh"
