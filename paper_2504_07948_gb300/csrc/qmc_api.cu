@@ -2866,14 +2866,24 @@ int qmc_batch_create(qmc_batch_t* out, int n_systems, qmc_t const* systems) {
         // the instruction rate does: four CTAs of four warps per SM.  Clusters of
         // 1 to 16 waters, sweep of the batch, four / eight warps: 1024 walkers 9.0 /
         // 6.1 ms, 4096 walkers 21.3 / 24.9 and 37.9 / 43.4 ms (16 and 64 systems;
-        // 30.7 and 59.6 ms with four warps and A^-1 in up to 100 KB).  The choice
+        // 30.7 and 59.6 ms with four warps and A^-1 in up to 100 KB).  Where two warps
+        // hold a move's partners in every system eight only wait for each other: 1024
+        // walkers of one, two, three and four waters, eight / four warps, 0.79 / 0.48,
+        // 1.54 / 0.91, 2.52 / 1.44 and 3.22 / 2.05 ms a step (6 waters 5.61 / 3.58, 8
+        // waters 4.47 / 3.35 with 512 walkers, 2.42 / 3.11 with 128; clusters of 1 to
+        // 8 waters 3.28 / 3.36, of 1 to 10 4.9 / 5.9 ms), unless every walker has a place
+        // at once (256 walkers of one water 0.26 / 0.28 ms).  The choice
         // orders the FP64 sums of a move, so a member's last bits follow it, as they
         // follow qmc_batch_set_options and the autotuner.
         long long walkers = 0;
-        for (int q = 0; q < n_systems; ++q) walkers += systems[q]->W;
+        int partners = 0;   // of a move, at most
+        for (int q = 0; q < n_systems; ++q) {
+            walkers += systems[q]->W;
+            partners = std::max(partners, systems[q]->N() + systems[q]->n_nuc);
+        }
         if (b->mode == QMC_MIXED)
             b->configure(128, 100 * 1024, 1, 0);
-        else if (walkers < 16LL * b->n_sm)
+        else if (walkers < (partners > 64 ? 16LL : 2LL) * b->n_sm)
             b->configure(256, 220 * 1024, 1, 0);
         else
             b->configure(128, 45 * 1024, 1, 0);
