@@ -497,7 +497,13 @@ __host__ __device__ inline int force_row_groups(int n) {
 // FP64 form: a spin in which some electron's row of A^-T weighs small entries
 // of B up (row_short; electrons shared out unevenly over distant fragments with
 // orbitals of their own) is taken as a determinant too large to stage is, in FP64 sums.
+// So is a spin of at most kForcePlain electrons: limbs, their scales and the
+// whole-warp row groups cost more than its short sums.  Pass in FP64 sums / limbs /
+// as before either: one water, 64 walkers 62 / 93 / 87 us, 2048 walkers 432 / 647 /
+// 950; 3 waters (15 electrons), 64 and 2048 walkers 148 / 178 / 292 and 1477 / 1617
+// us; 4 waters (20) 195 / 216 and 2255 / 2125 us; 6 waters (30) 4.6 / 3.6 ms.
 constexpr size_t kForceTwo = 113 * 1024;
+constexpr int kForcePlain = 16;
 template <typename T>
 struct ForceShape {
     bool stg;
@@ -599,7 +605,7 @@ __device__ __forceinline__ void force_walker(const DevSys& s, const DevWalkers& 
             if (nlB) b += nlB[(size_t)pp * n + qq];
             return b;
         };
-        bool stg = fs.stg;
+        bool stg = fs.stg && !(kFx && n <= kForcePlain);
         if (stg) {
             int lossy = 0;
             for (int r = wid; r < n; r += nw) {

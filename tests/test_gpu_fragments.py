@@ -9,7 +9,7 @@ from oracle import oracle as O
 from paper_2504_07948_gb300 import synth
 
 pytestmark = pytest.mark.gpu
-CASES = [(1, 8.0), (1, 11.0), (1, 14.0), (1, 17.0), (3, 12.0)]
+CASES = [(1, 8.0), (1, 11.0), (1, 14.0), (1, 17.0), (3, 12.0), (3, 16.0), (3, 19.0)]
 
 
 def fragments(m, D):
