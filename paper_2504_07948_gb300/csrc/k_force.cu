@@ -950,19 +950,11 @@ cudaError_t launch_force_prep(const DevSys& s, const DevWalkers& wk, int w0, int
     if (W == 0) return cudaSuccess;
     const size_t smem = force_head_bytes<T>(s.N, s.n_nuc);
     if (gtot) {
-        if (smem > 48 * 1024) {
-            cudaError_t e =
-                cudaFuncSetAttribute(k_force_prep<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
+        if (const cudaError_t e = allow_smem(k_force_prep<T, true>, smem)) return e;
         k_force_prep<T, true><<<W, 256, smem, st>>>(s, wk, w0, W, dvnn, (T*)Bw, gJw, accw, gtot, lossy);
         return cudaGetLastError();
     }
-    if (smem > 48 * 1024) {
-        cudaError_t e =
-            cudaFuncSetAttribute(k_force_prep<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_smem(k_force_prep<T, false>, smem)) return e;
     k_force_prep<T, false><<<W, 256, smem, st>>>(s, wk, w0, W, dvnn, (T*)Bw, gJw, accw, nullptr, lossy);
     return cudaGetLastError();
 }
@@ -984,22 +976,14 @@ cudaError_t launch_force_contract(const DevSys& s, const DevWalkers& wk, int w0,
     if (gEdet) {
         const int parts = contract_parts(W, s.n_nuc, true);
         const size_t smem = contract_smem<T>(s.N, s.n_nuc, parts, true);
-        if (smem > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(k_force_contract<T, true>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
+        if (const cudaError_t e = allow_smem(k_force_contract<T, true>, smem)) return e;
         k_force_contract<T, true><<<dim3(W, parts), 256, smem, st>>>(s, wk, w0, W, (const T*)Mw, (const T*)Yw, gJw, accw,
                                                                      dEL, dlog, gEdet);
         return cudaGetLastError();
     }
     const int parts = contract_parts(W, s.n_nuc, false);
     const size_t smem = contract_smem<T>(s.N, s.n_nuc, parts, false);
-    if (smem > 48 * 1024) {
-        cudaError_t e =
-            cudaFuncSetAttribute(k_force_contract<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_smem(k_force_contract<T, false>, smem)) return e;
     k_force_contract<T, false><<<dim3(W, parts), 256, smem, st>>>(s, wk, w0, W, (const T*)Mw, (const T*)Yw, gJw, accw, dEL,
                                                                   dlog, nullptr);
     return cudaGetLastError();
@@ -1029,7 +1013,7 @@ cudaError_t launch_force(const DevSys& s, const DevWalkers& wk, int w0, int W, c
     const size_t smem = ForceShape<T>(s.N, s.n_nuc, nmax, s.n_basis, kE, nw).total;
     const auto f = nw == 16 ? (kE ? k_force<T, true, 512> : k_force<T, false, 512>)
                             : (kE ? k_force<T, true, 256> : k_force<T, false, 256>);
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(f, smem);
     if (e != cudaSuccess) return e;
     f<<<W, 32 * nw, smem, st>>>(s, wk, w0, W, only, dvnn, Bscr, Pscr, dEL, dlog, gEdet, kE ? gtot : nullptr);
     return cudaGetLastError();
@@ -1192,10 +1176,7 @@ cudaError_t launch_space_warp(const DevSys& s, const DevWalkers& wk, int W, cons
                               double* dEL, double* dlog, cudaStream_t st) {
     if (W == 0) return cudaSuccess;
     const size_t smem = space_warp_smem<T>(s.N, s.n_nuc);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_space_warp<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_smem(k_space_warp<T>, smem)) return e;
     k_space_warp<T><<<W, 256, smem, st>>>(s, wk, W, gEdet, gtot, dEL, dlog);
     return cudaGetLastError();
 }
@@ -1280,7 +1261,7 @@ size_t space_warp_batch_smem_bytes(const DevSys& s, int elem) {
 template <typename T>
 int space_warp_batch_prepare(size_t smem) {
     int nb = 0;
-    if (cudaFuncSetAttribute(k_space_warp_batch<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+    if (allow_smem(k_space_warp_batch<T>, smem) !=
             cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_space_warp_batch<T>, 256, smem) != cudaSuccess) {
         cudaGetLastError();
@@ -1306,7 +1287,7 @@ template <typename T>
 int force_batch_prepare(size_t smem, int any_warp, int nw) {
     int nb = 0;
     const void* f = (const void*)force_batch_kernel<T>(any_warp, nw);
-    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+    if (allow_smem(f, smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, 32 * nw, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;

@@ -581,13 +581,13 @@ cudaError_t launch_force_msd(const DevSys& s, const DevWalkers& wk, int W, const
     if (gEdet) {
         const size_t smem_e = smem + sizeof(double) * 3 * (size_t)s.N;
         cudaError_t e =
-            cudaFuncSetAttribute(k_force_msd<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_e);
+            allow_smem(k_force_msd<T, true>, smem_e);
         if (e != cudaSuccess) return e;
         k_force_msd<T, true><<<W, 256, smem_e, st>>>(s, wk, W, dvnn, scr, force_msd_scratch_words(s), dEL, dlog,
                                                      gEdet, gtot);
         return cudaGetLastError();
     }
-    cudaError_t e = cudaFuncSetAttribute(k_force_msd<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_force_msd<T, false>, smem);
     if (e != cudaSuccess) return e;
     k_force_msd<T, false><<<W, 256, smem, st>>>(s, wk, W, dvnn, scr, force_msd_scratch_words(s), dEL, dlog, nullptr,
                                                 nullptr);

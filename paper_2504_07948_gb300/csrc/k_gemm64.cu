@@ -313,7 +313,7 @@ cudaError_t launch_gemm64(const Gemm64Operand& A, const Gemm64Operand& B, int M,
     if (batch <= 0 || M <= 0 || N <= 0) return cudaSuccess;
     if (K <= 0 || K > kGemm64MaxK) return cudaErrorInvalidValue;
     const size_t smem = kGSlots * kStageBytes;
-    cudaError_t e = cudaFuncSetAttribute(k_gemm64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_gemm64, smem);
     if (e != cudaSuccess) return e;
     const int n_sm = device_sms();
     const long long tiles = (long long)((M + kGm - 1) / kGm) * ((N + kGn - 1) / kGn) * batch;

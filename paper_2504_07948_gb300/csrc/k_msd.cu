@@ -794,7 +794,7 @@ template <typename T>
 cudaError_t launch_sweep_msd(const DevSys& s, const DevWalkers& wk, int W, const SweepParams& p, cudaStream_t st) {
     if (W == 0) return cudaSuccess;
     const size_t smem = msd_sweep_smem_bytes<T>(s);
-    cudaError_t e = cudaFuncSetAttribute(k_sweep_msd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_sweep_msd<T>, smem);
     if (e != cudaSuccess) return e;
     k_sweep_msd<T><<<W, 256, smem, st>>>(s, wk, W, p);
     return cudaGetLastError();
@@ -825,7 +825,7 @@ cudaError_t launch_msd_eloc(const DevSys& s, const DevWalkers& wk, int W, double
     };
     if (bytes() > 227 * 1024) n_tile = std::max(3 * nv, nmax);
     const size_t smem = bytes();
-    cudaError_t e = cudaFuncSetAttribute(k_msd_eloc<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_msd_eloc<T>, smem);
     if (e != cudaSuccess) return e;
     k_msd_eloc<T><<<W, 256, smem, st>>>(s, wk, W, eloc, logpsi, sign, grad, n_tile);
     return cudaGetLastError();

@@ -1003,7 +1003,7 @@ cudaError_t launch_nlpp(const DevSys& s, const DevWalkers& wk, int w0, int W, do
     }
     if (smem > 227 * 1024) return cudaErrorNotSupported;   // the host reports QMC_ERR_UNSUPPORTED
     auto f = ug ? k_nlpp<T, kNlEnergy, true> : k_nlpp<T, kNlEnergy, false>;
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(f, smem);
     if (e != cudaSuccess) return e;
     // slices until there are six waves of CTAs, while each still has a warp's
     // worth of electrons (a slice repeats the rotations and positions)
@@ -1033,7 +1033,7 @@ cudaError_t launch_nlpp_param(const DevSys& s, const DevWalkers& wk, int w0, int
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn, P = 4 + s.n_nuc * (1 + s.n3);
     const size_t smem = nl_layout<T>(s.N, nmax, s.n_basis, s.n_ecp, s.n_shell, s.n_nuc, kNlParam, P, false, s.pp_nq).total;
     if (smem > 227 * 1024) return cudaErrorNotSupported;   // the host reports QMC_ERR_UNSUPPORTED
-    cudaError_t e = cudaFuncSetAttribute(k_nlpp<T, kNlParam>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_nlpp<T, kNlParam>, smem);
     if (e != cudaSuccess) return e;
     k_nlpp<T, kNlParam><<<W - w0, kNlThreads, smem, st>>>(s, wk, w0, W, deloc, key, sweep, (const T*)U0, (const T*)U1,
                                                          nullptr, nullptr, nullptr);
@@ -1049,7 +1049,7 @@ cudaError_t launch_nlpp_force(const DevSys& s, const DevWalkers& wk, int w0, int
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
     const size_t smem = nl_layout<T>(s.N, nmax, s.n_basis, s.n_ecp, s.n_shell, s.n_nuc, kNlForce, 0, false, s.pp_nq).total;
     if (smem > 227 * 1024) return cudaErrorNotSupported;   // the host reports QMC_ERR_UNSUPPORTED
-    cudaError_t e = cudaFuncSetAttribute(k_nlpp<T, kNlForce>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_nlpp<T, kNlForce>, smem);
     if (e != cudaSuccess) return e;
     k_nlpp<T, kNlForce><<<W - w0, kNlThreads, smem, st>>>(s, wk, w0, W, nullptr, key, sweep, (const T*)U0,
                                                          (const T*)U1, (T*)nlB0, (T*)nlB1, nlF);

@@ -47,7 +47,7 @@ template <int kNt>
 static cudaError_t launch_sweep64(const DevSys& s, const DevWalkers& wk, int W, const SweepParams& p, size_t smem,
                                   cudaStream_t st) {
     const auto f = s.n3 > 0 ? k_sweep64<kNt, true> : k_sweep64<kNt, false>;
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(f, smem);
     if (e != cudaSuccess) return e;
     f<<<W, kNt, smem, st>>>(s, wk, W, p);
     return cudaGetLastError();
@@ -57,7 +57,7 @@ static cudaError_t launch_sweep64(const DevSys& s, const DevWalkers& wk, int W, 
 template <typename T, int kNt>
 static cudaError_t launch_sweep_j3(const DevSys& s, const DevWalkers& wk, int W, const SweepParams& p,
                                   const int* n_live, size_t smem, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(k_sweep<T, kNt, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_sweep<T, kNt, true>, smem);
     if (e != cudaSuccess) return e;
     k_sweep<T, kNt, true><<<W, kNt, smem, st>>>(s, wk, W, p, n_live);
     return cudaGetLastError();
@@ -84,11 +84,11 @@ cudaError_t launch_sweep(const DevSys& s, const DevWalkers& wk, int W, const Swe
         return nmax > 64 ? launch_sweep_j3<T, 256>(s, wk, W, p, n_live, smem, st)
                          : launch_sweep_j3<T, 128>(s, wk, W, p, n_live, smem, st);
     if (nmax > 64) {
-        cudaError_t e = cudaFuncSetAttribute(k_sweep<T, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(k_sweep<T, 256>, smem);
         if (e != cudaSuccess) return e;
         k_sweep<T, 256><<<W, 256, smem, st>>>(s, wk, W, p, n_live);
     } else {
-        cudaError_t e = cudaFuncSetAttribute(k_sweep<T, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(k_sweep<T, 128>, smem);
         if (e != cudaSuccess) return e;
         k_sweep<T, 128><<<W, 128, smem, st>>>(s, wk, W, p, n_live);
     }

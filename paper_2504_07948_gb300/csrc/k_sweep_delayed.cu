@@ -444,7 +444,7 @@ cudaError_t launch_sweep_delayed(const DevSys& s, const DevWalkers& wk, int W, c
                                  cudaStream_t st) {
     if (W == 0 || s.N == 0) return cudaSuccess;
     const size_t smem = delayed_smem_bytes<T>(s, kmax);
-    cudaError_t e = cudaFuncSetAttribute(k_sweep_delayed<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_sweep_delayed<T>, smem);
     if (e != cudaSuccess) return e;
     k_sweep_delayed<T><<<W, 256, smem, st>>>(s, wk, W, p, kmax);
     return cudaGetLastError();
@@ -500,7 +500,7 @@ template <typename T>
 int sweep_batch_prepare(int block, size_t smem, int delayed) {
     int nb = 0;
     const void* f = delayed ? (const void*)k_sweep_batch<T, true> : (const void*)k_sweep_batch<T, false>;
-    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+    if (allow_smem(f, smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, block, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;

@@ -291,7 +291,7 @@ static cudaError_t launch_tc_gemm_staged(int batch, int M, int N, int K, const f
     if (batch <= 0 || M <= 0 || N <= 0) return cudaSuccess;
     if (N > kTcMaxN || K < 0) return cudaErrorInvalidValue;
     const size_t smem = tc_gemm_smem_bytes(N);
-    cudaError_t e = cudaFuncSetAttribute(k_tc_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_tc_gemm, smem);
     if (e != cudaSuccess) return e;
     k_tc_gemm<<<dim3((M + kTcM - 1) / kTcM, batch), 256, smem, st>>>(M, N, K, A, sA, lda, B, sB, ldb, b_trans, D, sD,
                                                                      ldd, err);
@@ -902,7 +902,7 @@ cudaError_t launch_tc_gemm_ab(int batch, int M, int N, int K, float alpha, const
                               : make_map(&tb, B, K, N, ldb, sB, batch, kPK, Np);
     if (!ok_b) return cudaErrorNotSupported;
     const PipeSmem L = pipe_layout(Np);
-    cudaError_t e = cudaFuncSetAttribute(k_tc_gemm_pipe, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
+    cudaError_t e = allow_smem(k_tc_gemm_pipe, L.total);
     if (e != cudaSuccess) return e;
     // persistent: as many CTAs as are resident at once (tensor memory: two
     // accumulators of up to 256 columns each fit one CTA per SM at N > 128)
@@ -964,10 +964,6 @@ bool tc_split_plan(TcSplitPlan* p, int M, int N, int K, const float* Ah, const f
            make_map_sw128(reinterpret_cast<CUtensorMap*>(p->map[1]), Al, K, M, lda, kTcM) &&
            make_map_sw128(reinterpret_cast<CUtensorMap*>(p->map[2]), Bh, K, N, ldb, Np) &&
            make_map_sw128(reinterpret_cast<CUtensorMap*>(p->map[3]), Bl, K, N, ldb, Np);
-}
-
-cudaError_t tc_split_prepare() {
-    return cudaFuncSetAttribute(k_tc_gemm_split, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448 - 2048);
 }
 
 cudaError_t launch_tc_gemm_split(const TcSplitPlan& p, float* D, int ldd, unsigned* err, cudaStream_t st, bool after) {

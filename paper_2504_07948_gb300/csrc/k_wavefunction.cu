@@ -837,10 +837,7 @@ cudaError_t launch_jastrow_derivs(const DevSys& s, const double* R, const double
                                   double* deloc, cudaStream_t st) {
     if (W == 0) return cudaSuccess;
     const size_t smem = sizeof(double) * (6 * (size_t)s.N + 2 * (size_t)s.n_nuc);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_jastrow_derivs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_smem(k_jastrow_derivs, smem)) return e;
     k_jastrow_derivs<<<W, 256, smem, st>>>(s, R, G, W, dlog, deloc);
     return cudaGetLastError();
 }
@@ -874,11 +871,7 @@ cudaError_t launch_orbitals_all(const DevSys& s, const DevWalkers& wk, int W, cu
     if (W == 0 || s.N == 0) return cudaSuccess;
     if (sums || !orbitals_fx(s)) {
         const size_t smem = sizeof(double) * 5 * s.n_basis + (size_t)s.n_shell;
-        if (smem > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(k_orbitals_sums<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)smem);
-            if (e != cudaSuccess) return e;
-        }
+        if (const cudaError_t e = allow_smem(k_orbitals_sums<T>, smem)) return e;
         k_orbitals_sums<T><<<dim3(W, s.N), s.n_up > 32 ? 256 : 128, smem, st>>>(s, wk, W, only);
         return cudaGetLastError();
     }
@@ -891,11 +884,7 @@ cudaError_t launch_orbitals_all(const DevSys& s, const DevWalkers& wk, int W, cu
     // 2.76 -> 2.09 ms.  (At 20 orbitals 64 are ahead as well, 2.32 -> 1.88 ms for
     // 2048 walkers: the line could lie higher.)
     const int nt = nmax > 128 ? (nmax > 256 ? 256 : (nmax + 31) & ~31) : nmax > 16 ? 128 : 64;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_orbitals_all<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_smem(k_orbitals_all<T>, smem)) return e;
     k_orbitals_all<T><<<dim3(W, s.N), nt, smem, st>>>(s, wk, W, only);
     return cudaGetLastError();
 }
@@ -905,7 +894,7 @@ cudaError_t launch_invert(const DevSys& s, const DevWalkers& wk, int W, int stor
     if (W == 0) return cudaSuccess;
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
     const size_t smem = invert_smem_bytes(s, !sums);
-    cudaError_t e = cudaFuncSetAttribute(k_invert, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_invert, smem);
     if (e != cudaSuccess) return e;
     const int nt = nmax > 64 ? 512 : (nmax > 16 ? 256 : 128);
     k_invert<<<dim3(W, 2), nt, smem, st>>>(s, wk, W, store_fp32, !sums && orbitals_fx(s), err, only);
@@ -918,10 +907,7 @@ cudaError_t launch_eloc(const DevSys& s, const DevWalkers& wk, int W, double* el
     if (W == 0) return cudaSuccess;
     const int nt = std::min(kElocThreads, 2 * ((s.N + 31) & ~31));
     const size_t smem = eloc_smem_bytes(s, nt, sizeof(T));
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_eloc<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_smem(k_eloc<T>, smem)) return e;
     k_eloc<T><<<W, nt, smem, st>>>(s, wk, W, eloc_out, logpsi, grad, lap, err);
     return cudaGetLastError();
 }
@@ -1023,7 +1009,7 @@ int wf_batch_prepare(int family, int block, size_t smem) {
         case 4: f = (const void*)k_eloc_batch<float>; break;
         default: return 0;
     }
-    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+    if (allow_smem(f, smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, block, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;

@@ -1097,7 +1097,6 @@ struct qmc_ctx {
                                       tiled.Bl + off, tiled.nbp, tiled.Cth[spin], tiled.Ctl[spin], tiled.nbp),
                         QMC_ERR_UNSUPPORTED, "tensor maps of the tiled sweep's orbital GEMM could not be encoded");
             }
-        QMC_CK(tc_split_prepare());
         cudaEvent_t t0 = tm.mark(stream);
         int launches = 1;
         QMC_CK(tiled_begin(k, W, N(), tiled, stream));
@@ -3168,7 +3167,7 @@ int qmc_tc_gemm_split(int M, int N, int K, const float* A_hi, const float* A_lo,
     TcSplitPlan plan;
     if (!tc_split_plan(&plan, M, N, K, A_hi, A_lo, lda, B_hi, B_lo, ldb)) return QMC_ERR_UNSUPPORTED;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    if (tc_split_prepare() != cudaSuccess || launch_tc_gemm_split(plan, D, ldd, d_flag[dev], st) != cudaSuccess)
+    if (launch_tc_gemm_split(plan, D, ldd, d_flag[dev], st) != cudaSuccess)
         return QMC_ERR_CUDA;
     unsigned f = 0;
     if (cudaMemcpyAsync(&f, d_flag[dev], sizeof(unsigned), cudaMemcpyDeviceToHost, st) != cudaSuccess ||

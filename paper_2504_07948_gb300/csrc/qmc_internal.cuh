@@ -1318,6 +1318,27 @@ __device__ __forceinline__ float warp_sum(float v) {
 }
 
 
+// Lets a kernel be launched with smem bytes of dynamic shared memory.  The limit
+// goes to all that an SM has beside the kernel's static memory and stays there: set
+// to the size of each launch, a smaller system (another handle's, a batch
+// created later, another thread between this call and its launch) took the limit
+// of a larger one away.
+inline cudaError_t allow_smem(const void* f, size_t smem) {
+    if (smem <= 36 * 1024) return cudaSuccess;   // within the default limit, static memory included
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, f);
+    if (e != cudaSuccess) return e;
+    const int top = 227 * 1024 - (int)a.sharedSizeBytes;
+    if (smem > (size_t)top) return cudaErrorInvalidValue;
+    return a.maxDynamicSharedSizeBytes >= top
+               ? cudaSuccess
+               : cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, top);
+}
+template <typename... P>
+inline cudaError_t allow_smem(void (*f)(P...), size_t smem) {
+    return allow_smem((const void*)f, smem);
+}
+
 // Streaming multiprocessors of the current device.
 inline int device_sms() {
     int dev = 0, n = 152;
@@ -1337,10 +1358,7 @@ __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.la
 template <typename... P, typename... A>
 inline cudaError_t launch_after(void (*f)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, bool after,
                                 A&&... args) {
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_smem(f, smem)) return e;
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
@@ -1462,15 +1480,13 @@ cudaError_t launch_tc_gemm(int batch, int M, int N, int K, const float* A, long 
 // D = A B^T for operands given as TF32 hi / lo pairs ([M][K] and [N][K],
 // row strides lda, ldb, 16-byte aligned): the tensor maps are encoded once
 // by tc_split_plan (false when TMA cannot describe the operands) and the
-// launch reuses them; tc_split_prepare sets the kernel's shared-memory limit
-// (call it outside any stream capture).
+// launch reuses them.
 struct alignas(64) TcSplitPlan {
     unsigned char map[4][128];   // CUtensorMap of A_hi, A_lo, B_hi, B_lo
     int M, N, K, Np;             // Np: columns of a tile
 };
 bool tc_split_plan(TcSplitPlan* p, int M, int N, int K, const float* Ah, const float* Al, int lda, const float* Bh,
                    const float* Bl, int ldb);
-cudaError_t tc_split_prepare();
 // after: the launch may start before the kernel ahead of it ends (launch_after)
 cudaError_t launch_tc_gemm_split(const TcSplitPlan& p, float* D, int ldd, unsigned* err, cudaStream_t st,
                                  bool after = false);
