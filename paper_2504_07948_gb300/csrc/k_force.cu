@@ -771,11 +771,11 @@ __device__ __forceinline__ void force_walker(const DevSys& s, const DevWalkers& 
 // form keeps two (at three it spills).
 template <typename T, bool kE, int kNt>
 __global__ void __launch_bounds__(kNt, kNt == 512 ? 1 : sizeof(T) == 4 ? 3 : 2)
-    k_force(DevSys s, DevWalkers wk, int w0, int W, const int* only, const double* dvnn, double* Bscr, double* Pscr,
-            double* dEL, double* dlog, double* gEdet, double* gtot) {
+    k_force(DevSys s, DevWalkers wk, int W, const double* dvnn, double* Bscr, double* Pscr, double* dEL, double* dlog,
+            double* gEdet, double* gtot) {
     extern __shared__ double sm[];
-    if ((int)blockIdx.x >= W || (only && !only[blockIdx.x])) return;
-    const int w = w0 + blockIdx.x;
+    const int w = blockIdx.x;
+    if (w >= W) return;
     force_walker<T, kE>(s, wk, w, dvnn, Bscr, Pscr, dEL, dlog, sm, gEdet, gtot);
 }
 
@@ -794,8 +794,9 @@ __global__ void __launch_bounds__(kNt, kNt == 512 ? 1 : sizeof(T) == 4 ? 3 : 2)
 // its electron's row of B as soon as that electron's grad J is summed, so the
 // gradient cache is read from memory once (32-water cluster, 512 walkers, mixed:
 // 495 -> 398 us).
-// lossy (FP64 form): [W], whether some electron's row of A^-T weighs small entries
-// of B up (row_short): the walker's products are not left to bf16 digits then.
+// lossy (FP64 form): count (zero before the launch), then the walkers of the
+// launch in which some electron's row of A^-T weighs small entries of B up
+// (row_short): their products are not left to bf16 digits (k_force_products).
 template <typename T, bool kE>
 __global__ void k_force_prep(DevSys s, DevWalkers wk, int w0, int W, const double* dvnn, T* Bw, double* gJw,
                              double* accw, double* gtot, int* lossy) {
@@ -826,12 +827,106 @@ __global__ void k_force_prep(DevSys s, DevWalkers wk, int w0, int W, const doubl
     });
     if constexpr (sizeof(T) == 8) {
         low = __syncthreads_or(low);
-        if (threadIdx.x == 0) lossy[wl] = low;
+        if (threadIdx.x == 0 && low) lossy[1 + atomicAdd(lossy, 1)] = wl;
     }
     for (int q = threadIdx.x; q < 3 * N; q += blockDim.x) gJw[(size_t)wl * 3 * N + q] = double(h.gJ[q]);
     for (int q = threadIdx.x; q < 6 * nn; q += blockDim.x) accw[(size_t)wl * 6 * nn + q] = h.acc[q];
     if constexpr (kE)
         for (int q = threadIdx.x; q < 3 * N; q += blockDim.x) gtot[(size_t)w * 3 * N + q] = double(h.gt[q]);
+}
+
+// The four products of the listed walkers in FP64, in place of those that the
+// digits gave: stage 0 PT = AT B^T and M = C AT^T, 1 Q = PT AT, 2 Y = C Q^T.  Few
+// walkers, so each is spread over the chip: persistent CTAs over 32 x 32 tiles of
+// every listed walker and spin (a launch that finds none takes 2 us; one CTA a
+// walker by the fused kernel took 3 ms at 70 electrons per spin).  Bound by the FP64
+// pipe: four sums a thread, operands through shared memory.
+constexpr int kPt = 32;
+struct ProductArgs {
+    const double *AT[2], *C[2];                 // [wc][n][n] of the chunk, [n_basis][n]
+    double *B, *PT, *Q, *M, *Y;                 // [spin][wc][nmax^2] and [spin][wc] n_basis nmax
+    int n[2], nmax, nb, wc;
+};
+__global__ void __launch_bounds__(256) k_force_products(ProductArgs p, int stage, const int* lossy) {
+    __shared__ double sa[kPt][kPt + 1], sb[kPt][kPt + 1];
+    const int count = lossy[0];
+    const int tn[2] = {(p.n[0] + kPt - 1) / kPt, (p.n[1] + kPt - 1) / kPt}, tb = (p.nb + kPt - 1) / kPt;
+    // tiles per walker and spin: n x n in stages 0 and 1, n_basis x n in 0 and 2
+    auto tiles = [&](int s) { return (stage < 2 ? tn[s] * tn[s] : 0) + (stage != 1 ? tb * tn[s] : 0); };
+    const int per = tiles(0) + tiles(1);
+    const int c = threadIdx.x & 31, r0 = threadIdx.x >> 5;   // column, first of four rows
+    for (int it = blockIdx.x; it < count * per; it += gridDim.x) {
+        const int wl = lossy[1 + it / per];
+        int t = it % per;
+        const int s = t >= tiles(0);
+        if (s) t -= tiles(0);
+        const int n = p.n[s];
+        const size_t sq = ((size_t)s * p.wc + wl) * p.nmax * p.nmax;
+        const size_t bn = (size_t)s * p.wc * p.nb * p.nmax + (size_t)wl * p.nb * n;
+        const double* AT = p.AT[s] + (size_t)wl * n * n;
+        const bool square = stage < 2 && t < tn[s] * tn[s];
+        if (stage == 0 && !square) t -= tn[s] * tn[s];
+        const double *a = p.C[s], *b = stage == 0 ? AT : p.Q + sq;   // rows of both factors: M, Y
+        double* d = (stage == 0 ? p.M : p.Y) + bn;
+        int rows = p.nb;
+        if (square) {
+            a = stage == 0 ? AT : p.PT + sq;
+            b = stage == 0 ? p.B + sq : AT;
+            d = (stage == 0 ? p.PT : p.Q) + sq;
+            rows = n;
+        }
+        const int i0 = t / tn[s] * kPt, j0 = t % tn[s] * kPt;
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int k0 = 0; k0 < n; k0 += kPt) {
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int r = r0 + 8 * u;
+                sa[r][c] = i0 + r < rows && k0 + c < n ? a[(size_t)(i0 + r) * n + k0 + c] : 0.0;
+                // sb[j][k]: b's rows are the output's columns, in stage 1 its columns are
+                if (stage == 1)
+                    sb[c][r] = k0 + r < n && j0 + c < n ? b[(size_t)(k0 + r) * n + j0 + c] : 0.0;
+                else
+                    sb[r][c] = j0 + r < n && k0 + c < n ? b[(size_t)(j0 + r) * n + k0 + c] : 0.0;
+            }
+            __syncthreads();
+#pragma unroll 8
+            for (int k = 0; k < kPt; ++k) {
+                const double bv = sb[c][k];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) acc[u] += sa[r0 + 8 * u][k] * bv;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int r = i0 + r0 + 8 * u;
+            if (r < rows && j0 + c < n) d[(size_t)r * n + j0 + c] = acc[u];
+        }
+    }
+}
+
+cudaError_t launch_force_products(const DevSys& s, const DevWalkers& wk, int w0, int wc, double* B, double* PT, double* Q,
+                                  double* M, double* Y, const int* lossy, cudaStream_t st) {
+    ProductArgs p{};
+    for (int spin = 0; spin < 2; ++spin) {
+        p.n[spin] = spin ? s.n_dn : s.n_up;
+        p.AT[spin] = (const double*)wk.Ainv[spin] + (size_t)w0 * p.n[spin] * p.n[spin];
+        p.C[spin] = s.C[spin];
+    }
+    p.B = B;
+    p.PT = PT;
+    p.Q = Q;
+    p.M = M;
+    p.Y = Y;
+    p.nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
+    p.nb = s.n_basis;
+    p.wc = wc;
+    for (int stage = 0; stage < 3; ++stage) {
+        k_force_products<<<4 * device_sms(), 256, 0, st>>>(p, stage, lossy);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // CTAs per walker of k_force_contract: each takes a range of nuclei (the
@@ -1000,12 +1095,11 @@ template cudaError_t launch_force_contract<float>(const DevSys&, const DevWalker
                                                   const double*, const double*, double*, double*, double*,
                                                   cudaStream_t);
 
-// Walkers w0 .. w0 + W - 1, with only ([W]) those whose flag is set.
-// gEdet, gtot (both null, or both [.][N][3]): the space-warp form's
+// gEdet, gtot (both null, or both [W][N][3]): the space-warp form's
 // per-electron outputs (see force_walker).
 template <typename T>
-cudaError_t launch_force(const DevSys& s, const DevWalkers& wk, int w0, int W, const int* only, const double* dvnn,
-                         double* Bscr, double* Pscr, double* dEL, double* dlog, double* gEdet, double* gtot, cudaStream_t st) {
+cudaError_t launch_force(const DevSys& s, const DevWalkers& wk, int W, const double* dvnn, double* Bscr,
+                         double* Pscr, double* dEL, double* dlog, double* gEdet, double* gtot, cudaStream_t st) {
     if (W == 0) return cudaSuccess;
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
     const bool kE = gEdet != nullptr;
@@ -1015,7 +1109,7 @@ cudaError_t launch_force(const DevSys& s, const DevWalkers& wk, int w0, int W, c
                             : (kE ? k_force<T, true, 256> : k_force<T, false, 256>);
     cudaError_t e = allow_smem(f, smem);
     if (e != cudaSuccess) return e;
-    f<<<W, 32 * nw, smem, st>>>(s, wk, w0, W, only, dvnn, Bscr, Pscr, dEL, dlog, gEdet, kE ? gtot : nullptr);
+    f<<<W, 32 * nw, smem, st>>>(s, wk, W, dvnn, Bscr, Pscr, dEL, dlog, gEdet, kE ? gtot : nullptr);
     return cudaGetLastError();
 }
 
@@ -1309,9 +1403,9 @@ template cudaError_t launch_force_batch<double>(const BatchSys*, BatchPlan*, int
 template cudaError_t launch_force_batch<float>(const BatchSys*, BatchPlan*, int, int, int, size_t, int, int,
                                                cudaStream_t);
 
-template cudaError_t launch_force<double>(const DevSys&, const DevWalkers&, int, int, const int*, const double*, double*, double*,
+template cudaError_t launch_force<double>(const DevSys&, const DevWalkers&, int, const double*, double*, double*,
                                           double*, double*, double*, double*, cudaStream_t);
-template cudaError_t launch_force<float>(const DevSys&, const DevWalkers&, int, int, const int*, const double*, double*, double*,
+template cudaError_t launch_force<float>(const DevSys&, const DevWalkers&, int, const double*, double*, double*,
                                          double*, double*, double*, double*, cudaStream_t);
 
 }  // namespace qmc

@@ -20,8 +20,8 @@
 // K times that for the sum, some 2^-55 sqrt(K) with digits of random sign.  An
 // FP64 chain is off by 2^-53 of each of its partial sums instead, which is more
 // where the terms come near the product of the maxima and less where they lie far
-// below it; k_force_prep finds the walkers with such rows, and launch_force takes
-// them in FP64.  Elsewhere the error of A^-1 sets that of the derivatives: against
+// below it; k_force_prep finds the walkers with such rows, and k_force_products
+// takes them in FP64.  Elsewhere the error of A^-1 sets that of the derivatives: against
 // extended precision both paths, this one and FP64 GEMMs, give the same to all
 // digits shown (14 to 32 waters, electrons up to 12 bohr out, orbitals scaled by
 // 10^-9 to 10^9).

@@ -1272,7 +1272,7 @@ struct qmc_ctx {
                 d_fY = dalloc<T>(wk_allocs, 2 * (size_t)fc * nb * nmax);
                 d_fgJ = dalloc<double>(wk_allocs, (size_t)fc * N3);
                 d_faccw = dalloc<double>(wk_allocs, (size_t)fc * 6 * nn);
-                d_flossy = dalloc<int>(wk_allocs, fc);
+                d_flossy = dalloc<int>(wk_allocs, (size_t)fc + 1);
                 if (kFp64) {
                     // rows the tiles read: 128 of a left operand, 64 of a right one
                     const int n8 = (nmax + 7) / 8 * 8, rl = (nmax + 127) / 128 * 128, rr = (nmax + 63) / 64 * 64;
@@ -1303,6 +1303,7 @@ struct qmc_ctx {
         const DevWalkers& k = kw;
         for (int w0 = 0; w0 < W; w0 += Wc) {
             const int wc = std::min(Wc, W - w0);
+            if (kFp64) QMC_CK(cudaMemsetAsync(d_flossy, 0, sizeof(int), stream));
             QMC_CK(launch_force_prep<T>(ds, k, w0, wc, d_dvnn, d_fB, d_fgJ, d_faccw, d_gtot, d_flossy, stream));
             for (int spin = 0; spin < 2; ++spin) {
                 const int n = spin ? n_dn : n_up;
@@ -1355,12 +1356,12 @@ struct qmc_ctx {
                     gemm_sb<T>(CUBLAS_OP_T, CUBLAS_OP_N, n, nb, n, Q, n, nn2, Cs, n, 0, Y, n, (long long)nb * n, wc);
                 }
             }
+            // walkers that the digits would cost bits
+            if (kFp64)
+                QMC_CK(launch_force_products(ds, k, w0, wc, (double*)d_fB, (double*)d_fPT, (double*)d_fQ, (double*)d_fM,
+                                             (double*)d_fY, d_flossy, stream));
             QMC_CK(launch_force_contract<T>(ds, k, w0, wc, d_fM, d_fY, d_fgJ, d_faccw, d_dEL, d_dlog, d_gEdet,
                                             stream));
-            // walkers that fixed-point products would cost bits
-            if (kFp64)
-                QMC_CK(launch_force<T>(ds, k, w0, wc, d_flossy, d_dvnn, d_Bscr, d_Pscr, d_dEL, d_dlog, d_gEdet, d_gtot,
-                                       stream));
         }
     }
 
@@ -1430,9 +1431,9 @@ struct qmc_ctx {
         } else {
             tm.begin(stream);
             if (mode == QMC_MIXED) {
-                QMC_CK(launch_force<float>(ds, k, 0, W, nullptr, d_dvnn, d_Bscr, d_Pscr, d_dEL, d_dlog, gE, gt, stream));
+                QMC_CK(launch_force<float>(ds, k, W, d_dvnn, d_Bscr, d_Pscr, d_dEL, d_dlog, gE, gt, stream));
             } else {
-                QMC_CK(launch_force<double>(ds, k, 0, W, nullptr, d_dvnn, d_Bscr, d_Pscr, d_dEL, d_dlog, gE, gt, stream));
+                QMC_CK(launch_force<double>(ds, k, W, d_dvnn, d_Bscr, d_Pscr, d_dEL, d_dlog, gE, gt, stream));
             }
             tm.end(F_FORCE, 1, stream);
         }

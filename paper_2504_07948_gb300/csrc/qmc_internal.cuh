@@ -1438,15 +1438,16 @@ cudaError_t launch_sweep_delayed(const DevSys& s, const DevWalkers& wk, int W, c
                                  cudaStream_t st);
 // Ionic derivatives (k_force.cu).  gEdet, gtot: null, or the space-warp
 // form's per-electron outputs [W][N][3] (determinant part of dE_L/dr_i and
-// grad_i ln|psi|), consumed by launch_space_warp.  Walkers w0 .. w0 + W - 1,
-// with only ([W]) those whose flag is set; lossy ([W], FP64 form): walkers whose
-// products launch_force has to take.
+// grad_i ln|psi|), consumed by launch_space_warp.  lossy ([1 + W], FP64 form):
+// number and list of the walkers whose products launch_force_products takes.
 template <typename T>
-cudaError_t launch_force(const DevSys& s, const DevWalkers& wk, int w0, int W, const int* only, const double* dvnn,
-                         double* Bscr, double* Pscr, double* dEL, double* dlog, double* gEdet, double* gtot, cudaStream_t st);
+cudaError_t launch_force(const DevSys& s, const DevWalkers& wk, int W, const double* dvnn, double* Bscr,
+                         double* Pscr, double* dEL, double* dlog, double* gEdet, double* gtot, cudaStream_t st);
 template <typename T>
 cudaError_t launch_force_prep(const DevSys& s, const DevWalkers& wk, int w0, int W, const double* dvnn, void* Bw,
                               double* gJw, double* accw, double* gtot, int* lossy, cudaStream_t st);
+cudaError_t launch_force_products(const DevSys& s, const DevWalkers& wk, int w0, int wc, double* B, double* PT, double* Q,
+                                  double* M, double* Y, const int* lossy, cudaStream_t st);
 template <typename T>
 cudaError_t launch_force_contract(const DevSys& s, const DevWalkers& wk, int w0, int W, const void* Mw, const void* Yw,
                                   const double* gJw, const double* accw, double* dEL, double* dlog, double* gEdet,
