@@ -160,11 +160,14 @@ __global__ void k_orbitals_sums(DevSys s, DevWalkers wk, int W, const int* only)
 // with orbitals of their own.  So the inverse is held against its rows:
 // with x = A^-1 e_i, a row whose max|x_j| c_j max|A_ij / c_j| exceeds max|x_j
 // A_ij| by more than kFxSlack bits would lose accuracy against FP64 sums (their
-// error is some 2^-54 sqrt(rows) of the latter), and the orbitals of the spin's
-// electrons are taken again that way, as they are for a singular matrix.  On water
-// clusters with dense orbitals (1 to 32 waters) no row comes above 4 bits; with two
-// waters 11 bohr apart, six electrons of a spin on one of them, the rows
-// concerned stand at 8 to 20.
+// error is some 2^-54 sqrt(rows) of the latter).  The orbitals of such rows are
+// taken again that way (of all rows, if the matrix is singular) and the matrix is
+// inverted again, until no further row stands out.  On water clusters with dense
+// orbitals (1 to 32 waters) no row comes above 4 bits; with orbitals of a model
+// Hamiltonian one or two in a hundred pass 6, and with two waters 11 bohr apart, six
+// electrons of a spin on one of them, the rows concerned stand at 8 to 20.  Left to
+// fixed point, the model orbitals' E_L and gradients at 14 waters had 2 to 7
+// times the error of FP64 sums, now the same.
 
 // Pivot of column k from row k on (warp 0): row, value and reciprocal.
 __device__ __forceinline__ void find_pivot(const double* M, int n, int k, int* s_piv, double* s_val, double* s_pinv,
@@ -198,12 +201,14 @@ __device__ __forceinline__ void find_pivot(const double* M, int n, int k, int* s
     }
 }
 
-// The orbitals of the electrons of one spin as FP64 sums, by the whole CTA; ends
-// synchronised.  sm: 5 n_basis doubles and n_shell bytes of shared memory.
-__device__ __noinline__ void orbitals_again(const DevSys& s, const DevWalkers& wk, int w, int spin, int fp32, double* sm) {
+// The orbitals of one spin's electrons k with rows[k] as FP64 sums, by the whole
+// CTA; ends synchronised.  sm: 5 n_basis doubles and n_shell bytes of shared memory.
+__device__ __noinline__ void orbitals_again(const DevSys& s, const DevWalkers& wk, int w, int spin, int fp32,
+                                            const int* rows, double* sm) {
     const int i0 = spin ? s.n_up : 0, n = spin ? s.n_dn : s.n_up;
     unsigned char* live = reinterpret_cast<unsigned char*>(sm + 5 * s.n_basis);
     for (int k = 0; k < n; ++k) {
+        if (!rows[k]) continue;
         if (fp32)
             orbitals_sums_item<float>(s, wk, w, i0 + k, sm, live);
         else
@@ -213,25 +218,52 @@ __device__ __noinline__ void orbitals_again(const DevSys& s, const DevWalkers& w
 }
 
 // Whether row i of A (global memory) leaves the inverse x[j] = M[j n + c] short
-// of bits if taken in fixed point (see above).
+// of bits if taken in fixed point (see above); by one warp.
 __device__ __forceinline__ bool row_short(const double* A, const double* M, const double* __restrict__ sC, int n, int i,
                                           int c) {
-    int am = 0, rs = -0x10000, rf = 0;   // biased exponents: max|x_j| c_j, max|A_ij| / c_j, max|x_j A_ij|
-#pragma unroll 8
-    for (int j = 0; j < n; ++j) {
+    int am = 0, rs = 0, rf = 0;   // biased exponents: max|x_j| c_j, max|A_ij| / c_j, max|x_j A_ij|
+    for (int j = threadIdx.x & 31; j < n; j += 32) {
         const int ea = fx_expo(A[(size_t)i * n + j]), ex = fx_expo(M[j * n + c]), ec = fx_expo(sC[j]);
         am = max(am, ex + ec);
-        if (ea) rs = max(rs, ea - ec);
+        if (ea) rs = max(rs, ea - ec + 4096);
         if (ea && ex) rf = max(rf, ea + ex);
     }
-    return am + rs - rf > kFxSlack;
+    return warp_max_u(am) + warp_max_u(rs) - 4096 - warp_max_u(rf) > kFxSlack;
+}
+
+constexpr int kInvertWarps = 16;   // at most; words of shrt per walker and spin
+
+// Rows of A that fall short (of a singular matrix all) and are not FP64 sums yet,
+// after the elimination: warp w looks at the rows w, w + nw, .. (at most 32) and
+// returns a bit for each.  summed: those that are.  perm: the columns of the
+// inverse in M.
+__device__ __forceinline__ int short_rows(const DevSys& s, const double* A, int n, int spin, int sing, int summed,
+                                          const int* perm, const double* M) {
+    const int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    int now = 0;
+    for (int i = wid, q = 0; i < n; i += nw, ++q)
+        if (!(summed >> q & 1) && (sing || row_short(A, M, s.Ck_s[spin], n, i, perm[i]))) now |= 1 << q;
+    return now;
+}
+
+// Takes the rows of these bits again; rows: n integers of shared memory.
+__device__ __noinline__ void take_rows(const DevSys& s, const DevWalkers& wk, int w, int spin, int fp32, int now, int* rows,
+                                       double* M) {
+    const int n = spin ? s.n_dn : s.n_up, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if ((threadIdx.x & 31) == 0)
+        for (int i = wid, q = 0; i < n; i += nw, ++q) rows[i] = now >> q & 1;
+    __syncthreads();
+    orbitals_again(s, wk, w, spin, fp32, rows, M);
 }
 
 // Inversion of one (walker, spin) matrix (body of k_invert).  M: n^2 + n
 // doubles of shared memory (invert_smem_bytes); at least n threads.  fx: A was
-// taken in fixed point.
+// taken in fixed point.  kAgain: takes short rows again and inverts until none is
+// left; now: rows to take before the first inversion (short_rows).  Without it the
+// rows are left to a launch that does: shrt (fx) receives the bits of each warp.
+template <bool kAgain>
 __device__ __forceinline__ void invert_item(const DevSys& s, const DevWalkers& wk, int w, int spin, int store_fp32, int fx,
-                                            unsigned* err, double* M) {
+                                            int now, int* shrt, unsigned* err, double* M) {
     __shared__ int s_perm[256];
     __shared__ double s_val, s_pinv;
     __shared__ int s_piv, s_sing, s_row[2];
@@ -250,7 +282,13 @@ __device__ __forceinline__ void invert_item(const DevSys& s, const DevWalkers& w
     const int sub = n <= 8 ? 8 : n <= 16 ? 16 : 32, nrow = 32 / sub, lr = lane / sub, lc = lane % sub;
     int cur = 0, swaps = 0, neg = 0;   // where this thread's column ends up; interchanges; negative pivots
     double piv = 0.0;                  // this thread's pivot
+    int summed = 0;                    // rows of A that are FP64 sums (short_rows)
     for (;;) {
+        if constexpr (kAgain)
+            if (__syncthreads_or(now)) {
+                take_rows(s, wk, w, spin, store_fp32, now, s_perm, M);
+                summed |= now;
+            }
         if (threadIdx.x == 0) {
             s_sing = 0;
             s_row[0] = s_row[1] = 0;
@@ -313,13 +351,15 @@ __device__ __forceinline__ void invert_item(const DevSys& s, const DevWalkers& w
             }
         neg = __syncthreads_count(neg);
         if (!fx) break;
-        fx = 0;
-        int again = s_sing;
-        for (int i = threadIdx.x; !again && i < n; i += blockDim.x) again = row_short(A, M, s.Ck_s[spin], n, i, s_perm[i]);
-        if (!__syncthreads_or(again)) break;
-        orbitals_again(s, wk, w, spin, store_fp32, M);
+        now = short_rows(s, A, n, spin, s_sing, summed, s_perm, M);
+        if (!kAgain) {
+            if (lane == 0) shrt[(2 * w + spin) * kInvertWarps + wid] = now;
+            break;
+        }
+        if (!__syncthreads_or(now)) break;
     }
     if (s_sing) {
+        if (!kAgain && fx) return;   // not settled: every row is taken again
         if (threadIdx.x == 0) {
             wk.logdet[2 * w + spin] = -INFINITY;
             wk.sgn[2 * w + spin] = 0.0;
@@ -349,11 +389,24 @@ __device__ __forceinline__ void invert_item(const DevSys& s, const DevWalkers& w
     }
 }
 
-__global__ void k_invert(DevSys s, DevWalkers wk, int W, int store_fp32, int fx, unsigned* err, const int* only) {
+__global__ void k_invert(DevSys s, DevWalkers wk, int W, int store_fp32, int* shrt, unsigned* err, const int* only) {
     extern __shared__ double M[];  // [n][n], then fcol[n]
     const int w = blockIdx.x, spin = blockIdx.y;
     if (w >= W || (only && !only[w])) return;
-    invert_item(s, wk, w, spin, store_fp32, fx, err, M);
+    invert_item<false>(s, wk, w, spin, store_fp32, shrt != nullptr, 0, shrt, err, M);
+}
+
+// The matrices with rows that k_invert found short, taken again.  A kernel of its
+// own: with this work the elimination would need 112 registers, where 40 leave
+// room for three CTAs of the large size on an SM.
+__global__ void __launch_bounds__(32 * kInvertWarps) k_invert_again(DevSys s, DevWalkers wk, int W, int store_fp32,
+                                                                    const int* shrt, unsigned* err, const int* only) {
+    extern __shared__ double M[];
+    const int w = blockIdx.x, spin = blockIdx.y;
+    if (w >= W || (only && !only[w]) || (spin ? s.n_dn : s.n_up) == 0) return;
+    const int now = shrt[(2 * w + spin) * kInvertWarps + (threadIdx.x >> 5)];
+    if (!__syncthreads_or(now)) return;
+    invert_item<true>(s, wk, w, spin, store_fp32, 1, now, nullptr, err, M);
 }
 
 // Local energy, ln|psi| and (optionally) grad / Laplacian of ln|psi| from
@@ -889,15 +942,19 @@ cudaError_t launch_orbitals_all(const DevSys& s, const DevWalkers& wk, int W, cu
     return cudaGetLastError();
 }
 
-cudaError_t launch_invert(const DevSys& s, const DevWalkers& wk, int W, int store_fp32, bool sums, unsigned* err,
+cudaError_t launch_invert(const DevSys& s, const DevWalkers& wk, int W, int store_fp32, int* shrt, unsigned* err,
                           cudaStream_t st, const int* only) {
     if (W == 0) return cudaSuccess;
+    if (!orbitals_fx(s)) shrt = nullptr;
     const int nmax = s.n_up > s.n_dn ? s.n_up : s.n_dn;
-    const size_t smem = invert_smem_bytes(s, !sums);
-    cudaError_t e = allow_smem(k_invert, smem);
-    if (e != cudaSuccess) return e;
+    const size_t smem = invert_smem_bytes(s, false), smem_again = invert_smem_bytes(s, true);
+    if (const cudaError_t e = allow_smem(k_invert, smem)) return e;
     const int nt = nmax > 64 ? 512 : (nmax > 16 ? 256 : 128);
-    k_invert<<<dim3(W, 2), nt, smem, st>>>(s, wk, W, store_fp32, !sums && orbitals_fx(s), err, only);
+    k_invert<<<dim3(W, 2), nt, smem, st>>>(s, wk, W, store_fp32, shrt, err, only);
+    if (!shrt) return cudaGetLastError();
+    if (const cudaError_t e = cudaGetLastError()) return e;
+    if (const cudaError_t e = allow_smem(k_invert_again, smem_again)) return e;
+    k_invert_again<<<dim3(W, 2), nt, smem_again, st>>>(s, wk, W, store_fp32, shrt, err, only);
     return cudaGetLastError();
 }
 
@@ -940,7 +997,7 @@ __global__ void k_orbitals_batch(const BatchSys* __restrict__ sys, BatchPlan* pl
     }
 }
 
-__global__ void k_invert_batch(const BatchSys* __restrict__ sys, BatchPlan* plan, int parity, int store_fp32,
+__global__ void __launch_bounds__(256, 5) k_invert_batch(const BatchSys* __restrict__ sys, BatchPlan* plan, int parity, int store_fp32,
                                int ctr) {
     extern __shared__ double M[];
     __shared__ BatchSys bs;
@@ -952,7 +1009,8 @@ __global__ void k_invert_batch(const BatchSys* __restrict__ sys, BatchPlan* plan
         if (q < 0) break;
         batch_load(&bs, sys + q);
         __syncthreads();
-        invert_item(bs.s, bs.wk[parity], s_idx >> 1, s_idx & 1, store_fp32, orbitals_fx(bs.s), bs.err, M);
+        invert_item<true>(bs.s, bs.wk[parity], s_idx >> 1, s_idx & 1, store_fp32, orbitals_fx(bs.s), 0, nullptr, bs.err,
+                          M);
         __syncthreads();
     }
 }

@@ -301,6 +301,7 @@ struct qmc_ctx {
     double* d_facc = nullptr;
     double* d_sign = nullptr;
     int* d_refresh = nullptr;   // per-walker "rebuild in FP64" flags (determinant expansions)
+    int* d_short = nullptr;     // rows that a rebuild takes again (launch_invert)
     double* d_fmsd = nullptr;   // per-walker scratch of the multi-determinant force kernel
     void* d_nlB = nullptr;      // per-walker non-local matrix rows of both spins (force pass)
     double* d_nlF = nullptr;    // per-walker direct non-local derivative terms
@@ -856,6 +857,7 @@ struct qmc_ctx {
         }
         d_sign = dalloc<double>(wk_allocs, cap);
         d_refresh = dalloc<int>(wk_allocs, cap);
+        d_short = dalloc<int>(wk_allocs, 32 * (size_t)cap);
         QMC_CK(cudaMemsetAsync(d_refresh, 0, sizeof(int) * cap, stream));
         wk[0].refresh = d_refresh;
         wk[1].refresh = d_refresh;
@@ -899,8 +901,8 @@ struct qmc_ctx {
         } else {
             QMC_CK(launch_orbitals_all<double>(ds, k, W, stream));
         }
-        QMC_CK(launch_invert(ds, k, W, mode == QMC_MIXED, mode == QMC_MIXED && fresh, d_err, stream));
-        int nk = 2;
+        QMC_CK(launch_invert(ds, k, W, mode == QMC_MIXED, mode == QMC_MIXED && fresh ? nullptr : d_short, d_err, stream));
+        int nk = mode == QMC_MIXED && fresh ? 2 : 3;   // (a basis beyond the lists takes two)
         if (ds.msd) {
             if (mode == QMC_MIXED) {
                 QMC_CK(launch_msd_table<float>(ds, k, W, stream));
@@ -1180,7 +1182,7 @@ struct qmc_ctx {
             } else {
                 QMC_CK(launch_orbitals_all<double>(ds, k, W, stream, d_refresh));
             }
-            QMC_CK(launch_invert(ds, k, W, mode == QMC_MIXED, mode == QMC_MIXED, d_err, stream, d_refresh));
+            QMC_CK(launch_invert(ds, k, W, mode == QMC_MIXED, mode == QMC_MIXED ? nullptr : d_short, d_err, stream, d_refresh));
             if (mode == QMC_MIXED) {
                 QMC_CK(launch_msd_table<float>(ds, k, W, stream, d_refresh));
             } else {

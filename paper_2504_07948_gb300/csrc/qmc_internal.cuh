@@ -1391,8 +1391,9 @@ cudaError_t launch_orbitals_all(const DevSys& s, const DevWalkers& wk, int W, cu
                                 const int* only = nullptr, bool sums = false);
 // only (optional, [W]): rebuild just the walkers whose flag is nonzero.
 // launch_orbitals_all, sums: FP64 sums in index order (see k_orbitals_sums).
-// (launch_invert: the orbitals came from it)
-cudaError_t launch_invert(const DevSys& s, const DevWalkers& wk, int W, int store_fp32, bool sums, unsigned* err,
+// launch_invert, shrt ([W][2][16]): scratch that marks rows whose fixed-point
+// orbitals fall short; null where the orbitals are FP64 sums.
+cudaError_t launch_invert(const DevSys& s, const DevWalkers& wk, int W, int store_fp32, int* shrt, unsigned* err,
                           cudaStream_t st, const int* only = nullptr);
 // Jastrow parameter derivatives (k_wavefunction.cu): for P = 4 + n_nuc +
 // n_nuc n3 parameters (a_anti, a_par, b_ee, b_en, a_en[], c3[][]),
