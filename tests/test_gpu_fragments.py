@@ -87,3 +87,22 @@ def test_forces(m, D, path, monkeypatch):
     g.close()
     for c, ref in enumerate(O.Oracle(s).forces(R)):   # E_L, ln|psi|
         close(pw[:, c], ref, 1e-10)
+
+
+def test_forces_some_walkers(monkeypatch):
+    """More than a chunk of walkers, every third of them with the electrons shared out unevenly, spins of different size."""
+    from paper_2504_07948_gb300 import qmc as Q
+    monkeypatch.setenv("QMC_FORCE_GEMM_MIN_N", "1")
+    m, D = 3, 16.0
+    s = fragments(m, D)
+    s.n_dn -= 3
+    s.occ_dn = s.occ_dn[:s.n_dn]
+    few, even = walkers(m, D, 4)[:, :-3], walkers(m, D, 8, seed=7)[:, :-3]
+    even[:, 0, 0] -= D
+    R = np.stack([few, even[:4], even[4:]], 1).reshape(12, -1, 3)
+    g = Q.QMC(s, precision="fp64")
+    g.set_walkers(np.tile(R, (27, 1, 1)))
+    pw = g.forces()[1]
+    g.close()
+    for c, ref in enumerate(O.Oracle(s).forces(R)):
+        close(pw[:, c], np.tile(ref, (27, 1, 1)), 1e-10)
