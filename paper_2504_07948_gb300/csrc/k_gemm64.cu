@@ -33,7 +33,7 @@
 //
 // 32-water forces in FP64, 256 walkers (four products per spin, n = 160): with
 // cuBLAS DGEMM 46.6 ms of a 53.7 ms pass; with this kernel the pass takes
-// 10.4 ms, of which its products 3.2 and the digits 0.8 (the rest is FP64 pair
+// 10.5 ms, of which its products 3.2 and the digits 0.8 (the rest is FP64 pair
 // and basis terms).
 //
 // Roles of a CTA (one per SM, persistent over the tiles): warp 0 issues the

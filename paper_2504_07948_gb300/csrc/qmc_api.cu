@@ -902,7 +902,7 @@ struct qmc_ctx {
             QMC_CK(launch_orbitals_all<double>(ds, k, W, stream));
         }
         QMC_CK(launch_invert(ds, k, W, mode == QMC_MIXED, mode == QMC_MIXED && fresh ? nullptr : d_short, d_err, stream));
-        int nk = mode == QMC_MIXED && fresh ? 2 : 3;   // (a basis beyond the lists takes two)
+        int nk = mode == QMC_MIXED && fresh ? 2 : 3;   // (two for a basis too large for the lists)
         if (ds.msd) {
             if (mode == QMC_MIXED) {
                 QMC_CK(launch_msd_table<float>(ds, k, W, stream));
